@@ -88,7 +88,10 @@ typedef struct {
  *  prec          : bm_precision (default BM_FP64).
  *  refine_tol    : backward-error target of refinement (default 1e-9).
  *  refine_maxit  : refinement iteration cap (default 30).
- *  nb            : outer LU block size, a multiple of 32 in [32, 256] (0 = library default).
+ *  nb            : outer LU block size, a multiple of 32 in [32, 256] (0 = library default).  The CF32
+ *     precisions' default factors blocks of 128 columns without a pivot search, checks every candidate
+ *     against its pivot and continues with the search from the first block that needs an interchange
+ *     (the same pivots); a block size or a panel setting below asks for the search from the start.
  *  refine_residual: how refinement forms r = b - A x (bm_refine_residual):
  *     BM_RESID_TC_UPDATE (0, default): the first residual from exact integer products on the
  *        tensor cores - A (once, after assembly) and x split into seven base-128 digits per row /
@@ -432,7 +435,9 @@ bm_status bm_enqueue_probe(bm_ctx* ctx, int which, int reps);
  * launched directly (no graph replay) and each launch bracketed by two events on the handle's
  * stream, and reports the launches grouped by kernel name: count and summed device time.  The
  * factors and X are those of a normal call; the times add up to the serial device time of the two
- * calls (kernels that a normal call overlaps are timed one after another here).
+ * calls (kernels that a normal call overlaps are timed one after another here).  The FP32
+ * factorisation's panel eliminations are one group, panel_lc_kernel, whether they ran with or
+ * without the pivot search.
  *  out: cap entries (may be NULL to query the count); *count receives the number of groups.
  * Errors: those of bm_factor and bm_solve. */
 typedef struct {

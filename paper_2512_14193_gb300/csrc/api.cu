@@ -199,6 +199,7 @@ void free_problem(bm_ctx* c) {
     FREE(c->d_Up_i);
     FREE(c->d_Cp_r);
     FREE(c->d_Cp_i);
+    FREE(c->d_fd);
     for (int q = 0; q < 2; ++q) {
         FREE(c->d_dg[q]);
         FREE(c->d_dge[q]);
@@ -246,9 +247,12 @@ Plan make_plan(int N, int form, int prec, int nb_user, int bs, int nd) {
             p.ldk_c = round_up(split ? 3L * N : (long)N, 32);
             b += 2 * (size_t)N * p.ldk_c * 8;
         }
+        // packs of the trailing updates (the search-free blocks always take 3xTF32 products) and the
+        // search-free blocks' work buffer
         long kl = split ? 3L * p.nb : p.nb;
-        p.ldk_lu = round_up(kl, 32);
+        p.ldk_lu = round_up(nb_user > 0 ? kl : std::max(kl, 3L * 128), 32);
         b += 2 * (size_t)p.n * p.ldk_lu * 8;
+        if (nb_user == 0) b += lu_fast_bytes(p.n);
         // digit planes of the operator for the tensor-core residual, their row exponents, and the
         // row-maximum scratch of their construction
         const size_t planes = (size_t)rt_digit_planes(nd) * 2;
@@ -525,8 +529,11 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
     // Same shape as the assembled system: assemble again into the same buffers (no device
     // allocation or release - cudaFree would wait for every stream of the device - and the cached
     // graphs and tensor maps stay valid, as they depend only on these pointers and sizes).
+    // LU in search-free blocks, unless a block size or a panel setting asks for the panels (the contour
+    // solver's deferred assembly sets a cluster size for what its factorisations continue with)
+    const bool fast = prec != BM_FP64 && nb == 0 && pkern == 0 && (cl_cap == 0 || defer_kernels);
     const bool reuse = c->assembled && c->N == N && c->form == form && c->prec == prec && c->nb == p.nb &&
-                       c->rt_nd == nd && curve->kind != BM_CURVE_USER;
+                       (c->d_fd != nullptr) == fast && c->rt_nd == nd && curve->kind != BM_CURVE_USER;
     if (!reuse) free_problem(c);
     // the captured factorisation depends on the launch settings: capture again when they change
     if (reuse && (eager != c->eager || cl_cap != c->opt_cluster_cap || pkern != c->opt_panel_kernel))
@@ -534,6 +541,7 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
     c->eager = eager;
     c->opt_cluster_cap = cl_cap;
     c->opt_panel_kernel = pkern;
+    c->lu_fast = fast;
     c->bs_solve = 64;
     if (!reuse && c->held + p.bytes > c->budget) {
         bm_set_error("admission: system needs " + std::to_string(p.bytes) + " bytes, budget leaves " +
@@ -605,6 +613,7 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
         if (s == BM_OK) s = alloc_t(c, &c->d_Lp_i, lb);
         if (s == BM_OK) s = alloc_t(c, &c->d_Up_r, lb);
         if (s == BM_OK) s = alloc_t(c, &c->d_Up_i, lb);
+        if (s == BM_OK && fast) s = alloc_t(c, &c->d_fd, lu_fast_bytes(p.n));
     }
     if (s == BM_OK && c32) {
         // [0] Mtop (2N x N) or A (2N x 2N), [1] Mbot (N x 2N)
@@ -764,6 +773,7 @@ namespace {
 bm_status factor_sequence(bm_ctx* c) {
     cudaStream_t s = c->stream;
     BM_CUDA_TRY(cudaMemsetAsync(c->d_info, 0, 2 * sizeof(int), s));
+    BM_CUDA_TRY(cudaMemsetAsync(c->d_info + 4, 0, sizeof(int), s));
     if (c->prec == BM_FP64) {
         Z64 F{c->d_F64, c->ldF};
         if (c->form == BM_MIXED) {
@@ -848,10 +858,26 @@ bm_status factor_lu_enqueue(bm_ctx* c) {
     return run_captured(c, &c->g_lu, [&]() -> bm_status { return lu_factor_enqueue(c); });
 }
 
-bm_status factor_result(bm_ctx* c, int* info) {
-    int h[2] = {0, 0};
-    BM_CUDA_TRY(cudaMemcpyAsync(h, c->d_info, 2 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+// Waits for the factorisation; when it stopped at a block (lu_fast.cu), enqueues the rest of it with
+// the pivot search.
+bm_status factor_continue(bm_ctx* c) {
+    if (!c->lu_fast) return BM_OK;
+    int h[5] = {0, 0, 0, 0, 0};
+    BM_CUDA_TRY(cudaMemcpyAsync(h, c->d_info, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
     BM_CUDA_TRY(cudaStreamSynchronize(c->stream));
+    if (h[1] != 0 || h[4] == 0) return BM_OK;
+    return lu_resume_enqueue(c, h[4]);
+}
+
+bm_status factor_result(bm_ctx* c, int* info) {
+    int h[5] = {0, 0, 0, 0, 0};
+    BM_CUDA_TRY(cudaMemcpyAsync(h, c->d_info, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
+    BM_CUDA_TRY(cudaStreamSynchronize(c->stream));
+    if (c->lu_fast && h[1] == 0 && h[4] != 0) {
+        BM_TRY(lu_resume_enqueue(c, h[4]));
+        BM_CUDA_TRY(cudaMemcpyAsync(h, c->d_info, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
+        BM_CUDA_TRY(cudaStreamSynchronize(c->stream));
+    }
     if (info) *info = h[0];
     if (h[1] != 0) {
         bm_set_error("factorisation: a bounded device-side wait timed out");
@@ -884,22 +910,7 @@ extern "C" bm_status bm_factor(bm_ctx* c, int* info) {
     }
     BM_CUDA_TRY(cudaSetDevice(c->device));
     BM_TRY(run_captured(c, &c->g_factor, [&]() { return factor_sequence(c); }));
-    int h[2] = {0, 0};
-    BM_CUDA_TRY(cudaMemcpyAsync(h, c->d_info, 2 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    BM_CUDA_TRY(cudaStreamSynchronize(c->stream));
-    if (h[1] != 0) {
-        bm_set_error("factorisation: a bounded device-side wait timed out");
-        c->factored = false;
-        return BM_ETIMEOUT;
-    }
-    c->factored = true;
-    c->singular = h[0] != 0;
-    if (info) *info = h[0];
-    if (c->singular) {
-        bm_set_error("zero pivot in column " + std::to_string(h[0]));
-        return BM_ESINGULAR;
-    }
-    return BM_OK;
+    return factor_result(c, info);
 }
 
 // ------------------------------------------------------------------------------------------------

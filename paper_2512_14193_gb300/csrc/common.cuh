@@ -291,7 +291,9 @@ struct bm_ctx {
     int* d_ipiv = nullptr;
     int* d_perm = nullptr;
     int* d_info = nullptr;
-    int* d_err = nullptr;
+    int* d_err = nullptr;      // d_info + 1; d_info[2..3] test hooks, d_info[4] stop word of lu_fast.cu
+    bool lu_fast = false;      // FP32 LU in blocks without a pivot search (lu_fast.cu) and their
+    float* d_fd = nullptr;     //   work buffer: the default, unless bm_opts.nb or panel_kernel is set
     void* d_maps = nullptr;    // row-interchange maps used by the factorisation: big panel (even),
                                // sub-panel, big panel (odd)
     // look-ahead of the FP32 factorisation: the panel chain on la_hi (high priority), the rest of

@@ -396,7 +396,12 @@ __global__ void __launch_bounds__(192, 1)
     cgemm_tc_kernel(const __grid_constant__ CUtensorMap tmAr, const __grid_constant__ CUtensorMap tmAi,
                     const __grid_constant__ CUtensorMap tmBr, const __grid_constant__ CUtensorMap tmBi,
                     float* __restrict__ Cr, float* __restrict__ Ci, double2* __restrict__ C64, long ldc, long zstride,
-                    int m, int n, int kext, int S, float alpha, float beta, int* __restrict__ err) {
+                    int m, int n, int kext, int S, float alpha, float beta, int* __restrict__ err, TcGate gate) {
+    if (gate.first_tile && blockIdx.x == 0 && blockIdx.y == 0) return;
+    if (gate.fail) {  // a factorisation that stopped before this product's block (lu_fast.cu)
+        const int f = *reinterpret_cast<const volatile int*>(gate.fail);
+        if (f != 0 && (f >> 1) <= gate.block) return;
+    }
     cgemm_tc_body<OUT>(tmAr, tmAi, tmBr, tmBi, Cr, Ci, C64, ldc, zstride, m, n, kext, S, (int)blockIdx.z, alpha, beta,
                        err);
 }
@@ -462,7 +467,7 @@ namespace {
 template <int OUT>
 cudaError_t launch_tc(cudaStream_t s, dim3 grid, const void* tAr, const void* tAi, const void* tBr, const void* tBi,
                       float* Cr, float* Ci, double2* C64, long ldc, long zstride, int m, int n, int kext, int S,
-                      float alpha, float beta, int* d_err) {
+                      float alpha, float beta, int* d_err, TcGate gate = TcGate{}) {
     static DeviceFlags attr_set;
     if (attr_set.pending()) {
         cudaError_t e =
@@ -473,7 +478,7 @@ cudaError_t launch_tc(cudaStream_t s, dim3 grid, const void* tAr, const void* tA
     cgemm_tc_kernel<OUT><<<grid, tc_threads<OUT>(), SMEM_BYTES, s>>>(
         *reinterpret_cast<const CUtensorMap*>(tAr), *reinterpret_cast<const CUtensorMap*>(tAi),
         *reinterpret_cast<const CUtensorMap*>(tBr), *reinterpret_cast<const CUtensorMap*>(tBi), Cr, Ci, C64, ldc,
-        zstride, m, n, kext, S, alpha, beta, d_err);
+        zstride, m, n, kext, S, alpha, beta, d_err, gate);
     return cudaGetLastError();
 }
 
@@ -551,14 +556,14 @@ __global__ void pack_b_kernel(const float* __restrict__ Vr, const float* __restr
 
 // C = beta C + alpha A B^T, C FP32 planar column-major (m x n, ld ldc); one K range per CTA.
 cudaError_t gemm_tc(cudaStream_t s, const void* tAr, const void* tAi, const void* tBr, const void* tBi, float* Cr,
-                    float* Ci, long ldc, int m, int n, int kext, float alpha, float beta, int* d_err) {
+                    float* Ci, long ldc, int m, int n, int kext, float alpha, float beta, int* d_err, TcGate gate) {
     if (m <= 0 || n <= 0 || kext <= 0) return cudaSuccess;
     dim3 grid(ceil_div(m, BM), ceil_div(n, BN), 1);
     if (beta != 0.f)
         return launch_tc<OUT_C32_PRE>(s, grid, tAr, tAi, tBr, tBi, Cr, Ci, nullptr, ldc, 0, m, n, kext, 1, alpha,
-                                      beta, d_err);
+                                      beta, d_err, gate);
     return launch_tc<OUT_C32>(s, grid, tAr, tAi, tBr, tBi, Cr, Ci, nullptr, ldc, 0, m, n, kext, 1, alpha, beta,
-                              d_err);
+                              d_err, gate);
 }
 
 // Number of K splits for a product with few output tiles: about three waves of CTAs over the

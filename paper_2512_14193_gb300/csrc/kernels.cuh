@@ -25,8 +25,16 @@ cudaError_t gemm_update_z64_c32(cudaStream_t s, int m, int n, int k, float alpha
 
 // gemm_tc.cu (tensor maps are CUtensorMap, passed as opaque 128-byte blobs)
 bm_status tc_make_map(void* tmap, const float* base, long rows, long kext, long ldk, int box_rows);
+// TcGate: the launch skips its first 128 x 128 tile (another launch takes it), and does nothing when the
+// word *fail, if any, names a block of the factorisation up to `block` (lu_fast.cu)
+struct TcGate {
+    const int* fail = nullptr;
+    int block = 0;
+    int first_tile = 0;
+};
 cudaError_t gemm_tc(cudaStream_t s, const void* tAr, const void* tAi, const void* tBr, const void* tBi, float* Cr,
-                    float* Ci, long ldc, int m, int n, int kext, float alpha, float beta, int* d_err);
+                    float* Ci, long ldc, int m, int n, int kext, float alpha, float beta, int* d_err,
+                    TcGate gate = TcGate{});
 constexpr int TC_BM = 128;
 constexpr int TC_BN = 128;
 // destination of a split-K product: FP32 planar (re, im) or, when z is set, FP64 interleaved
@@ -49,6 +57,9 @@ cudaError_t gemm_tc_batch(cudaStream_t s, int B, const void* const* maps, float*
 // lu.cu
 bm_status lu_setup(bm_ctx* c, int cluster_cap, int panel_kernel);
 bm_status lu_factor_enqueue(bm_ctx* c);       // factor d_F64 / d_F32 in place (stream-ordered)
+// continue a factorisation that stopped at a block (the value of its stop word) with the pivot search
+bm_status lu_resume_enqueue(bm_ctx* c, int stop);
+size_t lu_fast_bytes(int n);                  // work buffer of the search-free blocks (d_fd)
 size_t swap_map_bytes();
 bm_status getrs_z64(bm_ctx* c, double2* Y, long ldy, int nrhs);   // in place; Y holds P B (rows gathered by perm)
 bm_status getrs_c32(bm_ctx* c, float* Yr, float* Yi, long ldy, int nrhs);
@@ -121,5 +132,6 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
                         const bm_opts* opts, bool defer_kernels);
 bm_status assemble_post(bm_ctx* c, bool run_assembly_kernel, bool wait);  // wait: synchronise the stream
 bm_status factor_lu_enqueue(bm_ctx* c);              // LU of the Schur complement in place (graph)
+bm_status factor_continue(bm_ctx* c);                // waits; enqueues the rest of a factorisation that stopped
 bm_status factor_result(bm_ctx* c, int* info);       // waits, reads info / timeout, sets the state
 bm_status set_panel_cluster(bm_ctx* c, int cap);     // panel cluster cap of an assembled handle

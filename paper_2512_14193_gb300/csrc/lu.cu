@@ -38,12 +38,6 @@ using namespace lu_detail;
 
 namespace {
 
-__device__ __forceinline__ float tf32_rna(float x) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return __uint_as_float(r);
-}
-
 // Row interchanges (from a swap map) for columns in [a0, a1) u [b0, b1); for columns of the
 // second range also X = L11^{-1} X on rows [t0, t0+tb) with the unit-lower L11 at (t0, t0),
 // staged in shared memory: whole when it fits, else in chunks of ST_KC columns that the CTA's
@@ -308,9 +302,9 @@ __global__ void pack_L_kernel(C32 A, long r0, long c0, int m, int kb, int split,
     }
 }
 
-__global__ void iota_kernel(int* p, int n) {
+__global__ void iota_kernel(int* p, int* q, int n) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) p[i] = i;
+    if (i < n) p[i] = q[i] = i;
 }
 
 // A ROWS x COLS tile of view A at (r0, c0) into shared memory (column-major, leading dimension
@@ -357,9 +351,10 @@ __device__ __forceinline__ void load_block(CV* dst, const CV* __restrict__ src, 
 // Entries outside the rb x rb leading block are zero.
 constexpr int TI_B = 64;
 template <class V, bool UPPER, int CG>
-__global__ void __launch_bounds__(256) tri_inv_kernel(V F, int n, typename V::cv* __restrict__ out) {
+__global__ void __launch_bounds__(256) tri_inv_kernel(V F, int n, typename V::cv* __restrict__ out, const int* fail) {
     using CV = typename V::cv;
     using Rl = typename V::real;
+    if (*fail != 0) return;  // the factorisation stopped (lu_fast.cu) and is continued first
     // CG column groups (blockIdx.y): the columns of the inverse are independent, so the FP64
     // factors, whose pipe is slow on each SM, spread one block over CG CTAs
     constexpr int B = TI_B, M = B * B / 256 / CG;
@@ -514,12 +509,12 @@ __global__ void __launch_bounds__(256) trsv_step_kernel(V F, V Y, V Z, int r0, i
 // in place (each CTA reads its whole tile before writing it).  bs == TS_BM == 64.
 template <class V>
 __global__ void __launch_bounds__(256) g_form_kernel(V F, int n, const typename V::cv* __restrict__ dinvL,
-                                                     const typename V::cv* __restrict__ dinvU) {
+                                                     const typename V::cv* __restrict__ dinvU, const int* fail) {
     using CV = typename V::cv;
     using Rl = typename V::real;
     constexpr int B = TS_BM;
     const int it = blockIdx.x, b = blockIdx.y;
-    if (it == b) return;
+    if (it == b || *fail != 0) return;
     extern __shared__ __align__(16) unsigned char sm[];
     CV* Ft = reinterpret_cast<CV*>(sm);  // [B][B] column-major tile of F
     CV* Ts = Ft + B * B;                 // [B][B] column-major T_b
@@ -877,8 +872,109 @@ cudaError_t gemm_any(cudaStream_t s, int m, int n, int k, C32 A, C32 B, C32 C) {
     return gemm_c32(s, m, n, k, -1.0f, A, false, B, 1.0f, C);
 }
 
+// What the solves need besides the factors: the inverted diagonal blocks and (FP32) the G form.
 template <class V>
-bm_status factor_t(bm_ctx* c, V F, bool tc, int split) {
+bm_status finish_t(bm_ctx* c, V F, cudaStream_t s) {
+    const int n = c->n;
+    const int* const fail = c->d_info + 4;
+    const int bs = c->bs_solve;
+    if (bs != TI_B || bs != TS_BM) {
+        bm_set_error("lu: the solve block size must be 64");
+        return BM_EINVAL;
+    }
+    const int nblk = ceil_div(n, bs);
+    size_t smem = ((size_t)bs * bs + 3 * (size_t)bs) * sizeof(typename V::cv);
+    using CV = typename V::cv;
+    constexpr int CG = std::is_same<V, C32>::value ? 1 : 4;  // column groups per block (FP64: 4)
+    LU_CUDA(cudaFuncSetAttribute(tri_inv_kernel<V, false, CG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)smem));
+    LU_CUDA(cudaFuncSetAttribute(tri_inv_kernel<V, true, CG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)smem));
+    {
+        BM_PROF(c, "tri_inv_kernel");
+        tri_inv_kernel<V, false, CG><<<dim3(nblk, CG), 256, smem, s>>>(F, n, reinterpret_cast<CV*>(c->d_dinvL), fail);
+        tri_inv_kernel<V, true, CG><<<dim3(nblk, CG), 256, smem, s>>>(F, n, reinterpret_cast<CV*>(c->d_dinvU), fail);
+        LU_CUDA(cudaGetLastError());
+    }
+    if constexpr (std::is_same<V, C32>::value) {
+        if (nblk > 1) {
+            BM_PROF(c, "g_form_kernel");
+            const size_t gsm = 2 * (size_t)TS_BM * TS_BM * sizeof(CV);
+            LU_CUDA(cudaFuncSetAttribute(g_form_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm));
+            g_form_kernel<V><<<dim3(nblk, nblk), 256, gsm, s>>>(F, n, reinterpret_cast<const CV*>(c->d_dinvL),
+                                                                reinterpret_cast<const CV*>(c->d_dinvU), fail);
+            LU_CUDA(cudaGetLastError());
+        }
+    }
+    return BM_OK;
+}
+
+// The FP32 LU in blocks of FD_B columns without a pivot search (lu_fast.cu).  Two streams: the chain
+// diagonal block -> solves -> next diagonal block's tile, and the rest of each trailing update beside
+// the next diagonal block.
+bm_status factor_fast(bm_ctx* c, C32 F) {
+    const int n = c->n;
+    int* const fail = c->d_info + 4;
+    const bool la = !c->prof && n > 2 * FD_B && c->la_hi != nullptr;
+    cudaStream_t s = la ? c->la_hi : c->stream;
+    cudaStream_t s2 = c->la_lo;
+    cudaEvent_t ev_start = c->la_ev[0], ev_fork = c->la_ev[1], ev_join = c->la_ev[2], ev_done = c->la_ev[3];
+    if (la) {
+        LU_CUDA(cudaEventRecord(ev_start, c->stream));
+        LU_CUDA(cudaStreamWaitEvent(s, ev_start, 0));
+    }
+    {
+        BM_PROF(c, "iota");
+        iota_kernel<<<ceil_div(n, 256), 256, 0, s>>>(c->d_perm, c->d_ipiv, n);
+        LU_CUDA(cudaGetLastError());
+    }
+    float* const packs[4] = {c->d_Lp_r, c->d_Lp_i, c->d_Up_r, c->d_Up_i};
+    bool rest = false;  // a trailing update is under way on s2
+    for (int J = 0; J < n; J += FD_B) {
+        const int db = std::min(FD_B, n - J), mm = n - J - db;
+        {
+            // (the profile keeps one name for the kernels that eliminate the panels)
+            BM_PROF(c, "panel_lc_kernel");
+            LU_CUDA(launch_lu_diag(s, F, J, db, c->d_fd, fail));
+        }
+        if (rest) LU_CUDA(cudaStreamWaitEvent(s, ev_join, 0));
+        {
+            BM_PROF(c, "lu_trsm_kernel");
+            LU_CUDA(launch_lu_trsm(s, F, J, db, mm, c->d_fd, n, packs, c->ldk_lu, c->num_sms, fail));
+        }
+        rest = false;
+        if (mm == 0) break;
+        BM_PROF(c, "cgemm_tc_kernel (trailing update)");
+        const C32 C = F.sub(J + FD_B, J + FD_B);
+        TcGate gate{fail, J + 1, 0};
+        auto update = [&](cudaStream_t st, int m) {
+            return gemm_tc(st, c->tm_lu[0], c->tm_lu[1], c->tm_lu[2], c->tm_lu[3], C.re, C.im, C.ld, m, m, 3 * FD_B, -1.0f,
+                           1.0f, c->d_err, gate);
+        };
+        if (!la || mm <= FD_B) {
+            LU_CUDA(update(s, mm));
+            continue;
+        }
+        LU_CUDA(cudaEventRecord(ev_fork, s));
+        LU_CUDA(update(s, FD_B));
+        LU_CUDA(cudaStreamWaitEvent(s2, ev_fork, 0));
+        gate.first_tile = 1;
+        LU_CUDA(update(s2, mm));
+        LU_CUDA(cudaEventRecord(ev_join, s2));
+        rest = true;
+    }
+    BM_TRY(finish_t<C32>(c, F, s));
+    if (la) {  // join the handle's stream
+        LU_CUDA(cudaEventRecord(ev_done, s));
+        LU_CUDA(cudaStreamWaitEvent(c->stream, ev_done, 0));
+    }
+    return BM_OK;
+}
+
+// The LU with the pivot search, from column J0 on (the columns before it are factored, their
+// interchanges and trailing updates applied).
+template <class V>
+bm_status factor_t(bm_ctx* c, V F, bool tc, int split, int J0 = 0) {
     const int n = c->n;
     const int NB = c->nb;
     const int cl_max = c->panel_cluster;
@@ -888,7 +984,7 @@ bm_status factor_t(bm_ctx* c, V F, bool tc, int split) {
     // U12 solve and trailing update of the next big panel's columns run first on the high-priority
     // stream, which then factors that panel while the low-priority stream finishes the rest of the
     // trailing update; the next block step waits for it.  Profiling keeps the serial order.
-    const bool la = std::is_same<V, C32>::value && tc && !c->prof && n > 2 * NB && c->la_hi != nullptr;
+    const bool la = std::is_same<V, C32>::value && tc && !c->prof && n - J0 > 2 * NB && c->la_hi != nullptr;
     cudaStream_t s = la ? c->la_hi : c->stream;
     cudaStream_t s2 = c->la_lo;
     cudaEvent_t ev_start = c->la_ev[0], ev_fork = c->la_ev[1], ev_join = c->la_ev[2], ev_done = c->la_ev[3];
@@ -897,12 +993,12 @@ bm_status factor_t(bm_ctx* c, V F, bool tc, int split) {
         LU_CUDA(cudaStreamWaitEvent(s, ev_start, 0));
         LU_CUDA(cudaStreamWaitEvent(s2, ev_start, 0));
     }
-    {
+    if (J0 == 0) {
         BM_PROF(c, "iota");
-        iota_kernel<<<ceil_div(n, 256), 256, 0, s>>>(c->d_perm, n);
+        iota_kernel<<<ceil_div(n, 256), 256, 0, s>>>(c->d_perm, c->d_ipiv, n);
         LU_CUDA(cudaGetLastError());
     }
-    for (int J = 0, blk = 0; J < n; J += NB, ++blk) {
+    for (int J = J0, blk = 0; J < n; J += NB, ++blk) {
         const int jb = std::min(NB, n - J);
         SwapMap* const d_map = (blk & 1) ? maps + 2 : maps;  // this big panel's map (two in flight)
         for (int j = J; j < J + jb;) {
@@ -992,36 +1088,7 @@ bm_status factor_t(bm_ctx* c, V F, bool tc, int split) {
         }
     }
     if (la) LU_CUDA(cudaStreamWaitEvent(s, ev_join, 0));
-    // inverted diagonal blocks for getrs
-    const int bs = c->bs_solve;
-    if (bs != TI_B || bs != TS_BM) {
-        bm_set_error("lu: the solve block size must be 64");
-        return BM_EINVAL;
-    }
-    const int nblk = ceil_div(n, bs);
-    size_t smem = ((size_t)bs * bs + 3 * (size_t)bs) * sizeof(typename V::cv);
-    using CV = typename V::cv;
-    constexpr int CG = std::is_same<V, C32>::value ? 1 : 4;  // column groups per block (FP64: 4)
-    LU_CUDA(cudaFuncSetAttribute(tri_inv_kernel<V, false, CG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem));
-    LU_CUDA(cudaFuncSetAttribute(tri_inv_kernel<V, true, CG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem));
-    {
-        BM_PROF(c, "tri_inv_kernel");
-        tri_inv_kernel<V, false, CG><<<dim3(nblk, CG), 256, smem, s>>>(F, n, reinterpret_cast<CV*>(c->d_dinvL));
-        tri_inv_kernel<V, true, CG><<<dim3(nblk, CG), 256, smem, s>>>(F, n, reinterpret_cast<CV*>(c->d_dinvU));
-        LU_CUDA(cudaGetLastError());
-    }
-    if constexpr (std::is_same<V, C32>::value) {
-        if (nblk > 1) {
-            BM_PROF(c, "g_form_kernel");
-            const size_t gsm = 2 * (size_t)TS_BM * TS_BM * sizeof(CV);
-            LU_CUDA(cudaFuncSetAttribute(g_form_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm));
-            g_form_kernel<V><<<dim3(nblk, nblk), 256, gsm, s>>>(F, n, reinterpret_cast<const CV*>(c->d_dinvL),
-                                                                reinterpret_cast<const CV*>(c->d_dinvU));
-            LU_CUDA(cudaGetLastError());
-        }
-    }
+    BM_TRY(finish_t<V>(c, F, s));
     if (la) {  // join the handle's stream
         LU_CUDA(cudaEventRecord(ev_done, s));
         LU_CUDA(cudaStreamWaitEvent(c->stream, ev_done, 0));
@@ -1216,8 +1283,19 @@ bm_status lu_factor_enqueue(bm_ctx* c) {
         return factor_t<Z64>(c, F, false, 0);
     }
     C32 F{c->d_F32r, c->d_F32i, c->ldF};
+    if (c->lu_fast) return factor_fast(c, F);
     return factor_t<C32>(c, F, true, c->prec == BM_CF32_3XTF32_IR ? 1 : 0);
 }
+
+bm_status lu_resume_enqueue(bm_ctx* c, int stop) {
+    C32 F{c->d_F32r, c->d_F32i, c->ldF};
+    const int J = (stop >> 1) - 1, db = std::min(FD_B, c->n - J);
+    LU_CUDA(cudaMemsetAsync(c->d_info + 4, 0, sizeof(int), c->stream));
+    if (stop & 1) LU_CUDA(launch_lu_restore(c->stream, F, J, db, c->n - J - db, c->d_fd, c->n));
+    return factor_t<C32>(c, F, true, c->prec == BM_CF32_3XTF32_IR ? 1 : 0, J);
+}
+
+size_t lu_fast_bytes(int n) { return fd_work_floats(n) * sizeof(float); }
 
 // Y holds P B already (rows gathered with d_perm); solves L U X = Y in place.
 bm_status getrs_z64(bm_ctx* c, double2* Y, long ldy, int nrhs) {

@@ -180,6 +180,28 @@ __device__ __forceinline__ float2 cinv_rcp(float2 a) {
     return make_float2(r * id, -id);
 }
 
+// 1 / a for a != 0: a is scaled by a power of two (exact) to |a|_inf in [1, 2), and
+// conj(a) / |a|^2 uses one hardware reciprocal refined by a Newton step (a few ulps, no overflow or
+// underflow for any finite a).
+__device__ __forceinline__ float2 cinv_fast(float2 a) {
+    const float s = fmaxf(fabsf(a.x), fabsf(a.y));
+    const int eb = min(max((int)((__float_as_uint(s) >> 23) & 0xff), 1), 253);  // biased exponent
+    const float sc = __uint_as_float((uint32_t)(254 - eb) << 23);                  // 2^-(eb - 127)
+    const float x = a.x * sc, y = a.y * sc;
+    const float d = fmaf(x, x, y * y);
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    r = r * fmaf(-d, r, 2.f);
+    const float rs = r * sc;
+    return make_float2(x * rs, -y * rs);
+}
+
+__device__ __forceinline__ float tf32_rna(float x) {
+    uint32_t r;
+    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
+    return __uint_as_float(r);
+}
+
 // ------------------------------------------------------------------------------------------------
 // panel factorisation
 // ------------------------------------------------------------------------------------------------
@@ -493,6 +515,30 @@ cudaError_t launch_panel(cudaStream_t s, C32 A, const PanelShape& ps, int j0, in
 cudaError_t launch_panel(cudaStream_t s, Z64 A, const PanelShape& ps, int j0, int m, int ib, int* ipiv, int* info,
                          int J, int jb, SwapMap* mi, SwapMap* mb, int* perm);
 int query_cluster_max_c32();
+
+// lu_fast.cu: blocks of FD_B columns whose pivots stay on the diagonal.  The work buffer holds the
+// factors of the current diagonal block (FdT) and what lu_trsm_kernel overwrote (FdBackup).
+constexpr int FD_B = 128, FD_PITCH = 132;
+constexpr long FD_T = 4L * FD_B * FD_PITCH + 4L * FD_B;
+struct FdT {
+    float *Ur, *Ui, *Lr, *Li;  // strict upper triangles of U and L^T, rows [p][k] of pitch FD_PITCH
+    float2 *inv, *piv;         // 1 / u_kk, u_kk
+    BM_HD explicit FdT(float* w)
+        : Ur(w), Ui(w + FD_B * FD_PITCH), Lr(w + 2 * FD_B * FD_PITCH), Li(w + 3 * FD_B * FD_PITCH),
+          inv(reinterpret_cast<float2*>(w + 4 * FD_B * FD_PITCH)),
+          piv(reinterpret_cast<float2*>(w + 4 * FD_B * FD_PITCH + 2 * FD_B)) {}
+};
+struct FdBackup {
+    float *Dr, *Di, *Lr, *Li, *Ur, *Ui;  // diagonal block; A21 (column-major, ld n); A12 (ld FD_B)
+    BM_HD FdBackup(float* w, long n)
+        : Dr(w), Di(w + FD_B * FD_B), Lr(w + 2 * FD_B * FD_B), Li(Lr + n * FD_B), Ur(Li + n * FD_B),
+          Ui(Ur + n * FD_B) {}
+};
+inline size_t fd_work_floats(long n) { return (size_t)FD_T + 2 * FD_B * FD_B + 4 * (size_t)n * FD_B; }
+cudaError_t launch_lu_diag(cudaStream_t s, C32 F, int J, int db, float* work, int* fail);
+cudaError_t launch_lu_trsm(cudaStream_t s, C32 F, int J, int db, int mm, float* work, long n, float* const* packs,
+                           long ldk, int num_sms, int* fail);
+cudaError_t launch_lu_restore(cudaStream_t s, C32 F, int J, int db, int mm, float* work, long n);
 int query_cluster_max_z64();
 
 }  // namespace lu_detail

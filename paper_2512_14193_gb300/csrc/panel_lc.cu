@@ -55,22 +55,6 @@ __device__ __forceinline__ u64 mul2(u64 a, u64 b) {
     return d;
 }
 
-// 1 / a for a != 0: a is scaled by a power of two (exact) to |a|_inf in [1, 2), and
-// conj(a) / |a|^2 uses one hardware reciprocal refined by a Newton step (a few ulps, no overflow or
-// underflow for any finite a).
-__device__ __forceinline__ float2 cinv_fast(float2 a) {
-    const float s = fmaxf(fabsf(a.x), fabsf(a.y));
-    const int eb = min(max((int)((__float_as_uint(s) >> 23) & 0xff), 1), 253);  // biased exponent
-    const float sc = __uint_as_float((uint32_t)(254 - eb) << 23);                  // 2^-(eb - 127)
-    const float x = a.x * sc, y = a.y * sc;
-    const float d = fmaf(x, x, y * y);
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
-    r = r * fmaf(-d, r, 2.f);
-    const float rs = r * sc;
-    return make_float2(x * rs, -y * rs);
-}
-
 // ------------------------------------------------------------------------------------------------
 // Net effect of the interchanges (a_k <-> p_k), k = 0 .. nk-1 in order, with a_k = base + k and
 // p_k >= a_k: the map new[dst] = old[src] over the rows they touch.  Row a_k is never touched after

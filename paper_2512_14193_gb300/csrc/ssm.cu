@@ -216,7 +216,10 @@ bm_status factor_batch(Batch& bt, int B) {
     bm_ctx* c0 = bt.h[0];
     const int N = c0->N;
     // the pivot / timeout words of every point, cleared ahead of everything that may set them
-    for (int b = 0; b < B; ++b) SSM_CUDA(cudaMemsetAsync(bt.h[b]->d_info, 0, 2 * sizeof(int), bt.s0));
+    for (int b = 0; b < B; ++b) {
+        SSM_CUDA(cudaMemsetAsync(bt.h[b]->d_info, 0, 2 * sizeof(int), bt.s0));
+        SSM_CUDA(cudaMemsetAsync(bt.h[b]->d_info + 4, 0, sizeof(int), bt.s0));
+    }
     SSM_CUDA(cudaEventRecord(bt.ev, bt.s0));
     for (int b = 0; b < B; ++b) SSM_CUDA(cudaStreamWaitEvent(bt.h[b]->stream, bt.ev, 0));
     if (c0->form == BM_MIXED && c0->prec != BM_FP64) {
@@ -252,6 +255,8 @@ bm_status factor_batch(Batch& bt, int B) {
         }
     }
     for (int b = 0; b < B; ++b) BM_TRY(factor_lu_enqueue(bt.h[b]));
+    // points that stopped at an interchange continue on their own streams, side by side
+    for (int b = 0; b < B; ++b) BM_TRY(factor_continue(bt.h[b]));
     for (int b = 0; b < B; ++b) {
         int info = 0;
         bm_status st = factor_result(bt.h[b], &info);
