@@ -940,7 +940,7 @@ bm_status factor_fast(bm_ctx* c, C32 F) {
         if (rest) LU_CUDA(cudaStreamWaitEvent(s, ev_join, 0));
         {
             BM_PROF(c, "lu_trsm_kernel");
-            LU_CUDA(launch_lu_trsm(s, F, J, db, mm, c->d_fd, n, packs, c->ldk_lu, c->num_sms, fail));
+            LU_CUDA(launch_lu_trsm(s, F, J, db, mm, c->d_fd, n, packs, c->ldk_lu, fail));
         }
         rest = false;
         if (mm == 0) break;

@@ -21,53 +21,72 @@
 namespace lu_detail {
 namespace {
 
-constexpr int B = FD_B, PITCH = FD_PITCH, W = 16;  // block, row pitch of the shared block, sub-step width
+constexpr int B = FD_B, PITCH = FD_PITCH, W = FD_W;  // block, row pitch of the shared block, sub-step
 constexpr int DT = 512;                            // threads of lu_diag_kernel
+
+// 1 / a for a != 0, as cinv_fast without its scaling where |a|^2 neither over- nor underflows
+__device__ __forceinline__ float2 cinv_near(float2 a) {
+    const float d = fmaf(a.x, a.x, a.y * a.y);
+    if (!(d > 1e-30f && d < 1e30f)) return cinv_fast(a);
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    r = r * fmaf(-d, r, 2.f);
+    return make_float2(a.x * r, -a.y * r);
+}
+__device__ __forceinline__ float2 shfl2(float2 v, int l) {
+    return make_float2(__shfl_sync(0xffffffffu, v.x, l), __shfl_sync(0xffffffffu, v.y, l));
+}
+// a - b c
+__device__ __forceinline__ float2 csubmul(float2 a, float2 b, float2 c) {
+    return make_float2(fmaf(-b.x, c.x, fmaf(b.y, c.y, a.x)), fmaf(-b.x, c.y, fmaf(-b.y, c.x, a.y)));
+}
 
 // Eliminates the 16 x 16 diagonal block at (c0, c0) of the shared block without interchanges: one
 // warp, lane = row (lanes 16-31 repeat lanes 0-15), the row in registers.  Returns false if a
-// candidate exceeds its pivot.  The chain per column is the pivot's broadcast, its reciprocal and one
-// multiply-add (about 90 cycles); sixteen columns keep the unrolled code small.
-__device__ __forceinline__ bool diag16(float* Sr, float* Si, int c0, float2* inv_s, float* thr_s) {
+// candidate exceeds its pivot.  The chain per column is one reciprocal: every lane forms the next
+// pivot itself from entries shuffled before the reciprocal is known (333 -> 110 cycles per column
+// against broadcasting the updated pivot).  Sixteen columns keep the unrolled code small.
+__device__ __forceinline__ bool diag16(float* Sr, float* Si, int c0, float2* inv_s, float2* piv_s) {
     const int lane = threadIdx.x & 31, r = lane & 15;
-    float ar[W], ai[W];
+    float2 x[W];
     float* pr = Sr + (c0 + r) * PITCH + c0;
     float* pi = Si + (c0 + r) * PITCH + c0;
 #pragma unroll
     for (int k = 0; k < W; k += 4) {
-        const float4 x = *reinterpret_cast<const float4*>(pr + k), y = *reinterpret_cast<const float4*>(pi + k);
-        ar[k] = x.x, ar[k + 1] = x.y, ar[k + 2] = x.z, ar[k + 3] = x.w;
-        ai[k] = y.x, ai[k + 1] = y.y, ai[k + 2] = y.z, ai[k + 3] = y.w;
+        const float4 u = *reinterpret_cast<const float4*>(pr + k), v = *reinterpret_cast<const float4*>(pi + k);
+        x[k] = make_float2(u.x, v.x);
+        x[k + 1] = make_float2(u.y, v.y);
+        x[k + 2] = make_float2(u.z, v.z);
+        x[k + 3] = make_float2(u.w, v.w);
     }
     bool ok = true;
+    float2 p = shfl2(x[0], 0);
+    float2 iv = cinv_near(p);
 #pragma unroll
     for (int c = 0; c < W; ++c) {
-        const float2 u = make_float2(__shfl_sync(0xffffffffu, ar[c], c), __shfl_sync(0xffffffffu, ai[c], c));
-        const float un = cnorm1(u);
-        const float2 iv = cinv_fast(u);
+        const float un = cnorm1(p);
         const bool below = r > c;
-        ok = ok && un > 0.f && (!below || cnorm1(make_float2(ar[c], ai[c])) <= un);
+        ok = ok && un > 0.f && (!below || cnorm1(x[c]) <= un);
         if (lane == c) {
             inv_s[c0 + c] = iv;
-            thr_s[c0 + c] = un;
+            piv_s[c0 + c] = p;
         }
-        const float2 l = below ? cmul(make_float2(ar[c], ai[c]), iv) : make_float2(0.f, 0.f);
+        if (c + 1 < W) {
+            const float2 ul = shfl2(x[c + 1], c), a0 = shfl2(x[c], c + 1), a1 = shfl2(x[c + 1], c + 1);
+            p = csubmul(a1, cmul(a0, iv), ul);  // the next pivot
+            const float2 l = below ? cmul(x[c], iv) : make_float2(0.f, 0.f);
+            iv = cinv_near(p);
+            x[c + 1] = csubmul(x[c + 1], l, ul);
 #pragma unroll
-        for (int k = c + 1; k < W; ++k) {
-            const float ur = __shfl_sync(0xffffffffu, ar[k], c), ui = __shfl_sync(0xffffffffu, ai[k], c);
-            ar[k] = fmaf(-l.x, ur, fmaf(l.y, ui, ar[k]));
-            ai[k] = fmaf(-l.x, ui, fmaf(-l.y, ur, ai[k]));
-        }
-        if (below) {
-            ar[c] = l.x;
-            ai[c] = l.y;
+            for (int k = c + 2; k < W; ++k) x[k] = csubmul(x[k], l, shfl2(x[k], c));
+            if (below) x[c] = l;
         }
     }
     if (lane < W) {
 #pragma unroll
         for (int k = 0; k < W; k += 4) {
-            *reinterpret_cast<float4*>(pr + k) = make_float4(ar[k], ar[k + 1], ar[k + 2], ar[k + 3]);
-            *reinterpret_cast<float4*>(pi + k) = make_float4(ai[k], ai[k + 1], ai[k + 2], ai[k + 3]);
+            *reinterpret_cast<float4*>(pr + k) = make_float4(x[k].x, x[k + 1].x, x[k + 2].x, x[k + 3].x);
+            *reinterpret_cast<float4*>(pi + k) = make_float4(x[k].y, x[k + 1].y, x[k + 2].y, x[k + 3].y);
         }
     }
     __syncwarp();
@@ -79,12 +98,11 @@ __device__ __forceinline__ bool diag16(float* Sr, float* Si, int c0, float2* inv
 // thread, then the rest takes the rank-16 update (a warp per 16 x 32 tile, 4 x 4 per thread) while warp
 // 0 updates and eliminates the next 16 x 16 block.  One SM's FP32 rate bounds the early sub-steps
 // (18k cycles of updates in all), the elimination chain the late ones.  The factors go to T for
-// lu_trsm_kernel, which also writes them to the matrix: U's and L^T's strict upper triangles as rows
-// [p][k], pitch 132, then the reciprocal pivots and the pivots' magnitudes.
+// lu_trsm_kernel, which also writes them to the matrix: U and L^T as packed rows of 16-row blocks with
+// the 16 x 16 diagonal blocks inverted, and both as they are (see FdT).
 __global__ void __launch_bounds__(DT, 1) lu_diag_kernel(C32 F, int J, int db, float* __restrict__ T, int* fail) {
     extern __shared__ __align__(16) float sm[];
-    __shared__ float2 inv_s[B];
-    __shared__ float thr_s[B];
+    __shared__ float2 inv_s[B], piv_s[B];
     __shared__ int bad;
     float* Sr = sm;
     float* Si = sm + B * PITCH;
@@ -94,7 +112,7 @@ __global__ void __launch_bounds__(DT, 1) lu_diag_kernel(C32 F, int J, int db, fl
     {
         // lane = 8 rows x 4 columns: 32-byte sectors of the matrix, all 32 shared banks
         const int r = warp * 8 + (lane & 7), cs = lane >> 3;
-#pragma unroll 8
+#pragma unroll 16
         for (int q = 0; q < B / 4; ++q) {
             const int c = 4 * q + cs;
             const bool in = r < db && c < db;
@@ -105,7 +123,7 @@ __global__ void __launch_bounds__(DT, 1) lu_diag_kernel(C32 F, int J, int db, fl
     }
     __syncthreads();
     bool ok = true;
-    if (warp == 0) ok = diag16(Sr, Si, 0, inv_s, thr_s);
+    if (warp == 0) ok = diag16(Sr, Si, 0, inv_s, piv_s);
     __syncthreads();
 #pragma unroll 1
     for (int c0 = 0; c0 + W < B; c0 += W) {
@@ -122,16 +140,21 @@ __global__ void __launch_bounds__(DT, 1) lu_diag_kernel(C32 F, int J, int db, fl
             }
 #pragma unroll
             for (int c = 0; c < W; ++c) {
-                ok = ok && cnorm1(make_float2(ar[c], ai[c])) <= thr_s[c0 + c];
+                ok = ok && cnorm1(make_float2(ar[c], ai[c])) <= cnorm1(piv_s[c0 + c]);
                 const float2 l = cmul(make_float2(ar[c], ai[c]), inv_s[c0 + c]);
                 ar[c] = l.x;
                 ai[c] = l.y;
-                const float* ur = Sr + (c0 + c) * PITCH + c0;
-                const float* ui = Si + (c0 + c) * PITCH + c0;
 #pragma unroll
-                for (int k = c + 1; k < W; ++k) {
-                    ar[k] = fmaf(-l.x, ur[k], fmaf(l.y, ui[k], ar[k]));
-                    ai[k] = fmaf(-l.x, ui[k], fmaf(-l.y, ur[k], ai[k]));
+                for (int k4 = (c + 1) & ~3; k4 < W; k4 += 4) {
+                    const float4 u = *reinterpret_cast<const float4*>(Sr + (c0 + c) * PITCH + c0 + k4);
+                    const float4 v = *reinterpret_cast<const float4*>(Si + (c0 + c) * PITCH + c0 + k4);
+                    const float ur[4] = {u.x, u.y, u.z, u.w}, ui[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (k4 + k > c) {
+                            ar[k4 + k] = fmaf(-l.x, ur[k], fmaf(l.y, ui[k], ar[k4 + k]));
+                            ai[k4 + k] = fmaf(-l.x, ui[k], fmaf(-l.y, ur[k], ai[k4 + k]));
+                        }
                 }
             }
 #pragma unroll
@@ -149,12 +172,18 @@ __global__ void __launch_bounds__(DT, 1) lu_diag_kernel(C32 F, int J, int db, fl
                 xi[k] = pi[k * PITCH];
             }
 #pragma unroll
-            for (int c = 0; c < W - 1; ++c) {
+            for (int k = 1; k < W; ++k) {  // x_k -= sum_{c<k} L[k][c] x_c
 #pragma unroll
-                for (int k = c + 1; k < W; ++k) {
-                    const float lr = Sr[(c0 + k) * PITCH + c0 + c], li = Si[(c0 + k) * PITCH + c0 + c];
-                    xr[k] = fmaf(-lr, xr[c], fmaf(li, xi[c], xr[k]));
-                    xi[k] = fmaf(-lr, xi[c], fmaf(-li, xr[c], xi[k]));
+                for (int c4 = 0; c4 < k; c4 += 4) {
+                    const float4 u = *reinterpret_cast<const float4*>(Sr + (c0 + k) * PITCH + c0 + c4);
+                    const float4 v = *reinterpret_cast<const float4*>(Si + (c0 + k) * PITCH + c0 + c4);
+                    const float lr[4] = {u.x, u.y, u.z, u.w}, li[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        if (c4 + c < k) {
+                            xr[k] = fmaf(-lr[c], xr[c4 + c], fmaf(li[c], xi[c4 + c], xr[k]));
+                            xi[k] = fmaf(-lr[c], xi[c4 + c], fmaf(-li[c], xr[c4 + c], xi[k]));
+                        }
                 }
             }
 #pragma unroll
@@ -193,7 +222,7 @@ __global__ void __launch_bounds__(DT, 1) lu_diag_kernel(C32 F, int J, int db, fl
                 pi[k] = ai[k];
             }
             __syncwarp();
-            ok = diag16(Sr, Si, t0, inv_s, thr_s) && ok;
+            ok = diag16(Sr, Si, t0, inv_s, piv_s) && ok;
         } else {
             const int nct = (rest + 31) / 32, units = (rest / W) * nct;
             const int rg = lane >> 3, cg = (lane & 7) * 4;
@@ -256,55 +285,85 @@ __global__ void __launch_bounds__(DT, 1) lu_diag_kernel(C32 F, int J, int db, fl
         return;
     }
     FdT t(T);
-    for (int e = tid; e < B * (B / 4); e += DT) {  // U's rows
-        const int p = e / (B / 4), k = 4 * (e % (B / 4));
-        float4 x = *reinterpret_cast<const float4*>(Sr + p * PITCH + k);
-        float4 y = *reinterpret_cast<const float4*>(Si + p * PITCH + k);
-        if (k <= p) x.x = y.x = 0.f;
-        if (k + 1 <= p) x.y = y.y = 0.f;
-        if (k + 2 <= p) x.z = y.z = 0.f;
-        if (k + 3 <= p) x.w = y.w = 0.f;
-        *reinterpret_cast<float4*>(t.Ur + p * PITCH + k) = x;
-        *reinterpret_cast<float4*>(t.Ui + p * PITCH + k) = y;
-    }
-    {  // L^T's rows: 8 columns p x 4 rows k of L per warp access (all banks)
-        const int ks = lane & 3, ps = lane >> 2;
-        for (int q = warp; q < (B / 8) * (B / 4); q += DT / 32) {
-            const int p = 8 * (q / (B / 4)) + ps, k = 4 * (q % (B / 4)) + ks;
-            t.Lr[p * PITCH + k] = k > p ? Sr[k * PITCH + p] : 0.f;
-            t.Li[p * PITCH + k] = k > p ? Si[k * PITCH + p] : 0.f;
+    {
+        // inverses of the sixteen 16 x 16 diagonal blocks of U (warps 0-7) and L^T (8-15), a column per
+        // lane: x_i = s_i (delta_ij - sum_{k>i} T[i][k] x_k)
+        const int b = warp & 7, d0 = W * b, j = lane & 15;
+        const bool up = warp < 8;
+        float xr[W], xi[W];
+#pragma unroll
+        for (int i = W - 1; i >= 0; --i) {
+            float sr = i == j ? 1.f : 0.f, si = 0.f;
+#pragma unroll
+            for (int k = i + 1; k < W; ++k) {
+                const int o = up ? (d0 + i) * PITCH + d0 + k : (d0 + k) * PITCH + d0 + i;
+                const float tr = Sr[o], ti = Si[o];
+                sr = fmaf(-tr, xr[k], fmaf(ti, xi[k], sr));
+                si = fmaf(-tr, xi[k], fmaf(-ti, xr[k], si));
+            }
+            const float2 s = up ? inv_s[d0 + i] : make_float2(1.f, 0.f);
+            xr[i] = sr * s.x - si * s.y;
+            xi[i] = sr * s.y + si * s.x;
+        }
+        if (lane < W) {
+            float* gr = (up ? t.Ur : t.Lr) + fd_row(d0);
+            float* gi = (up ? t.Ui : t.Li) + fd_row(d0);
+            const int w = B - d0;
+#pragma unroll
+            for (int i = 0; i < W; ++i) {
+                gr[i * w + j] = xr[i];
+                gi[i * w + j] = xi[i];
+            }
         }
     }
-    if (tid < B) {
-        t.inv[tid] = inv_s[tid];
-        t.piv[tid] = make_float2(Sr[tid * PITCH + tid], Si[tid * PITCH + tid]);
+    for (int e = tid; e < B * (B / 4); e += DT) {  // the factors as they are, and U right of the blocks
+        const int p = e / (B / 4), k = 4 * (e % (B / 4));
+        const float4 x = *reinterpret_cast<const float4*>(Sr + p * PITCH + k);
+        const float4 y = *reinterpret_cast<const float4*>(Si + p * PITCH + k);
+        *reinterpret_cast<float4*>(t.Fr + p * B + k) = x;
+        *reinterpret_cast<float4*>(t.Fi + p * B + k) = y;
+        if (k / W > p / W) {
+            const int o = fd_row(p) + k - (p & ~(W - 1));
+            *reinterpret_cast<float4*>(t.Ur + o) = x;
+            *reinterpret_cast<float4*>(t.Ui + o) = y;
+        }
     }
+    // L^T below the blocks: a lane reads 4 columns p of row k, a warp writes 32 k of each p
+    for (int q = warp; q < (B / 4) * (B / 32); q += DT / 32) {
+        const int p = 4 * (q % (B / 4)), k = 32 * (q / (B / 4)) + lane;
+        if (k / W <= p / W) continue;
+        const float4 x = *reinterpret_cast<const float4*>(Sr + k * PITCH + p);
+        const float4 y = *reinterpret_cast<const float4*>(Si + k * PITCH + p);
+        const int o = fd_row(p) + k - (p & ~(W - 1)), w = B - (p & ~(W - 1));
+        t.Lr[o] = x.x, t.Lr[o + w] = x.y, t.Lr[o + 2 * w] = x.z, t.Lr[o + 3 * w] = x.w;
+        t.Li[o] = y.x, t.Li[o + w] = y.y, t.Li[o + 2 * w] = y.z, t.Li[o + 3 * w] = y.w;
+    }
+    if (tid < B) t.piv[tid] = piv_s[tid];
 }
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(dst)), "l"(src) : "memory");
 }
 
-// L21 = A21 U11^{-1} (rows) and U12 = L11^{-1} A12 (columns): both are x_k = (a_k - sum_{p<k} x_p T[p][k]) s_k
-// with T = U, s_k = 1/u_kk for a row and T = L^T, s_k = 1 for a column.  A CTA takes R rows or columns
-// with Q = 256 / R threads each; a thread keeps 32 / Q entries of the current chunk of 32 in registers:
-// the chunk first takes the products with all earlier entries, then its own entries one after
-// another, each broadcast from its owner by shuffles.  FP32 rate and the shuffle chain share the time;
-// R = 32 halves both per CTA while the CTAs (one per SM: T takes 135 KB) still fit one wave.
-// The last CTA writes the diagonal block's factors to the matrix.  Every CTA saves what it overwrites.
-template <int R>
-__global__ void __launch_bounds__(256, 1) lu_trsm_kernel(C32 F, int J, int db, int mm, const float* __restrict__ T,
-                                                         float* __restrict__ bk, long ldb, float* __restrict__ Lpr,
-                                                         float* __restrict__ Lpi, float* __restrict__ Upr,
-                                                         float* __restrict__ Upi, long ldk, int* fail) {
-    constexpr int Q = 256 / R, CPT = 32 / Q, RW = R / 8, XP = R + 1;
+// L21 = A21 U11^{-1} (rows) and U12 = L11^{-1} A12 (columns): both are x T = a with T = U for a row and
+// T = L^T for a column, solved in chunks of 16 entries: y = a_b - sum_{b'<b} x_b' T[b'][b], then
+// x_b = y T[b][b]^{-1} with the inverted block.  A CTA takes R = 32 rows or columns, four threads each with
+// 4 of a chunk's 16 entries in registers; T (74 KB packed) and the 32 x 128 entries are in shared memory, so
+// two CTAs share an SM and one wave covers 4800 rows and columns.  The FP32 rate bounds it (9.2k cycles
+// of multiply-adds per CTA).  The pivot search's candidates l_ik u_kk are compared with their pivots.
+// The last eight CTAs write the diagonal block's factors to the matrix.  Every CTA saves what it
+// overwrites.
+constexpr int R = 32, RT = 4 * R, XP = R + 1;
+__global__ void __launch_bounds__(RT, 2) lu_trsm_kernel(C32 F, int J, int db, int mm, const float* __restrict__ T,
+                                                        float* __restrict__ bk, long ldb, float* __restrict__ Lpr,
+                                                        float* __restrict__ Lpi, float* __restrict__ Upr,
+                                                        float* __restrict__ Upi, long ldk, int* fail) {
     extern __shared__ __align__(16) float sm[];
     float* Tr = sm;
-    float* Ti = Tr + B * PITCH;
-    float* Xr = Ti + B * PITCH;  // [k][row]
+    float* Ti = Tr + FD_PACK;
+    float* Xr = Ti + FD_PACK;  // [k][row]
     float* Xi = Xr + B * XP;
-    __shared__ float2 inv_s[B];
-    __shared__ float thr_s[B];
+    __shared__ float2 piv_s[B];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     {
         const int f = *reinterpret_cast<volatile int*>(fail);
@@ -313,16 +372,33 @@ __global__ void __launch_bounds__(256, 1) lu_trsm_kernel(C32 F, int J, int db, i
     const FdT t(const_cast<float*>(T));
     const FdBackup b(bk, ldb);
     const int nr = (mm + R - 1) / R;
-    if ((int)blockIdx.x == 2 * nr) {  // the diagonal block
-        for (int e = tid; e < B * B; e += 256) {
-            const int i = e % B, j = e / B;
-            if (i >= db || j >= db) continue;
-            const long o = (long)(J + i) + (long)(J + j) * F.ld;
-            b.Dr[e] = F.re[o];
-            b.Di[e] = F.im[o];
-            const float2 p = t.piv[i];
-            F.re[o] = i == j ? p.x : (i < j ? t.Ur[i * PITCH + j] : t.Lr[j * PITCH + i]);
-            F.im[o] = i == j ? p.y : (i < j ? t.Ui[i * PITCH + j] : t.Li[j * PITCH + i]);
+    if ((int)blockIdx.x >= 2 * nr) {  // 16 columns of the diagonal block, a row of 4 columns at a time
+        const int i = tid, j0 = W * ((int)blockIdx.x - 2 * nr);
+        float4 x[W / 4], y[W / 4];
+#pragma unroll
+        for (int q = 0; q < W / 4; ++q) {
+            x[q] = *reinterpret_cast<const float4*>(t.Fr + i * B + j0 + 4 * q);
+            y[q] = *reinterpret_cast<const float4*>(t.Fi + i * B + j0 + 4 * q);
+        }
+        if (i < db) {
+            float orr[W], oi[W];
+#pragma unroll
+            for (int j = 0; j < W; ++j)
+                if (j0 + j < db) {
+                    const long o = (long)(J + i) + (long)(J + j0 + j) * F.ld;
+                    orr[j] = F.re[o];
+                    oi[j] = F.im[o];
+                }
+#pragma unroll
+            for (int j = 0; j < W; ++j)
+                if (j0 + j < db) {
+                    const long o = (long)(J + i) + (long)(J + j0 + j) * F.ld;
+                    b.Dr[i + (j0 + j) * B] = orr[j];
+                    b.Di[i + (j0 + j) * B] = oi[j];
+                    const float4 u = x[j / 4], v = y[j / 4];
+                    F.re[o] = j % 4 == 0 ? u.x : (j % 4 == 1 ? u.y : (j % 4 == 2 ? u.z : u.w));
+                    F.im[o] = j % 4 == 0 ? v.x : (j % 4 == 1 ? v.y : (j % 4 == 2 ? v.z : v.w));
+                }
         }
         return;
     }
@@ -331,22 +407,19 @@ __global__ void __launch_bounds__(256, 1) lu_trsm_kernel(C32 F, int J, int db, i
     {
         const float* sr = rows ? t.Ur : t.Lr;
         const float* si = rows ? t.Ui : t.Li;
-        for (int e = tid; e < B * PITCH / 4; e += 256) {
+        for (int e = tid; e < FD_PACK / 4; e += RT) {
             cp_async16(Tr + 4 * e, sr + 4 * e);
             cp_async16(Ti + 4 * e, si + 4 * e);
         }
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     }
-    if (tid < B) {
-        const float2 p = t.piv[tid];
-        inv_s[tid] = rows ? t.inv[tid] : make_float2(1.f, 0.f);
-        thr_s[tid] = cnorm1(p);
-    }
+    piv_s[tid] = t.piv[tid];
+    static_assert(RT == B, "a thread per pivot, row and K index");
     if (rows) {
-        const int r = tid % R;
-#pragma unroll 8
-        for (int i = 0; i < B * R / 256; ++i) {
-            const int k = tid / R + Q * i;
+        const int r = lane;
+#pragma unroll 16
+        for (int i = 0; i < B / 4; ++i) {
+            const int k = warp + 4 * i;
             float vr = 0.f, vi = 0.f;
             if (x0 + r < mm) {
                 const long o = (long)(J + B + x0 + r) + (long)(J + k) * F.ld;
@@ -359,123 +432,107 @@ __global__ void __launch_bounds__(256, 1) lu_trsm_kernel(C32 F, int J, int db, i
             Xi[k * XP + r] = vi;
         }
     } else {
-        const int k = tid % B;
-#pragma unroll 8
-        for (int i = 0; i < B * R / 256; ++i) {
-            const int c = tid / B + 2 * i;
+#pragma unroll 16
+        for (int c = 0; c < R; ++c) {
             float vr = 0.f, vi = 0.f;
             if (x0 + c < mm) {
-                const long o = (long)(J + k) + (long)(J + B + x0 + c) * F.ld;
+                const long o = (long)(J + tid) + (long)(J + B + x0 + c) * F.ld;
                 vr = F.re[o];
                 vi = F.im[o];
-                b.Ur[k + (long)(x0 + c) * B] = vr;
-                b.Ui[k + (long)(x0 + c) * B] = vi;
+                b.Ur[tid + (long)(x0 + c) * B] = vr;
+                b.Ui[tid + (long)(x0 + c) * B] = vi;
             }
-            Xr[k * XP + c] = vr;
-            Xi[k * XP + c] = vi;
+            Xr[tid * XP + c] = vr;
+            Xi[tid * XP + c] = vi;
         }
     }
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     __syncthreads();
-    const int rs = lane % RW, q = lane / RW, row = warp * RW + rs;
+    const int q = 4 * (lane & 3), row = warp * 8 + (lane >> 2);
+    // a -= (or +=) the products of entries p0 .. p0 + 15 with the 16 x 4 entries of T at tr, ti (row pitch w)
+    auto mac = [&](float (&ar)[4], float (&ai)[4], int p0, const float* tr, const float* ti, int w, float sign) {
+#pragma unroll
+        for (int p = 0; p < W; ++p) {
+            const float xr = sign * Xr[(p0 + p) * XP + row], xi = sign * Xi[(p0 + p) * XP + row];
+            const float4 u = *reinterpret_cast<const float4*>(tr + p * w);
+            const float4 v = *reinterpret_cast<const float4*>(ti + p * w);
+            ar[0] = fmaf(xr, u.x, fmaf(-xi, v.x, ar[0]));
+            ar[1] = fmaf(xr, u.y, fmaf(-xi, v.y, ar[1]));
+            ar[2] = fmaf(xr, u.z, fmaf(-xi, v.z, ar[2]));
+            ar[3] = fmaf(xr, u.w, fmaf(-xi, v.w, ar[3]));
+            ai[0] = fmaf(xr, v.x, fmaf(xi, u.x, ai[0]));
+            ai[1] = fmaf(xr, v.y, fmaf(xi, u.y, ai[1]));
+            ai[2] = fmaf(xr, v.z, fmaf(xi, u.z, ai[2]));
+            ai[3] = fmaf(xr, v.w, fmaf(xi, u.w, ai[3]));
+        }
+    };
     bool ok = true;
 #pragma unroll 1
-    for (int s0 = 0; s0 < B; s0 += 32) {
-        const int j0 = s0 + q * CPT;  // this thread's entries j0 .. j0 + CPT - 1
-        float ar[CPT], ai[CPT];
+    for (int j0 = 0; j0 < B; j0 += W) {
+        float ar[4], ai[4];
 #pragma unroll
-        for (int j = 0; j < CPT; ++j) {
-            ar[j] = Xr[(j0 + j) * XP + row];
-            ai[j] = Xi[(j0 + j) * XP + row];
+        for (int j = 0; j < 4; ++j) {
+            ar[j] = Xr[(j0 + q + j) * XP + row];
+            ai[j] = Xi[(j0 + q + j) * XP + row];
         }
-#pragma unroll 4
-        for (int p = 0; p < s0; ++p) {
-            const float xr = Xr[p * XP + row], xi = Xi[p * XP + row];
-            const float4* tr = reinterpret_cast<const float4*>(Tr + p * PITCH + j0);
-            const float4* ti = reinterpret_cast<const float4*>(Ti + p * PITCH + j0);
+        int o = j0 + q;  // T[p0 .. p0 + 15][j0 + q ..] in the packed rows
+#pragma unroll 1
+        for (int p0 = 0; p0 < j0; p0 += W) {
+            mac(ar, ai, p0, Tr + o, Ti + o, B - p0, -1.f);
+            o += W * (B - p0) - W;
+        }
+        __syncwarp();  // the chunk's entries have been read
 #pragma unroll
-            for (int j = 0; j < CPT; j += 4) {
-                const float4 u = tr[j / 4], v = ti[j / 4];
-                ar[j] = fmaf(-xr, u.x, fmaf(xi, v.x, ar[j]));
-                ar[j + 1] = fmaf(-xr, u.y, fmaf(xi, v.y, ar[j + 1]));
-                ar[j + 2] = fmaf(-xr, u.z, fmaf(xi, v.z, ar[j + 2]));
-                ar[j + 3] = fmaf(-xr, u.w, fmaf(xi, v.w, ar[j + 3]));
-                ai[j] = fmaf(-xr, v.x, fmaf(-xi, u.x, ai[j]));
-                ai[j + 1] = fmaf(-xr, v.y, fmaf(-xi, u.y, ai[j + 1]));
-                ai[j + 2] = fmaf(-xr, v.z, fmaf(-xi, u.z, ai[j + 2]));
-                ai[j + 3] = fmaf(-xr, v.w, fmaf(-xi, u.w, ai[j + 3]));
+        for (int j = 0; j < 4; ++j) {
+            Xr[(j0 + q + j) * XP + row] = ar[j];
+            Xi[(j0 + q + j) * XP + row] = ai[j];
+        }
+        __syncwarp();
+        float yr[4] = {0.f, 0.f, 0.f, 0.f}, yi[4] = {0.f, 0.f, 0.f, 0.f};
+        mac(yr, yi, j0, Tr + o, Ti + o, B - j0, 1.f);
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (rows) {
+                const float2 u = piv_s[j0 + q + j];
+                ok = ok && cnorm1(cmul(make_float2(yr[j], yi[j]), u)) <= cnorm1(u);
             }
+            Xr[(j0 + q + j) * XP + row] = yr[j];
+            Xi[(j0 + q + j) * XP + row] = yi[j];
         }
-#pragma unroll
-        for (int g = 0; g < Q; ++g) {
-#pragma unroll
-            for (int c = 0; c < CPT; ++c) {
-                const int k = s0 + g * CPT + c;
-                // the owner scales its entry (a row's entry is the pivot search's candidate first)
-                float2 x = make_float2(ar[c], ai[c]);
-                if (rows) {
-                    if (q == g) ok = ok && cnorm1(x) <= thr_s[k];
-                    x = cmul(x, inv_s[k]);
-                }
-                const float xr = __shfl_sync(0xffffffffu, x.x, g * RW + rs);
-                const float xi = __shfl_sync(0xffffffffu, x.y, g * RW + rs);
-                // T is zero at and left of the diagonal, so entries up to k stay
-                const float4* tr = reinterpret_cast<const float4*>(Tr + k * PITCH + j0);
-                const float4* ti = reinterpret_cast<const float4*>(Ti + k * PITCH + j0);
-#pragma unroll
-                for (int j = 0; j < CPT; j += 4) {
-                    const float4 u = tr[j / 4], v = ti[j / 4];
-                    ar[j] = fmaf(-xr, u.x, fmaf(xi, v.x, ar[j]));
-                    ar[j + 1] = fmaf(-xr, u.y, fmaf(xi, v.y, ar[j + 1]));
-                    ar[j + 2] = fmaf(-xr, u.z, fmaf(xi, v.z, ar[j + 2]));
-                    ar[j + 3] = fmaf(-xr, u.w, fmaf(xi, v.w, ar[j + 3]));
-                    ai[j] = fmaf(-xr, v.x, fmaf(-xi, u.x, ai[j]));
-                    ai[j + 1] = fmaf(-xr, v.y, fmaf(-xi, u.y, ai[j + 1]));
-                    ai[j + 2] = fmaf(-xr, v.z, fmaf(-xi, u.z, ai[j + 2]));
-                    ai[j + 3] = fmaf(-xr, v.w, fmaf(-xi, u.w, ai[j + 3]));
-                }
-                if (q == g) {
-                    ar[c] = x.x;
-                    ai[c] = x.y;
-                }
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < CPT; ++j) {
-            Xr[(j0 + j) * XP + row] = ar[j];
-            Xi[(j0 + j) * XP + row] = ai[j];
-        }
-        __syncwarp();  // a row's threads are lanes of one warp
+        __syncwarp();
     }
     if (!ok) atomicCAS(fail, 0, 2 * (J + 1) + 1);
     __syncthreads();
     if (rows) {
-        const int r = tid % R;
-        if (x0 + r < mm)
-            for (int k = tid / R; k < B; k += Q) {
-                const long o = (long)(J + B + x0 + r) + (long)(J + k) * F.ld;
-                F.re[o] = Xr[k * XP + r];
-                F.im[o] = Xi[k * XP + r];
+        if (x0 + lane < mm)
+#pragma unroll 8
+            for (int i = 0; i < B / 4; ++i) {
+                const int k = warp + 4 * i;
+                const long o = (long)(J + B + x0 + lane) + (long)(J + k) * F.ld;
+                F.re[o] = Xr[k * XP + lane];
+                F.im[o] = Xi[k * XP + lane];
             }
     } else {
-        const int k = tid % B;
-        for (int c = tid / B; c < R && x0 + c < mm; c += 2) {
-            const long o = (long)(J + k) + (long)(J + B + x0 + c) * F.ld;
-            F.re[o] = Xr[k * XP + c];
-            F.im[o] = Xi[k * XP + c];
-        }
+#pragma unroll 8
+        for (int c = 0; c < R; ++c)
+            if (x0 + c < mm) {
+                const long o = (long)(J + tid) + (long)(J + B + x0 + c) * F.ld;
+                F.re[o] = Xr[tid * XP + c];
+                F.im[o] = Xi[tid * XP + c];
+            }
     }
     // K-major packs, segments [hi | hi | lo] of L21 rows and [hi | lo | hi] of U12 columns
-    {
-        float* Pr = rows ? Lpr : Upr;
-        float* Pi = rows ? Lpi : Upi;
-        const int o1 = rows ? B : 2 * B, o2 = rows ? 2 * B : B;  // second hi, lo
-        const int k = tid % B;
-        for (int r = tid / B; r < R && x0 + r < mm; r += 2) {
-            const float vr = Xr[k * XP + r], vi = Xi[k * XP + r];
+    float* Pr = (rows ? Lpr : Upr) + tid;
+    float* Pi = (rows ? Lpi : Upi) + tid;
+    const int o1 = rows ? B : 2 * B, o2 = rows ? 2 * B : B;  // second hi, lo
+#pragma unroll 4
+    for (int r = 0; r < R; ++r)
+        if (x0 + r < mm) {
+            const float vr = Xr[tid * XP + r], vi = Xi[tid * XP + r];
             const float hr = tf32_rna(vr), hi = tf32_rna(vi);
-            float* pr = Pr + (long)(x0 + r) * ldk + k;
-            float* pi = Pi + (long)(x0 + r) * ldk + k;
+            float* pr = Pr + (long)(x0 + r) * ldk;
+            float* pi = Pi + (long)(x0 + r) * ldk;
             pr[0] = hr;
             pr[o1] = hr;
             pr[o2] = vr - hr;
@@ -483,7 +540,6 @@ __global__ void __launch_bounds__(256, 1) lu_trsm_kernel(C32 F, int J, int db, i
             pi[o1] = hi;
             pi[o2] = vi - hi;
         }
-    }
 }
 
 // the entries lu_trsm_kernel overwrote, back into the matrix
@@ -511,21 +567,6 @@ __global__ void lu_restore_kernel(C32 F, int J, int db, int mm, float* __restric
     }
 }
 
-template <int R>
-cudaError_t launch_trsm_t(cudaStream_t s, C32 F, int J, int db, int mm, float* T, float* bk, long ldb, float* const* P,
-                          long ldk, int* fail) {
-    constexpr int smem = (2 * B * PITCH + 2 * B * (R + 1)) * (int)sizeof(float);
-    static DeviceFlags attr;
-    if (attr.pending()) {
-        cudaError_t e = cudaFuncSetAttribute(lu_trsm_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        attr.done();
-    }
-    lu_trsm_kernel<R><<<2 * ceil_div(mm, R) + 1, 256, smem, s>>>(F, J, db, mm, T, bk, ldb, P[0], P[1], P[2], P[3], ldk,
-                                                                 fail);
-    return cudaGetLastError();
-}
-
 }  // namespace
 
 cudaError_t launch_lu_diag(cudaStream_t s, C32 F, int J, int db, float* work, int* fail) {
@@ -541,11 +582,18 @@ cudaError_t launch_lu_diag(cudaStream_t s, C32 F, int J, int db, float* work, in
 }
 
 cudaError_t launch_lu_trsm(cudaStream_t s, C32 F, int J, int db, int mm, float* work, long n, float* const* packs,
-                           long ldk, int num_sms, int* fail) {
+                           long ldk, int* fail) {
     if (mm > 0 && (db != B || ldk < 3 * B)) return cudaErrorInvalidValue;
-    if (2 * ceil_div(mm, 32) + 1 <= num_sms)
-        return launch_trsm_t<32>(s, F, J, db, mm, work, work + FD_T, n, packs, ldk, fail);
-    return launch_trsm_t<64>(s, F, J, db, mm, work, work + FD_T, n, packs, ldk, fail);
+    constexpr int smem = (2 * FD_PACK + 2 * B * XP) * (int)sizeof(float);
+    static DeviceFlags attr;
+    if (attr.pending()) {
+        cudaError_t e = cudaFuncSetAttribute(lu_trsm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        attr.done();
+    }
+    lu_trsm_kernel<<<2 * ceil_div(mm, R) + ceil_div(db, W), RT, smem, s>>>(
+        F, J, db, mm, work, work + FD_T, n, packs[0], packs[1], packs[2], packs[3], ldk, fail);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_lu_restore(cudaStream_t s, C32 F, int J, int db, int mm, float* work, long n) {

@@ -518,15 +518,21 @@ int query_cluster_max_c32();
 
 // lu_fast.cu: blocks of FD_B columns whose pivots stay on the diagonal.  The work buffer holds the
 // factors of the current diagonal block (FdT) and what lu_trsm_kernel overwrote (FdBackup).
-constexpr int FD_B = 128, FD_PITCH = 132;
-constexpr long FD_T = 4L * FD_B * FD_PITCH + 4L * FD_B;
+constexpr int FD_B = 128, FD_PITCH = 132, FD_W = 16;
+constexpr int FD_PACK = FD_W * (FD_B + FD_W) * (FD_B / FD_W) / 2;  // packed floats of a block upper triangle
+// offset of row p of a packed block upper triangle: rows of 16-row block q hold columns 16 q .. 127
+BM_HD constexpr int fd_row(int p) {
+    const int q = p / FD_W;
+    return FD_W * (q * FD_B - FD_W * q * (q - 1) / 2) + (p - FD_W * q) * (FD_B - FD_W * q);
+}
+constexpr long FD_T = 4L * FD_PACK + 2L * FD_B * FD_B + 2L * FD_B;
 struct FdT {
-    float *Ur, *Ui, *Lr, *Li;  // strict upper triangles of U and L^T, rows [p][k] of pitch FD_PITCH
-    float2 *inv, *piv;         // 1 / u_kk, u_kk
+    float *Ur, *Ui, *Lr, *Li;  // U and L^T packed, the 16 x 16 diagonal blocks inverted
+    float *Fr, *Fi;            // the factors as they are, [row][column]
+    float2* piv;               // u_kk
     BM_HD explicit FdT(float* w)
-        : Ur(w), Ui(w + FD_B * FD_PITCH), Lr(w + 2 * FD_B * FD_PITCH), Li(w + 3 * FD_B * FD_PITCH),
-          inv(reinterpret_cast<float2*>(w + 4 * FD_B * FD_PITCH)),
-          piv(reinterpret_cast<float2*>(w + 4 * FD_B * FD_PITCH + 2 * FD_B)) {}
+        : Ur(w), Ui(w + FD_PACK), Lr(w + 2 * FD_PACK), Li(w + 3 * FD_PACK), Fr(w + 4 * FD_PACK),
+          Fi(Fr + FD_B * FD_B), piv(reinterpret_cast<float2*>(Fi + FD_B * FD_B)) {}
 };
 struct FdBackup {
     float *Dr, *Di, *Lr, *Li, *Ur, *Ui;  // diagonal block; A21 (column-major, ld n); A12 (ld FD_B)
@@ -537,7 +543,7 @@ struct FdBackup {
 inline size_t fd_work_floats(long n) { return (size_t)FD_T + 2 * FD_B * FD_B + 4 * (size_t)n * FD_B; }
 cudaError_t launch_lu_diag(cudaStream_t s, C32 F, int J, int db, float* work, int* fail);
 cudaError_t launch_lu_trsm(cudaStream_t s, C32 F, int J, int db, int mm, float* work, long n, float* const* packs,
-                           long ldk, int num_sms, int* fail);
+                           long ldk, int* fail);
 cudaError_t launch_lu_restore(cudaStream_t s, C32 F, int J, int db, int mm, float* work, long n);
 int query_cluster_max_z64();
 
