@@ -948,8 +948,9 @@ bm_status ensure_ws(bm_ctx* c, int nrhs) {
     }
     if (c->prec != BM_FP64) {
         // x digit planes and split-K workspace of the tensor-core residual
-        const int N = c->N, np = rt_digit_planes(c->rt_nd);
+        const int N = c->N, np = rt_x_planes(c->rt_nd);
         const int npad = (int)round_up(w, rt_col_tile(c->rt_nd));
+        c->dx_cols = npad;
         const int nprod = (c->form == BM_MIXED) ? 2 : 1;
         long mq[2], Kq[2];
         for (int q = 0; q < nprod; ++q) {
@@ -961,8 +962,7 @@ bm_status ensure_ws(bm_ctx* c, int nrhs) {
             c->dx_ldk[q] = rt_ldk(K);
             BM_TRY(alloc_t(c, &c->d_dx[q], (size_t)np * npad * c->dx_ldk[q] * 2));
             BM_TRY(alloc_t(c, &c->d_dxe[q], (size_t)npad * 4));
-            BM_TRY(rt_make_map(c->tm_dx[q], c->d_dx[q], npad, K, c->dx_ldk[q], (long)npad * c->dx_ldk[q],
-                               rt_col_tile(c->rt_nd), c->rt_nd));
+            BM_TRY(rt_make_map_x(c->tm_dx[q], c->d_dx[q], npad, K, c->dx_ldk[q], c->rt_nd));
         }
         // the split count depends on the number of right-hand sides: size for the largest need
         size_t wsz = 0;

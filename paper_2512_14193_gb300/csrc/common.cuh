@@ -279,7 +279,8 @@ struct bm_ctx {
     void* d_dx[2] = {nullptr, nullptr};
     int* d_dxe[2] = {nullptr, nullptr};
     long dx_ldk[2] = {0, 0};
-    alignas(64) unsigned char tm_dx[2][128];
+    long dx_cols = 0;         // columns of a plane (the workspace's, not the call's)
+    alignas(64) unsigned char tm_dx[2][256];
     double* d_rtw = nullptr;
     size_t rtw_elems = 0;
 

@@ -114,16 +114,18 @@ struct RtArgs {
     int m, K, S;
 };
 long rt_ldk(long K);                 // leading dimension of a digit plane row (K rounded to 64)
-int rt_digit_planes(int nd);         // planes per operand (nd digits x Re, Im)
+int rt_digit_planes(int nd);         // planes of A (nd digits x Re, Im)
+int rt_x_planes(int nd);             // planes of x
 int rt_col_tile(int nd);             // right-hand sides per CTA
 // K splits S[q] of the nprod products (m[q] rows, K[q] columns) of one launch with n right-hand sides
 void rt_plan_splits(int nprod, const long* m, const long* K, int n, int nd, int num_sms, int* S);
 bm_status rt_make_map(void* tmap, const void* base, long rows, long K, long ldk, long plane_elems, int box_rows,
                       int nd);
+bm_status rt_make_map_x(void* tmaps, const void* base, long cols, long K, long ldk, int nd);  // two blobs
 cudaError_t launch_digits_a(cudaStream_t s, const double2* A, long lda, int rows, int K, int* e, void* D, long ldk,
                             void* rowmax, int nd);
 cudaError_t launch_digits_x(cudaStream_t s, const double2* X, long ldx, int r0, int K, int n, int npad, int* f,
-                            void* D, long ldk, int nd);
+                            void* D, long ldk, long plane, int nd);
 cudaError_t gemm_rt(cudaStream_t s, const RtArgs* prods, int nprod, int n, double alpha, int* d_err, int* launched,
                     int nd);
 

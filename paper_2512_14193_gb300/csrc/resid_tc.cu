@@ -17,18 +17,24 @@
 //     the hardware adds in;
 //   * after each chunk the seven level sums are combined and added to a running double-float sum
 //     (pairs of FP32) per output; the dropped pairs (d + d' > 8) weigh below 2^-56.
-// The complex product uses four real products per digit pair with the A-negate bit of the
-// instruction descriptor for -Im A Im x (as the TF32 kernel does).  The x digit tiles sit one after
-// another in shared memory (digit d' at rows 32 d'), and level l's accumulator at tensor-memory
-// column 32 l, so one MMA of width N = 32 (7 - d) multiplies A digit d by all the x digits it pairs
-// with and lands each pair in its level: four MMAs per A digit and 16-wide K step.
+// The x digit tiles sit one after another in shared memory and the levels' accumulators one after
+// another in tensor memory, so one MMA multiplies A digit d by all the x digits it pairs with and
+// lands each pair in its level.  Seven digits (32 right-hand sides per CTA): four MMAs of width
+// 32 (7 - d) per A digit and 16-wide K step, the A-negate bit of the instruction descriptor giving
+// -Im A Im x.  Nine digits (16 right-hand sides): the real and imaginary parts of a level share an
+// accumulator, [Re | Im], and x is staged as two stacks per digit, [Re x | Im x] for Re A and
+// [-Im x | Re x] for Im A, so each A tile is read from shared memory once per K step by two MMAs of width
+// 32 (9 - d) instead of four half as wide: the narrow ones left the tensor pipe waiting for A.
+// The digits of A are taken from the last to the first: digit d reaches levels d and up, so the next
+// chunk's products start on level D - 1 as soon as it has been read while the readers go on with the lower
+// levels (reading all of them first left the tensor pipe idle for a third of the time).
 //
-// CTA: 128 output rows x up to 32 right-hand sides, K range [kbeg, kend) (split K, deterministic
+// CTA: 128 output rows x up to 32 (16) right-hand sides, K range [kbeg, kend) (split K, deterministic
 // reduction afterwards when there is more than one split).  Warp 0 issues TMA loads (per 64-wide
-// K block: the 14 digit planes of x, then the 7 digit pairs (Re, Im) of A one stage at a time),
-// warp 1 issues the MMAs, warps 2-9 read the level sums from tensor memory after each chunk (warps
-// 2-5 the real parts, 6-9 the imaginary parts, one output row per thread) and keep the running
-// sums.  All waits are bounded (2 s); a timeout sets *err and the CTA drains what it issued.
+// K block: the digit planes of x, then the digit tiles of A one stage at a time), warp 1 issues the
+// MMAs, warps 2-9 read the level sums from tensor memory after each chunk (warps 2-5 the real parts,
+// 6-9 the imaginary parts, one output row per thread) and keep the running sums.  All waits are
+// bounded (2 s); a timeout sets *err and the CTA drains what it issued.
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -38,32 +44,40 @@
 
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 
 namespace {
 
 constexpr int RT_BM = 128;   // output rows per CTA
 constexpr int RT_BK = 64;    // K elements per stage: bf16 rows of 128 bytes (one swizzle span)
-constexpr int RT_AST = 3;    // stages of A digit pairs
 constexpr int RT_TILE_A = RT_BM * RT_BK * 2;  // one digit plane of A: 16 KB
-constexpr int RT_A_STAGE = 2 * RT_TILE_A;     // Re and Im of one digit
 constexpr int RT_THREADS = 320;
 constexpr uint64_t RT_WAIT_NS = 2000000000ull;
 // D digits per operand (7: pairs to level 6, 2^-50; 9: to level 8, 2^-64) and NT right-hand sides
 // per CTA (32 for D = 7, 16 for D = 9).  Level sums over a chunk stay below 2^24: D pairs x 2
-// products x 4096 x chunk K, so the chunk is 256 for D = 7 and 128 for D = 9.  Tensor memory:
-// real parts of levels 0..D-1 at columns NT l, imaginary parts at NT (D + l).
+// products x 4096 x chunk K, so the chunk is 256 for D = 7 and 192 for D = 9.
 template <int D>
 struct RtCfg {
-    static constexpr int NT = D <= 7 ? 32 : 16;         // right-hand sides per CTA
+    static constexpr bool STACK = D > 7;                // [Re | Im] levels, two x stacks, single-plane A stages
+    static constexpr int NT = STACK ? 16 : 32;          // right-hand sides per CTA
     static constexpr int TILE_X = NT * RT_BK * 2;       // one digit plane of x
-    static constexpr int KB_CHUNK = D <= 7 ? 4 : 2;     // K blocks of 64 per exact chunk
-    static constexpr int X_BUF = 2 * D * TILE_X;        // all digits of x, Re and Im
-    static constexpr int SMEM = RT_AST * RT_A_STAGE + 2 * X_BUF + 1024 + 256;
+    static constexpr int KB_CHUNK = STACK ? 3 : 4;      // K blocks of 64 per exact chunk
+    static constexpr int X_STACK = 2 * D * TILE_X;      // one stack: all digits, two planes each
+    static constexpr int X_BUF = (STACK ? 2 : 1) * X_STACK;
+    static constexpr int A_PL = STACK ? 1 : 2;          // A planes per stage
+    static constexpr int A_STAGE = A_PL * RT_TILE_A;
+    static constexpr int AST = STACK ? 5 : 3;           // A stages
+    static constexpr int USES = 2 * D / A_PL;           // stage uses per K block
+    static constexpr int SMEM = AST * A_STAGE + 2 * X_BUF + 1024 + 256;
     static_assert(2 * D * NT <= 512, "the level accumulators fit tensor memory");
-    static_assert(D * NT <= 256, "the widest MMA (A digit 0 against all x digits) has N <= 256");
+    static_assert(D * NT <= 256, "the widest single MMA has N <= 256");
     static_assert(D * 2 * 4096L * 64 * KB_CHUNK <= (1L << 24), "chunk sums stay exact in FP32");
     static_assert(SMEM <= 232448, "shared memory");
 };
+
+// Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 bytes apart.
+constexpr uint32_t DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (1u << 16); }
 
 __device__ __forceinline__ uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ uint64_t gtimer() {
@@ -109,14 +123,26 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const void* tmap, uint
         "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar), "r"(x), "r"(y), "r"(z)
         : "memory");
 }
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const void* tmap, uint32_t bar, int x, int y, int z, int w) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], "
+        "[%2];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar), "r"(x), "r"(y), "r"(z), "r"(w)
+        : "memory");
+}
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
-            d),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
-        : "memory");
+// D += A B (acc: a literal 0 or 1) from the low words of the two shared-memory descriptors, issued by the
+// lanes with `leader` set.  The operands are warp-uniform, so that they live in uniform registers and a
+// product costs a handful of instructions: one thread's issue rate bounds the narrow products otherwise.
+__device__ __forceinline__ void mma_bf16(bool leader, uint32_t d, uint32_t alo, uint32_t blo, uint32_t idesc,
+                                         uint32_t acc) {
+    if (leader)
+        asm volatile(
+            "{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, %4, 0;\n mov.b64 a, {%1, %5};\n mov.b64 b, {%2, %5};\n"
+            " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n}\n" ::"r"(d),
+            "r"(alo), "r"(blo), "r"(idesc), "r"(acc), "n"(DESC_HI)
+            : "memory");
 }
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -134,13 +160,8 @@ __device__ __forceinline__ void tmem_ld16(uint32_t ta, float* v) {
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(a[i]);
 }
-// Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 bytes apart.
-__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
-           ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
-}
 // Instruction descriptor, kind::f16: D = F32, A = B = BF16, both K-major, M = 128, N = n.
-__device__ __forceinline__ uint32_t idesc_bf16(uint32_t neg_a, uint32_t n) {
+__device__ constexpr uint32_t idesc_bf16(uint32_t neg_a, uint32_t n) {
     return (1u << 4) | (1u << 7) | (1u << 10) | (neg_a << 13) | ((n >> 3) << 17) | ((uint32_t)(RT_BM >> 4) << 24);
 }
 // s + t exactly as hi + lo (Knuth's TwoSum); the rn intrinsics keep the steps from being contracted
@@ -153,7 +174,7 @@ __device__ __forceinline__ void two_sum(float& hi, float& lo, float a, float b) 
 
 struct RtProd {
     CUtensorMap tmA;   // the A digit planes (3-D: K, rows, 14 planes)
-    CUtensorMap tmX;   // the x digit planes (3-D: K, columns, 14 planes)
+    CUtensorMap tmX[2];  // the x digit planes: 3-D (K, columns, 14 planes), or the two stacks (4-D)
     const int* eA;     // row exponents of A
     const int* fX;     // column exponents of x
     double2* C;        // output (FP64 complex), C += alpha A x
@@ -171,17 +192,19 @@ struct RtJob {
 
 template <int D>
 __global__ void __launch_bounds__(RT_THREADS, 1) resid_tc_kernel(const __grid_constant__ RtJob J, int* __restrict__ err) {
-    constexpr int RT_D = D, RT_KB_CHUNK = RtCfg<D>::KB_CHUNK, RT_X_BUF = RtCfg<D>::X_BUF;
-    constexpr int RT_NT = RtCfg<D>::NT, RT_TILE_X = RtCfg<D>::TILE_X;
+    using Cfg = RtCfg<D>;
+    constexpr int RT_D = D, RT_KB_CHUNK = Cfg::KB_CHUNK, RT_X_BUF = Cfg::X_BUF, RT_AST = Cfg::AST;
+    constexpr int RT_NT = Cfg::NT, RT_TILE_X = Cfg::TILE_X, RT_A_STAGE = Cfg::A_STAGE, USES = Cfg::USES;
+    constexpr bool STACK = Cfg::STACK;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t* sA = smem;                               // RT_AST stages of (Re, Im) digit tiles of A
-    uint8_t* sX = smem + RT_AST * RT_A_STAGE;         // 2 buffers of all 14 digit tiles of x
+    uint8_t* sA = smem;                               // RT_AST stages of digit tiles of A
+    uint8_t* sX = smem + RT_AST * RT_A_STAGE;         // 2 buffers of all digit tiles of x
     uint64_t* bars = reinterpret_cast<uint64_t*>(sX + 2 * RT_X_BUF);
-    // afull[3], aempty[3], xfull[2], xempty[2], accfull, accempty, drain
+    // afull[AST], aempty[AST], xfull[2], xempty[2], accfull, drain, levfree[D]
     const uint32_t afull = su32(bars), aempty = afull + 8 * RT_AST, xfull = aempty + 8 * RT_AST;
-    const uint32_t xempty = xfull + 16, accfull = xempty + 16, accempty = accfull + 8, drain = accempty + 8;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * RT_AST + 7);
+    const uint32_t xempty = xfull + 16, accfull = xempty + 16, drain = accfull + 8, levfree = drain + 8;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * RT_AST + 6 + RT_D);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     // ---- work unit: product q, row tile, K split z, column tile ----
@@ -197,7 +220,8 @@ __global__ void __launch_bounds__(RT_THREADS, 1) resid_tc_kernel(const __grid_co
     const int nchunks = (nkb + RT_KB_CHUNK - 1) / RT_KB_CHUNK;
     const int row0 = it * RT_BM, col0 = tn * RT_NT;
     const int ncols = min(RT_NT, J.n - col0);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // (the shuffle tells the compiler that the warp index is uniform)
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < RT_AST; ++s) {
@@ -209,8 +233,8 @@ __global__ void __launch_bounds__(RT_THREADS, 1) resid_tc_kernel(const __grid_co
             mbar_init(xempty + 8 * s, 1);
         }
         mbar_init(accfull, 1);
-        mbar_init(accempty, 256);  // the eight reading warps
         mbar_init(drain, 1);
+        for (int l = 0; l < RT_D; ++l) mbar_init(levfree + 8 * l, 8);  // the eight reading warps
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -234,18 +258,28 @@ __global__ void __launch_bounds__(RT_THREADS, 1) resid_tc_kernel(const __grid_co
             const int kx = (kb0 + kb) * RT_BK;
             mbar_expect_tx(xfull + 8 * xb, RT_X_BUF);
             uint8_t* xbuf = sX + xb * RT_X_BUF;
-            // shared layout: the seven real-part digit tiles, then the seven imaginary-part ones
-            for (int pl = 0; pl < 2 * RT_D; ++pl)
-                tma_load_3d(su32(xbuf + ((pl & 1) * RT_D + (pl >> 1)) * RT_TILE_X), &P.tmX, xfull + 8 * xb, kx, col0,
-                            pl);
+            if constexpr (STACK) {
+                tma_load_4d(su32(xbuf), &P.tmX[0], xfull + 8 * xb, kx, col0, 0, 0);
+                tma_load_4d(su32(xbuf + Cfg::X_STACK), &P.tmX[1], xfull + 8 * xb, kx, col0, 0, 0);
+            } else {
+                // shared layout: the real-part digit tiles, then the imaginary-part ones
+                for (int pl = 0; pl < 2 * RT_D; ++pl)
+                    tma_load_3d(su32(xbuf + ((pl & 1) * RT_D + (pl >> 1)) * RT_TILE_X), &P.tmX[0], xfull + 8 * xb, kx,
+                                col0, pl);
+            }
             x_issued = kb + 1;
-            for (int d = 0; d < RT_D; ++d) {
-                const int idx = kb * RT_D + d, s = idx % RT_AST;
+            for (int u2 = 0; u2 < USES; ++u2) {
+                const int idx = kb * USES + u2, s = idx % RT_AST;
                 if (idx >= RT_AST && !mbar_wait(aempty + 8 * s, (uint32_t)(idx / RT_AST - 1) & 1u, abort_flag)) break;
                 uint8_t* as = sA + s * RT_A_STAGE;
                 mbar_expect_tx(afull + 8 * s, RT_A_STAGE);
-                tma_load_3d(su32(as), &P.tmA, afull + 8 * s, kx, row0, 2 * d);
-                tma_load_3d(su32(as + RT_TILE_A), &P.tmA, afull + 8 * s, kx, row0, 2 * d + 1);
+                const int d = RT_D - 1 - u2 * Cfg::A_PL / 2;  // from the last digit to the first
+                if constexpr (STACK) {
+                    tma_load_3d(su32(as), &P.tmA, afull + 8 * s, kx, row0, 2 * d + (u2 & 1));
+                } else {
+                    tma_load_3d(su32(as), &P.tmA, afull + 8 * s, kx, row0, 2 * d);
+                    tma_load_3d(su32(as + RT_TILE_A), &P.tmA, afull + 8 * s, kx, row0, 2 * d + 1);
+                }
                 a_issued = idx + 1;
             }
         }
@@ -262,55 +296,103 @@ __global__ void __launch_bounds__(RT_THREADS, 1) resid_tc_kernel(const __grid_co
                 }
             }
         }
-    } else if (warp == 1 && lane == 0) {
-        // ---------------- MMA issuer ----------------
+    } else if (warp == 1) {
+        // ---------------- MMA issuer (the whole warp walks the loop, lane 0 issues) ----------------
+        const bool leader = lane == 0;
+        const uint32_t xlo0 = desc_lo(su32(sX)), alo0 = desc_lo(su32(sA));
         bool ok = true;
+        int s = 0;             // stage
+        uint32_t sph = 0;      // its phase
         for (int kb = 0; kb < nkb && ok; ++kb) {
-            const int ch = kb / RT_KB_CHUNK, first_of_chunk = (kb % RT_KB_CHUNK) == 0;
-            // the readers have taken the previous chunk's level sums out of tensor memory
-            if (first_of_chunk && ch > 0 && !mbar_wait(accempty, (uint32_t)(ch - 1) & 1u, abort_flag)) break;
+            const int ch = kb / RT_KB_CHUNK;
             const int xb = kb & 1;
             if (!mbar_wait(xfull + 8 * xb, (uint32_t)(kb >> 1) & 1u, abort_flag)) break;
             fence_after();
-            const uint32_t xbase = su32(sX + xb * RT_X_BUF);
-            for (int d = 0; d < RT_D; ++d) {
-                const int idx = kb * RT_D + d, s = idx % RT_AST;
-                if (!mbar_wait(afull + 8 * s, (uint32_t)(idx / RT_AST) & 1u, abort_flag)) {
-                    ok = false;
-                    break;
-                }
-                fence_after();
-                const uint32_t ar = su32(sA + s * RT_A_STAGE), ai = ar + RT_TILE_A;
-                // x digits 0 .. 6 - d (rows 0 .. 32 (7 - d) of the stacked tiles) into levels d .. 6
-                const uint32_t nw = (uint32_t)(RT_NT * (RT_D - d));
-                const uint32_t idp = idesc_bf16(0, nw), idn = idesc_bf16(1, nw);
-                const uint32_t Dr = tmem + (uint32_t)(d * RT_NT), Di = Dr + RT_D * RT_NT;
-                const uint32_t xr = xbase, xi = xbase + RT_D * RT_TILE_X;
+            const uint32_t xlo = xlo0 + (uint32_t)xb * (RT_X_BUF >> 4);
+            // one K block; FIRST: of a chunk.  The first products of a chunk overwrite level d (and add to
+            // the levels above, which the digits before have overwritten), once the readers have taken it
+            // out of tensor memory.
+            auto block = [&](auto first) {
+                constexpr bool FIRST = decltype(first)::value;
 #pragma unroll
-                for (int kk = 0; kk < RT_BK / 16; ++kk) {
-                    const uint32_t off = kk * 32;  // 16 bf16 = 32 bytes along K inside the swizzle span
-                    const uint64_t dar = desc_sw128(ar + off), dai = desc_sw128(ai + off);
-                    const uint64_t dxr = desc_sw128(xr + off), dxi = desc_sw128(xi + off);
-                    // digit 0 of A reaches every level: its first product of a chunk overwrites them
-                    const uint32_t acc = (first_of_chunk && d == 0 && kk == 0) ? 0u : 1u;
-                    mma_bf16(Dr, dar, dxr, idp, acc);
-                    mma_bf16(Dr, dai, dxi, idn, 1u);
-                    mma_bf16(Di, dar, dxi, idp, acc);
-                    mma_bf16(Di, dai, dxr, idp, 1u);
+                for (int u2 = 0; u2 < USES; ++u2) {
+                    const int d = RT_D - 1 - u2 * Cfg::A_PL / 2;
+                    const bool fresh = FIRST && (!STACK || (u2 & 1) == 0);
+                    if ((fresh && ch > 0 && !mbar_wait(levfree + 8 * d, (uint32_t)(ch - 1) & 1u, abort_flag)) ||
+                        !mbar_wait(afull + 8 * s, sph, abort_flag)) {
+                        ok = false;
+                        return;
+                    }
+                    fence_after();
+                    const uint32_t alo = alo0 + (uint32_t)s * (RT_A_STAGE >> 4);
+                    if constexpr (STACK) {
+                        // x digits 0 .. D - 1 - d (both parts) into levels d .. D - 1
+                        const uint32_t blo = xlo + (uint32_t)(u2 & 1) * (Cfg::X_STACK >> 4);
+                        const uint32_t Dl = tmem + (uint32_t)(2 * RT_NT * d);
+                        const uint32_t n1 = 2 * RT_NT, nw = n1 * (uint32_t)(RT_D - d);
+#pragma unroll
+                        for (int kk = 0; kk < RT_BK / 16; ++kk) {
+                            const uint32_t off = kk * 2;  // 16 bf16 = 32 bytes along K inside the swizzle span
+                            const bool over = fresh && kk == 0;
+                            if (over || nw > 256) {
+                                mma_bf16(leader, Dl, alo + off, blo + off, idesc_bf16(0, n1), over ? 0u : 1u);
+                                if (nw > n1)
+                                    mma_bf16(leader, Dl + n1, alo + off, blo + (2 * RT_TILE_X >> 4) + off,
+                                             idesc_bf16(0, nw - n1), 1u);
+                            } else {
+                                mma_bf16(leader, Dl, alo + off, blo + off, idesc_bf16(0, nw), 1u);
+                            }
+                        }
+                    } else {
+                        const uint32_t ail = alo + (RT_TILE_A >> 4);
+                        const uint32_t nw = (uint32_t)(RT_NT * (RT_D - d));
+                        const uint32_t idp = idesc_bf16(0, nw), idn = idesc_bf16(1, nw);
+                        const uint32_t Dr = tmem + (uint32_t)(d * RT_NT), Di = Dr + RT_D * RT_NT;
+                        const uint32_t xr = xlo, xi = xlo + (RT_D * RT_TILE_X >> 4);
+#pragma unroll
+                        for (int kk = 0; kk < RT_BK / 16; ++kk) {
+                            const uint32_t off = kk * 2;
+                            if (fresh && kk == 0) {
+                                const uint32_t id1 = idesc_bf16(0, RT_NT), idw = idesc_bf16(0, nw - RT_NT);
+                                mma_bf16(leader, Dr, alo, xr, id1, 0u);
+                                mma_bf16(leader, Di, alo, xi, id1, 0u);
+                                if (nw > RT_NT) {
+                                    mma_bf16(leader, Dr + RT_NT, alo, xr + (RT_TILE_X >> 4), idw, 1u);
+                                    mma_bf16(leader, Di + RT_NT, alo, xi + (RT_TILE_X >> 4), idw, 1u);
+                                }
+                            } else {
+                                mma_bf16(leader, Dr, alo + off, xr + off, idp, 1u);
+                                mma_bf16(leader, Di, alo + off, xi + off, idp, 1u);
+                            }
+                            mma_bf16(leader, Dr, ail + off, xi + off, idn, 1u);
+                            mma_bf16(leader, Di, ail + off, xr + off, idp, 1u);
+                        }
+                    }
+                    if (leader) mma_commit(aempty + 8 * s);
+                    if (++s == RT_AST) {
+                        s = 0;
+                        sph ^= 1u;
+                    }
                 }
-                mma_commit(aempty + 8 * s);
-            }
+            };
+            if (kb % RT_KB_CHUNK == 0)
+                block(std::true_type{});
+            else
+                block(std::false_type{});
             if (!ok) break;
-            mma_commit(xempty + 8 * xb);
-            if ((kb % RT_KB_CHUNK) == RT_KB_CHUNK - 1 || kb == nkb - 1) mma_commit(accfull);
+            if (leader) {
+                mma_commit(xempty + 8 * xb);
+                if ((kb % RT_KB_CHUNK) == RT_KB_CHUNK - 1 || kb == nkb - 1) mma_commit(accfull);
+            }
         }
-        if (*abort_flag) {
+        if (*abort_flag && leader) {
             // products already issued finish before tensor memory and shared memory are released
             mma_commit(drain);
             const uint64_t t0 = gtimer();
             while (!mbar_try(drain, 0u) && gtimer() - t0 < RT_WAIT_NS) {
             }
         }
+        __syncwarp();
     } else if (warp >= 2) {
         // ---------------- level-sum readers: warps 2-5 real parts, 6-9 imaginary parts ----------------
         const int qw = warp & 3;  // tensor-memory lane quarter this warp may read
@@ -322,38 +404,43 @@ __global__ void __launch_bounds__(RT_THREADS, 1) resid_tc_kernel(const __grid_co
         for (int ch = 0; ch < nchunks; ++ch) {
             if (!mbar_wait(accfull, (uint32_t)ch & 1u, abort_flag)) break;
             fence_after();
+            float th[RT_NT], tl[RT_NT];
 #pragma unroll
-            for (int g = 0; g < RT_NT / 16; ++g) {
-                float th[16], tl[16];
-#pragma unroll
-                for (int j = 0; j < 16; ++j) th[j] = tl[j] = 0.f;
-                // level sums are exact integers; scale by 128^-l (exact) and add in double-float
+            for (int j = 0; j < RT_NT; ++j) th[j] = tl[j] = 0.f;
+            // level sums are exact integers; scale by 128^-l (exact) and add in double-float, the last
+            // level first, each released to the next chunk's products when it has been read
 #pragma unroll 1
-                for (int lev = 0; lev < RT_D; ++lev) {
+            for (int lev = RT_D - 1; lev >= 0; --lev) {
+                const float w = __int_as_float((127 - 7 * lev) << 23);  // 2^(-7 lev)
+#pragma unroll
+                for (int g = 0; g < RT_NT / 16; ++g) {
                     float v[16];
-                    tmem_ld16(tmem + lane_off + (uint32_t)(part * RT_D * RT_NT + lev * RT_NT + g * 16), v);
-                    const float w = __int_as_float((127 - 7 * lev) << 23);  // 2^(-7 lev)
+                    tmem_ld16(tmem + lane_off + (uint32_t)(STACK ? 2 * RT_NT * lev + RT_NT * part + g * 16
+                                                                 : part * RT_D * RT_NT + lev * RT_NT + g * 16), v);
+                    if (g == RT_NT / 16 - 1) {
+                        fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(levfree + 8 * lev);
+                    }
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
                         float hi, lo;
-                        two_sum(hi, lo, th[j], v[j] * w);
-                        th[j] = hi;
-                        tl[j] = __fadd_rn(tl[j], lo);
+                        two_sum(hi, lo, th[g * 16 + j], v[j] * w);
+                        th[g * 16 + j] = hi;
+                        tl[g * 16 + j] = __fadd_rn(tl[g * 16 + j], lo);
                     }
                 }
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    // (sh, sl) += (th, tl)
-                    float hi, lo;
-                    two_sum(hi, lo, sh[g * 16 + j], th[j]);
-                    lo = __fadd_rn(lo, __fadd_rn(sl[g * 16 + j], tl[j]));
-                    const float s2 = __fadd_rn(hi, lo);
-                    sl[g * 16 + j] = __fsub_rn(lo, __fsub_rn(s2, hi));
-                    sh[g * 16 + j] = s2;
-                }
             }
-            fence_before();
-            mbar_arrive(accempty);
+#pragma unroll
+            for (int j = 0; j < RT_NT; ++j) {
+                // (sh, sl) += (th, tl)
+                float hi, lo;
+                two_sum(hi, lo, sh[j], th[j]);
+                lo = __fadd_rn(lo, __fadd_rn(sl[j], tl[j]));
+                const float s2 = __fadd_rn(hi, lo);
+                sl[j] = __fsub_rn(lo, __fsub_rn(s2, hi));
+                sh[j] = s2;
+            }
         }
         if (!*abort_flag) {
             const int row = row0 + qw * 32 + lane;
@@ -506,6 +593,9 @@ __global__ void digits_a_kernel(const double2* __restrict__ A, long lda, int row
     }
 }
 
+// minus a bf16 bit pattern (zero stays +0)
+__device__ __forceinline__ unsigned short bf16_neg(unsigned short b) { return b == 0 ? b : (unsigned short)(b ^ 0x8000u); }
+
 // Column exponents of x over rows [r0, r0 + K) for the n columns (one block per column).
 __global__ void col_exponent_kernel(const double2* __restrict__ X, long ldx, int r0, int K, int* __restrict__ f) {
     const int c = blockIdx.x;
@@ -526,23 +616,31 @@ __global__ void col_exponent_kernel(const double2* __restrict__ X, long ldx, int
     }
 }
 
-// Digit planes of x rows [r0, r0 + K) (columns c < n; columns up to npad are zero): plane 2d + part,
-// layout [col][ldk].
+// Digit planes of x rows [r0, r0 + K) (columns c < n; columns up to npad are zero), layout [col][ldk]:
+// plane 2 d + part, or (stack) planes 3 d .. 3 d + 2 = -Im, Re, Im.
 __global__ void digits_x_kernel(const double2* __restrict__ X, long ldx, int r0, int K, int n, int npad,
                                 const int* __restrict__ f, __nv_bfloat16* __restrict__ D, long ldk, long plane,
-                                int nd) {
+                                int nd, int stack) {
     const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (long)npad * K) return;
     const int c = (int)(idx / K), k = (int)(idx % K);
     __nv_bfloat16* o = D + (long)c * ldk + k;
     if (c >= n) {
-        for (int p = 0; p < 2 * nd; ++p) o[p * plane] = __float2bfloat16_rn(0.f);
+        for (int p = 0; p < (stack ? 3 : 2) * nd; ++p) o[p * plane] = __float2bfloat16_rn(0.f);
         return;
     }
     const double2 v = X[r0 + k + (long)c * ldx];
     const int ex = f[c];
-    digits_of(v.x, ex, nd, o, 2 * plane);
-    digits_of(v.y, ex, nd, o + plane, 2 * plane);
+    if (stack) {
+        digits_of(-v.y, ex, nd, o, 3 * plane);
+        digits_of(v.x, ex, nd, o + plane, 3 * plane);
+        for (int d = 0; d < nd; ++d)
+            reinterpret_cast<unsigned short*>(o)[(3 * d + 2) * plane] =
+                bf16_neg(reinterpret_cast<unsigned short*>(o)[3 * d * plane]);
+    } else {
+        digits_of(v.x, ex, nd, o, 2 * plane);
+        digits_of(v.y, ex, nd, o + plane, 2 * plane);
+    }
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 rt_encode() {
@@ -587,8 +685,42 @@ bm_status rt_make_map(void* tmap, const void* base, long rows, long K, long ldk,
     return BM_OK;
 }
 
+// Tensor maps of the x digit planes (two blobs): the 3-D map of seven digits, or the two stacks of nine,
+// [Re | Im] and [-Im | Re] per digit (4-D: K, columns, two consecutive planes, digits three planes apart).
+bm_status rt_make_map_x(void* tmaps, const void* base, long cols, long K, long ldk, int nd) {
+    const long plane = cols * ldk;
+    if (nd <= 7) return rt_make_map(tmaps, base, cols, K, ldk, plane, rt_col_tile(nd), nd);
+    PFN_cuTensorMapEncodeTiled_v12000 enc = rt_encode();
+    if (enc == nullptr) {
+        bm_set_error("cuTensorMapEncodeTiled is unavailable from the driver");
+        return BM_ECUDA;
+    }
+    if ((reinterpret_cast<uintptr_t>(base) & 15) != 0 || (ldk * 2) % 16 != 0) {
+        bm_set_error("digit-plane tensor map: base or stride not 16-byte aligned");
+        return BM_EINVAL;
+    }
+    for (int q = 0; q < 2; ++q) {
+        cuuint64_t dims[4] = {(cuuint64_t)K, (cuuint64_t)cols, 2, (cuuint64_t)nd};
+        cuuint64_t strides[3] = {(cuuint64_t)ldk * 2, (cuuint64_t)plane * 2, (cuuint64_t)plane * 6};
+        cuuint32_t box[4] = {(cuuint32_t)RT_BK, (cuuint32_t)rt_col_tile(nd), 2, (cuuint32_t)nd};
+        cuuint32_t estr[4] = {1, 1, 1, 1};
+        // q = 0: planes Re, Im of each digit; q = 1: planes -Im, Re
+        unsigned char* from = const_cast<unsigned char*>(static_cast<const unsigned char*>(base)) + (q == 0 ? plane * 2 : 0);
+        CUresult r = enc(reinterpret_cast<CUtensorMap*>(static_cast<unsigned char*>(tmaps) + 128 * q),
+                         CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, from, dims, strides, box, estr,
+                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (r != CUDA_SUCCESS) {
+            bm_set_error("cuTensorMapEncodeTiled (digit stacks) failed with code " + std::to_string((int)r));
+            return BM_ECUDA;
+        }
+    }
+    return BM_OK;
+}
+
 long rt_ldk(long K) { return (K + RT_BK - 1) / RT_BK * RT_BK; }
 int rt_digit_planes(int nd) { return 2 * nd; }
+int rt_x_planes(int nd) { return nd <= 7 ? 2 * nd : 3 * nd; }
 int rt_col_tile(int nd) { return nd <= 7 ? RtCfg<7>::NT : RtCfg<9>::NT; }
 
 // Row exponents and digit planes of A; rowmax is scratch of `rows` 8-byte words.
@@ -607,12 +739,12 @@ cudaError_t launch_digits_a(cudaStream_t s, const double2* A, long lda, int rows
 }
 
 cudaError_t launch_digits_x(cudaStream_t s, const double2* X, long ldx, int r0, int K, int n, int npad, int* f,
-                            void* D, long ldk, int nd) {
+                            void* D, long ldk, long plane, int nd) {
     if (n <= 0 || K <= 0) return cudaSuccess;
     col_exponent_kernel<<<n, 256, 0, s>>>(X, ldx, r0, K, f);
     const long t = (long)npad * K;
     digits_x_kernel<<<ceil_div(t, 256L), 256, 0, s>>>(X, ldx, r0, K, n, npad, f, reinterpret_cast<__nv_bfloat16*>(D),
-                                                      ldk, (long)npad * ldk, nd);
+                                                      ldk, plane, nd, nd > 7);
     return cudaGetLastError();
 }
 
@@ -665,7 +797,7 @@ cudaError_t gemm_rt(cudaStream_t s, const RtArgs* prods, int nprod, int n, doubl
             const RtArgs& a = prods[q];
             RtProd& p = J.p[q];
             std::memcpy(&p.tmA, a.tmA, sizeof(CUtensorMap));
-            std::memcpy(&p.tmX, a.tmX, sizeof(CUtensorMap));
+            std::memcpy(p.tmX, a.tmX, (nd <= 7 ? 1 : 2) * sizeof(CUtensorMap));
             p.eA = a.eA;
             p.fX = a.fX;
             p.C = a.C;

@@ -283,7 +283,8 @@ bm_status residual_tc(bm_ctx* c, const double2* B, const double2* X, double2* R,
         for (int q = 0; q < nprod; ++q) {
             const int r0 = (c->form == BM_MIXED && q == 0) ? 2 * N : 0;
             const int K = (c->form == BM_MIXED && q == 0) ? N : 2 * N;
-            SV_CUDA(launch_digits_x(s, X, ld, r0, K, nrhs, npad, c->d_dxe[q], c->d_dx[q], c->dx_ldk[q], c->rt_nd));
+            SV_CUDA(launch_digits_x(s, X, ld, r0, K, nrhs, npad, c->d_dxe[q], c->d_dx[q], c->dx_ldk[q],
+                                    c->dx_cols * c->dx_ldk[q], c->rt_nd));
         }
     }
     // mixed: Mbot (K = 2N, the longer units) first, then Mtop; ordinary: A
