@@ -65,9 +65,13 @@ cudaMemPool_t device_pool(int dev) {
 }
 }  // namespace
 
+namespace {
+void dg_release(bm_ctx* c);
+}
 bm_status ctx_alloc(bm_ctx* c, void** p, size_t bytes) {
     *p = nullptr;
     if (bytes == 0) return BM_OK;
+    if (c->held + bytes > c->budget && c->d_dgw) dg_release(c);
     if (c->held + bytes > c->budget) {
         bm_set_error("allocation of " + std::to_string(bytes) + " bytes exceeds the HBM budget");
         return BM_ENOMEM;
@@ -76,7 +80,15 @@ bm_status ctx_alloc(bm_ctx* c, void** p, size_t bytes) {
     // waits for the rest of the device, so handles that come and go (a serving loop, contour
     // workers) do not stall each other's streams
     cudaMemPool_t pool = device_pool(c->device);
-    cudaError_t e = pool ? cudaMallocFromPoolAsync(p, bytes, pool, c->stream) : cudaMallocAsync(p, bytes, c->stream);
+    auto get = [&]() {
+        return pool ? cudaMallocFromPoolAsync(p, bytes, pool, c->stream) : cudaMallocAsync(p, bytes, c->stream);
+    };
+    cudaError_t e = get();
+    if (e != cudaSuccess && c->d_dgw) {
+        cudaGetLastError();
+        dg_release(c);
+        e = get();
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         *p = nullptr;
@@ -118,6 +130,14 @@ void drop_slot(bm_ctx::GraphSlot& g) {
     if (g.exec) cudaGraphExecDestroy(g.exec);
     g.exec = nullptr;
     g.kernels = 0;
+}
+
+// Gives the optional workspace of the FP64 factorisation back (with the graphs that use it).
+void dg_release(bm_ctx* c) {
+    drop_slot(c->g_factor);
+    drop_slot(c->g_lu);
+    FREE(c->d_dgw);
+    c->dgw_bytes = 0;
 }
 
 void drop_solve_graphs(bm_ctx* c) {
@@ -183,6 +203,8 @@ void free_problem(bm_ctx* c) {
     FREE(c->d_Qbot);
     FREE(c->d_QA);
     FREE(c->d_F64);
+    FREE(c->d_dgw);
+    c->dgw_bytes = 0;
     FREE(c->d_F32r);
     FREE(c->d_F32i);
     FREE(c->d_ipiv);
@@ -205,6 +227,7 @@ void free_problem(bm_ctx* c) {
         FREE(c->d_dge[q]);
     }
     c->assembled = c->factored = c->singular = false;
+    c->fast_denied = false;
     c->tm_ok = false;
     c->tc_skinny = false;
 }
@@ -214,7 +237,8 @@ double2 d2(bm_c64 z) { return make_double2(z.re, z.im); }
 
 long round_up(long a, long b) { return (a + b - 1) / b * b; }
 
-Plan make_plan(int N, int form, int prec, int nb_user, int bs, int nd) {
+// fast: the FP32 LU in search-free blocks (lu_fast.cu), with its work buffer
+Plan make_plan(int N, int form, int prec, int nb_user, int bs, int nd, bool fast) {
     Plan p;
     const bool c32 = prec != BM_FP64;
     const bool split = prec == BM_CF32_3XTF32_IR;
@@ -250,9 +274,9 @@ Plan make_plan(int N, int form, int prec, int nb_user, int bs, int nd) {
         // packs of the trailing updates (the search-free blocks always take 3xTF32 products) and the
         // search-free blocks' work buffer
         long kl = split ? 3L * p.nb : p.nb;
-        p.ldk_lu = round_up(nb_user > 0 ? kl : std::max(kl, 3L * 128), 32);
+        p.ldk_lu = round_up(fast ? std::max(kl, 3L * 128) : kl, 32);
         b += 2 * (size_t)p.n * p.ldk_lu * 8;
-        if (nb_user == 0) b += lu_fast_bytes(p.n);
+        if (fast) b += lu_fast_bytes(p.n);
         // digit planes of the operator for the tensor-core residual, their row exponents, and the
         // row-maximum scratch of their construction
         const size_t planes = (size_t)rt_digit_planes(nd) * 2;
@@ -272,9 +296,11 @@ Plan make_plan(int N, int form, int prec, int nb_user, int bs, int nd) {
 
 // Device bytes one request needs: the assembled system and its factorisation, plus the solve
 // workspace for nrhs right-hand sides (an estimate from the same sizes ensure_ws uses, with a
-// margin for the split-K partial sums).
-size_t request_bytes(int N, int form, int prec, int nb, int nrhs) {
-    Plan p = make_plan(N, form, prec, nb, 64, 9);
+// margin for the split-K partial sums).  optional: with what a handle also takes when its budget has room
+// (the search-free LU's buffers, the FP64 digit workspace).
+size_t request_bytes(int N, int form, int prec, int nb, int nrhs, bool optional, int num_sms) {
+    Plan p = make_plan(N, form, prec, nb, 64, 9, optional && prec != BM_FP64 && nb == 0);
+    if (optional && prec == BM_FP64 && form == BM_MIXED) p.bytes += dg_bytes(N, N, 2 * N, num_sms);
     const size_t w = (size_t)std::max(nrhs, 8);
     size_t b = p.bytes + 7 * (size_t)N * 8 + (size_t)p.nsys * w * 16 * 3 + (size_t)p.n * w * 16 * 2;
     if (prec == BM_FP64) {
@@ -525,23 +551,28 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
     cudaStreamSynchronize(c->stream);
     const int rmode = opts ? opts->refine_residual : BM_RESID_TC_UPDATE;
     const int nd = rmode == BM_RESID_TC_ALL ? 9 : 7;
-    Plan p = make_plan(N, form, prec, nb, 64, nd);
-    // Same shape as the assembled system: assemble again into the same buffers (no device
-    // allocation or release - cudaFree would wait for every stream of the device - and the cached
-    // graphs and tensor maps stay valid, as they depend only on these pointers and sizes).
     // LU in search-free blocks, unless a block size or a panel setting asks for the panels (the contour
     // solver's deferred assembly sets a cluster size for what its factorisations continue with)
     const bool fast = prec != BM_FP64 && nb == 0 && pkern == 0 && (cl_cap == 0 || defer_kernels);
+    Plan p = make_plan(N, form, prec, nb, 64, nd, fast);
+    // Same shape as the assembled system: assemble again into the same buffers (no device
+    // allocation or release - cudaFree would wait for every stream of the device - and the cached
+    // graphs and tensor maps stay valid, as they depend only on these pointers and sizes).
     const bool reuse = c->assembled && c->N == N && c->form == form && c->prec == prec && c->nb == p.nb &&
-                       (c->d_fd != nullptr) == fast && c->rt_nd == nd && curve->kind != BM_CURVE_USER;
-    if (!reuse) free_problem(c);
+                       (c->d_fd != nullptr || c->fast_denied) == fast && c->rt_nd == nd && curve->kind != BM_CURVE_USER;
+    if (!reuse) {
+        free_problem(c);
+        // a budget without room for the search-free LU's buffers keeps the panels
+        c->fast_denied = fast && c->held + p.bytes > c->budget;
+    }
+    if (c->fast_denied) p = make_plan(N, form, prec, nb, 64, nd, false);
     // the captured factorisation depends on the launch settings: capture again when they change
     if (reuse && (eager != c->eager || cl_cap != c->opt_cluster_cap || pkern != c->opt_panel_kernel))
         drop_graphs(c);
     c->eager = eager;
     c->opt_cluster_cap = cl_cap;
     c->opt_panel_kernel = pkern;
-    c->lu_fast = fast;
+    c->lu_fast = fast && !c->fast_denied;
     c->bs_solve = 64;
     if (!reuse && c->held + p.bytes > c->budget) {
         bm_set_error("admission: system needs " + std::to_string(p.bytes) + " bytes, budget leaves " +
@@ -613,7 +644,7 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
         if (s == BM_OK) s = alloc_t(c, &c->d_Lp_i, lb);
         if (s == BM_OK) s = alloc_t(c, &c->d_Up_r, lb);
         if (s == BM_OK) s = alloc_t(c, &c->d_Up_i, lb);
-        if (s == BM_OK && fast) s = alloc_t(c, &c->d_fd, lu_fast_bytes(p.n));
+        if (s == BM_OK && c->lu_fast) s = alloc_t(c, &c->d_fd, lu_fast_bytes(p.n));
     }
     if (s == BM_OK && c32) {
         // [0] Mtop (2N x N) or A (2N x 2N), [1] Mbot (N x 2N)
@@ -766,6 +797,29 @@ bm_status assemble_post(bm_ctx* c, bool run_assembly_kernel, bool wait) {
     return BM_OK;
 }
 
+// Reserves the digit workspace of an FP64 factorisation where the budget and the device have room for it
+// (without it the products run on the CUDA cores).
+void dg_reserve(bm_ctx* c) {
+    if (c->prec != BM_FP64 || c->d_dgw) return;
+    const size_t b = c->form == BM_MIXED ? dg_bytes(c->N, c->N, 2 * c->N, c->num_sms) : 0;
+    if (b == 0 || c->held + b > c->budget) return;
+    if (alloc_t(c, &c->d_dgw, b) == BM_OK) c->dgw_bytes = b;
+}
+
+bm_status schur_z64(bm_ctx* c, cudaStream_t s) {
+    const int N = c->N;
+    const Z64 F{c->d_F64, c->ldF}, A{c->d_Mbot, c->ldbot}, B{c->d_Mtop, c->ldtop};
+    const size_t b = dg_bytes(N, N, 2 * N, c->num_sms);
+    if (b == 0 || b > c->dgw_bytes) {
+        BM_PROF(c, "cgemm_simt_kernel<Z64> (Schur complement)");
+        BM_CUDA_TRY(gemm_z64(s, N, N, 2 * N, -1.0, A, false, B, 0.0, F));
+        return BM_OK;
+    }
+    BM_PROF(c, "resid_tc_kernel (Schur complement)");
+    BM_CUDA_TRY(cudaMemset2DAsync(F.p, (size_t)F.ld * 16, 0, (size_t)N * 16, N, s));
+    return gemm_z64_dg(s, c->d_dgw, c->num_sms, N, N, 2 * N, -1.0, A, B, F, c->d_err);
+}
+
 // ------------------------------------------------------------------------------------------------
 namespace {
 
@@ -777,10 +831,7 @@ bm_status factor_sequence(bm_ctx* c) {
     if (c->prec == BM_FP64) {
         Z64 F{c->d_F64, c->ldF};
         if (c->form == BM_MIXED) {
-            // U33 = -[M31 M32] [M13; M23]
-            BM_PROF(c, "cgemm_simt_kernel<Z64> (Schur complement)");
-            BM_CUDA_TRY(gemm_z64(s, c->N, c->N, 2 * c->N, -1.0, Z64{c->d_Mbot, c->ldbot}, false,
-                                 Z64{c->d_Mtop, c->ldtop}, 0.0, F));
+            BM_TRY(schur_z64(c, s));  // U33 = -[M31 M32] [M13; M23]
         } else {
             BM_PROF(c, "copy_z64_kernel");
             BM_CUDA_TRY(launch_copy_z64(s, c->d_A, c->ldA, c->n, c->n, c->d_F64, c->ldF));
@@ -909,6 +960,7 @@ extern "C" bm_status bm_factor(bm_ctx* c, int* info) {
         return BM_ESTATE;
     }
     BM_CUDA_TRY(cudaSetDevice(c->device));
+    dg_reserve(c);
     BM_TRY(run_captured(c, &c->g_factor, [&]() { return factor_sequence(c); }));
     return factor_result(c, info);
 }

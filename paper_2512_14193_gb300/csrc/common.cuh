@@ -286,6 +286,8 @@ struct bm_ctx {
 
     // factorisation storage
     double2* d_F64 = nullptr;  // FP64 LU (n x n, ld ldF)
+    void* d_dgw = nullptr;     // FP64: workspace of the digit products of the factorisation.  Optional: it
+    size_t dgw_bytes = 0;      //   is given back when another allocation needs the room (ctx_alloc)
     float* d_F32r = nullptr;   // FP32 planar LU
     float* d_F32i = nullptr;
     long ldF = 0;
@@ -294,7 +296,8 @@ struct bm_ctx {
     int* d_info = nullptr;
     int* d_err = nullptr;      // d_info + 1; d_info[2..3] test hooks, d_info[4] stop word of lu_fast.cu
     bool lu_fast = false;      // FP32 LU in blocks without a pivot search (lu_fast.cu) and their
-    float* d_fd = nullptr;     //   work buffer: the default, unless bm_opts.nb or panel_kernel is set
+    float* d_fd = nullptr;     //   work buffer: the default, unless bm_opts.nb or a panel setting is set
+    bool fast_denied = false;  //   or the budget has no room for the buffer
     void* d_maps = nullptr;    // row-interchange maps used by the factorisation: big panel (even),
                                // sub-panel, big panel (odd)
     // look-ahead of the FP32 factorisation: the panel chain on la_hi (high priority), the rest of
@@ -420,7 +423,7 @@ struct ProfScope {
 // allocation helpers (api.cu)
 bm_status ctx_alloc(bm_ctx* c, void** p, size_t bytes);
 void ctx_free(bm_ctx* c, void* p);
-size_t request_bytes(int N, int form, int prec, int nb, int nrhs);  // api.cu
+size_t request_bytes(int N, int form, int prec, int nb, int nrhs, bool optional, int num_sms);  // api.cu
 void ctx_release(bm_ctx* c);                                        // api.cu
 
 // ---------------------------------------------------------------------------------------------

@@ -129,6 +129,15 @@ cudaError_t launch_digits_x(cudaStream_t s, const double2* X, long ldx, int r0, 
 cudaError_t gemm_rt(cudaStream_t s, const RtArgs* prods, int nprod, int n, double alpha, int* d_err, int* launched,
                     int nd);
 
+// FP64 products from nine-digit products (FP64 precision): workspace (0: the CUDA cores are the better
+// place), and C += alpha A B
+size_t dg_bytes(int m, int n, int K, int num_sms);
+bm_status gemm_z64_dg(cudaStream_t s, void* work, int num_sms, int m, int n, int K, double alpha, Z64 A, Z64 B, Z64 C,
+                      int* d_err);
+
+// api.cu: the Schur complement of the FP64 precision into d_F64 (the workspace reserved before any capture)
+void dg_reserve(bm_ctx* c);
+bm_status schur_z64(bm_ctx* c, cudaStream_t s);
 // api.cu: assembly in two halves (the batched contour solver assembles many handles at once)
 bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, bm_c64 k_in, bm_formulation form,
                         const bm_opts* opts, bool defer_kernels);

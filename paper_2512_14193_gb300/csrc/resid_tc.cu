@@ -828,3 +828,84 @@ cudaError_t gemm_rt(cudaStream_t s, const RtArgs* prods, int nprod, int n, doubl
     }
     return cudaGetLastError();
 }
+
+// ------------------------------------------------------------------------------------------------
+// FP64 products C += alpha A B (column-major, C initialised) from nine-digit products: the Schur
+// complement and the trailing updates of the FP64 precision.  Each row of A and column of B is good to
+// 2^-64 of its largest entry, ten bits past FP64's own rounding of that entry, and sums are kept in
+// double-float: the error against 64 bits is that of an FP64 product or below (N = 1000 Schur
+// complement 14.0 -> 0.9 ms; the FP64 pipe runs 304 multiply-adds a cycle on the whole chip).
+// The operands' digit planes are made per call in the workspace, in chunks of rows and columns when it
+// does not hold them all.
+// ------------------------------------------------------------------------------------------------
+namespace {
+constexpr int DG_ND = 9;
+struct DgPlan {
+    int mr, nc;       // rows and columns per chunk
+    size_t a, x, w;   // bytes: A planes with exponents and row maxima, X planes with exponents, K-split sums
+};
+size_t al256(size_t v) { return (v + 255) / 256 * 256; }
+size_t dg_a_bytes(int mr, int K) { return al256((size_t)2 * DG_ND * mr * rt_ldk(K) * 2) + al256((size_t)mr * 4) + al256((size_t)mr * 8); }
+size_t dg_x_bytes(int nc, int K) { return al256((size_t)rt_x_planes(DG_ND) * nc * rt_ldk(K) * 2) + al256((size_t)nc * 4); }
+DgPlan dg_plan(int m, int n, int K, int num_sms) {
+    constexpr size_t CAP = (size_t)512 << 20;  // per operand
+    DgPlan p{};
+    const int nt = rt_col_tile(DG_ND);
+    const long ar = (long)(CAP / ((size_t)4 * DG_ND * rt_ldk(K))) / RT_BM * RT_BM;
+    const long xc = (long)(CAP / ((size_t)2 * rt_x_planes(DG_ND) * rt_ldk(K))) / nt * nt;
+    p.mr = (int)std::min<long>(m, std::max<long>(ar, RT_BM));
+    p.nc = (int)std::min<long>(ceil_div(n, nt) * (long)nt, std::max<long>(xc, nt));
+    p.a = dg_a_bytes(p.mr, K);
+    p.x = dg_x_bytes(p.nc, K);
+    const long mq = p.mr, kq = K;
+    int S = 1;
+    rt_plan_splits(1, &mq, &kq, std::min(p.nc, n), DG_ND, num_sms, &S);
+    p.w = S > 1 ? al256((size_t)2 * S * p.mr * std::min(p.nc, n) * 8) : 0;
+    return p;
+}
+}  // namespace
+
+// Workspace one product needs, and whether it is worth it: below about 60 us of FP64 multiply-adds the
+// digit conversions cost more than they save.
+size_t dg_bytes(int m, int n, int K, int num_sms) {
+    if ((double)m * n * K < 9e6) return 0;
+    const DgPlan p = dg_plan(m, n, K, num_sms);
+    return p.a + p.x + p.w;
+}
+
+bm_status gemm_z64_dg(cudaStream_t s, void* work, int num_sms, int m, int n, int K, double alpha, Z64 A, Z64 B, Z64 C,
+                      int* d_err) {
+    const DgPlan p = dg_plan(m, n, K, num_sms);
+    const int nt = rt_col_tile(DG_ND);
+    const long ldk = rt_ldk(K);
+    unsigned char* w = static_cast<unsigned char*>(work);
+    void* ap = w;
+    int* ea = reinterpret_cast<int*>(w + al256((size_t)2 * DG_ND * p.mr * ldk * 2));
+    void* rmax = reinterpret_cast<unsigned char*>(ea) + al256((size_t)p.mr * 4);
+    unsigned char* xp = w + p.a;
+    int* fx = reinterpret_cast<int*>(xp + al256((size_t)rt_x_planes(DG_ND) * p.nc * ldk * 2));
+    double* ws = reinterpret_cast<double*>(xp + p.x);
+    alignas(64) unsigned char tma[128], tmx[256];
+    BM_TRY(rt_make_map_x(tmx, xp, p.nc, K, ldk, DG_ND));
+    for (int i0 = 0; i0 < m; i0 += p.mr) {
+        const int mr = std::min(p.mr, m - i0);
+        BM_CUDA_TRY(launch_digits_a(s, A.p + i0, A.ld, mr, K, ea, ap, ldk, rmax, DG_ND));
+        BM_TRY(rt_make_map(tma, ap, mr, K, ldk, (long)mr * ldk, RT_BM, DG_ND));
+        for (int j0 = 0; j0 < n; j0 += p.nc) {
+            const int nc = std::min(p.nc, n - j0);
+            BM_CUDA_TRY(launch_digits_x(s, B.p + (long)j0 * B.ld, B.ld, 0, K, nc, ceil_div(nc, nt) * nt, fx, xp, ldk,
+                                        (long)p.nc * ldk, DG_ND));
+            const long mq = mr, kq = K;
+            int S = 1, nl = 0;
+            rt_plan_splits(1, &mq, &kq, nc, DG_ND, num_sms, &S);
+            while (S > 1 && (size_t)2 * S * mr * nc * 8 > p.w) --S;
+            RtArgs a{tma, tmx, ea, fx, C.p + i0 + (long)j0 * C.ld, C.ld, nullptr, nullptr, mr, K, S};
+            if (S > 1) {
+                a.Wr = ws;
+                a.Wi = ws + (size_t)S * mr * nc;
+            }
+            BM_CUDA_TRY(gemm_rt(s, &a, 1, nc, alpha, d_err, &nl, DG_ND));
+        }
+    }
+    return BM_OK;
+}

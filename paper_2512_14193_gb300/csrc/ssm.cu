@@ -244,8 +244,8 @@ bm_status factor_batch(Batch& bt, int B) {
         for (int b = 0; b < B; ++b) {
             bm_ctx* c = bt.h[b];
             if (c->form == BM_MIXED) {
-                SSM_CUDA(gemm_z64(c->stream, N, N, 2 * N, -1.0, Z64{c->d_Mbot, c->ldbot}, false, Z64{c->d_Mtop, c->ldtop},
-                                  0.0, Z64{c->d_F64, c->ldF}));
+                dg_reserve(c);
+                BM_TRY(schur_z64(c, c->stream));
             } else if (c->prec == BM_FP64) {
                 SSM_CUDA(launch_copy_z64(c->stream, c->d_A, c->ldA, c->n, c->n, c->d_F64, c->ldF));
             } else {
