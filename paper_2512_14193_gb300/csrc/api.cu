@@ -981,6 +981,8 @@ bm_status ensure_ws(bm_ctx* c, int nrhs) {
     BM_TRY(alloc_t(c, &c->d_Y64b, yb));
     if (c->prec == BM_FP64) {
         BM_TRY(alloc_t(c, &c->d_Zw64, yb));
+        c->flow_len = 2L * ceil_div(c->n, 16) * ceil_div(w, 4);  // two triangles x (16-row tiles) x (4-column tiles)
+        BM_TRY(alloc_t(c, &c->d_flow, (size_t)c->flow_len * sizeof(int)));
     } else {
         size_t fb = (size_t)c->nsys * w * 4;
         BM_TRY(alloc_t(c, &c->d_Wr, fb));
@@ -1120,6 +1122,15 @@ extern "C" bm_status bm_solve(bm_ctx* c, int nrhs, const bm_c64* B, int ldb, bm_
     bm_status st = BM_OK;
     if (c->prec == BM_FP64) {
         st = run_captured(c, &c->g_fp64[nrhs], [&]() { return solve_fp64(c, c->d_Bw, c->d_X, ld, nrhs); });
+        if (st == BM_OK && !info) {  // (with info the device-wait word comes with the backward error)
+            int herr = 0;
+            BM_CUDA_TRY(cudaMemcpyAsync(&herr, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
+            BM_CUDA_TRY(cudaStreamSynchronize(s));
+            if (herr != 0) {
+                bm_set_error("a bounded device wait timed out (triangular solve)");
+                st = BM_ETIMEOUT;
+            }
+        }
         if (st == BM_OK && info) {
             cudaEventRecord(r0, s);
             st = residual_fp64(c, c->d_Bw, c->d_X, c->d_R, ld, nrhs);

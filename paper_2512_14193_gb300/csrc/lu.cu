@@ -350,20 +350,17 @@ __device__ __forceinline__ void load_block(CV* dst, const CV* __restrict__ src, 
 // (the reciprocals 1 / U_kk are formed before the sweep).
 // Entries outside the rb x rb leading block are zero.
 constexpr int TI_B = 64;
-template <class V, bool UPPER, int CG>
+template <class V, bool UPPER>
 __global__ void __launch_bounds__(256) tri_inv_kernel(V F, int n, typename V::cv* __restrict__ out, const int* fail) {
     using CV = typename V::cv;
     using Rl = typename V::real;
     if (*fail != 0) return;  // the factorisation stopped (lu_fast.cu) and is continued first
-    // CG column groups (blockIdx.y): the columns of the inverse are independent, so the FP64
-    // factors, whose pipe is slow on each SM, spread one block over CG CTAs
-    constexpr int B = TI_B, M = B * B / 256 / CG;
+    constexpr int B = TI_B, M = B * B / 256;
     extern __shared__ __align__(16) unsigned char sm[];
     CV* T = reinterpret_cast<CV*>(sm);  // [B][B] column-major
     CV* buf = T + B * B;                // [2][B]
     CV* dg = buf + 2 * B;               // [B] 1 / U_kk
     const int t = threadIdx.x, i = t % B, c0 = t / B;
-    const int mg = (int)blockIdx.y * M;  // this CTA's columns: c0 + 4 (mg + m), m < M
     const long r0 = (long)blockIdx.x * B;
     const int rb = (int)min((long)B, n - r0);
     load_tile<B, B>(T, F, r0, r0, rb, rb);
@@ -372,7 +369,7 @@ __global__ void __launch_bounds__(256) tri_inv_kernel(V F, int n, typename V::cv
 #pragma unroll
     for (int m = 0; m < M; ++m) {
         x[m] = czero<Rl>();
-        if (i == c0 + 4 * (mg + m) && i < rb) x[m].x = (Rl)1;
+        if (i == c0 + 4 * m && i < rb) x[m].x = (Rl)1;
     }
     __syncthreads();
     for (int s = 0; s < rb; ++s) {
@@ -385,7 +382,7 @@ __global__ void __launch_bounds__(256) tri_inv_kernel(V F, int n, typename V::cv
                 for (int m = 0; m < M; ++m) x[m] = cmul(x[m], d);
             }
 #pragma unroll
-            for (int m = 0; m < M; ++m) bk[c0 + 4 * (mg + m)] = x[m];
+            for (int m = 0; m < M; ++m) bk[c0 + 4 * m] = x[m];
         }
         __syncthreads();
         if (UPPER ? i < k : (i > k && i < rb)) {
@@ -393,117 +390,15 @@ __global__ void __launch_bounds__(256) tri_inv_kernel(V F, int n, typename V::cv
             tik.x = -tik.x;
             tik.y = -tik.y;
 #pragma unroll
-            for (int m = 0; m < M; ++m) cfma(x[m], tik, bk[c0 + 4 * (mg + m)]);
+            for (int m = 0; m < M; ++m) cfma(x[m], tik, bk[c0 + 4 * m]);
         }
     }
     CV* o = out + (long)blockIdx.x * B * B;
 #pragma unroll
-    for (int m = 0; m < M; ++m) o[i + (c0 + 4 * (mg + m)) * B] = x[m];
+    for (int m = 0; m < M; ++m) o[i + (c0 + 4 * m) * B] = x[m];
 }
 
-// One block step of a blocked triangular solve with inverted diagonal blocks (one launch per
-// block, all right-hand sides):
-//   Zb = Tinv Y[r0:r0+rb, :]                          (written to Z by the CTAs of row tile 0)
-//   Y[rest0:rest0+nrest, :] -= F[rest0.., r0:r0+rb] Zb (each CTA one 64-row tile of the rest)
-// Forward (unit L) and backward (U) passes use the same kernel with the rows below or above the
-// block as the rest; Z is a second buffer, so no CTA reads a block that another one rewrites.
 constexpr int TS_BM = 64;
-template <class V, int BN>
-__global__ void __launch_bounds__(256) trsv_step_kernel(V F, V Y, V Z, int r0, int rb, int rest0, int nrest, int nrhs,
-                                                        int bs, const typename V::cv* __restrict__ Tinv) {
-    using CV = typename V::cv;
-    using Rl = typename V::real;
-    extern __shared__ __align__(16) unsigned char sm[];
-    CV* Ts = reinterpret_cast<CV*>(sm);  // [bs][bs] column-major
-    CV* Yb = Ts + bs * bs;               // [BN][bs]
-    CV* Zb = Yb + BN * bs;               // [BN][bs]
-    CV* Ft = Zb + BN * bs;               // [bs][TS_BM] column-major tile of F
-    const int t = threadIdx.x;
-    const int j0 = blockIdx.y * BN;
-    const int nc = min(BN, nrhs - j0);
-    for (int e = t; e < bs * bs; e += 256) Ts[e] = Tinv[e];
-    for (int e = t; e < bs * BN; e += 256) {
-        int i = e % bs, jj = e / bs;
-        Yb[jj * bs + i] = (i < rb && jj < nc) ? Y.get((long)r0 + i, (long)j0 + jj) : czero<Rl>();
-    }
-    const long tr0 = (long)rest0 + (long)blockIdx.x * TS_BM;
-    const int tm = (int)min((long)TS_BM, (long)rest0 + nrest - tr0);
-    if (nrest > 0)
-        for (int e = t; e < TS_BM * bs; e += 256) {
-            int i = e % TS_BM, k = e / TS_BM;
-            Ft[k * TS_BM + i] = (i < tm && k < rb) ? F.get(tr0 + i, (long)r0 + k) : czero<Rl>();
-        }
-    __syncthreads();
-    // register micro-tiles: thread (tx, ty) owns rows tx + 16a (a < bs/16) and columns ty + 16b
-    constexpr int TN = BN / 16;
-    const int tx = t % 16, ty = t / 16;
-    const int TMb = bs / 16;  // bs is 64: 4 rows per thread
-    {
-        CV acc[4][TN];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < TN; ++b) acc[a][b] = czero<Rl>();
-        // threads whose columns all lie past the last right-hand side skip the products (with one
-        // right-hand side, 15 of 16 column slots: the FP64 pipe is the bound of these small steps)
-        const int kend = (ty < nc) ? rb : 0;
-        for (int k = 0; k < kend; ++k) {
-            CV tv[4], yv[TN];
-#pragma unroll
-            for (int a = 0; a < 4; ++a) tv[a] = (a < TMb) ? Ts[tx + 16 * a + k * bs] : czero<Rl>();
-#pragma unroll
-            for (int b = 0; b < TN; ++b) yv[b] = Yb[(ty + 16 * b) * bs + k];
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int b = 0; b < TN; ++b) cfma(acc[a][b], tv[a], yv[b]);
-        }
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < TN; ++b)
-                if (a < TMb) Zb[(ty + 16 * b) * bs + tx + 16 * a] = acc[a][b];
-    }
-    __syncthreads();
-    if (blockIdx.x == 0)
-        for (int e = t; e < bs * BN; e += 256) {
-            int i = e % bs, jj = e / bs;
-            if (i < rb && jj < nc) Z.set((long)r0 + i, (long)j0 + jj, Zb[jj * bs + i]);
-        }
-    if (nrest <= 0) return;
-    CV acc[4][TN];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < TN; ++b) acc[a][b] = czero<Rl>();
-    const int kend2 = (ty < nc) ? rb : 0;
-    for (int k = 0; k < kend2; ++k) {
-        CV fv[4], zv[TN];
-#pragma unroll
-        for (int a = 0; a < 4; ++a) fv[a] = Ft[k * TS_BM + tx + 16 * a];
-#pragma unroll
-        for (int b = 0; b < TN; ++b) zv[b] = Zb[(ty + 16 * b) * bs + k];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < TN; ++b) cfma(acc[a][b], fv[a], zv[b]);
-    }
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        const int i = tx + 16 * a;
-        if (i >= tm) continue;
-#pragma unroll
-        for (int b = 0; b < TN; ++b) {
-            const int jj = ty + 16 * b;
-            if (jj >= nc) continue;
-            CV y = Y.get(tr0 + i, (long)j0 + jj);
-            y.x -= acc[a][b].x;
-            y.y -= acc[a][b].y;
-            Y.set(tr0 + i, (long)j0 + jj, y);
-        }
-    }
-}
-
 // G form of the factors (C32): every off-diagonal bs x bs tile F[it, b] (it != b) becomes
 // F[it, b] T_b with T_b = L_bb^{-1} below the diagonal and U_bb^{-1} above it.  One CTA per tile,
 // in place (each CTA reads its whole tile before writing it).  bs == TS_BM == 64.
@@ -816,6 +711,119 @@ __global__ void __launch_bounds__(256, 4) trsv_flow_kernel(C32 F, C32 Y, C32 Z, 
     }
 }
 
+// Inverses of the 16 x 16 diagonal blocks of the FP64 factors: a block per half warp, lane = column,
+// the unit lower triangles for blockIdx.y = 0, the upper ones for 1.  Rows and columns past n are the
+// identity's.  out: column-major 16 x 16 blocks.
+constexpr int FZ_B = 16, FZ_NC = 4;
+__global__ void __launch_bounds__(32) tri_inv16_kernel(Z64 F, int n, double2* __restrict__ outL,
+                                                       double2* __restrict__ outU, const int* fail) {
+    if (*fail != 0) return;
+    const int lane = threadIdx.x & 31, j = lane & 15, blk = (int)blockIdx.x * 2 + (lane >> 4);
+    const long r0 = (long)blk * FZ_B;
+    const bool upper = blockIdx.y == 1;
+    double2 x[FZ_B];
+    auto at = [&](int i, int k) {
+        return r0 + max(i, k) < n ? F.get(r0 + i, r0 + k) : (i == k ? make_double2(1.0, 0.0) : make_double2(0.0, 0.0));
+    };
+    if (upper) {
+        const double2 dinv = cinv(at(j, j));
+#pragma unroll
+        for (int i = FZ_B - 1; i >= 0; --i) {
+            double2 s = make_double2(i == j ? 1.0 : 0.0, 0.0);
+#pragma unroll
+            for (int k = i + 1; k < FZ_B; ++k) {
+                const double2 t = at(i, k);
+                cfma(s, make_double2(-t.x, -t.y), x[k]);
+            }
+            const int src = (lane & 16) + i;
+            x[i] = cmul(s, make_double2(__shfl_sync(0xffffffffu, dinv.x, src), __shfl_sync(0xffffffffu, dinv.y, src)));
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < FZ_B; ++i) {
+            double2 s = make_double2(i == j ? 1.0 : 0.0, 0.0);
+#pragma unroll
+            for (int k = 0; k < i; ++k) {
+                const double2 t = at(i, k);
+                cfma(s, make_double2(-t.x, -t.y), x[k]);
+            }
+            x[i] = s;
+        }
+    }
+    if (r0 >= n) return;
+    double2* o = (upper ? outU : outL) + (long)blk * FZ_B * FZ_B + j * FZ_B;
+#pragma unroll
+    for (int i = 0; i < FZ_B; ++i) o[i] = x[i];
+}
+
+// The FP64 triangular solve as one persistent cooperative launch per triangle (the scheme of
+// trsv_flow_kernel).  Work item (i, j): tile row i of 16 rows, 4 right-hand sides; it takes
+// Y[i, j] - sum_b F[i, b] X[b, j] over the tile rows before it, each as soon as ready[b, j] is set, then
+// X[i, j] = T_i (that) with the inverted 16 x 16 diagonal block, and publishes.  An SM does two FP64
+// multiply-adds a cycle, so a link of the chain costs its two 16 x 16 x 4 products (2 us) besides the flag
+// and the loads; 64-row block steps cost 77 us per block instead (each CTA recomputed the diagonal block's
+// product, padded to 16 columns).  N = 1000, four right-hand sides: 2.46 -> 0.6 ms.  Thread: row t % 16,
+// column, half of the k range.
+template <bool UPPER>
+__global__ void __launch_bounds__(128, 8) trsv_flow_z64_kernel(Z64 F, Z64 Y, Z64 X, int n, int nrhs,
+                                                               const double2* __restrict__ Tinv, int* ready, int* err) {
+    constexpr int B = FZ_B, NC = FZ_NC, KH = B / 2;
+    __shared__ double2 red[2][NC][B];
+    __shared__ double2 ys[NC][B];
+    const int t = threadIdx.x, r = t % B, c = (t / B) % NC, ks = t / (B * NC), k0 = ks * KH;
+    const int nblk = (n + B - 1) / B, ct = (nrhs + NC - 1) / NC, items = nblk * ct;
+    pdl_wait();
+    pdl_trigger();
+    for (int q = blockIdx.x; q < items; q += gridDim.x) {
+        const int i = UPPER ? nblk - 1 - q / ct : q / ct, j = q % ct;
+        const long r0 = (long)i * B, row = r0 + r;
+        const int col = j * NC + c;
+        const bool in = row < n && col < nrhs;
+        double2 f[KH], ti[KH];
+        auto load_f = [&](int b) {
+#pragma unroll
+            for (int k = 0; k < KH; ++k) {
+                const long fc = (long)b * B + k0 + k;
+                f[k] = (row < n && fc < n) ? F.get(row, fc) : make_double2(0.0, 0.0);
+            }
+        };
+        const int nsteps = UPPER ? nblk - 1 - i : i;
+        if (nsteps > 0) load_f(UPPER ? nblk - 1 : 0);
+        const double2 y0 = in ? Y.get(row, col) : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int k = 0; k < KH; ++k) ti[k] = Tinv[(long)i * B * B + (k0 + k) * B + r];
+        double2 acc = make_double2(0.0, 0.0);
+        for (int st = 0; st < nsteps; ++st) {
+            const int b = UPPER ? nblk - 1 - st : st;
+            double2 g[KH];
+#pragma unroll
+            for (int k = 0; k < KH; ++k) g[k] = f[k];
+            if (st + 1 < nsteps) load_f(UPPER ? b - 1 : b + 1);  // the next tile, while this one waits
+            flow_wait(ready + b * ct + j, err);
+            double2 x[KH];
+#pragma unroll
+            for (int k = 0; k < KH; ++k) {
+                const long xr = (long)b * B + k0 + k;
+                x[k] = (xr < n && col < nrhs) ? __ldcg(X.p + xr + (long)col * X.ld) : make_double2(0.0, 0.0);
+            }
+#pragma unroll
+            for (int k = 0; k < KH; ++k) cfma(acc, g[k], x[k]);
+        }
+        red[ks][c][r] = acc;
+        __syncthreads();
+        if (ks == 0) ys[c][r] = csub(y0, cadd(red[0][c][r], red[1][c][r]));
+        __syncthreads();
+        double2 z = make_double2(0.0, 0.0);
+#pragma unroll
+        for (int k = 0; k < KH; ++k) cfma(z, ti[k], ys[c][k0 + k]);
+        red[ks][c][r] = z;
+        __syncthreads();
+        if (ks == 0 && in) X.set(row, col, cadd(red[0][c][r], red[1][c][r]));
+        __syncthreads();  // orders every thread's rows before the release (cumulative at gpu scope)
+        if (t == 0) asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(ready + i * ct + j), "r"(1) : "memory");
+    }
+}
+
 __global__ void gather_rows_z64_kernel(const int* __restrict__ perm, int n, int nrhs, const double2* __restrict__ B,
                                        long ldb, double2* __restrict__ Y, long ldy) {
     long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -877,6 +885,14 @@ template <class V>
 bm_status finish_t(bm_ctx* c, V F, cudaStream_t s) {
     const int n = c->n;
     const int* const fail = c->d_info + 4;
+    using CV = typename V::cv;
+    if constexpr (std::is_same<V, Z64>::value) {
+        BM_PROF(c, "tri_inv_kernel");
+        tri_inv16_kernel<<<dim3(ceil_div(ceil_div(n, FZ_B), 2), 2), 32, 0, s>>>(
+            F, n, reinterpret_cast<double2*>(c->d_dinvL), reinterpret_cast<double2*>(c->d_dinvU), fail);
+        LU_CUDA(cudaGetLastError());
+        return BM_OK;
+    }
     const int bs = c->bs_solve;
     if (bs != TI_B || bs != TS_BM) {
         bm_set_error("lu: the solve block size must be 64");
@@ -884,16 +900,12 @@ bm_status finish_t(bm_ctx* c, V F, cudaStream_t s) {
     }
     const int nblk = ceil_div(n, bs);
     size_t smem = ((size_t)bs * bs + 3 * (size_t)bs) * sizeof(typename V::cv);
-    using CV = typename V::cv;
-    constexpr int CG = std::is_same<V, C32>::value ? 1 : 4;  // column groups per block (FP64: 4)
-    LU_CUDA(cudaFuncSetAttribute(tri_inv_kernel<V, false, CG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem));
-    LU_CUDA(cudaFuncSetAttribute(tri_inv_kernel<V, true, CG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem));
-    {
+    if constexpr (std::is_same<V, C32>::value) {
+        LU_CUDA(cudaFuncSetAttribute(tri_inv_kernel<V, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        LU_CUDA(cudaFuncSetAttribute(tri_inv_kernel<V, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         BM_PROF(c, "tri_inv_kernel");
-        tri_inv_kernel<V, false, CG><<<dim3(nblk, CG), 256, smem, s>>>(F, n, reinterpret_cast<CV*>(c->d_dinvL), fail);
-        tri_inv_kernel<V, true, CG><<<dim3(nblk, CG), 256, smem, s>>>(F, n, reinterpret_cast<CV*>(c->d_dinvU), fail);
+        tri_inv_kernel<V, false><<<nblk, 256, smem, s>>>(F, n, reinterpret_cast<CV*>(c->d_dinvL), fail);
+        tri_inv_kernel<V, true><<<nblk, 256, smem, s>>>(F, n, reinterpret_cast<CV*>(c->d_dinvU), fail);
         LU_CUDA(cudaGetLastError());
     }
     if constexpr (std::is_same<V, C32>::value) {
@@ -1097,18 +1109,6 @@ bm_status factor_t(bm_ctx* c, V F, bool tc, int split, int J0 = 0) {
 }
 
 template <class V, int BN>
-cudaError_t launch_trsv_step(cudaStream_t s, V F, V Y, V Z, int r0, int rb, int rest0, int nrest, int nrhs, int bs,
-                             const typename V::cv* Tinv) {
-    size_t smem = ((size_t)bs * bs + 2 * (size_t)BN * bs + (size_t)bs * TS_BM) * sizeof(typename V::cv);
-    auto kern = trsv_step_kernel<V, BN>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    dim3 grid(std::max(1, ceil_div(nrest, TS_BM)), ceil_div(nrhs, BN));
-    kern<<<grid, 256, smem, s>>>(F, Y, Z, r0, rb, rest0, nrest, nrhs, bs, Tinv);
-    return cudaGetLastError();
-}
-
-template <class V, int BN>
 cudaError_t launch_trsv_g_step(cudaStream_t s, V F, V Y, int r0, int rb, int rest0, int nrest, int nrhs) {
     size_t smem = ((size_t)BN * TS_BM + (size_t)TS_BM * TS_BM) * sizeof(typename V::cv);
     dim3 grid(ceil_div(nrest, TS_BM), ceil_div(nrhs, BN));
@@ -1128,35 +1128,34 @@ cudaError_t launch_trsv_diag(cudaStream_t s, V Y, V Z, int n, int nrhs, const ty
     return launch_pdl(kern, grid, dim3(256), smem, s, Y, Z, n, nrhs, Tinv);
 }
 
-// one cooperative launch of the persistent triangular solve: as many CTAs as the items, at most
-// the number the device keeps resident (queried once per process and device)
-template <bool UPPER>
-cudaError_t launch_trsv_flow(cudaStream_t s, C32 F, C32 Y, C32 Z, int n, int nrhs, const float2* T, int* ready,
-                             int* err, const int* never, const int* hook, int items, int num_sms) {
-    auto kern = trsv_flow_kernel<UPPER>;
-    const int smem = (TS_BM * TS_BM + 2 * FL_BN * TS_BM) * (int)sizeof(float2);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+// one cooperative launch of a persistent triangular solve: as many CTAs as the items, at most the number the
+// device keeps resident (queried once per process, device and kernel)
+template <class... KArgs, class... Args>
+cudaError_t launch_flow(cudaStream_t s, void (*kern)(KArgs...), int threads, int smem, int items, int num_sms,
+                        Args... args) {
+    cudaError_t e = cudaSuccess;
+    if (smem > 0) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     static std::mutex mu;
-    static std::map<int, int> per_sm_cache;
+    static std::map<std::pair<const void*, int>, int> per_sm_cache;
     int dev = 0;
     e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     {
         std::lock_guard<std::mutex> lock(mu);
-        auto it = per_sm_cache.find(dev);
+        const std::pair<const void*, int> key{reinterpret_cast<const void*>(kern), dev};
+        auto it = per_sm_cache.find(key);
         if (it == per_sm_cache.end()) {
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem);
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
             if (e != cudaSuccess) return e;
-            it = per_sm_cache.emplace(dev, per_sm).first;
+            it = per_sm_cache.emplace(key, per_sm).first;
         }
         per_sm = it->second;
     }
-    const int grid = std::max(1, std::min(items, std::max(per_sm, 1) * std::max(num_sms, 1)));
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid, 1, 1);
-    cfg.blockDim = dim3(256, 1, 1);
+    cfg.gridDim = dim3(std::max(1, std::min(items, std::max(per_sm, 1) * std::max(num_sms, 1))), 1, 1);
+    cfg.blockDim = dim3(threads, 1, 1);
     cfg.dynamicSmemBytes = (size_t)smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -1164,7 +1163,7 @@ cudaError_t launch_trsv_flow(cudaStream_t s, C32 F, C32 Y, C32 Z, int n, int nrh
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, F, Y, Z, n, nrhs, T, ready, err, never, hook);
+    return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
 // Solve L U X = Y in place (Y holds P B); Zw is an n x nrhs work buffer.
@@ -1188,10 +1187,11 @@ bm_status getrs_t(bm_ctx* c, V F, V Y, V Zw, int nrhs, const typename V::cv* din
             // (test hook: with d_info[3] set at assembly, one wait of the forward sweep is on the
             // never-set word after the flags)
             LU_CUDA(cudaMemsetAsync(c->d_flow, 0, (size_t)2 * items * sizeof(int), s));
-            LU_CUDA(launch_trsv_flow<false>(s, F, Y, Zw, n, nrhs, dinvL, c->d_flow, c->d_err, c->d_flow + c->flow_len,
-                                            c->d_info + 3, items, c->num_sms));
-            LU_CUDA(launch_trsv_flow<true>(s, F, Zw, Y, n, nrhs, dinvU, c->d_flow + items, c->d_err, nullptr,
-                                           c->d_info + 3, items, c->num_sms));
+            const int smem = (TS_BM * TS_BM + 2 * FL_BN * TS_BM) * (int)sizeof(float2);
+            LU_CUDA(launch_flow(s, trsv_flow_kernel<false>, 256, smem, items, c->num_sms, F, Y, Zw, n, nrhs, dinvL,
+                                c->d_flow, c->d_err, c->d_flow + c->flow_len, c->d_info + 3));
+            LU_CUDA(launch_flow(s, trsv_flow_kernel<true>, 256, smem, items, c->num_sms, F, Zw, Y, n, nrhs, dinvU,
+                                c->d_flow + items, c->d_err, nullptr, c->d_info + 3));
             return BM_OK;
         }
         auto gstep = [&](V Yv, int r0, int rb, int rest0, int nrest) {
@@ -1219,20 +1219,17 @@ bm_status getrs_t(bm_ctx* c, V F, V Y, V Zw, int nrhs, const typename V::cv* din
         BM_PROF(c, "trsv_diag_kernel");
         LU_CUDA(diag(Zw, Y, dinvU));  // Y = U^{-1} Zw
     } else {
-        auto step = [&](V Yv, V Zv, int r0, int rb, int rest0, int nrest, const typename V::cv* T) {
-            return narrow ? launch_trsv_step<V, 16>(s, F, Yv, Zv, r0, rb, rest0, nrest, nrhs, bs, T)
-                          : launch_trsv_step<V, 32>(s, F, Yv, Zv, r0, rb, rest0, nrest, nrhs, bs, T);
-        };
-        for (int b = 0; b < nblk; ++b) {  // Zw = L^{-1} Y
-            int r0 = b * bs, rb = std::min(bs, n - r0);
-            BM_PROF(c, "trsv_step_kernel");
-            LU_CUDA(step(Y, Zw, r0, rb, r0 + rb, n - r0 - rb, dinvL + (long)b * bs * bs));
+        const int items = ceil_div(n, FZ_B) * ceil_div(nrhs, FZ_NC);
+        if (c->d_flow == nullptr || 2L * items > c->flow_len) {
+            bm_set_error("lu: the triangular solve's flags are missing");
+            return BM_EINVAL;
         }
-        for (int b = nblk - 1; b >= 0; --b) {  // Y = U^{-1} Zw
-            int r0 = b * bs, rb = std::min(bs, n - r0);
-            BM_PROF(c, "trsv_step_kernel");
-            LU_CUDA(step(Zw, Y, r0, rb, 0, r0, dinvU + (long)b * bs * bs));
-        }
+        BM_PROF(c, "trsv_flow_z64_kernel");
+        LU_CUDA(cudaMemsetAsync(c->d_flow, 0, (size_t)2 * items * sizeof(int), s));
+        LU_CUDA(launch_flow(s, trsv_flow_z64_kernel<false>, 128, 0, items, c->num_sms, F, Y, Zw, n, nrhs, dinvL,
+                            c->d_flow, c->d_err));
+        LU_CUDA(launch_flow(s, trsv_flow_z64_kernel<true>, 128, 0, items, c->num_sms, F, Zw, Y, n, nrhs, dinvU,
+                            c->d_flow + items, c->d_err));
     }
     return BM_OK;
 }

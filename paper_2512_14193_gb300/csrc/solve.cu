@@ -169,8 +169,8 @@ bm_status solve_fp64(bm_ctx* c, const double2* B, double2* X, long ld, int nrhs)
             SV_CUDA(copy_z64(s, B + 2 * N, ld, N, nrhs, c->d_Y64b, ldy));
         }
         {
-            BM_PROF(c, "cgemm_simt_kernel<Z64> (solve product)");
-            SV_CUDA(gemm_z64(s, N, nrhs, 2 * N, -1.0, Z64{c->d_Mbot, c->ldbot}, false, Z64{const_cast<double2*>(B), ld},
+            BM_PROF(c, "skinny_z64_kernel (solve product)");
+            SV_CUDA(gemm_z64_skinny(s, c->num_sms, N, nrhs, 2 * N, -1.0, Z64{c->d_Mbot, c->ldbot}, Z64{const_cast<double2*>(B), ld},
                              1.0, Z64{c->d_Y64b, ldy}));
         }
         {
@@ -188,8 +188,8 @@ bm_status solve_fp64(bm_ctx* c, const double2* B, double2* X, long ld, int nrhs)
             SV_CUDA(copy_z64(s, B, ld, 2 * N, nrhs, X, ld));
         }
         {
-            BM_PROF(c, "cgemm_simt_kernel<Z64> (solve product)");
-            SV_CUDA(gemm_z64(s, 2 * N, nrhs, N, -1.0, Z64{c->d_Mtop, c->ldtop}, false, Z64{X + 2 * N, ld}, 1.0,
+            BM_PROF(c, "skinny_z64_kernel (solve product)");
+            SV_CUDA(gemm_z64_skinny(s, c->num_sms, 2 * N, nrhs, N, -1.0, Z64{c->d_Mtop, c->ldtop}, Z64{X + 2 * N, ld}, 1.0,
                              Z64{X, ld}));
         }
     } else {
@@ -217,14 +217,14 @@ bm_status residual_fp64(bm_ctx* c, const double2* B, const double2* X, double2* 
         resid_init_kernel<<<ceil_div(t, 256), 256, 0, s>>>(B, X, ld, c->nsys, nsub, nrhs, R);
         SV_CUDA(cudaGetLastError());
     }
-    BM_PROF(c, "cgemm_simt_kernel<Z64> (FP64 residual)");
+    BM_PROF(c, "skinny_z64_kernel (FP64 residual)");
     if (c->form == BM_MIXED) {
-        SV_CUDA(gemm_z64(s, 2 * N, nrhs, N, -1.0, Z64{c->d_Mtop, c->ldtop}, false,
+        SV_CUDA(gemm_z64_skinny(s, c->num_sms, 2 * N, nrhs, N, -1.0, Z64{c->d_Mtop, c->ldtop},
                          Z64{const_cast<double2*>(X) + 2 * N, ld}, 1.0, Z64{R, ld}));
-        SV_CUDA(gemm_z64(s, N, nrhs, 2 * N, -1.0, Z64{c->d_Mbot, c->ldbot}, false, Z64{const_cast<double2*>(X), ld},
+        SV_CUDA(gemm_z64_skinny(s, c->num_sms, N, nrhs, 2 * N, -1.0, Z64{c->d_Mbot, c->ldbot}, Z64{const_cast<double2*>(X), ld},
                          1.0, Z64{R + 2 * N, ld}));
     } else {
-        SV_CUDA(gemm_z64(s, 2 * N, nrhs, 2 * N, -1.0, Z64{c->d_A, c->ldA}, false, Z64{const_cast<double2*>(X), ld},
+        SV_CUDA(gemm_z64_skinny(s, c->num_sms, 2 * N, nrhs, 2 * N, -1.0, Z64{c->d_A, c->ldA}, Z64{const_cast<double2*>(X), ld},
                          1.0, Z64{R, ld}));
     }
     c->launches += (c->form == BM_MIXED) ? 3 : 2;
