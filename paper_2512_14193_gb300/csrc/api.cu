@@ -294,13 +294,21 @@ Plan make_plan(int N, int form, int prec, int nb_user, int bs, int nd, bool fast
 
 }  // namespace
 
+// Digit workspace of an FP64 factorisation: the Schur complement's, and the first trailing update's
+static size_t dg_request(int N, int form, bool fast, int num_sms) {
+    size_t b = form == BM_MIXED ? dg_bytes(N, N, 2 * N, num_sms) : 0;
+    const int m = (form == BM_MIXED ? N : 2 * N) - 128;
+    if (fast && m > 0) b = std::max(b, dg_bytes(m, m, 128, num_sms));
+    return b;
+}
+
 // Device bytes one request needs: the assembled system and its factorisation, plus the solve
 // workspace for nrhs right-hand sides (an estimate from the same sizes ensure_ws uses, with a
 // margin for the split-K partial sums).  optional: with what a handle also takes when its budget has room
 // (the search-free LU's buffers, the FP64 digit workspace).
 size_t request_bytes(int N, int form, int prec, int nb, int nrhs, bool optional, int num_sms) {
     Plan p = make_plan(N, form, prec, nb, 64, 9, optional && prec != BM_FP64 && nb == 0);
-    if (optional && prec == BM_FP64 && form == BM_MIXED) p.bytes += dg_bytes(N, N, 2 * N, num_sms);
+    if (optional && prec == BM_FP64) p.bytes += dg_request(N, form, true, num_sms) + lu_fast_z_bytes();
     const size_t w = (size_t)std::max(nrhs, 8);
     size_t b = p.bytes + 7 * (size_t)N * 8 + (size_t)p.nsys * w * 16 * 3 + (size_t)p.n * w * 16 * 2;
     if (prec == BM_FP64) {
@@ -559,7 +567,7 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
     // allocation or release - cudaFree would wait for every stream of the device - and the cached
     // graphs and tensor maps stay valid, as they depend only on these pointers and sizes).
     const bool reuse = c->assembled && c->N == N && c->form == form && c->prec == prec && c->nb == p.nb &&
-                       (c->d_fd != nullptr || c->fast_denied) == fast && c->rt_nd == nd && curve->kind != BM_CURVE_USER;
+                       (prec == BM_FP64 || (c->d_fd != nullptr || c->fast_denied) == fast) && c->rt_nd == nd && curve->kind != BM_CURVE_USER;
     if (!reuse) {
         free_problem(c);
         // a budget without room for the search-free LU's buffers keeps the panels
@@ -572,7 +580,8 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
     c->eager = eager;
     c->opt_cluster_cap = cl_cap;
     c->opt_panel_kernel = pkern;
-    c->lu_fast = fast && !c->fast_denied;
+    c->fast_z = prec == BM_FP64 && nb == 0 && pkern == 0 && (cl_cap == 0 || defer_kernels);
+    c->lu_fast = prec == BM_FP64 ? c->fast_z && c->d_fd != nullptr : fast && !c->fast_denied;
     c->bs_solve = 64;
     if (!reuse && c->held + p.bytes > c->budget) {
         bm_set_error("admission: system needs " + std::to_string(p.bytes) + " bytes, budget leaves " +
@@ -644,7 +653,7 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
         if (s == BM_OK) s = alloc_t(c, &c->d_Lp_i, lb);
         if (s == BM_OK) s = alloc_t(c, &c->d_Up_r, lb);
         if (s == BM_OK) s = alloc_t(c, &c->d_Up_i, lb);
-        if (s == BM_OK && c->lu_fast) s = alloc_t(c, &c->d_fd, lu_fast_bytes(p.n));
+        if (s == BM_OK && c32 && c->lu_fast) s = alloc_t(c, &c->d_fd, lu_fast_bytes(p.n));
     }
     if (s == BM_OK && c32) {
         // [0] Mtop (2N x N) or A (2N x 2N), [1] Mbot (N x 2N)
@@ -797,11 +806,20 @@ bm_status assemble_post(bm_ctx* c, bool run_assembly_kernel, bool wait) {
     return BM_OK;
 }
 
-// Reserves the digit workspace of an FP64 factorisation where the budget and the device have room for it
-// (without it the products run on the CUDA cores).
+// Reserves, where the budget and the device have room, the small buffer of the search-free FP64 blocks
+// (without it the panels search) and the digit workspace (without it the products run on the CUDA cores).
 void dg_reserve(bm_ctx* c) {
-    if (c->prec != BM_FP64 || c->d_dgw) return;
-    const size_t b = c->form == BM_MIXED ? dg_bytes(c->N, c->N, 2 * c->N, c->num_sms) : 0;
+    if (c->prec != BM_FP64) return;
+    if (c->fast_z && !c->d_fd && c->held + lu_fast_z_bytes() <= c->budget &&
+        alloc_t(c, &c->d_fd, lu_fast_z_bytes()) != BM_OK)
+        c->d_fd = nullptr;
+    if (c->lu_fast != (c->fast_z && c->d_fd)) {
+        c->lu_fast = !c->lu_fast;
+        drop_slot(c->g_factor);
+        drop_slot(c->g_lu);
+    }
+    if (c->d_dgw) return;
+    const size_t b = dg_request(c->N, c->form, c->lu_fast, c->num_sms);
     if (b == 0 || c->held + b > c->budget) return;
     if (alloc_t(c, &c->d_dgw, b) == BM_OK) c->dgw_bytes = b;
 }

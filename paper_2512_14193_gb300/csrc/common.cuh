@@ -297,6 +297,7 @@ struct bm_ctx {
     int* d_err = nullptr;      // d_info + 1; d_info[2..3] test hooks, d_info[4] stop word of lu_fast.cu
     bool lu_fast = false;      // FP32 LU in blocks without a pivot search (lu_fast.cu) and their
     float* d_fd = nullptr;     //   work buffer: the default, unless bm_opts.nb or a panel setting is set
+    bool fast_z = false;       // FP64: the same (lu_fast_z.cu), where dg_reserve finds room
     bool fast_denied = false;  //   or the budget has no room for the buffer
     void* d_maps = nullptr;    // row-interchange maps used by the factorisation: big panel (even),
                                // sub-panel, big panel (odd)

@@ -62,6 +62,7 @@ bm_status lu_factor_enqueue(bm_ctx* c);       // factor d_F64 / d_F32 in place (
 // continue a factorisation that stopped at a block (the value of its stop word) with the pivot search
 bm_status lu_resume_enqueue(bm_ctx* c, int stop);
 size_t lu_fast_bytes(int n);                  // work buffer of the search-free blocks (d_fd)
+size_t lu_fast_z_bytes();                     // and of the FP64 ones
 size_t swap_map_bytes();
 bm_status getrs_z64(bm_ctx* c, double2* Y, long ldy, int nrhs);   // in place; Y holds P B (rows gathered by perm)
 bm_status getrs_c32(bm_ctx* c, float* Yr, float* Yi, long ldy, int nrhs);
@@ -137,7 +138,8 @@ size_t dg_bytes(int m, int n, int K, int num_sms);
 bm_status gemm_z64_dg(cudaStream_t s, void* work, int num_sms, int m, int n, int K, double alpha, Z64 A, Z64 B, Z64 C,
                       int* d_err);
 
-// api.cu: the Schur complement of the FP64 precision into d_F64 (the workspace reserved before any capture)
+// api.cu: what an FP64 factorisation takes where the budget has room (before any capture); the Schur
+// complement of the FP64 precision into d_F64
 void dg_reserve(bm_ctx* c);
 bm_status schur_z64(bm_ctx* c, cudaStream_t s);
 // api.cu: assembly in two halves (the batched contour solver assembles many handles at once)

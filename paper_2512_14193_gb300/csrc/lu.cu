@@ -983,6 +983,50 @@ bm_status factor_fast(bm_ctx* c, C32 F) {
     return BM_OK;
 }
 
+// The FP64 LU in blocks of FZ_BLOCK columns without a pivot search (lu_fast_z.cu), outer blocks of FZ_OUTER:
+// inside one, each block updates the rest of the outer block's columns and rows on the FP64 pipe; then the
+// trailing matrix takes the outer block's product, by digits on the tensor cores where that is the faster
+// (dg_bytes), else on the FP64 pipe.
+bm_status factor_fast_z(bm_ctx* c, Z64 F) {
+    const int n = c->n;
+    cudaStream_t s = c->stream;
+    int* const fail = c->d_info + 4;
+    double2* const work = reinterpret_cast<double2*>(c->d_fd);
+    {
+        BM_PROF(c, "iota");
+        iota_kernel<<<ceil_div(n, 256), 256, 0, s>>>(c->d_perm, c->d_ipiv, n);
+        LU_CUDA(cudaGetLastError());
+    }
+    for (int J = 0; J < n; J += FZ_OUTER) {
+        const int je = std::min(J + FZ_OUTER, n);
+        for (int j = J; j < je; j += FZ_BLOCK) {
+            const int db = std::min(FZ_BLOCK, n - j), e = j + db, mm = n - e;
+            {
+                BM_PROF(c, "panel_kernel");  // (the profile keeps one name for the panels' elimination)
+                LU_CUDA(launch_lu_diag_z(s, F, j, db, work, fail));
+            }
+            {
+                BM_PROF(c, "lu_trsm_z_kernel");
+                LU_CUDA(launch_lu_trsm_z(s, F, j, db, mm, work, fail));
+            }
+            if (mm == 0 || e >= je) continue;
+            BM_PROF(c, "cgemm_simt_kernel (panel update)");
+            LU_CUDA(gemm_z64(s, mm, je - e, db, -1.0, F.sub(e, j), false, F.sub(j, e), 1.0, F.sub(e, e)));
+            if (je < n)
+                LU_CUDA(gemm_z64(s, je - e, n - je, db, -1.0, F.sub(e, j), false, F.sub(j, je), 1.0, F.sub(e, je)));
+        }
+        const int m = n - je, k = je - J;
+        if (m == 0) break;
+        BM_PROF(c, "cgemm_simt_kernel (trailing update)");
+        const size_t need = dg_bytes(m, m, k, c->num_sms);
+        if (need > 0 && need <= c->dgw_bytes)
+            BM_TRY(gemm_z64_dg(s, c->d_dgw, c->num_sms, m, m, k, -1.0, F.sub(je, J), F.sub(J, je), F.sub(je, je), c->d_err));
+        else
+            LU_CUDA(gemm_z64(s, m, m, k, -1.0, F.sub(je, J), false, F.sub(J, je), 1.0, F.sub(je, je)));
+    }
+    return finish_t<Z64>(c, F, s);
+}
+
 // The LU with the pivot search, from column J0 on (the columns before it are factored, their
 // interchanges and trailing updates applied).
 template <class V>
@@ -1277,7 +1321,7 @@ bm_status lu_setup(bm_ctx* c, int cluster_cap, int panel_kernel) {
 bm_status lu_factor_enqueue(bm_ctx* c) {
     if (c->prec == BM_FP64) {
         Z64 F{c->d_F64, c->ldF};
-        return factor_t<Z64>(c, F, false, 0);
+        return c->lu_fast ? factor_fast_z(c, F) : factor_t<Z64>(c, F, false, 0);
     }
     C32 F{c->d_F32r, c->d_F32i, c->ldF};
     if (c->lu_fast) return factor_fast(c, F);
@@ -1285,6 +1329,14 @@ bm_status lu_factor_enqueue(bm_ctx* c) {
 }
 
 bm_status lu_resume_enqueue(bm_ctx* c, int stop) {
+    if (c->prec == BM_FP64) {  // from the start, with the matrix formed again
+        LU_CUDA(cudaMemsetAsync(c->d_info + 4, 0, sizeof(int), c->stream));
+        if (c->form == BM_MIXED)
+            BM_TRY(schur_z64(c, c->stream));
+        else
+            LU_CUDA(launch_copy_z64(c->stream, c->d_A, c->ldA, c->n, c->n, c->d_F64, c->ldF));
+        return factor_t<Z64>(c, Z64{c->d_F64, c->ldF}, false, 0);
+    }
     C32 F{c->d_F32r, c->d_F32i, c->ldF};
     const int J = (stop >> 1) - 1, db = std::min(FD_B, c->n - J);
     LU_CUDA(cudaMemsetAsync(c->d_info + 4, 0, sizeof(int), c->stream));
@@ -1293,6 +1345,7 @@ bm_status lu_resume_enqueue(bm_ctx* c, int stop) {
 }
 
 size_t lu_fast_bytes(int n) { return fd_work_floats(n) * sizeof(float); }
+size_t lu_fast_z_bytes() { return FZ_T * sizeof(double2); }
 
 // Y holds P B already (rows gathered with d_perm); solves L U X = Y in place.
 bm_status getrs_z64(bm_ctx* c, double2* Y, long ldy, int nrhs) {

@@ -514,6 +514,16 @@ cudaError_t launch_panel(cudaStream_t s, C32 A, const PanelShape& ps, int j0, in
                          int J, int jb, SwapMap* mi, SwapMap* mb, int* perm);
 cudaError_t launch_panel(cudaStream_t s, Z64 A, const PanelShape& ps, int j0, int m, int ib, int* ipiv, int* info,
                          int J, int jb, SwapMap* mi, SwapMap* mb, int* perm);
+// lu_fast_z.cu: the same for FP64 in blocks of FZ_BLOCK columns
+constexpr int FZ_BLOCK = 32, FZ_OUTER = 128;
+constexpr long FZ_T = 3L * FZ_BLOCK * FZ_BLOCK + FZ_BLOCK;
+struct FzT {
+    double2 *U, *L, *F, *piv;  // U and L^T with inverted 8 x 8 diagonal blocks, the factors, the pivots
+    BM_HD explicit FzT(double2* w)
+        : U(w), L(w + FZ_BLOCK * FZ_BLOCK), F(w + 2 * FZ_BLOCK * FZ_BLOCK), piv(w + 3 * FZ_BLOCK * FZ_BLOCK) {}
+};
+cudaError_t launch_lu_diag_z(cudaStream_t s, Z64 F, int J, int db, double2* work, int* fail);
+cudaError_t launch_lu_trsm_z(cudaStream_t s, Z64 F, int J, int db, int mm, const double2* work, int* fail);
 int query_cluster_max_c32();
 
 // lu_fast.cu: blocks of FD_B columns whose pivots stay on the diagonal.  The work buffer holds the

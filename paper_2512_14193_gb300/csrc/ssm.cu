@@ -243,8 +243,8 @@ bm_status factor_batch(Batch& bt, int B) {
     } else {
         for (int b = 0; b < B; ++b) {
             bm_ctx* c = bt.h[b];
+            dg_reserve(c);
             if (c->form == BM_MIXED) {
-                dg_reserve(c);
                 BM_TRY(schur_z64(c, c->stream));
             } else if (c->prec == BM_FP64) {
                 SSM_CUDA(launch_copy_z64(c->stream, c->d_A, c->ldA, c->n, c->n, c->d_F64, c->ldF));

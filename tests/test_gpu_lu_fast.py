@@ -15,6 +15,9 @@ pytestmark = pytest.mark.gpu
 FREE, SEARCH = "lu_trsm_kernel", "swap_trsm_kernel (block row)"
 
 
+FREE_Z = "lu_trsm_z_kernel"
+
+
 def _solve(bmlib, curve, N, k0, k1, form, opts, seed=3, ncols=5):
     h = bmlib.bm_create(0)
     try:
@@ -30,7 +33,10 @@ def _solve(bmlib, curve, N, k0, k1, form, opts, seed=3, ncols=5):
     g, P = O.nodes(curve, N), O.default_params(k0, k1)
     eta = (O.backward_error_mixed(O.mixed_blocks(g, P), X, B) if form == W.MIXED
            else O.backward_error_dense(O.ordinary_matrix(g, P), X, B))
-    assert info.backward_error <= 1e-9 and eta <= 1.5e-9
+    if opts.prec == bmlib.BM_FP64:
+        assert info.backward_error < 1e-13 and eta < 1e-13  # the suite's bound for the FP64 path
+    else:
+        assert info.backward_error <= 1e-9 and eta <= 1.5e-9
     return kernels
 
 
@@ -43,6 +49,14 @@ def test_block_edges(bmlib, prec, form, N):
     assert FREE in kernels and SEARCH not in kernels
 
 
+# FP64: block 32, sub-step 8, outer block 128 (digits above 265 rows), 16 rows per CTA
+@pytest.mark.parametrize("form,N", [(0, n) for n in (8, 9, 31, 32, 33, 40, 127, 128, 129, 160, 161, 257, 420)] +
+                                   [(1, n) for n in (8, 16, 17, 64, 66, 210)])
+def test_fp64_block_edges(bmlib, form, N):
+    kernels = _solve(bmlib, W.circle(), N, 2.0, 3.0, form, bmlib.make_opts(0))
+    assert FREE_Z in kernels and SEARCH not in kernels
+
+
 # partial pivoting interchanges rows of these systems, first in the column given: in the first block, in a
 # later one, near the end; inside a diagonal block and below it
 @pytest.mark.parametrize("curve,N,k0,form", [
@@ -51,9 +65,10 @@ def test_block_edges(bmlib, prec, form, N):
     (W.ellipse(1.0, 0.6), 400, 4.901444581998341 - 1.0794051420988682j, 1),    # column 657 of 800
     (W.kite(), 600, 30.0 - 0.6j, 1),                                           # column 790 of 1200
 ])
-def test_interchanges_continue_with_the_search(bmlib, curve, N, k0, form):
-    kernels = _solve(bmlib, curve, N, k0, 1.5 * k0, form, bmlib.make_opts(2))
-    assert FREE in kernels and SEARCH in kernels
+@pytest.mark.parametrize("prec", [0, 2])
+def test_interchanges_continue_with_the_search(bmlib, curve, N, k0, form, prec):
+    kernels = _solve(bmlib, curve, N, k0, 1.5 * k0, form, bmlib.make_opts(prec))
+    assert (FREE if prec else FREE_Z) in kernels and SEARCH in kernels
 
 
 def test_an_explicit_block_size_keeps_the_search(bmlib):
