@@ -237,8 +237,17 @@ double2 d2(bm_c64 z) { return make_double2(z.re, z.im); }
 
 long round_up(long a, long b) { return (a + b - 1) / b * b; }
 
+// Split planes of the operator a residual mode reads: all of them for double-float residuals, the hi/lo ones
+// where residual updates run on the CUDA cores (the ordinary system and single TF32), none else.
+int planes_needed(int form, int prec, int resid_mode) {
+    if (prec == BM_FP64) return 0;
+    if (resid_mode == BM_RESID_DF_UPDATE) return 2;
+    if (resid_mode == BM_RESID_FP64_ALL || resid_mode == BM_RESID_TC_ALL) return 0;
+    return form == BM_ORDINARY || prec == BM_CF32_TF32_IR ? 1 : 0;
+}
+
 // fast: the FP32 LU in search-free blocks (lu_fast.cu), with its work buffer
-Plan make_plan(int N, int form, int prec, int nb_user, int bs, int nd, bool fast) {
+Plan make_plan(int N, int form, int prec, int nb_user, int bs, int nd, bool fast, int planes) {
     Plan p;
     const bool c32 = prec != BM_FP64;
     const bool split = prec == BM_CF32_3XTF32_IR;
@@ -260,8 +269,8 @@ Plan make_plan(int N, int form, int prec, int nb_user, int bs, int nd, bool fast
     } else {
         b += (size_t)p.ldF * p.n * 8;
         // split hi/lo planes of the FP64 operator (same size as the FP64 blocks) and of re + im
-        b += (form == BM_MIXED) ? (size_t)p.ldtop * N * 24 + (size_t)p.ldbot * 2 * N * 24
-                                : (size_t)p.ldA * 2 * N * 24;
+        const size_t pb = planes == 2 ? 24 : (planes == 1 ? 16 : 0);
+        b += (form == BM_MIXED) ? (size_t)p.ldtop * N * pb + (size_t)p.ldbot * 2 * N * pb : (size_t)p.ldA * 2 * N * pb;
         if (form == BM_MIXED) {
             p.kseg = 2 * N;
             long kext = split ? 3L * p.kseg : p.kseg;
@@ -306,8 +315,9 @@ static size_t dg_request(int N, int form, bool fast, int num_sms) {
 // workspace for nrhs right-hand sides (an estimate from the same sizes ensure_ws uses, with a
 // margin for the split-K partial sums).  optional: with what a handle also takes when its budget has room
 // (the search-free LU's buffers, the FP64 digit workspace).
-size_t request_bytes(int N, int form, int prec, int nb, int nrhs, bool optional, int num_sms) {
-    Plan p = make_plan(N, form, prec, nb, 64, 9, optional && prec != BM_FP64 && nb == 0);
+size_t request_bytes(int N, int form, int prec, int nb, int nrhs, int resid_mode, bool optional, int num_sms) {
+    Plan p = make_plan(N, form, prec, nb, 64, 9, optional && prec != BM_FP64 && nb == 0,
+                       planes_needed(form, prec, resid_mode));
     if (optional && prec == BM_FP64) p.bytes += dg_request(N, form, true, num_sms) + lu_fast_z_bytes();
     const size_t w = (size_t)std::max(nrhs, 8);
     size_t b = p.bytes + 7 * (size_t)N * 8 + (size_t)p.nsys * w * 16 * 3 + (size_t)p.n * w * 16 * 2;
@@ -371,7 +381,7 @@ extern "C" bm_status bm_create(bm_ctx** out, int device, void* cuda_stream, size
         return s;
     }
     c->d_err = c->d_info + 1;
-    c->htab = HankelTable{tab, nx, ny, re0, im0, step, 1.0 / step};
+    c->htab = HankelTable{tab, nx, ny, re0, im0, step, 1.0 / step, (int)std::lround(-im0 / step)};
     *out = c;
     return BM_OK;
 }
@@ -562,18 +572,20 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
     // LU in search-free blocks, unless a block size or a panel setting asks for the panels (the contour
     // solver's deferred assembly sets a cluster size for what its factorisations continue with)
     const bool fast = prec != BM_FP64 && nb == 0 && pkern == 0 && (cl_cap == 0 || defer_kernels);
-    Plan p = make_plan(N, form, prec, nb, 64, nd, fast);
+    const int planes = planes_needed(form, prec, rmode);
+    Plan p = make_plan(N, form, prec, nb, 64, nd, fast, planes);
     // Same shape as the assembled system: assemble again into the same buffers (no device
     // allocation or release - cudaFree would wait for every stream of the device - and the cached
     // graphs and tensor maps stay valid, as they depend only on these pointers and sizes).
     const bool reuse = c->assembled && c->N == N && c->form == form && c->prec == prec && c->nb == p.nb &&
-                       (prec == BM_FP64 || (c->d_fd != nullptr || c->fast_denied) == fast) && c->rt_nd == nd && curve->kind != BM_CURVE_USER;
+                       (prec == BM_FP64 || (c->d_fd != nullptr || c->fast_denied) == fast) && c->rt_nd == nd && c->planes == planes &&
+                       curve->kind != BM_CURVE_USER;
     if (!reuse) {
         free_problem(c);
         // a budget without room for the search-free LU's buffers keeps the panels
         c->fast_denied = fast && c->held + p.bytes > c->budget;
     }
-    if (c->fast_denied) p = make_plan(N, form, prec, nb, 64, nd, false);
+    if (c->fast_denied) p = make_plan(N, form, prec, nb, 64, nd, false, planes);
     // the captured factorisation depends on the launch settings: capture again when they change
     if (reuse && (eager != c->eager || cl_cap != c->opt_cluster_cap || pkern != c->opt_panel_kernel))
         drop_graphs(c);
@@ -604,6 +616,7 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
     c->refine_maxit = (opts && opts->refine_maxit > 0) ? opts->refine_maxit : 30;
     c->resid_mode = rmode;
     c->rt_nd = nd;
+    c->planes = planes;
     c->ldtop = p.ldtop;
     c->ldbot = p.ldbot;
     c->ldA = p.ldA;
@@ -624,15 +637,15 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
         s = alloc_t(c, &c->d_A, (size_t)p.ldA * 2 * N * 16);
     }
     if (s == BM_OK && !c32) s = alloc_t(c, &c->d_F64, (size_t)p.ldF * p.n * 16);
-    if (s == BM_OK && c32) {
+    if (s == BM_OK && planes >= 1) {
         if (form == BM_MIXED) {
             s = alloc_t(c, &c->d_Ptop, (size_t)p.ldtop * N * 16);
             if (s == BM_OK) s = alloc_t(c, &c->d_Pbot, (size_t)p.ldbot * 2 * N * 16);
-            if (s == BM_OK) s = alloc_t(c, &c->d_Qtop, (size_t)p.ldtop * N * 8);
-            if (s == BM_OK) s = alloc_t(c, &c->d_Qbot, (size_t)p.ldbot * 2 * N * 8);
+            if (s == BM_OK && planes == 2) s = alloc_t(c, &c->d_Qtop, (size_t)p.ldtop * N * 8);
+            if (s == BM_OK && planes == 2) s = alloc_t(c, &c->d_Qbot, (size_t)p.ldbot * 2 * N * 8);
         } else {
             s = alloc_t(c, &c->d_PA, (size_t)p.ldA * 2 * N * 16);
-            if (s == BM_OK) s = alloc_t(c, &c->d_QA, (size_t)p.ldA * 2 * N * 8);
+            if (s == BM_OK && planes == 2) s = alloc_t(c, &c->d_QA, (size_t)p.ldA * 2 * N * 8);
         }
     }
     if (s == BM_OK && c32) {
@@ -739,10 +752,13 @@ bm_status assemble_post(bm_ctx* c, bool run_assembly_kernel, bool wait) {
     if (c32) {
         if (form == BM_MIXED) {
             BM_CUDA_TRY(launch_pack_solve(st, c, prec == BM_CF32_3XTF32_IR));
-            BM_CUDA_TRY(launch_split_planes(st, c->d_Mtop, c->ldtop, 2 * N, N, c->d_Ptop, c->d_Qtop, c->ldtop));
-            BM_CUDA_TRY(launch_split_planes(st, c->d_Mbot, c->ldbot, N, 2 * N, c->d_Pbot, c->d_Qbot, c->ldbot));
-            c->launches += 3;
-        } else {
+            c->launches += 1;
+            if (c->planes) {
+                BM_CUDA_TRY(launch_split_planes(st, c->d_Mtop, c->ldtop, 2 * N, N, c->d_Ptop, c->d_Qtop, c->ldtop));
+                BM_CUDA_TRY(launch_split_planes(st, c->d_Mbot, c->ldbot, N, 2 * N, c->d_Pbot, c->d_Qbot, c->ldbot));
+                c->launches += 2;
+            }
+        } else if (c->planes) {
             BM_CUDA_TRY(launch_split_planes(st, c->d_A, c->ldA, 2 * N, 2 * N, c->d_PA, c->d_QA, c->ldA));
             c->launches += 1;
         }
@@ -1010,9 +1026,11 @@ bm_status ensure_ws(bm_ctx* c, int nrhs) {
         BM_TRY(alloc_t(c, &c->d_W2i, vb));
         BM_TRY(alloc_t(c, &c->d_Zwr, vb));
         BM_TRY(alloc_t(c, &c->d_Zwi, vb));
-        BM_TRY(alloc_t(c, &c->d_XP, (size_t)c->nsys * w * 16));
-        BM_TRY(alloc_t(c, &c->d_XQ, (size_t)c->nsys * w * 8));
-        BM_TRY(alloc_t(c, &c->d_Wdf, (size_t)4 * c->N * w * 16));
+        if (c->planes == 2) {  // double-float residuals
+            BM_TRY(alloc_t(c, &c->d_XP, (size_t)c->nsys * w * 16));
+            BM_TRY(alloc_t(c, &c->d_XQ, (size_t)c->nsys * w * 8));
+            BM_TRY(alloc_t(c, &c->d_Wdf, (size_t)4 * c->N * w * 16));
+        }
         // two triangles x (64-row tiles) x (8-column tiles)
         c->flow_len = 2L * ceil_div(c->n, 64) * ceil_div(w, 8);
         BM_TRY(alloc_t(c, &c->d_flow, (size_t)(c->flow_len + 1) * sizeof(int)));  // + a flag never set (test hook)

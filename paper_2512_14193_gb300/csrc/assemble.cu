@@ -18,6 +18,7 @@
 // [M31, M32; D1 + I/2, -eps1 S1].
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "common.cuh"
 #include "hankel.cuh"
@@ -93,61 +94,63 @@ struct AsmArgs {
     int N;
     double h;
     double2 k0, k1, eps0, eps1, beta;
+    // products of the constants (kd = i k0 / 4): the entries' factors, formed once on the host
+    double2 eS, eD, kd, b0, b1, q0, q1;
     HankelTable T;
     const double* g;
     double2* o[4];  // output quadrants (see header comment)
     long ld[4];
 };
 
+// What both entries of an unordered pair share.  With ws the source weight, dn_t and dn_s the normal
+// projections of the target and the source, and the constants folded (AsmArgs):
+//   M31 = ws (D dn_s + bB)         D  = kd H1(k0 r)/r,  bB = beta kd [k0 H0 dni dnj/r^2 + H1 (ninj - 2 dni dnj/r^2)/r]
+//   M32 = ws (eS + eD dn_t)        eS = -eps0 (i/4) H0, eD = eps0 beta kd H1/r
+//   q0 ws, q1 dn ws                M13 and M23 (dn = dn_t) or -eps1 S1 and D1 (dn = dn_s)
+// so a pair takes about 70 FP64 operations besides its two Hankel evaluations (130 with each operator
+// formed by itself).
 struct PairVals {
-    // per wavenumber: cS = (i/4) H0, cD = (ik/4) H1 / r, B = N bracket (without weight)
-    double2 cS0, cD0, B0, cS1, cD1;
+    double2 D, bB, eS, eD, q0, q1;
 };
 
+template <bool REAL>
 __device__ __forceinline__ void pair_vals(const AsmArgs& a, double dx, double dy, double dni, double dnj, double ninj,
                                           PairVals& v) {
-    double r = sqrt(dx * dx + dy * dy);
-    double ir = 1.0 / r;
+    const double r2 = dx * dx + dy * dy;
+    const double ir = rsqrt(r2);
+    double r = r2 * ir;
+    r = fma(0.5 * ir, fma(-r, r, r2), r);  // sqrt(r2): one correction of the product
     double2 h0, h1;
-    hk::hankel01(cscale(a.k0, r), a.T, h0, h1);
-    double2 ik0 = cscale(cmuli(a.k0), 0.25);  // i k0 / 4
-    v.cS0 = cscale(cmuli(h0), 0.25);
-    v.cD0 = cscale(cmul(ik0, h1), ir);
-    // N bracket: k H0 dni dnj / r^2 - 2 H1 dni dnj / r^3 + H1 ninj / r
-    double pp = dni * dnj * ir * ir;
-    double2 br = cscale(cmul(a.k0, h0), pp);
-    br = cadd(br, cscale(h1, (ninj - 2.0 * pp) * ir));
-    v.B0 = cmul(ik0, br);
-    hk::hankel01(cscale(a.k1, r), a.T, h0, h1);
-    double2 ik1 = cscale(cmuli(a.k1), 0.25);
-    v.cS1 = cscale(cmuli(h0), 0.25);
-    v.cD1 = cscale(cmul(ik1, h1), ir);
+    if (REAL) hk::hankel01_real(a.k0.x * r, a.T, h0, h1);
+    else hk::hankel01(cscale(a.k0, r), a.T, h0, h1);
+    const double pp = dni * dnj * ir * ir;
+    h1 = cscale(h1, ir);
+    v.D = cmul(a.kd, h1);
+    v.eS = cmul(a.eS, h0);
+    v.eD = cmul(a.eD, h1);
+    v.bB = cadd(cscale(cmul(a.b0, h0), pp), cscale(cmul(a.b1, h1), ninj - 2.0 * pp));
+    if (REAL) hk::hankel01_real(a.k1.x * r, a.T, h0, h1);
+    else hk::hankel01(cscale(a.k1, r), a.T, h0, h1);
+    v.q0 = cmul(a.q0, h0);
+    v.q1 = cmul(a.q1, cscale(h1, ir));
 }
 
-// Entries of the four output quadrants for an ordered pair with given target/source normal
-// projections (dn_t = d.nu_target, dn_s = d.nu_source) and source weight ws.
+// Entries of the four output quadrants for an ordered pair
 template <int FORM>
-__device__ __forceinline__ void outputs(const AsmArgs& a, const PairVals& v, double dn_t, double dn_s, double ws,
-                                        double2 out[4]) {
-    double2 S0 = cscale(v.cS0, ws);
-    double2 D0 = cscale(v.cD0, dn_s * ws);
-    double2 Ds0 = cscale(v.cD0, -dn_t * ws);
-    double2 N0 = cscale(v.B0, ws);
-    double2 S1 = cscale(v.cS1, ws);
-    double2 M31 = cadd(D0, cmul(a.beta, N0));
-    double2 M32 = cneg(cmul(a.eps0, cadd(S0, cmul(a.beta, Ds0))));
+__device__ __forceinline__ void outputs(const PairVals& v, double dn_t, double dn_s, double ws, double2 out[4]) {
+    const double2 M31 = make_double2(ws * fma(v.D.x, dn_s, v.bB.x), ws * fma(v.D.y, dn_s, v.bB.y));
+    const double2 M32 = make_double2(ws * fma(v.eD.x, dn_t, v.eS.x), ws * fma(v.eD.y, dn_t, v.eS.y));
+    const double2 a = cscale(v.q0, ws), b = cscale(v.q1, (FORM == BM_MIXED ? dn_t : dn_s) * ws);
     if (FORM == BM_MIXED) {
-        double2 Ds1 = cscale(v.cD1, -dn_t * ws);
-        out[0] = cneg(S1);                      // M13
-        out[1] = cneg(cdiv(Ds1, a.eps1));       // M23
+        out[0] = a;    // M13
+        out[1] = b;    // M23
         out[2] = M31;
         out[3] = M32;
     } else {
-        double2 D1 = cscale(v.cD1, dn_s * ws);
         out[0] = M31;
         out[1] = M32;
-        out[2] = D1;
-        out[3] = cneg(cmul(a.eps1, S1));
+        out[2] = b;
+        out[3] = a;
     }
 }
 
@@ -184,12 +187,10 @@ __device__ __forceinline__ void diag_outputs(const AsmArgs& a, int i, double2 ou
     }
 }
 
-constexpr int AT = 32;  // assembly tile
-constexpr int AY = 8;   // threads in y
-
-// One 32 x 32 tile pair (I <= J) of the assembled blocks, chosen by blockIdx.x.
-template <int FORM>
+// One AT x AT tile pair (I <= J) of the assembled blocks, chosen by blockIdx.x; 256 threads, AT in x.
+template <int FORM, bool REAL, int AT>
 __device__ __forceinline__ void assemble_tile(const AsmArgs& a) {
+    constexpr int AY = 256 / AT;     // threads in y
     extern __shared__ double2 st[];  // [4][AT][AT+1] staging of the transposed tile
     // decode the upper-triangular tile pair (I <= J) from the linear block index
     long idx = blockIdx.x;
@@ -224,12 +225,12 @@ __device__ __forceinline__ void assemble_tile(const AsmArgs& a) {
                 double dx = xi - xj, dy = yi - yj;
                 double dni = dx * nxi + dy * nyi, dnj = dx * nxj + dy * nyj, ninj = nxi * nxj + nyi * nyj;
                 PairVals v;
-                pair_vals(a, dx, dy, dni, dnj, ninj, v);
+                pair_vals<REAL>(a, dx, dy, dni, dnj, ninj, v);
                 // (i, j): target i, source j
-                outputs<FORM>(a, v, dni, dnj, wj, o1);
+                outputs<FORM>(v, dni, dnj, wj, o1);
                 if (!diag_tile) {
                     // (j, i): d -> -d, target j (d.nu_j -> -dnj), source i (-dni)
-                    outputs<FORM>(a, v, -dnj, -dni, wi, o2);
+                    outputs<FORM>(v, -dnj, -dni, wi, o2);
                 }
             }
 #pragma unroll
@@ -255,16 +256,16 @@ __device__ __forceinline__ void assemble_tile(const AsmArgs& a) {
     }
 }
 
-template <int FORM>
-__global__ void __launch_bounds__(AT* AY) assemble_kernel(AsmArgs a) {
-    assemble_tile<FORM>(a);
+template <int FORM, bool REAL, int AT>
+__global__ void __launch_bounds__(256) assemble_kernel(AsmArgs a) {
+    assemble_tile<FORM, REAL, AT>(a);
 }
 
 // Several systems of the same size at once (contour points of one curve): system blockIdx.z takes
 // its wavenumbers, material constants and output blocks from args[blockIdx.z].
-template <int FORM>
-__global__ void __launch_bounds__(AT* AY) assemble_batch_kernel(const AsmArgs* __restrict__ args) {
-    assemble_tile<FORM>(args[blockIdx.z]);
+template <int FORM, int AT>
+__global__ void __launch_bounds__(256) assemble_batch_kernel(const AsmArgs* __restrict__ args) {
+    assemble_tile<FORM, false, AT>(args[blockIdx.z]);
 }
 
 // row sums of |A| for ||A||_inf; rows of an m x ncols column-major block, plus `add` per row
@@ -757,10 +758,19 @@ static AsmArgs asm_args(const bm_ctx* c) {
     a.eps0 = c->eps0;
     a.eps1 = c->eps1;
     a.beta = c->beta;
+    const bool mixed = c->form == BM_MIXED;
+    const double2 i4 = make_double2(0.0, 0.25), kd1 = cmul(i4, a.k1);
+    a.kd = cmul(i4, a.k0);
+    a.eS = cneg(cmul(a.eps0, i4));
+    a.eD = cmul(a.eps0, cmul(a.beta, a.kd));
+    a.b1 = cmul(a.beta, a.kd);
+    a.b0 = cmul(a.b1, a.k0);
+    a.q0 = mixed ? cneg(i4) : cneg(cmul(a.eps1, i4));
+    a.q1 = mixed ? cdiv(kd1, a.eps1) : kd1;
     a.T = c->htab;
     a.g = c->d_geom;
     long N = c->N;
-    if (c->form == BM_MIXED) {
+    if (mixed) {
         a.o[0] = c->d_Mtop;
         a.o[1] = c->d_Mtop + N;
         a.o[2] = c->d_Mbot;
@@ -777,23 +787,36 @@ static AsmArgs asm_args(const bm_ctx* c) {
     return a;
 }
 
+// Tile size: the FP64 pipe bounds the kernel, so every SM has to have its share.  32 x 32 tiles from eight
+// per SM on; below, 16 x 16 ones (N = 256: 136 CTAs instead of 36, 0.30 -> 0.10 ms).
+static bool big_tiles(const bm_ctx* c, int B) {
+    const long T = ceil_div(c->N, 32);
+    return T * (T + 1) / 2 * B >= 8L * c->num_sms;
+}
+
+template <int AT, class... KArgs, class... Args>
+static cudaError_t launch_tiles(cudaStream_t s, void (*kern)(KArgs...), int N, int B, Args... args) {
+    const long T = ceil_div(N, AT);
+    const int smem = 4 * AT * (AT + 1) * (int)sizeof(double2);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    kern<<<dim3((unsigned)(T * (T + 1) / 2), 1, (unsigned)B), dim3(AT, 256 / AT), smem, s>>>(args...);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_assemble(cudaStream_t s, const bm_ctx* c) {
     const AsmArgs a = asm_args(c);
-    long T = ceil_div(c->N, AT);
-    long nblk = T * (T + 1) / 2;
-    size_t smem = 4 * AT * (AT + 1) * sizeof(double2);
-    dim3 blk(AT, AY);
-    cudaError_t e;
-    if (c->form == BM_MIXED) {
-        e = cudaFuncSetAttribute(assemble_kernel<BM_MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        assemble_kernel<BM_MIXED><<<(unsigned)nblk, blk, smem, s>>>(a);
-    } else {
-        e = cudaFuncSetAttribute(assemble_kernel<BM_ORDINARY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        assemble_kernel<BM_ORDINARY><<<(unsigned)nblk, blk, smem, s>>>(a);
-    }
-    return cudaGetLastError();
+    const bool big = big_tiles(c, 1), real = a.k0.y == 0.0 && a.k1.y == 0.0;
+    auto go = [&](auto form) {
+        constexpr int F = decltype(form)::value;
+        if (big)
+            return real ? launch_tiles<32>(s, assemble_kernel<F, true, 32>, c->N, 1, a)
+                        : launch_tiles<32>(s, assemble_kernel<F, false, 32>, c->N, 1, a);
+        return real ? launch_tiles<16>(s, assemble_kernel<F, true, 16>, c->N, 1, a)
+                    : launch_tiles<16>(s, assemble_kernel<F, false, 16>, c->N, 1, a);
+    };
+    return c->form == BM_MIXED ? go(std::integral_constant<int, BM_MIXED>{})
+                               : go(std::integral_constant<int, BM_ORDINARY>{});
 }
 
 // One launch assembling the systems of B handles of equal N and formulation (grid.z = handle);
@@ -805,24 +828,16 @@ cudaError_t launch_assemble_batch(cudaStream_t s, bm_ctx* const* cs, int B, void
     for (int b = 0; b < B; ++b) h[b] = asm_args(cs[b]);
     cudaError_t e = cudaMemcpyAsync(d_args, h.data(), sizeof(AsmArgs) * B, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return e;
-    const int N = cs[0]->N;
-    long T = ceil_div(N, AT);
-    long nblk = T * (T + 1) / 2;
-    size_t smem = 4 * AT * (AT + 1) * sizeof(double2);
-    dim3 blk(AT, AY), grid((unsigned)nblk, 1, (unsigned)B);
+    const bm_ctx* c = cs[0];
     const AsmArgs* args = reinterpret_cast<const AsmArgs*>(d_args);
-    if (cs[0]->form == BM_MIXED) {
-        e = cudaFuncSetAttribute(assemble_batch_kernel<BM_MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem);
-        if (e != cudaSuccess) return e;
-        assemble_batch_kernel<BM_MIXED><<<grid, blk, smem, s>>>(args);
-    } else {
-        e = cudaFuncSetAttribute(assemble_batch_kernel<BM_ORDINARY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem);
-        if (e != cudaSuccess) return e;
-        assemble_batch_kernel<BM_ORDINARY><<<grid, blk, smem, s>>>(args);
-    }
-    return cudaGetLastError();
+    const bool big = big_tiles(c, B);
+    auto go = [&](auto form) {
+        constexpr int F = decltype(form)::value;
+        return big ? launch_tiles<32>(s, assemble_batch_kernel<F, 32>, c->N, B, args)
+                   : launch_tiles<16>(s, assemble_batch_kernel<F, 16>, c->N, B, args);
+    };
+    return c->form == BM_MIXED ? go(std::integral_constant<int, BM_MIXED>{})
+                               : go(std::integral_constant<int, BM_ORDINARY>{});
 }
 
 cudaError_t launch_zeta_band(cudaStream_t s, const bm_ctx* c) {

@@ -191,6 +191,7 @@ struct HankelTable {
     const double2* c;  // coefficient blocks, HT_SLOTS per anchor
     int nx, ny;
     double re0, im0, step, inv_step;
+    int iy_real;       // the row of anchors on the real axis
 };
 // Builds (once per process) the host copy of the anchor table: {H0(z0), H1(z0)} per anchor.
 const std::vector<double2>& hankel_anchor_host(int& nx, int& ny, double& re0, double& im0, double& step);
@@ -260,6 +261,8 @@ struct bm_ctx {
     double* d_normA = nullptr;  // ||A||_inf (device scalar)
     // the FP64 operator split into FP32 hi/lo planes (CF32 precisions; same layout and leading
     // dimensions as d_Mtop / d_Mbot / d_A) for the double-float residual
+    // (planes: 0 none, 1 the hi/lo planes, whose hi parts the FP32 residual updates read, 2 also the sums)
+    int planes = 0;
     float4* d_Ptop = nullptr;
     float4* d_Pbot = nullptr;
     float4* d_PA = nullptr;
@@ -424,7 +427,7 @@ struct ProfScope {
 // allocation helpers (api.cu)
 bm_status ctx_alloc(bm_ctx* c, void** p, size_t bytes);
 void ctx_free(bm_ctx* c, void* p);
-size_t request_bytes(int N, int form, int prec, int nb, int nrhs, bool optional, int num_sms);  // api.cu
+size_t request_bytes(int N, int form, int prec, int nb, int nrhs, int resid_mode, bool optional, int num_sms);  // api.cu
 void ctx_release(bm_ctx* c);                                        // api.cu
 
 // ---------------------------------------------------------------------------------------------

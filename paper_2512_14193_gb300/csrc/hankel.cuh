@@ -118,14 +118,21 @@ __device__ __forceinline__ void series(double2 z, double2& h0, double2& h1) {
     h1 = make_double2(J1.x - Y1.y, J1.y + Y1.x);
 }
 
+// Index of the grid line (origin a0, spacing step = 1 / inv_step, a power of two) nearest to a, and a's
+// offset from it: adding 1.5 2^52 rounds to an integer, whose low word is the index (three FP64
+// operations instead of seven).
+__device__ __forceinline__ int grid_line(double a, double a0, double step, double inv_step, int n, double& d) {
+    const double c = 6755399441055744.0 - a0 * inv_step;  // (a0 inv_step is an integer: exact)
+    const double t = fma(a, inv_step, c);
+    d = fma(-step, t - c, a);
+    return min(max(__double2loint(t), 0), n - 1);
+}
+
 __device__ __forceinline__ void taylor(double2 z, const HankelTable& T, double2& h0, double2& h1) {
-    int ix = __double2int_rn((z.x - T.re0) * T.inv_step);
-    int iy = __double2int_rn((z.y - T.im0) * T.inv_step);
-    ix = min(max(ix, 0), T.nx - 1);
-    iy = min(max(iy, 0), T.ny - 1);
-    const double2 z0 = make_double2(T.re0 + ix * T.step, T.im0 + iy * T.step);
+    double2 d;
+    const int ix = grid_line(z.x, T.re0, T.step, T.inv_step, T.nx, d.x);
+    const int iy = grid_line(z.y, T.im0, T.step, T.inv_step, T.ny, d.y);
     const double2* C = T.c + (long)HT_SLOTS * ((long)iy * T.nx + ix);
-    const double2 d = csub(z, z0);
     // Horner's scheme for P(d) = sum a_k d^k and its derivative together (Q <- Q d + P before
     // P <- P d + a_k): a_18 .. a_9 in FP32, then a_8 .. a_0 in FP64.  H0 = P, H1 = -P'.
     const float4* C32 = reinterpret_cast<const float4*>(C + HT_K64);
@@ -202,6 +209,91 @@ __device__ __forceinline__ void hankel01(double2 z, const HankelTable& T, double
     if (r2 < R_SERIES * R_SERIES) series(z, h0, h1);
     else if (r2 < R_ASYM * R_ASYM) taylor(z, T, h0, h1);
     else asym(z, h0, h1);
+}
+
+// ---- real arguments: the same zones with real arithmetic where the terms are real (a real wavenumber's
+//      operator; the FP64 operations of an evaluation halve) ----
+__device__ __forceinline__ void series_real(double z, double2& h0, double2& h1) {
+    const double w = -0.25 * z * z;
+    constexpr float THR[15] = {1e-17f,    6.32456e-9f, 7.11379e-6f, 2.75490e-4f, 2.70192e-3f,
+                               1.31556e-2f, 4.25859e-2f, 0.106263f,  0.222133f,  0.409216f,
+                               0.686394f, 1.07166f,    1.58169f,    2.23167f,    3.03529f};  // as in series()
+    const float zf = (float)z, wa = 0.25f * zf * zf;
+    double t0 = 1.0, t1 = 1.0, J0 = 1.0, J1 = 1.0, S0 = 0.0, S1 = -2.0 * EULER_GAMMA + 1.0;
+    constexpr int M64 = 10;
+    double Hm = 0.0;
+#pragma unroll
+    for (int m = 1; m < M64; ++m) {
+        if (wa <= THR[m - 1]) break;
+        const double dm = (double)m;
+        t0 *= w * (1.0 / (dm * dm));
+        t1 *= w * (1.0 / (dm * (dm + 1.0)));
+        Hm += 1.0 / dm;
+        J0 += t0;
+        J1 += t1;
+        S0 = fma(t0, Hm, S0);
+        S1 = fma(t1, -2.0 * EULER_GAMMA + 2.0 * Hm + 1.0 / (dm + 1.0), S1);
+    }
+    if (wa > THR[M64 - 1]) {
+        const float fw = (float)w;
+        float ft0 = (float)t0, ft1 = (float)t1, fJ0 = 0.f, fJ1 = 0.f, fS0 = 0.f, fS1 = 0.f, fH = (float)Hm;
+#pragma unroll
+        for (int m = M64; m < 16; ++m) {
+            if (wa <= THR[m - 1]) break;
+            const float dm = (float)m;
+            ft0 *= fw * (1.0f / (dm * dm));
+            ft1 *= fw * (1.0f / (dm * (dm + 1.0f)));
+            fH += 1.0f / dm;
+            fJ0 += ft0;
+            fJ1 += ft1;
+            fS0 += ft0 * fH;
+            fS1 += ft1 * ((float)(-2.0 * EULER_GAMMA) + 2.0f * fH + 1.0f / (dm + 1.0f));
+        }
+        J0 += fJ0;
+        J1 += fJ1;
+        S0 += fS0;
+        S1 += fS1;
+    }
+    const double zh = 0.5 * z, L = log(zh);
+    J1 *= zh;
+    h0 = make_double2(J0, TWO_OVER_PI * (fma(L + EULER_GAMMA, J0, -S0)));
+    h1 = make_double2(J1, fma(TWO_OVER_PI, fma(L, J1, -1.0 / z), -ONE_OVER_PI * zh * S1));
+}
+
+__device__ __forceinline__ void taylor_real(double z, const HankelTable& T, double2& h0, double2& h1) {
+    double d;
+    const int ix = grid_line(z, T.re0, T.step, T.inv_step, T.nx, d);
+    const double2* C = T.c + (long)HT_SLOTS * ((long)T.iy_real * T.nx + ix);
+    const float4* C32 = reinterpret_cast<const float4*>(C + HT_K64);
+    float2 c32[HT_K32];
+#pragma unroll
+    for (int j = 0; j < HT_K32 / 2; ++j) {
+        const float4 v = __ldg(C32 + j);
+        c32[2 * j] = make_float2(v.x, v.y);
+        c32[2 * j + 1] = make_float2(v.z, v.w);
+    }
+    const float fd = (float)d;
+    float2 fp = c32[HT_K32 - 1], fq = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int j = HT_K32 - 2; j >= 0; --j) {
+        fq = make_float2(fmaf(fq.x, fd, fp.x), fmaf(fq.y, fd, fp.y));
+        fp = make_float2(fmaf(fp.x, fd, c32[j].x), fmaf(fp.y, fd, c32[j].y));
+    }
+    double2 P = make_double2(fp.x, fp.y), Q = make_double2(fq.x, fq.y);
+#pragma unroll
+    for (int k = HT_K64 - 1; k >= 0; --k) {
+        const double2 ak = __ldg(C + k);
+        Q = make_double2(fma(Q.x, d, P.x), fma(Q.y, d, P.y));
+        P = make_double2(fma(P.x, d, ak.x), fma(P.y, d, ak.y));
+    }
+    h0 = P;
+    h1 = cneg(Q);
+}
+
+__device__ __forceinline__ void hankel01_real(double z, const HankelTable& T, double2& h0, double2& h1) {
+    if (z < R_SERIES) series_real(z, h0, h1);
+    else if (z < R_ASYM) taylor_real(z, T, h0, h1);
+    else asym(make_double2(z, 0.0), h0, h1);
 }
 
 }  // namespace hk

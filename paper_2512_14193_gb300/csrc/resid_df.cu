@@ -178,7 +178,7 @@ __global__ void split_planes_kernel(const double2* __restrict__ A, long lda, int
     const double2 v = A[i + (long)j * lda];
     const float2 r = split1(v.x), im = split1(v.y);
     P[i + (long)j * ldp] = make_float4(r.x, r.y, im.x, im.y);
-    Q[i + (long)j * ldp] = split1(v.x + v.y);
+    if (Q != nullptr) Q[i + (long)j * ldp] = split1(v.x + v.y);
 }
 
 }  // namespace

@@ -144,9 +144,9 @@ extern "C" bm_status bm_server_submit(bm_server* s, const bm_request* r, unsigne
     const int nsys = (r->formulation == BM_MIXED) ? 3 * r->N : 2 * r->N;
     if (r->ldb < nsys || r->ldx < nsys) return BM_EINVAL;
     const int sms = s->handles[0]->num_sms;
-    size_t bytes = request_bytes(r->N, r->formulation, s->opts.prec, s->opts.nb, r->nrhs, true, sms);
+    size_t bytes = request_bytes(r->N, r->formulation, s->opts.prec, s->opts.nb, r->nrhs, s->opts.refine_residual, true, sms);
     if (bytes > s->budget)
-        bytes = request_bytes(r->N, r->formulation, s->opts.prec, s->opts.nb, r->nrhs, false, sms);
+        bytes = request_bytes(r->N, r->formulation, s->opts.prec, s->opts.nb, r->nrhs, s->opts.refine_residual, false, sms);
     if (bytes > s->budget) {
         bm_set_error("bm_server_submit: the request needs " + std::to_string(bytes) + " bytes, more than the budget " +
                      std::to_string(s->budget));
