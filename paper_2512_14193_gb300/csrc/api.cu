@@ -170,6 +170,7 @@ void free_solve_ws(bm_ctx* c) {
     FREE(c->d_Bx1i);
     FREE(c->d_Bx2r);
     FREE(c->d_Bx2i);
+    FREE(c->d_Bxe);
     FREE(c->d_Pkr);
     FREE(c->d_Pki);
     FREE(c->d_XP);
@@ -215,10 +216,12 @@ void free_problem(bm_ctx* c) {
     FREE(c->d_Ap_i);
     FREE(c->d_Bp_r);
     FREE(c->d_Bp_i);
+    FREE(c->d_Bpe);
     FREE(c->d_Lp_r);
     FREE(c->d_Lp_i);
     FREE(c->d_Up_r);
     FREE(c->d_Up_i);
+    FREE(c->d_Upe);
     FREE(c->d_Cp_r);
     FREE(c->d_Cp_i);
     FREE(c->d_fd);
@@ -238,19 +241,18 @@ double2 d2(bm_c64 z) { return make_double2(z.re, z.im); }
 long round_up(long a, long b) { return (a + b - 1) / b * b; }
 
 // Split planes of the operator a residual mode reads: all of them for double-float residuals, the hi/lo ones
-// where residual updates run on the CUDA cores (the ordinary system and single TF32), none else.
+// where residual updates run on the CUDA cores (the ordinary system), none else.
 int planes_needed(int form, int prec, int resid_mode) {
     if (prec == BM_FP64) return 0;
     if (resid_mode == BM_RESID_DF_UPDATE) return 2;
     if (resid_mode == BM_RESID_FP64_ALL || resid_mode == BM_RESID_TC_ALL) return 0;
-    return form == BM_ORDINARY || prec == BM_CF32_TF32_IR ? 1 : 0;
+    return form == BM_ORDINARY ? 1 : 0;
 }
 
 // fast: the FP32 LU in search-free blocks (lu_fast.cu), with its work buffer
 Plan make_plan(int N, int form, int prec, int nb_user, int bs, int nd, bool fast, int planes) {
     Plan p;
     const bool c32 = prec != BM_FP64;
-    const bool split = prec == BM_CF32_3XTF32_IR;
     p.n = (form == BM_MIXED) ? N : 2 * N;
     p.nsys = (form == BM_MIXED) ? 3 * N : 2 * N;
     p.nb = nb_user > 0 ? nb_user : (c32 ? 256 : 64);
@@ -272,19 +274,15 @@ Plan make_plan(int N, int form, int prec, int nb_user, int bs, int nd, bool fast
         const size_t pb = planes == 2 ? 24 : (planes == 1 ? 16 : 0);
         b += (form == BM_MIXED) ? (size_t)p.ldtop * N * pb + (size_t)p.ldbot * 2 * N * pb : (size_t)p.ldA * 2 * N * pb;
         if (form == BM_MIXED) {
-            p.kseg = 2 * N;
-            long kext = split ? 3L * p.kseg : p.kseg;
-            p.ldk_schur = round_up(kext, 32);
-            b += 2 * (size_t)N * p.ldk_schur * 8;
+            p.ldk_schur = tc_ldk(2L * N);
+            b += 2 * (size_t)N * p.ldk_schur * 4 + (size_t)N * 4;
             // [M13; M23] rows for the skinny products of the solve
-            p.ldk_c = round_up(split ? 3L * N : (long)N, 32);
-            b += 2 * (size_t)N * p.ldk_c * 8;
+            p.ldk_c = tc_ldk(N);
+            b += 2 * (size_t)N * p.ldk_c * 4;
         }
-        // packs of the trailing updates (the search-free blocks always take 3xTF32 products) and the
-        // search-free blocks' work buffer
-        long kl = split ? 3L * p.nb : p.nb;
-        p.ldk_lu = round_up(fast ? std::max(kl, 3L * 128) : kl, 32);
-        b += 2 * (size_t)p.n * p.ldk_lu * 8;
+        // packs of the trailing updates and the search-free blocks' work buffer
+        p.ldk_lu = tc_ldk(fast ? std::max(p.nb, 128) : p.nb);
+        b += 2 * (size_t)p.n * p.ldk_lu * 4 + (size_t)p.n * 4;
         if (fast) b += lu_fast_bytes(p.n);
         // digit planes of the operator for the tensor-core residual, their row exponents, and the
         // row-maximum scratch of their construction
@@ -325,7 +323,7 @@ size_t request_bytes(int N, int form, int prec, int nb, int nrhs, int resid_mode
         b += (size_t)p.n * w * 16;
     } else {
         b += (size_t)p.nsys * w * 8 + (size_t)p.n * w * 16 + (size_t)p.nsys * w * 24 + 4 * (size_t)N * w * 16;
-        if (form == BM_MIXED) b += 2 * w * (size_t)(p.ldk_schur + p.ldk_c) * 4 + ((size_t)64 << 20);
+        if (form == BM_MIXED) b += 2 * w * (size_t)(p.ldk_schur + p.ldk_c) * 2 + 8 * w + ((size_t)64 << 20);
     }
     return b;
 }
@@ -421,9 +419,9 @@ extern "C" bm_status bm_enqueue_probe(bm_ctx* c, int which, int reps) {
                 BM_CUDA_TRY(gemm_z64(s, c->N, c->N, 2 * c->N, -1.0, Z64{c->d_Mbot, c->ldbot}, false,
                                      Z64{c->d_Mtop, c->ldtop}, 0.0, Z64{c->d_F64, c->ldF}));
             } else {
-                long kext = (c->prec == BM_CF32_3XTF32_IR) ? 3L * c->kseg_schur : c->kseg_schur;
                 BM_CUDA_TRY(gemm_tc(s, c->tm_schur[0], c->tm_schur[1], c->tm_schur[2], c->tm_schur[3], c->d_F32r,
-                                    c->d_F32i, c->ldF, c->N, c->N, (int)kext, -1.0f, 0.0f, c->d_err));
+                                    c->d_F32i, c->ldF, c->N, c->N, 2 * c->N, -1.0f, 0.0f,
+                                    TcScale{c->d_dge[1], c->d_Bpe, TC_E_DGE}, c->d_err));
             }
             c->launches += 1;
         }
@@ -622,7 +620,6 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
     c->ldA = p.ldA;
     c->ldF = p.ldF;
     c->ldk_schur = p.ldk_schur;
-    c->kseg_schur = p.kseg;
     c->ldk_lu = p.ldk_lu;
     c->ldk_c = p.ldk_c;
     const bool c32 = prec != BM_FP64;
@@ -652,20 +649,22 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
         s = alloc_t(c, &c->d_F32r, (size_t)p.ldF * p.n * 4);
         if (s == BM_OK) s = alloc_t(c, &c->d_F32i, (size_t)p.ldF * p.n * 4);
         if (s == BM_OK && form == BM_MIXED) {
-            size_t pb = (size_t)N * p.ldk_schur * 4;
+            size_t pb = (size_t)N * p.ldk_schur * 2;
             if (s == BM_OK) s = alloc_t(c, &c->d_Ap_r, pb);
             if (s == BM_OK) s = alloc_t(c, &c->d_Ap_i, pb);
             if (s == BM_OK) s = alloc_t(c, &c->d_Bp_r, pb);
             if (s == BM_OK) s = alloc_t(c, &c->d_Bp_i, pb);
-            size_t cb = (size_t)2 * N * p.ldk_c * 4;
+            if (s == BM_OK) s = alloc_t(c, &c->d_Bpe, (size_t)N * 4);
+            size_t cb = (size_t)2 * N * p.ldk_c * 2;
             if (s == BM_OK) s = alloc_t(c, &c->d_Cp_r, cb);
             if (s == BM_OK) s = alloc_t(c, &c->d_Cp_i, cb);
         }
-        size_t lb = (size_t)p.n * p.ldk_lu * 4;
+        size_t lb = (size_t)p.n * p.ldk_lu * 2;
         if (s == BM_OK) s = alloc_t(c, &c->d_Lp_r, lb);
         if (s == BM_OK) s = alloc_t(c, &c->d_Lp_i, lb);
         if (s == BM_OK) s = alloc_t(c, &c->d_Up_r, lb);
         if (s == BM_OK) s = alloc_t(c, &c->d_Up_i, lb);
+        if (s == BM_OK) s = alloc_t(c, &c->d_Upe, (size_t)p.n * 4);
         if (s == BM_OK && c32 && c->lu_fast) s = alloc_t(c, &c->d_fd, lu_fast_bytes(p.n));
     }
     if (s == BM_OK && c32) {
@@ -693,7 +692,7 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
     }  // !reuse
     cudaStream_t st = c->stream;
     if (c32 && !reuse) {
-        size_t lb = (size_t)p.n * p.ldk_lu * 4;
+        size_t lb = (size_t)p.n * p.ldk_lu * 2;
         BM_CUDA_TRY(cudaMemsetAsync(c->d_Lp_r, 0, lb, st));
         BM_CUDA_TRY(cudaMemsetAsync(c->d_Lp_i, 0, lb, st));
         BM_CUDA_TRY(cudaMemsetAsync(c->d_Up_r, 0, lb, st));
@@ -751,8 +750,6 @@ bm_status assemble_post(bm_ctx* c, bool run_assembly_kernel, bool wait) {
     c->launches += ((form == BM_MIXED) ? 2 : 1) + (c->zeta_p > 0 ? 1 : 0);
     if (c32) {
         if (form == BM_MIXED) {
-            BM_CUDA_TRY(launch_pack_solve(st, c, prec == BM_CF32_3XTF32_IR));
-            c->launches += 1;
             if (c->planes) {
                 BM_CUDA_TRY(launch_split_planes(st, c->d_Mtop, c->ldtop, 2 * N, N, c->d_Ptop, c->d_Qtop, c->ldtop));
                 BM_CUDA_TRY(launch_split_planes(st, c->d_Mbot, c->ldbot, N, 2 * N, c->d_Pbot, c->d_Qbot, c->ldbot));
@@ -774,7 +771,8 @@ bm_status assemble_post(bm_ctx* c, bool run_assembly_kernel, bool wait) {
                                         nd));
             BM_CUDA_TRY(launch_digits_a(st, c->d_Mbot, c->ldbot, N, 2 * N, c->d_dge[1], c->d_dg[1], c->dg_ldk[1], rowmax,
                                         nd));
-            c->launches += 6;
+            BM_CUDA_TRY(launch_pack_solve(st, c));
+            c->launches += 7;
         } else {
             BM_CUDA_TRY(launch_digits_a(st, c->d_A, c->ldA, 2 * N, 2 * N, c->d_dge[0], c->d_dg[0], c->dg_ldk[0], rowmax,
                                         nd));
@@ -789,16 +787,13 @@ bm_status assemble_post(bm_ctx* c, bool run_assembly_kernel, bool wait) {
     BM_CUDA_TRY(cudaMemsetAsync(c->d_info + 3, c->opt_test_wait == 2 ? 1 : 0, sizeof(int), c->stream));
     if (wait) BM_CUDA_TRY(cudaStreamSynchronize(c->stream));
     if (c32) {
-        const bool split = prec == BM_CF32_3XTF32_IR;
         if (form == BM_MIXED) {
-            long kext = split ? 3L * p.kseg : p.kseg;
-            BM_TRY(tc_make_map(c->tm_schur[0], c->d_Ap_r, N, kext, p.ldk_schur, TC_BM));
-            BM_TRY(tc_make_map(c->tm_schur[1], c->d_Ap_i, N, kext, p.ldk_schur, TC_BM));
-            BM_TRY(tc_make_map(c->tm_schur[2], c->d_Bp_r, N, kext, p.ldk_schur, TC_BN));
-            BM_TRY(tc_make_map(c->tm_schur[3], c->d_Bp_i, N, kext, p.ldk_schur, TC_BN));
-            long kext_c = split ? 3L * N : (long)N;
-            BM_TRY(tc_make_map(c->tm_skinny[0], c->d_Cp_r, 2L * N, kext_c, p.ldk_c, TC_BM));
-            BM_TRY(tc_make_map(c->tm_skinny[1], c->d_Cp_i, 2L * N, kext_c, p.ldk_c, TC_BM));
+            BM_TRY(tc_make_map(c->tm_schur[0], c->d_Ap_r, N, 2L * N, p.ldk_schur, TC_BM));
+            BM_TRY(tc_make_map(c->tm_schur[1], c->d_Ap_i, N, 2L * N, p.ldk_schur, TC_BM));
+            BM_TRY(tc_make_map(c->tm_schur[2], c->d_Bp_r, N, 2L * N, p.ldk_schur, TC_BN));
+            BM_TRY(tc_make_map(c->tm_schur[3], c->d_Bp_i, N, 2L * N, p.ldk_schur, TC_BN));
+            BM_TRY(tc_make_map(c->tm_skinny[0], c->d_Cp_r, 2L * N, N, p.ldk_c, TC_BM));
+            BM_TRY(tc_make_map(c->tm_skinny[1], c->d_Cp_i, 2L * N, N, p.ldk_c, TC_BM));
             c->tc_skinny = true;
         }
         {
@@ -807,7 +802,7 @@ bm_status assemble_post(bm_ctx* c, bool run_assembly_kernel, bool wait) {
             if (form == BM_MIXED)
                 BM_TRY(rt_make_map(c->tm_dg[1], c->d_dg[1], N, 2L * N, c->dg_ldk[1], (long)N * c->dg_ldk[1], 128, nd));
         }
-        long klu = p.ldk_lu;
+        const long klu = p.ldk_lu / 2;
         BM_TRY(tc_make_map(c->tm_lu[0], c->d_Lp_r, p.n, klu, p.ldk_lu, TC_BM));
         BM_TRY(tc_make_map(c->tm_lu[1], c->d_Lp_i, p.n, klu, p.ldk_lu, TC_BM));
         BM_TRY(tc_make_map(c->tm_lu[2], c->d_Up_r, p.n, klu, p.ldk_lu, TC_BN));
@@ -872,15 +867,15 @@ bm_status factor_sequence(bm_ctx* c) {
         }
     } else {
         if (c->form == BM_MIXED) {
-            // the FP32 operands of the Schur product, then U33 = -[M31 M32] [M13; M23]
+            // the packed operands of the Schur product, then U33 = -[M31 M32] [M13; M23]
             {
                 BM_PROF(c, "pack_schur (pack_rowmajor/colmajor_kernel)");
-                BM_CUDA_TRY(launch_pack_schur(s, c, c->prec == BM_CF32_3XTF32_IR));
+                BM_CUDA_TRY(launch_pack_schur(s, c));
             }
-            long kext = (c->prec == BM_CF32_3XTF32_IR) ? 3L * c->kseg_schur : c->kseg_schur;
             BM_PROF(c, "cgemm_tc_kernel (Schur complement)");
             BM_CUDA_TRY(gemm_tc(s, c->tm_schur[0], c->tm_schur[1], c->tm_schur[2], c->tm_schur[3], c->d_F32r,
-                                c->d_F32i, c->ldF, c->N, c->N, (int)kext, -1.0f, 0.0f, c->d_err));
+                                c->d_F32i, c->ldF, c->N, c->N, 2 * c->N, -1.0f, 0.0f,
+                                TcScale{c->d_dge[1], c->d_Bpe, TC_E_DGE}, c->d_err));
         } else {
             BM_PROF(c, "to_c32_kernel");
             BM_CUDA_TRY(launch_to_c32(s, c->d_A, c->ldA, c->n, c->n, c->d_F32r, c->d_F32i, c->ldF));
@@ -1069,31 +1064,30 @@ bm_status ensure_ws(bm_ctx* c, int nrhs) {
     }
     if (c->tc_skinny) {
         const int N = c->N;
-        const bool split = c->prec == BM_CF32_3XTF32_IR;
-        const long k1 = split ? 6L * N : 2L * N, k2 = split ? 3L * N : (long)N;
-        BM_TRY(alloc_t(c, &c->d_Bx1r, (size_t)w * c->ldk_schur * 4));
-        BM_TRY(alloc_t(c, &c->d_Bx1i, (size_t)w * c->ldk_schur * 4));
-        BM_TRY(alloc_t(c, &c->d_Bx2r, (size_t)w * c->ldk_c * 4));
-        BM_TRY(alloc_t(c, &c->d_Bx2i, (size_t)w * c->ldk_c * 4));
+        BM_TRY(alloc_t(c, &c->d_Bx1r, (size_t)w * c->ldk_schur * 2));
+        BM_TRY(alloc_t(c, &c->d_Bx1i, (size_t)w * c->ldk_schur * 2));
+        BM_TRY(alloc_t(c, &c->d_Bx2r, (size_t)w * c->ldk_c * 2));
+        BM_TRY(alloc_t(c, &c->d_Bx2i, (size_t)w * c->ldk_c * 2));
+        BM_TRY(alloc_t(c, &c->d_Bxe, 2 * (size_t)w * sizeof(int)));
         // rows past a call's nrhs only feed output columns that are never stored; zero them anyway
-        BM_CUDA_TRY(cudaMemsetAsync(c->d_Bx1r, 0, (size_t)w * c->ldk_schur * 4, c->stream));
-        BM_CUDA_TRY(cudaMemsetAsync(c->d_Bx1i, 0, (size_t)w * c->ldk_schur * 4, c->stream));
-        BM_CUDA_TRY(cudaMemsetAsync(c->d_Bx2r, 0, (size_t)w * c->ldk_c * 4, c->stream));
-        BM_CUDA_TRY(cudaMemsetAsync(c->d_Bx2i, 0, (size_t)w * c->ldk_c * 4, c->stream));
+        BM_CUDA_TRY(cudaMemsetAsync(c->d_Bx1r, 0, (size_t)w * c->ldk_schur * 2, c->stream));
+        BM_CUDA_TRY(cudaMemsetAsync(c->d_Bx1i, 0, (size_t)w * c->ldk_schur * 2, c->stream));
+        BM_CUDA_TRY(cudaMemsetAsync(c->d_Bx2r, 0, (size_t)w * c->ldk_c * 2, c->stream));
+        BM_CUDA_TRY(cudaMemsetAsync(c->d_Bx2i, 0, (size_t)w * c->ldk_c * 2, c->stream));
         // partial sums of the two product shapes (N x nrhs over 2N, 2N x nrhs over N) for every
         // nrhs up to w (the split count falls when nrhs crosses a tile boundary)
         size_t pe = 0;
         for (int q = 1; q <= w; ++q) {
-            pe = std::max(pe, (size_t)tc_split_k(N, q, (int)k1, c->num_sms) * N * q);
-            pe = std::max(pe, (size_t)tc_split_k(2 * N, q, (int)k2, c->num_sms) * 2 * N * q);
+            pe = std::max(pe, (size_t)tc_split_k(N, q, 2 * N, c->num_sms) * N * q);
+            pe = std::max(pe, (size_t)tc_split_k(2 * N, q, N, c->num_sms) * 2 * N * q);
         }
         BM_TRY(alloc_t(c, &c->d_Pkr, pe * 4));
         BM_TRY(alloc_t(c, &c->d_Pki, pe * 4));
         c->pk_elems = pe;
-        BM_TRY(tc_make_map(c->tm_skinny[2], c->d_Bx1r, w, k1, c->ldk_schur, TC_BN));
-        BM_TRY(tc_make_map(c->tm_skinny[3], c->d_Bx1i, w, k1, c->ldk_schur, TC_BN));
-        BM_TRY(tc_make_map(c->tm_skinny[4], c->d_Bx2r, w, k2, c->ldk_c, TC_BN));
-        BM_TRY(tc_make_map(c->tm_skinny[5], c->d_Bx2i, w, k2, c->ldk_c, TC_BN));
+        BM_TRY(tc_make_map(c->tm_skinny[2], c->d_Bx1r, w, 2L * N, c->ldk_schur, TC_BN));
+        BM_TRY(tc_make_map(c->tm_skinny[3], c->d_Bx1i, w, 2L * N, c->ldk_schur, TC_BN));
+        BM_TRY(tc_make_map(c->tm_skinny[4], c->d_Bx2r, w, N, c->ldk_c, TC_BN));
+        BM_TRY(tc_make_map(c->tm_skinny[5], c->d_Bx2i, w, N, c->ldk_c, TC_BN));
     }
     c->ws_nrhs = w;
     return BM_OK;

@@ -23,6 +23,7 @@
 #include "common.cuh"
 #include "hankel.cuh"
 #include "kernels.cuh"
+#include "tc_pack.cuh"
 
 namespace {
 
@@ -472,86 +473,54 @@ __global__ void hankel_probe_kernel(const double2* __restrict__ z, int n, Hankel
     h1[i] = b;
 }
 
-__device__ __forceinline__ float tf32_rna(float x) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return __uint_as_float(r);
-}
-
-// Schur A operand: Mbot (N x 2N col-major FP64) -> row-major [N][ldk] planar FP32, segments
-// (3xTF32: [hi | hi | lo]); B operand: Mtop (2N x N) -> [N][ldk] with column n of Mtop as row n
-// (3xTF32: [hi | lo | hi]).  Padding columns [nseg*K, ldk) are zeroed.
-__global__ void pack_rowmajor_kernel(const double2* __restrict__ M, long ldm, int rows, int K, int split,
-                                     float* __restrict__ Pr, float* __restrict__ Pi, long ldk) {
+// A operands: rows of an FP64 column-major block (rows x K) as pack rows, scaled by the digit planes' row
+// exponents e (entries below 2^(e - 1); TC_E_DGE).  One 32 x 32 tile per CTA through shared memory, so that
+// both sides are coalesced; a warp writes the 128 bytes of a row.
+__global__ void pack_rowmajor_kernel(const double2* __restrict__ M, long ldm, int rows, int K,
+                                     const int* __restrict__ e, __half* __restrict__ Pr, __half* __restrict__ Pi,
+                                     long ldk) {
     __shared__ float2 t[32][33];
-    int k0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-    int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
+    const int k0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
+    const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
+#pragma unroll
     for (int q = ty; q < 32; q += 8) {
-        int r = r0 + tx, k = k0 + q;
-        double2 v = (r < rows && k < K) ? M[r + (long)k * ldm] : make_double2(0, 0);
+        const int r = r0 + tx, k = k0 + q;
+        const double2 v = (r < rows && k < K) ? M[r + (long)k * ldm] : make_double2(0, 0);
         t[q][tx] = make_float2((float)v.x, (float)v.y);
     }
     __syncthreads();
+#pragma unroll
     for (int q = ty; q < 32; q += 8) {
-        int r = r0 + q, k = k0 + tx;
-        if (r >= rows || k >= K) continue;
-        float2 v = t[tx][q];
-        long o = (long)r * ldk + k;
-        if (!split) {
-            Pr[o] = v.x;
-            Pi[o] = v.y;
-        } else {
-            float hr = tf32_rna(v.x), hi = tf32_rna(v.y);
-            Pr[o] = hr;
-            Pi[o] = hi;
-            Pr[o + K] = hr;
-            Pi[o + K] = hi;
-            Pr[o + 2 * K] = v.x - hr;
-            Pi[o + 2 * K] = v.y - hi;
-        }
+        const int r = r0 + q;
+        if (r >= rows) continue;
+        // lanes 0-15: the hi parts of entries 2 l and 2 l + 1, lanes 16-31: the lo parts
+        const TcRowScale sc(-TC_E_DGE - e[r]);
+        const int l = 2 * (tx & 15);
+        __half2 hr, lr, hi, li;
+        tc_split(sc(t[l][q].x), hr.x, lr.x);
+        tc_split(sc(t[l + 1][q].x), hr.y, lr.y);
+        tc_split(sc(t[l][q].y), hi.x, li.x);
+        tc_split(sc(t[l + 1][q].y), hi.y, li.y);
+        const long o = (long)r * ldk + 2 * k0 + 2 * tx;
+        *reinterpret_cast<__half2*>(Pr + o) = tx < 16 ? hr : lr;
+        *reinterpret_cast<__half2*>(Pi + o) = tx < 16 ? hi : li;
     }
 }
 
-__global__ void pack_colmajor_kernel(const double2* __restrict__ M, long ldm, int K, int cols, int split,
-                                     float* __restrict__ Pr, float* __restrict__ Pi, long ldk) {
-    long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    long kext = split ? 3L * K : (long)K;
-    long total = (long)cols * ldk;
-    if (idx >= total) return;
-    int n = (int)(idx / ldk);
-    long kk = idx - (long)n * ldk;
-    float vr = 0.f, vi = 0.f;
-    if (kk < kext) {
-        long k = kk % K;
-        int seg = (int)(kk / K);
-        double2 v = M[k + (long)n * ldm];
-        float fr = (float)v.x, fi = (float)v.y;
-        if (!split) {
-            vr = fr;
-            vi = fi;
-        } else {
-            float hr = tf32_rna(fr), hi = tf32_rna(fi);
-            if (seg == 1) {
-                vr = fr - hr;
-                vi = fi - hi;
-            } else {
-                vr = hr;
-                vi = hi;
-            }
-        }
+// B operand of the Schur product: column n of an FP64 block as pack row n, one CTA per column.
+struct ColZ64 {
+    const double2* p;
+    __device__ __forceinline__ float2 operator()(long k) const {
+        const double2 v = p[k];
+        return make_float2((float)v.x, (float)v.y);
     }
-    Pr[idx] = vr;
-    Pi[idx] = vi;
-}
-
-__global__ void pad_zero_rows_kernel(float* Pr, float* Pi, long ldk, int rows, long kext) {
-    // zero the K padding [kext, ldk) of each row of a row-major pack
-    long pad = ldk - kext;
-    long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (pad <= 0 || idx >= (long)rows * pad) return;
-    long r = idx / pad, c = kext + idx % pad;
-    Pr[r * ldk + c] = 0.f;
-    Pi[r * ldk + c] = 0.f;
+};
+__global__ void __launch_bounds__(TC_PACK_THREADS) pack_colmajor_kernel(const double2* __restrict__ M, long ldm, int K,
+                                                                        __half* __restrict__ Pr,
+                                                                        __half* __restrict__ Pi, long ldk,
+                                                                        int* __restrict__ e) {
+    const long n = blockIdx.x;
+    tc_pack_column(ColZ64{M + n * ldm}, K, Pr + n * ldk, Pi + n * ldk, e + n);
 }
 
 __global__ void to_c32_kernel(const double2* __restrict__ A, long lda, int m, int n, float* Fr, float* Fi, long ldf) {
@@ -957,29 +926,21 @@ cudaError_t launch_hankel_probe(cudaStream_t s, const bm_ctx* c, const double2* 
 
 // Operands of the Schur-complement product (part of the factorisation, like the FP32 copy of the
 // ordinary matrix): A = [M31 M32] row-major, B = [M13; M23] column by column.
-cudaError_t launch_pack_schur(cudaStream_t s, const bm_ctx* c, int split) {
-    int N = c->N;
-    int K = 2 * N;
-    dim3 blk(32, 8);
-    dim3 grid(ceil_div(K, 32), ceil_div(N, 32));
-    pack_rowmajor_kernel<<<grid, blk, 0, s>>>(c->d_Mbot, c->ldbot, N, K, split, c->d_Ap_r, c->d_Ap_i, c->ldk_schur);
-    long kext = split ? 3L * K : (long)K;
-    long padn = (long)N * (c->ldk_schur - kext);
-    if (padn > 0) pad_zero_rows_kernel<<<ceil_div(padn, 256), 256, 0, s>>>(c->d_Ap_r, c->d_Ap_i, c->ldk_schur, N, kext);
-    long total = (long)N * c->ldk_schur;
-    pack_colmajor_kernel<<<ceil_div(total, 256), 256, 0, s>>>(c->d_Mtop, c->ldtop, K, N, split, c->d_Bp_r, c->d_Bp_i,
-                                                               c->ldk_schur);
+cudaError_t launch_pack_schur(cudaStream_t s, const bm_ctx* c) {
+    const int N = c->N, K = 2 * N;
+    pack_rowmajor_kernel<<<dim3(ceil_div(K, 32), ceil_div(N, 32)), dim3(32, 8), 0, s>>>(
+        c->d_Mbot, c->ldbot, N, K, c->d_dge[1], c->d_Ap_r, c->d_Ap_i, c->ldk_schur);
+    pack_colmajor_kernel<<<N, TC_PACK_THREADS, 0, s>>>(c->d_Mtop, c->ldtop, K, c->d_Bp_r, c->d_Bp_i, c->ldk_schur,
+                                                       c->d_Bpe);
     return cudaGetLastError();
 }
 
 // Rows of [M13; M23] (2N x N) for the skinny products [M13; M23] z of the solve (made once at
-// assembly, like the split planes of the residual); only the tensor maps read this pack, which
-// stop at K, so its padding columns stay unset.
-cudaError_t launch_pack_solve(cudaStream_t s, const bm_ctx* c, int split) {
-    int N = c->N;
-    dim3 blk(32, 8);
-    dim3 gridc(ceil_div(N, 32), ceil_div(2 * N, 32));
-    pack_rowmajor_kernel<<<gridc, blk, 0, s>>>(c->d_Mtop, c->ldtop, 2 * N, N, split, c->d_Cp_r, c->d_Cp_i, c->ldk_c);
+// assembly, after the digit planes, whose row exponents scale them).
+cudaError_t launch_pack_solve(cudaStream_t s, const bm_ctx* c) {
+    const int N = c->N;
+    pack_rowmajor_kernel<<<dim3(ceil_div(N, 32), ceil_div(2 * N, 32)), dim3(32, 8), 0, s>>>(
+        c->d_Mtop, c->ldtop, 2 * N, N, c->d_dge[0], c->d_Cp_r, c->d_Cp_i, c->ldk_c);
     return cudaGetLastError();
 }
 

@@ -2,6 +2,7 @@
 // launch helpers and the handle layout.  Not part of the public ABI (include/bm.h is).
 #pragma once
 
+#include <cuda_fp16.h>
 #include <atomic>
 #include <cuda_runtime.h>
 #include <cstdint>
@@ -217,7 +218,7 @@ struct DevBuf {
 // Sizes and leading dimensions of one assembled system (api.cu make_plan).
 struct Plan {
     long ldtop = 0, ldbot = 0, ldA = 0, ldF = 0, ldk_schur = 0, ldk_lu = 0, ldk_c = 0;
-    int n = 0, nsys = 0, nb = 0, kseg = 0, nblk = 0;
+    int n = 0, nsys = 0, nb = 0, nblk = 0;
     size_t bytes = 0;
 };
 
@@ -313,20 +314,22 @@ struct bm_ctx {
     void* d_dinvU = nullptr;
     int bs_solve = 64;
 
-    // tensor-core operand packs (FP32 planar, K-major, segments for 3xTF32)
-    float* d_Ap_r = nullptr;  // Schur A operand [M31 M32] (N rows x Kext)
-    float* d_Ap_i = nullptr;
-    float* d_Bp_r = nullptr;  // Schur B operand [M13; M23]^T rows (N rows x Kext)
-    float* d_Bp_i = nullptr;
+    // tensor-core operand packs (tc_pack.cuh; planar, ldk halves a row) and the exponents of their rows that
+    // are not the digit planes' d_dge
+    __half* d_Ap_r = nullptr;  // Schur A operand [M31 M32] (N rows, K = 2N; exponents d_dge[1])
+    __half* d_Ap_i = nullptr;
+    __half* d_Bp_r = nullptr;  // Schur B operand [M13; M23]^T rows (N rows, K = 2N; exponents d_Bpe)
+    __half* d_Bp_i = nullptr;
+    int* d_Bpe = nullptr;
     long ldk_schur = 0;
-    int kseg_schur = 0;       // K of one segment (2N)
-    float* d_Lp_r = nullptr;  // LU trailing-update packs
-    float* d_Lp_i = nullptr;
-    float* d_Up_r = nullptr;
-    float* d_Up_i = nullptr;
+    __half* d_Lp_r = nullptr;  // LU trailing-update packs (L21 times 2^TC_SHIFT_L; exponents d_Upe of U12)
+    __half* d_Lp_i = nullptr;
+    __half* d_Up_r = nullptr;
+    __half* d_Up_i = nullptr;
+    int* d_Upe = nullptr;
     long ldk_lu = 0;
-    float* d_Cp_r = nullptr;  // [M13; M23] rows, K = N (2N rows x Kext): A operand of the skinny
-    float* d_Cp_i = nullptr;  //   products [M13; M23] z of the mixed correction and residual update
+    __half* d_Cp_r = nullptr;  // [M13; M23] rows, K = N (2N rows; exponents d_dge[0]): A operand of the skinny
+    __half* d_Cp_i = nullptr;  //   products [M13; M23] z of the mixed correction and residual update
     long ldk_c = 0;
     float* d_O32r = nullptr;  // ordinary: FP32 copy of A is the LU buffer (d_F32*)
 
@@ -350,10 +353,11 @@ struct bm_ctx {
     double* d_colred = nullptr;  // per-column reductions (4 x nrhs)
     // mixed CF32: B operand packs of the skinny tensor-core products (ws_nrhs rows, K-major) and
     // the split-K partial-sum workspace
-    float* d_Bx1r = nullptr;  // [W1; W2] columns, K = 2N (ld ldk_schur)
-    float* d_Bx1i = nullptr;
-    float* d_Bx2r = nullptr;  // z3 columns, K = N (ld ldk_c)
-    float* d_Bx2i = nullptr;
+    __half* d_Bx1r = nullptr;  // [W1; W2] columns, K = 2N (ld ldk_schur)
+    __half* d_Bx1i = nullptr;
+    __half* d_Bx2r = nullptr;  // z3 columns, K = N (ld ldk_c)
+    __half* d_Bx2i = nullptr;
+    int* d_Bxe = nullptr;      // their exponents: ws_nrhs of [W1; W2], then of z3
     float* d_Pkr = nullptr;
     float* d_Pki = nullptr;
     float4* d_XP = nullptr;   // CF32: the iterate split for the double-float residual (nsys x nrhs)

@@ -1,17 +1,25 @@
 // Complex GEMM on the 5th-generation tensor cores (sm_103a): C = beta C + alpha A B^T with
-// A (m x K) and B (n x K) given as K-major planar FP32 packs, computed in TF32 with FP32
-// accumulation in tensor memory.  This is the contraction of Theorem thm:LU
-// (U33 = -[M31 M32][M13; M23]) and of every LU trailing update A22 -= L21 U12.
+// A (m x K) and B (n x K) given as K-major planar packs.  This is the contraction of Theorem thm:LU
+// (U33 = -[M31 M32][M13; M23]), of every LU trailing update A22 -= L21 U12 and of the skinny products of
+// the solve.
 //
-// Complex product with four real products ("4M") on planar operands:
-//     Dr = Ar Br^T - Ai Bi^T,  Di = Ar Bi^T + Ai Br^T
-// Two TMEM accumulators (128 lanes x 128 columns each); the minus sign uses the A-negate bit of
-// the instruction descriptor.  The 3xTF32 variant needs no kernel change: its packs repeat the
-// K range as [A_hi | A_hi | A_lo] and [B_hi | B_lo | B_hi], so one K-extended product sums
-// A_hi B_hi + A_hi B_lo + A_lo B_hi.
+// Operand split: every entry is an FP32 value scaled by a power of two of its row (A) or of its column
+// (rows of B) to below 2^15, and held as two FP16 numbers hi + lo (11 + 11 significant bits; entries below
+// 2^-18 of their row's largest keep 2^-40 of that one).  The product is A_hi B_hi + A_hi B_lo + A_lo B_hi,
+// the terms and significands of a 3xTF32 product, at twice its rate and from a third of its bytes: hi
+// and lo of 32 consecutive K are adjacent, [32 hi | 32 lo], one 128-byte shared row, so each is loaded
+// once for the three products.  Exponents: TcScale.  Schur complement N = 4096 (per-launch times):
+// 3.50 -> 1.58 ms against the same kernel on three-segment TF32 packs.
 //
-// CTA tile 128 x 128, K step 32 (128-byte rows), 3-stage TMA -> shared-memory pipeline with
-// mbarriers.  Warp 0 lane 0 issues TMA loads, warp 1 lane 0 issues tcgen05.mma; all four warps
+// Complex product with planar operands and one accumulator [Dr | Di] (128 lanes x 256 columns of TMEM):
+//     [Dr | Di] += Ar [Br; Bi]^T,  Dr -= Ai Bi^T,  Di += Ai Br^T
+// The real and imaginary tiles of B lie one after another in shared memory, so the first is one MMA of
+// width 256 (a narrower MMA reads A again: shared-memory bandwidth bounds 128 x 128 FP16 products); the
+// minus sign is the A-negate bit of the instruction descriptor.
+//
+// CTA tile 128 x 128, 32 K elements per stage (64 KB), 3-stage TMA -> shared-memory pipeline with
+// mbarriers.  Warp 0 lane 0 issues TMA loads, warp 1 the tcgen05.mma (the whole warp walks the loop so
+// that the operands live in uniform registers, lane 0 issues); all four warps
 // then read the accumulators (tcgen05.ld 32x32b, warp w owns TMEM lanes 32(w mod 4) .. +31 = rows)
 // and update C with coalesced column-major stores.  For C = C + alpha A B^T (the LU trailing
 // updates) a six-warp form loads the C tile into the upper half of TMEM during the main loop, so
@@ -21,6 +29,7 @@
 // up after 1 ms and takes that timeout path without issuing any product.
 #include "common.cuh"
 #include "kernels.cuh"
+#include "tc_pack.cuh"
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -31,15 +40,19 @@
 namespace {
 
 constexpr int BM = TC_BM, BN = TC_BN;
-constexpr int BKE = 32;  // K elements per stage (fp32: 128-byte rows, one swizzle span)
+constexpr int BKE = 32;  // K elements per stage: 32 hi and 32 lo halves, a 128-byte row (one swizzle span)
 constexpr int STAGES = 3;
-constexpr int TILE_A = BM * BKE * 4;
-constexpr int TILE_B = BN * BKE * 4;
+constexpr int TILE_A = BM * 2 * BKE * 2;
+constexpr int TILE_B = BN * 2 * BKE * 2;
 constexpr int STAGE_BYTES = 2 * TILE_A + 2 * TILE_B;
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
 constexpr uint32_t TMEM_COLS = 2 * BN;  // Dr, Di
 constexpr uint64_t WAIT_NS = 2000000000ull;
 constexpr uint64_t TEST_WAIT_NS = 1000000ull;  // the test hook's wait limit
+
+// Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 bytes apart.
+constexpr uint32_t DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (1u << 16); }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -97,12 +110,16 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-__device__ __forceinline__ void mma_tf32(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(
-            d),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
-        : "memory");
+// D (+)= A B from the low words of the two shared-memory descriptors, issued by the lanes with `leader` set;
+// the operands are warp-uniform.
+__device__ __forceinline__ void mma_f16(bool leader, uint32_t d, uint32_t alo, uint32_t blo, uint32_t idesc,
+                                        uint32_t acc) {
+    if (leader)
+        asm volatile(
+            "{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, %4, 0;\n mov.b64 a, {%1, %5};\n mov.b64 b, {%2, %5};\n"
+            " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n}\n" ::"r"(d),
+            "r"(alo), "r"(blo), "r"(idesc), "r"(acc), "n"(DESC_HI)
+            : "memory");
 }
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -130,16 +147,9 @@ __device__ __forceinline__ void tmem_ld16x2(uint32_t ta, uint32_t tb, float* va,
     }
 }
 
-// Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 bytes apart.
-__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
-           ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
-}
-
-// Instruction descriptor, kind::tf32: D = F32, A = B = TF32, both K-major, M = 128, N = BN.
-__host__ __device__ constexpr uint32_t idesc_tf32(uint32_t neg_a) {
-    return (1u << 4) | (2u << 7) | (2u << 10) | (neg_a << 13) | ((uint32_t)(BN >> 3) << 17) |
-           ((uint32_t)(BM >> 4) << 24);
+// Instruction descriptor, kind::f16: D = F32, A = B = F16, both K-major, M = 128, N = n.
+__host__ __device__ constexpr uint32_t idesc_f16(uint32_t neg_a, uint32_t n) {
+    return (1u << 4) | (neg_a << 13) | ((n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 }
 
 // Output modes: OUT_C32 C (FP32 planar) = beta C + alpha D; OUT_Z64 C64 (FP64) = beta C64 + alpha D;
@@ -172,18 +182,20 @@ __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.
 template <int OUT>
 __device__ __forceinline__ void cgemm_tc_body(const CUtensorMap& tmAr, const CUtensorMap& tmAi, const CUtensorMap& tmBr,
                                               const CUtensorMap& tmBi, float* __restrict__ Cr, float* __restrict__ Ci,
-                                              double2* __restrict__ C64, long ldc, long zstride, int m, int n, int kext,
-                                              int S, int zsplit, float alpha, float beta, int* __restrict__ err) {
+                                              double2* __restrict__ C64, long ldc, long zstride, int m, int n, int K,
+                                              int S, int zsplit, float alpha, float beta, const TcScale& sc,
+                                              int* __restrict__ err) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     // full[S], empty[S], done, never (the test hook's barrier: initialised, never arrived on)
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // (the shuffle tells the compiler that the warp index is uniform)
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int tm = blockIdx.x, tn = blockIdx.y;
     // this CTA's K split: k-blocks [kb_begin, kb_begin + nkb)
-    const int nkb_all = (kext + BKE - 1) / BKE;
+    const int nkb_all = (K + BKE - 1) / BKE;
     const int kb_begin = (int)((long)zsplit * nkb_all / S);
     const int nkb = (int)((long)(zsplit + 1) * nkb_all / S) - kb_begin;
     const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES), done = smem_u32(bars + 2 * STAGES);
@@ -216,7 +228,7 @@ __device__ __forceinline__ void cgemm_tc_body(const CUtensorMap& tmAr, const CUt
             uint8_t* st = smem + s * STAGE_BYTES;
             const uint32_t fb = full0 + 8 * s;
             mbar_expect_tx(fb, STAGE_BYTES);
-            const int kx = (kb_begin + kb) * BKE;
+            const int kx = (kb_begin + kb) * 2 * BKE;
             tma_load_2d(smem_u32(st), &tmAr, fb, kx, tm * BM);
             tma_load_2d(smem_u32(st + TILE_A), &tmAi, fb, kx, tm * BM);
             tma_load_2d(smem_u32(st + 2 * TILE_A), &tmBr, fb, kx, tn * BN);
@@ -231,9 +243,10 @@ __device__ __forceinline__ void cgemm_tc_body(const CUtensorMap& tmAr, const CUt
                 }
             }
         }
-    } else if (warp == 1 && lane == 0) {
-        // ---------------- MMA issuer ----------------
-        const uint32_t idp = idesc_tf32(0), idn = idesc_tf32(1);
+    } else if (warp == 1) {
+        // ---------------- MMA issuer (the whole warp walks the loop, lane 0 issues) ----------------
+        const bool leader = lane == 0;
+        constexpr uint32_t IDW = idesc_f16(0, 2 * BN), IDP = idesc_f16(0, BN), IDN = idesc_f16(1, BN);
         if (err[1] != 0) {
             // test hook: a wait that nothing ends, bounded like every other wait
             const uint64_t t0 = gtimer();
@@ -241,32 +254,42 @@ __device__ __forceinline__ void cgemm_tc_body(const CUtensorMap& tmAr, const CUt
             }
             *abort_flag = 1;
         }
+        const uint32_t lo0 = desc_lo(smem_u32(smem));
+        int s = 0;
+        uint32_t ph = 0;
         for (int kb = 0; kb < nkb && !*abort_flag; ++kb) {
-            const int s = kb % STAGES;
-            const uint32_t ph = (uint32_t)(kb / STAGES) & 1u;
             if (!mbar_wait(full0 + 8 * s, ph, abort_flag)) break;
             fence_after();
-            const uint32_t ar = smem_u32(smem + s * STAGE_BYTES);
-            const uint32_t ai = ar + TILE_A, br = ar + 2 * TILE_A, bi = br + TILE_B;
+            const uint32_t ar = lo0 + (uint32_t)s * (STAGE_BYTES >> 4);
+            const uint32_t ai = ar + (TILE_A >> 4), br = ar + (2 * TILE_A >> 4), bi = br + (TILE_B >> 4);
+            // [Dr | Di] (+)= A B^T at offsets oa and ob (16-byte units) of the 128-byte rows
+            auto product = [&](uint32_t oa, uint32_t ob, uint32_t acc) {
+                mma_f16(leader, Dr, ar + oa, br + ob, IDW, acc);
+                mma_f16(leader, Dr, ai + oa, bi + ob, IDN, 1u);
+                mma_f16(leader, Di, ai + oa, br + ob, IDP, 1u);
+            };
 #pragma unroll
-            for (int kk = 0; kk < BKE / 8; ++kk) {
-                const uint32_t off = kk * 32;  // 8 tf32 = 32 bytes along K inside the swizzle span
-                const uint64_t dar = desc_sw128(ar + off), dai = desc_sw128(ai + off);
-                const uint64_t dbr = desc_sw128(br + off), dbi = desc_sw128(bi + off);
-                const uint32_t acc = (kb | kk) ? 1u : 0u;
-                mma_tf32(Dr, dar, dbr, idp, acc);
-                mma_tf32(Dr, dai, dbi, idn, 1u);
-                mma_tf32(Di, dar, dbi, idp, acc);
-                mma_tf32(Di, dai, dbr, idp, 1u);
+            for (uint32_t kk = 0; kk < BKE / 16; ++kk) {
+                const uint32_t hi = 2 * kk, lo = hi + 4;  // 16 halves = 32 bytes; lo 64 bytes after hi
+                product(hi, hi, kb > 0 || kk > 0 ? 1u : 0u);
+                product(hi, lo, 1u);
+                product(lo, hi, 1u);
             }
-            mma_commit(empty0 + 8 * s);
+            if (leader) mma_commit(empty0 + 8 * s);
+            if (++s == STAGES) {
+                s = 0;
+                ph ^= 1u;
+            }
         }
-        mma_commit(done);
-        if (*abort_flag) {
-            // the products already issued finish (and the commit lands) before TMEM and shared
-            // memory are released
-            const uint64_t t0 = gtimer();
-            while (!mbar_try(done, 0u) && gtimer() - t0 < WAIT_NS) {
+        __syncwarp();
+        if (leader) {
+            mma_commit(done);
+            if (*abort_flag) {
+                // the products already issued finish (and the commit lands) before TMEM and shared
+                // memory are released
+                const uint64_t t0 = gtimer();
+                while (!mbar_try(done, 0u) && gtimer() - t0 < WAIT_NS) {
+                }
             }
         }
     }
@@ -302,10 +325,19 @@ __device__ __forceinline__ void cgemm_tc_body(const CUtensorMap& tmAr, const CUt
         const long row = (long)tm * BM + qw * 32 + lane;
         const uint32_t lane_off = (uint32_t)(qw * 32) << 16;
         const long col0 = (long)tn * BN;
+        const int er = sc.e0 + (sc.eA != nullptr && row < m ? __ldg(sc.eA + row) : 0);
 #pragma unroll 1
         for (int c0 = 0; c0 < BN; c0 += 16) {
             float vr[16], vi[16];
             tmem_ld16x2(Dr + lane_off + c0, Di + lane_off + c0, vr, vi);
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+                const long col = col0 + c0 + q;
+                const int e = er + (col < n ? __ldg(sc.eB + col) : 0);
+                const float f = tc_pow2(e >> 1), g = tc_pow2(e - (e >> 1));  // e may exceed one factor's range
+                vr[q] = vr[q] * f * g;
+                vi[q] = vi[q] * f * g;
+            }
             if (OUT == OUT_C32_PRE) {
                 float cr[16], ci[16];
                 tmem_ld16x2(Dr + 2 * BN + lane_off + c0, Di + 2 * BN + lane_off + c0, cr, ci);
@@ -396,14 +428,15 @@ __global__ void __launch_bounds__(192, 1)
     cgemm_tc_kernel(const __grid_constant__ CUtensorMap tmAr, const __grid_constant__ CUtensorMap tmAi,
                     const __grid_constant__ CUtensorMap tmBr, const __grid_constant__ CUtensorMap tmBi,
                     float* __restrict__ Cr, float* __restrict__ Ci, double2* __restrict__ C64, long ldc, long zstride,
-                    int m, int n, int kext, int S, float alpha, float beta, int* __restrict__ err, TcGate gate) {
+                    int m, int n, int K, int S, float alpha, float beta, int* __restrict__ err, TcScale sc,
+                    TcGate gate) {
     if (gate.first_tile && blockIdx.x == 0 && blockIdx.y == 0) return;
     if (gate.fail) {  // a factorisation that stopped before this product's block (lu_fast.cu)
         const int f = *reinterpret_cast<const volatile int*>(gate.fail);
         if (f != 0 && (f >> 1) <= gate.block) return;
     }
-    cgemm_tc_body<OUT>(tmAr, tmAi, tmBr, tmBi, Cr, Ci, C64, ldc, zstride, m, n, kext, S, (int)blockIdx.z, alpha, beta,
-                       err);
+    cgemm_tc_body<OUT>(tmAr, tmAi, tmBr, tmBi, Cr, Ci, C64, ldc, zstride, m, n, K, S, (int)blockIdx.z, alpha, beta,
+                       sc, err);
 }
 
 // One product per blockIdx.z: C_z = beta C_z + alpha A_z B_z^T for a batch of equal-shape products
@@ -413,12 +446,13 @@ struct alignas(64) TcBatchEntry {
     float* Cr;
     float* Ci;
     long ldc;
+    TcScale sc;
 };
 __global__ void __launch_bounds__(128, 1)
-    cgemm_tc_batch_kernel(const TcBatchEntry* __restrict__ E, int m, int n, int kext, float alpha, int* __restrict__ err) {
+    cgemm_tc_batch_kernel(const TcBatchEntry* __restrict__ E, int m, int n, int K, float alpha, int* __restrict__ err) {
     const TcBatchEntry& e = E[blockIdx.z];
-    cgemm_tc_body<OUT_C32>(e.map[0], e.map[1], e.map[2], e.map[3], e.Cr, e.Ci, nullptr, e.ldc, 0, m, n, kext, 1, 0,
-                           alpha, 0.f, err);
+    cgemm_tc_body<OUT_C32>(e.map[0], e.map[1], e.map[2], e.map[3], e.Cr, e.Ci, nullptr, e.ldc, 0, m, n, K, 1, 0,
+                           alpha, 0.f, e.sc, err);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
@@ -436,23 +470,23 @@ PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
 
 }  // namespace
 
-// 2-D tensor map over a row-major [rows][ldk] FP32 pack: dims {kext, rows}, box {32, box_rows},
-// 128-byte swizzle; reads outside {kext, rows} return zeros.
-bm_status tc_make_map(void* tmap, const float* base, long rows, long kext, long ldk, int box_rows) {
+// 2-D tensor map over a row-major [rows][ldk] pack of K entries a row (tc_ldk): dims {2 K rounded to 64,
+// rows} halves, box {64, box_rows}, 128-byte swizzle; reads outside return zeros.
+bm_status tc_make_map(void* tmap, const __half* base, long rows, long K, long ldk, int box_rows) {
     PFN_cuTensorMapEncodeTiled_v12000 enc = get_encode();
     if (enc == nullptr) {
         bm_set_error("cuTensorMapEncodeTiled is unavailable from the driver");
         return BM_ECUDA;
     }
-    if ((reinterpret_cast<uintptr_t>(base) & 15) != 0 || (ldk * 4) % 16 != 0) {
+    if ((reinterpret_cast<uintptr_t>(base) & 15) != 0 || (ldk * 2) % 16 != 0) {
         bm_set_error("tensor map: base or stride not 16-byte aligned");
         return BM_EINVAL;
     }
-    cuuint64_t dims[2] = {(cuuint64_t)kext, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)ldk * 4};
-    cuuint32_t box[2] = {(cuuint32_t)BKE, (cuuint32_t)box_rows};
+    cuuint64_t dims[2] = {(cuuint64_t)tc_ldk(K), (cuuint64_t)rows};
+    cuuint64_t strides[1] = {(cuuint64_t)ldk * 2};
+    cuuint32_t box[2] = {(cuuint32_t)(2 * BKE), (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
-    CUresult r = enc(reinterpret_cast<CUtensorMap*>(tmap), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base),
+    CUresult r = enc(reinterpret_cast<CUtensorMap*>(tmap), CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<__half*>(base),
                      dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
@@ -466,8 +500,8 @@ namespace {
 
 template <int OUT>
 cudaError_t launch_tc(cudaStream_t s, dim3 grid, const void* tAr, const void* tAi, const void* tBr, const void* tBi,
-                      float* Cr, float* Ci, double2* C64, long ldc, long zstride, int m, int n, int kext, int S,
-                      float alpha, float beta, int* d_err, TcGate gate = TcGate{}) {
+                      float* Cr, float* Ci, double2* C64, long ldc, long zstride, int m, int n, int K, int S,
+                      float alpha, float beta, int* d_err, TcScale sc, TcGate gate = TcGate{}) {
     static DeviceFlags attr_set;
     if (attr_set.pending()) {
         cudaError_t e =
@@ -478,7 +512,7 @@ cudaError_t launch_tc(cudaStream_t s, dim3 grid, const void* tAr, const void* tA
     cgemm_tc_kernel<OUT><<<grid, tc_threads<OUT>(), SMEM_BYTES, s>>>(
         *reinterpret_cast<const CUtensorMap*>(tAr), *reinterpret_cast<const CUtensorMap*>(tAi),
         *reinterpret_cast<const CUtensorMap*>(tBr), *reinterpret_cast<const CUtensorMap*>(tBi), Cr, Ci, C64, ldc,
-        zstride, m, n, kext, S, alpha, beta, d_err, gate);
+        zstride, m, n, K, S, alpha, beta, d_err, sc, gate);
     return cudaGetLastError();
 }
 
@@ -526,51 +560,40 @@ __global__ void splitk_reduce_z64_kernel(const float* __restrict__ Pr, const flo
     c = make_double2(cr, ci);
 }
 
-// B operand of a skinny product: V (K x nrhs FP32 planar, column-major) -> row c of a [nrhs][ldk]
-// K-major pack; 3xTF32 segments [hi | lo | hi] with hi = tf32(v), lo = v - hi.
-__global__ void pack_b_kernel(const float* __restrict__ Vr, const float* __restrict__ Vi, long ldv, int K, int nrhs,
-                              int split, float* __restrict__ Br, float* __restrict__ Bi, long ldk) {
-    const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long)K * nrhs) return;
-    const int c = (int)(idx / K), k = (int)(idx % K);
-    const float vr = __ldg(Vr + k + (long)c * ldv), vi = __ldg(Vi + k + (long)c * ldv);
-    const long o = (long)c * ldk + k;
-    if (!split) {
-        Br[o] = vr;
-        Bi[o] = vi;
-        return;
-    }
-    uint32_t hr, hi;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(hr) : "f"(vr));
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(hi) : "f"(vi));
-    const float fr = __uint_as_float(hr), fi = __uint_as_float(hi);
-    Br[o] = fr;
-    Bi[o] = fi;
-    Br[o + K] = vr - fr;
-    Bi[o + K] = vi - fi;
-    Br[o + 2L * K] = fr;
-    Bi[o + 2L * K] = fi;
+// B operand of a skinny product: V (K x nrhs FP32 planar, column-major) -> row c of a [nrhs][ldk] pack and
+// its exponent eB[c].  One CTA per column, which it reads twice (the second time from L2).
+struct PlanarCol {
+    const float *re, *im;
+    __device__ __forceinline__ float2 operator()(long k) const { return make_float2(__ldg(re + k), __ldg(im + k)); }
+};
+__global__ void __launch_bounds__(TC_PACK_THREADS) pack_b_kernel(const float* __restrict__ Vr,
+                                                                 const float* __restrict__ Vi, long ldv, int K,
+                                                                 __half* __restrict__ Br, __half* __restrict__ Bi,
+                                                                 long ldk, int* __restrict__ eB) {
+    const long c = blockIdx.x;
+    tc_pack_column(PlanarCol{Vr + c * ldv, Vi + c * ldv}, K, Br + c * ldk, Bi + c * ldk, eB + c);
 }
 
 }  // namespace
 
 // C = beta C + alpha A B^T, C FP32 planar column-major (m x n, ld ldc); one K range per CTA.
 cudaError_t gemm_tc(cudaStream_t s, const void* tAr, const void* tAi, const void* tBr, const void* tBi, float* Cr,
-                    float* Ci, long ldc, int m, int n, int kext, float alpha, float beta, int* d_err, TcGate gate) {
-    if (m <= 0 || n <= 0 || kext <= 0) return cudaSuccess;
+                    float* Ci, long ldc, int m, int n, int K, float alpha, float beta, TcScale sc, int* d_err,
+                    TcGate gate) {
+    if (m <= 0 || n <= 0 || K <= 0) return cudaSuccess;
     dim3 grid(ceil_div(m, BM), ceil_div(n, BN), 1);
     if (beta != 0.f)
-        return launch_tc<OUT_C32_PRE>(s, grid, tAr, tAi, tBr, tBi, Cr, Ci, nullptr, ldc, 0, m, n, kext, 1, alpha,
-                                      beta, d_err, gate);
-    return launch_tc<OUT_C32>(s, grid, tAr, tAi, tBr, tBi, Cr, Ci, nullptr, ldc, 0, m, n, kext, 1, alpha, beta,
-                              d_err, gate);
+        return launch_tc<OUT_C32_PRE>(s, grid, tAr, tAi, tBr, tBi, Cr, Ci, nullptr, ldc, 0, m, n, K, 1, alpha,
+                                      beta, d_err, sc, gate);
+    return launch_tc<OUT_C32>(s, grid, tAr, tAi, tBr, tBi, Cr, Ci, nullptr, ldc, 0, m, n, K, 1, alpha, beta,
+                              d_err, sc, gate);
 }
 
 // Number of K splits for a product with few output tiles: about three waves of CTAs over the
 // SMs (one CTA per SM fits), at most 32 splits and at least one 32-wide K step per split.
-int tc_split_k(int m, int n, int kext, int num_sms) {
+int tc_split_k(int m, int n, int K, int num_sms) {
     const long tiles = (long)ceil_div(m, BM) * ceil_div(n, BN);
-    const int nkb = ceil_div(kext, BKE);
+    const int nkb = ceil_div(K, BKE);
     long S = (3L * num_sms) / tiles;
     if (S > 32) S = 32;
     if (S > nkb) S = nkb;
@@ -583,24 +606,24 @@ int tc_split_k(int m, int n, int kext, int num_sms) {
 // workspace (Pr, Pi: S m n floats each) and one reduction kernel sums the slices in a fixed order
 // (deterministic).  Returns the number of kernels launched in *launched.
 cudaError_t gemm_tc_split(cudaStream_t s, const void* tAr, const void* tAi, const void* tBr, const void* tBi, int m,
-                          int n, int kext, float alpha, float beta, TcDest dst, int S, float* Pr, float* Pi,
+                          int n, int K, float alpha, float beta, TcScale sc, TcDest dst, int S, float* Pr, float* Pi,
                           int* d_err, int* launched) {
     *launched = 0;
-    if (m <= 0 || n <= 0 || kext <= 0) return cudaSuccess;
+    if (m <= 0 || n <= 0 || K <= 0) return cudaSuccess;
     const bool z64 = dst.z != nullptr;
     if (S <= 1) {
         dim3 grid(ceil_div(m, BM), ceil_div(n, BN), 1);
         *launched = 1;
         if (z64)
-            return launch_tc<OUT_Z64>(s, grid, tAr, tAi, tBr, tBi, nullptr, nullptr, dst.z, dst.ld, 0, m, n, kext, 1,
-                                      alpha, beta, d_err);
-        return launch_tc<OUT_C32>(s, grid, tAr, tAi, tBr, tBi, dst.re, dst.im, nullptr, dst.ld, 0, m, n, kext, 1,
-                                  alpha, beta, d_err);
+            return launch_tc<OUT_Z64>(s, grid, tAr, tAi, tBr, tBi, nullptr, nullptr, dst.z, dst.ld, 0, m, n, K, 1,
+                                      alpha, beta, d_err, sc);
+        return launch_tc<OUT_C32>(s, grid, tAr, tAi, tBr, tBi, dst.re, dst.im, nullptr, dst.ld, 0, m, n, K, 1,
+                                  alpha, beta, d_err, sc);
     }
     dim3 grid(ceil_div(m, BM), ceil_div(n, BN), S);
     const long zs = (long)m * n;
-    cudaError_t e = launch_tc<OUT_PART>(s, grid, tAr, tAi, tBr, tBi, Pr, Pi, nullptr, m, zs, m, n, kext, S, 1.f, 0.f,
-                                        d_err);
+    cudaError_t e = launch_tc<OUT_PART>(s, grid, tAr, tAi, tBr, tBi, Pr, Pi, nullptr, m, zs, m, n, K, S, 1.f, 0.f,
+                                        d_err, sc);
     if (e != cudaSuccess) return e;
     const int nb = (int)ceil_div(zs, 256L);
     if (z64)
@@ -611,11 +634,10 @@ cudaError_t gemm_tc_split(cudaStream_t s, const void* tAr, const void* tAi, cons
     return cudaGetLastError();
 }
 
-cudaError_t launch_pack_b(cudaStream_t s, const float* Vr, const float* Vi, long ldv, int K, int nrhs, int split,
-                          float* Br, float* Bi, long ldk) {
-    const long t = (long)K * nrhs;
-    if (t == 0) return cudaSuccess;
-    pack_b_kernel<<<ceil_div(t, 256L), 256, 0, s>>>(Vr, Vi, ldv, K, nrhs, split, Br, Bi, ldk);
+cudaError_t launch_pack_b(cudaStream_t s, const float* Vr, const float* Vi, long ldv, int K, int nrhs, __half* Br,
+                          __half* Bi, long ldk, int* eB) {
+    if (K <= 0 || nrhs <= 0) return cudaSuccess;
+    pack_b_kernel<<<nrhs, TC_PACK_THREADS, 0, s>>>(Vr, Vi, ldv, K, Br, Bi, ldk, eB);
     return cudaGetLastError();
 }
 
@@ -624,8 +646,9 @@ cudaError_t launch_pack_b(cudaStream_t s, const float* Vr, const float* Vi, long
 // B * tc_batch_entry_bytes() bytes, filled here.
 size_t tc_batch_entry_bytes() { return sizeof(TcBatchEntry); }
 cudaError_t gemm_tc_batch(cudaStream_t s, int B, const void* const* maps, float* const* Cr, float* const* Ci,
-                          const long* ldc, int m, int n, int kext, float alpha, void* d_entries, int* d_err) {
-    if (B < 1 || m <= 0 || n <= 0 || kext <= 0) return cudaSuccess;
+                          const long* ldc, const TcScale* sc, int m, int n, int K, float alpha, void* d_entries,
+                          int* d_err) {
+    if (B < 1 || m <= 0 || n <= 0 || K <= 0) return cudaSuccess;
     static DeviceFlags attr;
     if (attr.pending()) {
         cudaError_t e = cudaFuncSetAttribute(cgemm_tc_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -640,11 +663,12 @@ cudaError_t gemm_tc_batch(cudaStream_t s, int B, const void* const* maps, float*
         h[b].Cr = Cr[b];
         h[b].Ci = Ci[b];
         h[b].ldc = ldc[b];
+        h[b].sc = sc[b];
     }
     cudaError_t e = cudaMemcpyAsync(d_entries, h.data(), sizeof(TcBatchEntry) * B, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return e;
     dim3 grid(ceil_div(m, BM), ceil_div(n, BN), B);
-    cgemm_tc_batch_kernel<<<grid, 128, SMEM_BYTES, s>>>(reinterpret_cast<const TcBatchEntry*>(d_entries), m, n, kext,
+    cgemm_tc_batch_kernel<<<grid, 128, SMEM_BYTES, s>>>(reinterpret_cast<const TcBatchEntry*>(d_entries), m, n, K,
                                                         alpha, d_err);
     return cudaGetLastError();
 }

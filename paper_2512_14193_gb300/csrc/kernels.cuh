@@ -2,6 +2,8 @@
 #pragma once
 #include "common.cuh"
 
+#include <cuda_fp16.h>
+
 // assemble.cu
 cudaError_t launch_geometry(cudaStream_t s, int kind, const double p[4], int N, const double* d_user, double* d_geom);
 cudaError_t launch_assemble(cudaStream_t s, const bm_ctx* c);
@@ -14,8 +16,8 @@ cudaError_t launch_far_field(cudaStream_t s, const bm_ctx* c, const double2* X, 
                              int M, double2* U, long ldu);
 cudaError_t launch_hankel_probe(cudaStream_t s, const bm_ctx* c, const double2* z, int n, double2* h0, double2* h1);
 cudaError_t launch_f32_convert(cudaStream_t s, const double* x, int n, float* rn);
-cudaError_t launch_pack_schur(cudaStream_t s, const bm_ctx* c, int split);  // Schur operands (in bm_factor)
-cudaError_t launch_pack_solve(cudaStream_t s, const bm_ctx* c, int split);  // [M13; M23] rows (assembly)
+cudaError_t launch_pack_schur(cudaStream_t s, const bm_ctx* c);  // Schur operands (in bm_factor)
+cudaError_t launch_pack_solve(cudaStream_t s, const bm_ctx* c);  // [M13; M23] rows (assembly)
 cudaError_t launch_to_c32(cudaStream_t s, const double2* A, long lda, int m, int n, float* Fr, float* Fi, long ldf);
 
 // gemm_simt.cu
@@ -26,7 +28,17 @@ cudaError_t gemm_c32(cudaStream_t s, int m, int n, int k, float alpha, C32 A, bo
 cudaError_t gemm_update_z64_c32(cudaStream_t s, int m, int n, int k, float alpha, Z64 A, C32 B, Z64 C);
 
 // gemm_tc.cu (tensor maps are CUtensorMap, passed as opaque 128-byte blobs)
-bm_status tc_make_map(void* tmap, const float* base, long rows, long kext, long ldk, int box_rows);
+bm_status tc_make_map(void* tmap, const __half* base, long rows, long K, long ldk, int box_rows);
+constexpr long tc_ldk(long K) { return (K + 31) / 32 * 64; }  // halves per pack row of K entries (hi and lo)
+// Scales of a product's packs: entry (i, j) of A B^T is the packed product times 2^(eA[i] + eB[j] + e0)
+// (eA null: zeros)
+struct TcScale {
+    const int* eA = nullptr;
+    const int* eB = nullptr;
+    int e0 = 0;
+};
+constexpr int TC_E_DGE = -16;  // e0 of rows scaled by the digit planes' exponents (entries below 2^(e - 1))
+constexpr int TC_SHIFT_L = 14; // L21 is packed times 2^14 (its entries are below sqrt 2 in modulus)
 // TcGate: the launch skips its first 128 x 128 tile (another launch takes it), and does nothing when the
 // word *fail, if any, names a block of the factorisation up to `block` (lu_fast.cu)
 struct TcGate {
@@ -35,7 +47,7 @@ struct TcGate {
     int first_tile = 0;
 };
 cudaError_t gemm_tc(cudaStream_t s, const void* tAr, const void* tAi, const void* tBr, const void* tBi, float* Cr,
-                    float* Ci, long ldc, int m, int n, int kext, float alpha, float beta, int* d_err,
+                    float* Ci, long ldc, int m, int n, int K, float alpha, float beta, TcScale sc, int* d_err,
                     TcGate gate = TcGate{});
 constexpr int TC_BM = 128;
 constexpr int TC_BN = 128;
@@ -46,15 +58,16 @@ struct TcDest {
     double2* z;
     long ld;
 };
-int tc_split_k(int m, int n, int kext, int num_sms);
+int tc_split_k(int m, int n, int K, int num_sms);
 cudaError_t gemm_tc_split(cudaStream_t s, const void* tAr, const void* tAi, const void* tBr, const void* tBi, int m,
-                          int n, int kext, float alpha, float beta, TcDest dst, int S, float* Pr, float* Pi,
+                          int n, int K, float alpha, float beta, TcScale sc, TcDest dst, int S, float* Pr, float* Pi,
                           int* d_err, int* launched);
-cudaError_t launch_pack_b(cudaStream_t s, const float* Vr, const float* Vi, long ldv, int K, int nrhs, int split,
-                          float* Br, float* Bi, long ldk);
+cudaError_t launch_pack_b(cudaStream_t s, const float* Vr, const float* Vi, long ldv, int K, int nrhs, __half* Br,
+                          __half* Bi, long ldk, int* eB);
 size_t tc_batch_entry_bytes();
 cudaError_t gemm_tc_batch(cudaStream_t s, int B, const void* const* maps, float* const* Cr, float* const* Ci,
-                          const long* ldc, int m, int n, int kext, float alpha, void* d_entries, int* d_err);
+                          const long* ldc, const TcScale* sc, int m, int n, int K, float alpha, void* d_entries,
+                          int* d_err);
 
 // lu.cu
 bm_status lu_setup(bm_ctx* c, int cluster_cap, int panel_kernel);

@@ -17,7 +17,7 @@
 //        gemm (SIMT)       : rank-nbp update of the rest of the big panel
 //     swap_trsm_kernel     : interchanges for all other columns, U12 = L11^{-1} A12 (and its
 //                            K-major pack for the tensor cores)
-//     trailing update      : A22 -= L21 U12  (tensor-core TF32 / 3xTF32 for C32, SIMT for Z64)
+//     trailing update      : A22 -= L21 U12  (tensor cores, split FP16 (gemm_tc.cu) for C32, SIMT for Z64)
 // Pivot = first row index of max |Re| + |Im| (the LAPACK izamax rule).  An exactly zero pivot
 // records the 1-based column in *info and skips the scaling, as LAPACK getrf does.
 //
@@ -72,8 +72,8 @@ constexpr int ST_WARPS = 16, ST_COLS = 1;
 constexpr int ST_KC = 32;  // L11 columns per shared-memory chunk when L11 does not fit whole
 template <class V>
 __global__ void __launch_bounds__(ST_WARPS * 32) swap_trsm_kernel(V A, const SwapMap* __restrict__ map, int a0, int a1,
-                                                                   int b0, int b1, int t0, int tb, float* Upr,
-                                                                   float* Upi, long ldk, int split, int l_in_smem) {
+                                                                   int b0, int b1, int t0, int tb, __half* Upr,
+                                                                   __half* Upi, long ldk, int* Upe, int l_in_smem) {
     using CV = typename V::cv;
     using Rl = typename V::real;
     constexpr int QMAX = 8;  // rows per lane: tb <= 256
@@ -228,77 +228,47 @@ __global__ void __launch_bounds__(ST_WARPS * 32) swap_trsm_kernel(V A, const Swa
             if (i < tb) A.set((long)t0 + i, col, x[q]);
         }
         if (Upr != nullptr) {
-            // K-major pack of this column (row index = col - b0); segments [hi | lo | hi] when split
-            long rowp = col - b0;
-            float* pr = Upr + rowp * ldk;
-            float* pi = Upi + rowp * ldk;
+            // pack row col - b0 (tb is a multiple of 32: the last panel has no pack) and its exponent, which
+            // also takes L21's shift back
+            const long rowp = col - b0;
+            float mx = 0.f;
 #pragma unroll
-            for (int q = 0; q < QMAX; ++q) {
-                int i = lane + 32 * q;
-                if (i < tb) {
-                    float vr = (float)x[q].x, vi = (float)x[q].y;
-                    if (!split) {
-                        pr[i] = vr;
-                        pi[i] = vi;
-                    } else {
-                        float hr = tf32_rna(vr), hi = tf32_rna(vi);
-                        pr[i] = hr;
-                        pi[i] = hi;
-                        pr[tb + i] = vr - hr;
-                        pi[tb + i] = vi - hi;
-                        pr[2 * tb + i] = hr;
-                        pi[2 * tb + i] = hi;
-                    }
+            for (int q = 0; q < QMAX; ++q)
+                if (lane + 32 * q < tb) mx = fmaxf(mx, fmaxf(fabsf((float)x[q].x), fabsf((float)x[q].y)));
+            for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            const TcRowScale sc(mx);
+            if (lane == 0) Upe[rowp] = sc.ex - 15 - TC_SHIFT_L;
+            __half* pr = Upr + rowp * ldk + lane;
+            __half* pi = Upi + rowp * ldk + lane;
+#pragma unroll
+            for (int q = 0; q < QMAX; ++q)
+                if (lane + 32 * q < tb) {
+                    tc_split(sc((float)x[q].x), pr[64 * q], pr[64 * q + 32]);
+                    tc_split(sc((float)x[q].y), pi[64 * q], pi[64 * q + 32]);
                 }
-            }
-            long kext = split ? 3L * tb : (long)tb;
-            long kpad = (kext + 31) / 32 * 32;
-            for (long i = kext + lane; i < kpad; i += 32) {
-                pr[i] = 0.f;
-                pi[i] = 0.f;
-            }
         }
     }
 }
 
-// L21 pack: rows [r0, r0+m) x columns [c0, c0+kb) of A -> row-major [m][ldk] planar, segments
-// [hi | hi | lo] when split (K padded with zeros to a multiple of 32).
-__global__ void pack_L_kernel(C32 A, long r0, long c0, int m, int kb, int split, float* Pr, float* Pi, long ldk) {
+// L21 pack: rows [r0, r0+m) x columns [c0, c0+kb) of A (kb a multiple of 32) -> pack rows, times 2^TC_SHIFT_L.
+__global__ void pack_L_kernel(C32 A, long r0, long c0, int m, __half* Pr, __half* Pi, long ldk) {
     __shared__ float2 t[32][33];
-    int k0 = blockIdx.x * 32, i0 = blockIdx.y * 32;
-    int tx = threadIdx.x, ty = threadIdx.y;
+    const int k0 = blockIdx.x * 32, i0 = blockIdx.y * 32;
+    const int tx = threadIdx.x, ty = threadIdx.y;
     for (int q = ty; q < 32; q += 8) {
-        int i = i0 + tx, k = k0 + q;
-        t[q][tx] = (i < m && k < kb) ? A.get(r0 + i, c0 + k) : make_float2(0.f, 0.f);
+        const int i = i0 + tx;
+        t[q][tx] = i < m ? A.get(r0 + i, c0 + k0 + q) : make_float2(0.f, 0.f);
     }
     __syncthreads();
-    long kext = split ? 3L * kb : (long)kb;
-    long kpad = (kext + 31) / 32 * 32;
+    const TcRowScale sc(TC_SHIFT_L);
     for (int q = ty; q < 32; q += 8) {
-        int i = i0 + q, k = k0 + tx;
+        const int i = i0 + q;
         if (i >= m) continue;
-        float* pr = Pr + (long)i * ldk;
-        float* pi = Pi + (long)i * ldk;
-        if (k < kb) {
-            float2 v = t[tx][q];
-            if (!split) {
-                pr[k] = v.x;
-                pi[k] = v.y;
-            } else {
-                float hr = tf32_rna(v.x), hi = tf32_rna(v.y);
-                pr[k] = hr;
-                pi[k] = hi;
-                pr[kb + k] = hr;
-                pi[kb + k] = hi;
-                pr[2 * kb + k] = v.x - hr;
-                pi[2 * kb + k] = v.y - hi;
-            }
-        }
-        if (blockIdx.x == 0)
-            for (long kk = kext + tx; kk < kpad; kk += 32) {
-                pr[kk] = 0.f;
-                pi[kk] = 0.f;
-            }
+        const float2 v = t[tx][q];
+        __half* pr = Pr + (long)i * ldk + 2 * k0 + tx;
+        __half* pi = Pi + (long)i * ldk + 2 * k0 + tx;
+        tc_split(sc(v.x), pr[0], pr[32]);
+        tc_split(sc(v.y), pi[0], pi[32]);
     }
 }
 
@@ -855,7 +825,7 @@ __global__ void gather_rows_c32_kernel(const int* __restrict__ perm, int n, int 
 
 template <class V>
 cudaError_t launch_swap_trsm(cudaStream_t s, V A, const SwapMap* map, int a0, int a1, int b0, int b1, int t0, int tb,
-                             float* Upr, float* Upi, long ldk, int split) {
+                             __half* Upr, __half* Upi, long ldk, int* Upe) {
     using CV = typename V::cv;
     long ncols = (long)(a1 - a0) + (b1 - b0);
     if (ncols <= 0) return cudaSuccess;
@@ -870,7 +840,7 @@ cudaError_t launch_swap_trsm(cudaStream_t s, V A, const SwapMap* map, int a0, in
     }
     int grid = ceil_div(ncols, ST_WARPS * ST_COLS);
     return launch_pdl(kern, dim3(grid), dim3(ST_WARPS * 32), smem, s, A, map, a0, a1, b0, b1, t0, tb, Upr, Upi, ldk,
-                      split, l_in_smem);
+                      Upe, l_in_smem);
 }
 
 cudaError_t gemm_any(cudaStream_t s, int m, int n, int k, Z64 A, Z64 B, Z64 C) {
@@ -940,7 +910,7 @@ bm_status factor_fast(bm_ctx* c, C32 F) {
         iota_kernel<<<ceil_div(n, 256), 256, 0, s>>>(c->d_perm, c->d_ipiv, n);
         LU_CUDA(cudaGetLastError());
     }
-    float* const packs[4] = {c->d_Lp_r, c->d_Lp_i, c->d_Up_r, c->d_Up_i};
+    const TcPacks packs{c->d_Lp_r, c->d_Lp_i, c->d_Up_r, c->d_Up_i, c->d_Upe, c->ldk_lu};
     bool rest = false;  // a trailing update is under way on s2
     for (int J = 0; J < n; J += FD_B) {
         const int db = std::min(FD_B, n - J), mm = n - J - db;
@@ -952,7 +922,7 @@ bm_status factor_fast(bm_ctx* c, C32 F) {
         if (rest) LU_CUDA(cudaStreamWaitEvent(s, ev_join, 0));
         {
             BM_PROF(c, "lu_trsm_kernel");
-            LU_CUDA(launch_lu_trsm(s, F, J, db, mm, c->d_fd, n, packs, c->ldk_lu, fail));
+            LU_CUDA(launch_lu_trsm(s, F, J, db, mm, c->d_fd, n, packs, fail));
         }
         rest = false;
         if (mm == 0) break;
@@ -960,8 +930,8 @@ bm_status factor_fast(bm_ctx* c, C32 F) {
         const C32 C = F.sub(J + FD_B, J + FD_B);
         TcGate gate{fail, J + 1, 0};
         auto update = [&](cudaStream_t st, int m) {
-            return gemm_tc(st, c->tm_lu[0], c->tm_lu[1], c->tm_lu[2], c->tm_lu[3], C.re, C.im, C.ld, m, m, 3 * FD_B, -1.0f,
-                           1.0f, c->d_err, gate);
+            return gemm_tc(st, c->tm_lu[0], c->tm_lu[1], c->tm_lu[2], c->tm_lu[3], C.re, C.im, C.ld, m, m, FD_B, -1.0f,
+                           1.0f, TcScale{nullptr, c->d_Upe, 0}, c->d_err, gate);
         };
         if (!la || mm <= FD_B) {
             LU_CUDA(update(s, mm));
@@ -1030,7 +1000,7 @@ bm_status factor_fast_z(bm_ctx* c, Z64 F) {
 // The LU with the pivot search, from column J0 on (the columns before it are factored, their
 // interchanges and trailing updates applied).
 template <class V>
-bm_status factor_t(bm_ctx* c, V F, bool tc, int split, int J0 = 0) {
+bm_status factor_t(bm_ctx* c, V F, bool tc, int J0 = 0) {
     const int n = c->n;
     const int NB = c->nb;
     const int cl_max = c->panel_cluster;
@@ -1082,7 +1052,7 @@ bm_status factor_t(bm_ctx* c, V F, bool tc, int split, int J0 = 0) {
             if (jb > ib) {
                 if (!fused) {
                     BM_PROF(c, "swap_trsm_kernel (sub-panel)");
-                    LU_CUDA(launch_swap_trsm<V>(s, F, d_map2, J, j, j + ib, J + jb, j, ib, nullptr, nullptr, 0, 0));
+                    LU_CUDA(launch_swap_trsm<V>(s, F, d_map2, J, j, j + ib, J + jb, j, ib, nullptr, nullptr, 0, nullptr));
                 }
                 if (j + ib < J + jb) {
                     BM_PROF(c, "cgemm_simt_kernel (panel update)");
@@ -1102,7 +1072,7 @@ bm_status factor_t(bm_ctx* c, V F, bool tc, int split, int J0 = 0) {
             // on s: the next big panel's columns (all trailing columns without look-ahead), and the
             // columns left of this panel unless the rest stream takes them
             LU_CUDA(launch_swap_trsm<V>(s, F, d_map, 0, la ? 0 : J, J + jb, J + jb + nnext, J, jb,
-                                        pack ? c->d_Up_r : nullptr, pack ? c->d_Up_i : nullptr, c->ldk_lu, split));
+                                        pack ? c->d_Up_r : nullptr, pack ? c->d_Up_i : nullptr, c->ldk_lu, c->d_Upe));
         }
         if (mm > 0) {
             if (tc) {
@@ -1110,16 +1080,14 @@ bm_status factor_t(bm_ctx* c, V F, bool tc, int split, int J0 = 0) {
                     dim3 blk2(32, 8), grid(ceil_div(jb, 32), ceil_div(mm, 32));
                     {
                         BM_PROF(c, "pack_L_kernel");
-                        pack_L_kernel<<<grid, blk2, 0, s>>>(F, J + jb, J, mm, jb, split, c->d_Lp_r, c->d_Lp_i,
-                                                            c->ldk_lu);
+                        pack_L_kernel<<<grid, blk2, 0, s>>>(F, J + jb, J, mm, c->d_Lp_r, c->d_Lp_i, c->ldk_lu);
                         LU_CUDA(cudaGetLastError());
                     }
-                    const int kext = split ? 3 * jb : jb;
                     C32 Cv = F.sub(J + jb, J + jb);
                     {
                         BM_PROF(c, "cgemm_tc_kernel (trailing update)");
                         LU_CUDA(gemm_tc(s, c->tm_lu[0], c->tm_lu[1], c->tm_lu[2], c->tm_lu[3], Cv.re, Cv.im, Cv.ld, mm,
-                                        nnext, kext, -1.0f, 1.0f, c->d_err));
+                                        nnext, jb, -1.0f, 1.0f, TcScale{nullptr, c->d_Upe, 0}, c->d_err));
                     }
                     if (la) {
                         // the rest on s2: interchanges of the columns left of this panel and right of
@@ -1128,11 +1096,12 @@ bm_status factor_t(bm_ctx* c, V F, bool tc, int split, int J0 = 0) {
                         LU_CUDA(cudaStreamWaitEvent(s2, ev_fork, 0));
                         LU_CUDA(launch_swap_trsm<V>(s2, F, d_map, 0, J, J + jb + nnext, n, J, jb,
                                                     c->d_Up_r + (long)NB * c->ldk_lu, c->d_Up_i + (long)NB * c->ldk_lu,
-                                                    c->ldk_lu, split));
+                                                    c->ldk_lu, c->d_Upe + NB));
                         if (mm > nnext) {
                             C32 Cr = F.sub(J + jb, J + jb + nnext);
                             LU_CUDA(gemm_tc(s2, c->tm_lu[0], c->tm_lu[1], c->tm_lu[4], c->tm_lu[5], Cr.re, Cr.im, Cr.ld,
-                                            mm, mm - nnext, kext, -1.0f, 1.0f, c->d_err));
+                                            mm, mm - nnext, jb, -1.0f, 1.0f, TcScale{nullptr, c->d_Upe + NB, 0},
+                                            c->d_err));
                         }
                         LU_CUDA(cudaEventRecord(ev_join, s2));
                     }
@@ -1321,11 +1290,11 @@ bm_status lu_setup(bm_ctx* c, int cluster_cap, int panel_kernel) {
 bm_status lu_factor_enqueue(bm_ctx* c) {
     if (c->prec == BM_FP64) {
         Z64 F{c->d_F64, c->ldF};
-        return c->lu_fast ? factor_fast_z(c, F) : factor_t<Z64>(c, F, false, 0);
+        return c->lu_fast ? factor_fast_z(c, F) : factor_t<Z64>(c, F, false);
     }
     C32 F{c->d_F32r, c->d_F32i, c->ldF};
     if (c->lu_fast) return factor_fast(c, F);
-    return factor_t<C32>(c, F, true, c->prec == BM_CF32_3XTF32_IR ? 1 : 0);
+    return factor_t<C32>(c, F, true);
 }
 
 bm_status lu_resume_enqueue(bm_ctx* c, int stop) {
@@ -1335,13 +1304,13 @@ bm_status lu_resume_enqueue(bm_ctx* c, int stop) {
             BM_TRY(schur_z64(c, c->stream));
         else
             LU_CUDA(launch_copy_z64(c->stream, c->d_A, c->ldA, c->n, c->n, c->d_F64, c->ldF));
-        return factor_t<Z64>(c, Z64{c->d_F64, c->ldF}, false, 0);
+        return factor_t<Z64>(c, Z64{c->d_F64, c->ldF}, false);
     }
     C32 F{c->d_F32r, c->d_F32i, c->ldF};
     const int J = (stop >> 1) - 1, db = std::min(FD_B, c->n - J);
     LU_CUDA(cudaMemsetAsync(c->d_info + 4, 0, sizeof(int), c->stream));
     if (stop & 1) LU_CUDA(launch_lu_restore(c->stream, F, J, db, c->n - J - db, c->d_fd, c->n));
-    return factor_t<C32>(c, F, true, c->prec == BM_CF32_3XTF32_IR ? 1 : 0, J);
+    return factor_t<C32>(c, F, true, J);
 }
 
 size_t lu_fast_bytes(int n) { return fd_work_floats(n) * sizeof(float); }

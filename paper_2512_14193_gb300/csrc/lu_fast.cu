@@ -14,7 +14,7 @@
 //   lu_trsm_kernel  all SMs: L21 = A21 U11^{-1} by rows (stage 1 of the check) and U12 = L11^{-1} A12
 //                   by columns, written to the matrix and packed for the tensor cores; the original
 //                   entries are kept in a backup until the next block
-//   gemm_tc         A22 -= L21 U12 in 3xTF32: the next diagonal block's tile first, so that the next
+//   gemm_tc         A22 -= L21 U12, split FP16 operands (gemm_tc.cu): the next diagonal block's tile first, so that the next
 //                   lu_diag_kernel runs beside the rest (look-ahead on two streams)
 #include "lu_internal.cuh"
 
@@ -355,9 +355,7 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
 // overwrites.
 constexpr int R = 32, RT = 4 * R, XP = R + 1;
 __global__ void __launch_bounds__(RT, 2) lu_trsm_kernel(C32 F, int J, int db, int mm, const float* __restrict__ T,
-                                                        float* __restrict__ bk, long ldb, float* __restrict__ Lpr,
-                                                        float* __restrict__ Lpi, float* __restrict__ Upr,
-                                                        float* __restrict__ Upi, long ldk, int* fail) {
+                                                        float* __restrict__ bk, long ldb, TcPacks packs, int* fail) {
     extern __shared__ __align__(16) float sm[];
     float* Tr = sm;
     float* Ti = Tr + FD_PACK;
@@ -522,23 +520,28 @@ __global__ void __launch_bounds__(RT, 2) lu_trsm_kernel(C32 F, int J, int db, in
                 F.im[o] = Xi[tid * XP + c];
             }
     }
-    // K-major packs, segments [hi | hi | lo] of L21 rows and [hi | lo | hi] of U12 columns
-    float* Pr = (rows ? Lpr : Upr) + tid;
-    float* Pi = (rows ? Lpi : Upi) + tid;
-    const int o1 = rows ? B : 2 * B, o2 = rows ? 2 * B : B;  // second hi, lo
+    // packs of L21 rows (times 2^TC_SHIFT_L) and U12 columns (by their exponents, which take that shift back)
+    __shared__ float mx_s[RT / 32][R];
+    if (!rows) {
+        float mx = 0.f;  // of a quarter of column `lane`
+#pragma unroll 8
+        for (int k = warp; k < B; k += RT / 32)
+            mx = fmaxf(mx, fmaxf(fabsf(Xr[k * XP + lane]), fabsf(Xi[k * XP + lane])));
+        mx_s[warp][lane] = mx;
+        __syncthreads();
+    }
+    __half* Pr = (rows ? packs.Lr : packs.Ur) + tc_pos(tid);
+    __half* Pi = (rows ? packs.Li : packs.Ui) + tc_pos(tid);
 #pragma unroll 4
     for (int r = 0; r < R; ++r)
         if (x0 + r < mm) {
-            const float vr = Xr[tid * XP + r], vi = Xi[tid * XP + r];
-            const float hr = tf32_rna(vr), hi = tf32_rna(vi);
-            float* pr = Pr + (long)(x0 + r) * ldk;
-            float* pi = Pi + (long)(x0 + r) * ldk;
-            pr[0] = hr;
-            pr[o1] = hr;
-            pr[o2] = vr - hr;
-            pi[0] = hi;
-            pi[o1] = hi;
-            pi[o2] = vi - hi;
+            const TcRowScale sc = rows ? TcRowScale(TC_SHIFT_L)
+                                       : TcRowScale(fmaxf(fmaxf(mx_s[0][r], mx_s[1][r]), fmaxf(mx_s[2][r], mx_s[3][r])));
+            if (!rows && tid == 0) packs.Ue[x0 + r] = sc.ex - 15 - TC_SHIFT_L;
+            __half* pr = Pr + (long)(x0 + r) * packs.ldk;
+            __half* pi = Pi + (long)(x0 + r) * packs.ldk;
+            tc_split(sc(Xr[tid * XP + r]), pr[0], pr[32]);
+            tc_split(sc(Xi[tid * XP + r]), pi[0], pi[32]);
         }
 }
 
@@ -581,9 +584,9 @@ cudaError_t launch_lu_diag(cudaStream_t s, C32 F, int J, int db, float* work, in
     return cudaGetLastError();
 }
 
-cudaError_t launch_lu_trsm(cudaStream_t s, C32 F, int J, int db, int mm, float* work, long n, float* const* packs,
-                           long ldk, int* fail) {
-    if (mm > 0 && (db != B || ldk < 3 * B)) return cudaErrorInvalidValue;
+cudaError_t launch_lu_trsm(cudaStream_t s, C32 F, int J, int db, int mm, float* work, long n, TcPacks packs,
+                           int* fail) {
+    if (mm > 0 && (db != B || packs.ldk < tc_ldk(B))) return cudaErrorInvalidValue;
     constexpr int smem = (2 * FD_PACK + 2 * B * XP) * (int)sizeof(float);
     static DeviceFlags attr;
     if (attr.pending()) {
@@ -592,7 +595,7 @@ cudaError_t launch_lu_trsm(cudaStream_t s, C32 F, int J, int db, int mm, float* 
         attr.done();
     }
     lu_trsm_kernel<<<2 * ceil_div(mm, R) + ceil_div(db, W), RT, smem, s>>>(
-        F, J, db, mm, work, work + FD_T, n, packs[0], packs[1], packs[2], packs[3], ldk, fail);
+        F, J, db, mm, work, work + FD_T, n, packs, fail);
     return cudaGetLastError();
 }
 

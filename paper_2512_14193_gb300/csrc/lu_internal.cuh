@@ -3,6 +3,7 @@
 #pragma once
 #include "common.cuh"
 #include "kernels.cuh"
+#include "tc_pack.cuh"
 
 #include <cooperative_groups.h>
 #include <algorithm>
@@ -196,11 +197,6 @@ __device__ __forceinline__ float2 cinv_fast(float2 a) {
     return make_float2(x * rs, -y * rs);
 }
 
-__device__ __forceinline__ float tf32_rna(float x) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return __uint_as_float(r);
-}
 
 // ------------------------------------------------------------------------------------------------
 // panel factorisation
@@ -552,8 +548,12 @@ struct FdBackup {
 };
 inline size_t fd_work_floats(long n) { return (size_t)FD_T + 2 * FD_B * FD_B + 4 * (size_t)n * FD_B; }
 cudaError_t launch_lu_diag(cudaStream_t s, C32 F, int J, int db, float* work, int* fail);
-cudaError_t launch_lu_trsm(cudaStream_t s, C32 F, int J, int db, int mm, float* work, long n, float* const* packs,
-                           long ldk, int* fail);
+struct TcPacks {  // the trailing update's packs and U12's exponents
+    __half *Lr, *Li, *Ur, *Ui;
+    int* Ue;
+    long ldk;
+};
+cudaError_t launch_lu_trsm(cudaStream_t s, C32 F, int J, int db, int mm, float* work, long n, TcPacks packs, int* fail);
 cudaError_t launch_lu_restore(cudaStream_t s, C32 F, int J, int db, int mm, float* work, long n);
 int query_cluster_max_z64();
 

@@ -226,17 +226,18 @@ bm_status factor_batch(Batch& bt, int B) {
         std::vector<const void*> maps(B);
         std::vector<float*> Cr(B), Ci(B);
         std::vector<long> ld(B);
+        std::vector<TcScale> sc(B);
         for (int b = 0; b < B; ++b) {
             bm_ctx* c = bt.h[b];
-            SSM_CUDA(launch_pack_schur(bt.s0, c, c->prec == BM_CF32_3XTF32_IR));
+            SSM_CUDA(launch_pack_schur(bt.s0, c));
             maps[b] = c->tm_schur;
             Cr[b] = c->d_F32r;
             Ci[b] = c->d_F32i;
             ld[b] = c->ldF;
+            sc[b] = TcScale{c->d_dge[1], c->d_Bpe, TC_E_DGE};
         }
-        const long kext = (c0->prec == BM_CF32_3XTF32_IR) ? 3L * c0->kseg_schur : c0->kseg_schur;
-        SSM_CUDA(gemm_tc_batch(bt.s0, B, maps.data(), Cr.data(), Ci.data(), ld.data(), N, N, (int)kext, -1.0f, bt.d_tc,
-                               c0->d_err));
+        SSM_CUDA(gemm_tc_batch(bt.s0, B, maps.data(), Cr.data(), Ci.data(), ld.data(), sc.data(), N, N, 2 * N, -1.0f,
+                               bt.d_tc, c0->d_err));
         c0->launches += 3 * B + 1;
         SSM_CUDA(cudaEventRecord(bt.ev, bt.s0));
         for (int b = 0; b < B; ++b) SSM_CUDA(cudaStreamWaitEvent(bt.h[b]->stream, bt.ev, 0));
