@@ -420,7 +420,7 @@ extern "C" bm_status bm_enqueue_probe(bm_ctx* c, int which, int reps) {
                                      Z64{c->d_Mtop, c->ldtop}, 0.0, Z64{c->d_F64, c->ldF}));
             } else {
                 BM_CUDA_TRY(gemm_tc(s, c->tm_schur[0], c->tm_schur[1], c->tm_schur[2], c->tm_schur[3], c->d_F32r,
-                                    c->d_F32i, c->ldF, c->N, c->N, 2 * c->N, -1.0f, 0.0f,
+                                    c->d_F32i, c->ldF, c->N, c->N, 2 * c->N, -1.0f,
                                     TcScale{c->d_dge[1], c->d_Bpe, TC_E_DGE}, c->d_err));
             }
             c->launches += 1;
@@ -874,7 +874,7 @@ bm_status factor_sequence(bm_ctx* c) {
             }
             BM_PROF(c, "cgemm_tc_kernel (Schur complement)");
             BM_CUDA_TRY(gemm_tc(s, c->tm_schur[0], c->tm_schur[1], c->tm_schur[2], c->tm_schur[3], c->d_F32r,
-                                c->d_F32i, c->ldF, c->N, c->N, 2 * c->N, -1.0f, 0.0f,
+                                c->d_F32i, c->ldF, c->N, c->N, 2 * c->N, -1.0f,
                                 TcScale{c->d_dge[1], c->d_Bpe, TC_E_DGE}, c->d_err));
         } else {
             BM_PROF(c, "to_c32_kernel");

@@ -21,9 +21,8 @@
 // mbarriers.  Warp 0 lane 0 issues TMA loads, warp 1 the tcgen05.mma (the whole warp walks the loop so
 // that the operands live in uniform registers, lane 0 issues); all four warps
 // then read the accumulators (tcgen05.ld 32x32b, warp w owns TMEM lanes 32(w mod 4) .. +31 = rows)
-// and update C with coalesced column-major stores.  For C = C + alpha A B^T (the LU trailing
-// updates) a six-warp form loads the C tile into the upper half of TMEM during the main loop, so
-// the epilogue only stores.  Every mbarrier wait is bounded (2 s by the global timer); a timeout
+// and update C with coalesced column-major stores; the LU trailing updates have a persistent form
+// (cgemm_tc_upd_kernel).  Every mbarrier wait is bounded (2 s by the global timer); a timeout
 // sets *err, skips the epilogue, waits for issued copies and products and frees TMEM.  err[1] is
 // a test hook: when it is set the MMA warp first waits on a barrier that nothing completes, gives
 // up after 1 ms and takes that timeout path without issuing any product.
@@ -34,6 +33,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cstring>
 #include <vector>
 
@@ -67,6 +67,9 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
 }
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
     uint32_t ok;
@@ -152,30 +155,29 @@ __host__ __device__ constexpr uint32_t idesc_f16(uint32_t neg_a, uint32_t n) {
     return (1u << 4) | (neg_a << 13) | ((n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 }
 
-// Output modes: OUT_C32 C (FP32 planar) = beta C + alpha D; OUT_Z64 C64 (FP64) = beta C64 + alpha D;
-// OUT_PART the raw D of this K split to a workspace slice (split-K partial sums); OUT_C32_PRE as
-// OUT_C32 for beta != 0, with six warps: warps 2-5 copy the C tile into TMEM columns 2BN..4BN while
-// the MMAs run, so the epilogue reads D and C from TMEM and only stores (the C loads no longer
-// follow the main loop; one CTA per SM leaves nothing else to overlap them with).
-enum { OUT_C32 = 0, OUT_Z64 = 1, OUT_PART = 2, OUT_C32_PRE = 3 };
-
-template <int OUT>
-__host__ __device__ constexpr int tc_threads() { return OUT == OUT_C32_PRE ? 192 : 128; }
-template <int OUT>
-__host__ __device__ constexpr uint32_t tc_tmem_cols() { return OUT == OUT_C32_PRE ? 2 * TMEM_COLS : TMEM_COLS; }
-
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float* v) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};\n" ::"r"(
-            taddr),
-        "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(__float_as_uint(v[3])),
-        "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])), "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])),
-        "r"(__float_as_uint(v[8])), "r"(__float_as_uint(v[9])), "r"(__float_as_uint(v[10])),
-        "r"(__float_as_uint(v[11])), "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])),
-        "r"(__float_as_uint(v[14])), "r"(__float_as_uint(v[15]))
-        : "memory");
+// The products of one stage (its descriptor's low word ar: A re, A im, B re, B im tiles) into [Dr | Di], issued
+// by the lanes with `leader` set; acc = 0 overwrites.
+__device__ __forceinline__ void tc_stage_products(bool leader, uint32_t Dr, uint32_t Di, uint32_t ar, uint32_t acc) {
+    constexpr uint32_t IDW = idesc_f16(0, 2 * BN), IDP = idesc_f16(0, BN), IDN = idesc_f16(1, BN);
+    const uint32_t ai = ar + (TILE_A >> 4), br = ar + (2 * TILE_A >> 4), bi = br + (TILE_B >> 4);
+    // [Dr | Di] (+)= A B^T at offsets oa and ob (16-byte units) of the 128-byte rows
+    auto product = [&](uint32_t oa, uint32_t ob, uint32_t ac) {
+        mma_f16(leader, Dr, ar + oa, br + ob, IDW, ac);
+        mma_f16(leader, Dr, ai + oa, bi + ob, IDN, 1u);
+        mma_f16(leader, Di, ai + oa, br + ob, IDP, 1u);
+    };
+#pragma unroll
+    for (uint32_t kk = 0; kk < BKE / 16; ++kk) {
+        const uint32_t hi = 2 * kk, lo = hi + 4;  // 16 halves = 32 bytes; lo 64 bytes after hi
+        product(hi, hi, kk > 0 ? 1u : acc);
+        product(hi, lo, 1u);
+        product(lo, hi, 1u);
+    }
 }
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// Output modes: OUT_C32 C (FP32 planar) = beta C + alpha D; OUT_Z64 C64 (FP64) = beta C64 + alpha D;
+// OUT_PART the D of this K split to a workspace slice (split-K partial sums).
+enum { OUT_C32 = 0, OUT_Z64 = 1, OUT_PART = 2 };
 
 // The body of one CTA: tile (tm, tn) of C, K split z of S.  The four tensor maps are param-space
 // copies (single product) or global-memory entries of a batch.
@@ -211,7 +213,7 @@ __device__ __forceinline__ void cgemm_tc_body(const CUtensorMap& tmAr, const CUt
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) tmem_alloc(smem_u32(tmem_slot), tc_tmem_cols<OUT>());
+    if (warp == 0) tmem_alloc(smem_u32(tmem_slot), TMEM_COLS);
     fence_before();
     __syncthreads();
     fence_after();
@@ -246,7 +248,6 @@ __device__ __forceinline__ void cgemm_tc_body(const CUtensorMap& tmAr, const CUt
     } else if (warp == 1) {
         // ---------------- MMA issuer (the whole warp walks the loop, lane 0 issues) ----------------
         const bool leader = lane == 0;
-        constexpr uint32_t IDW = idesc_f16(0, 2 * BN), IDP = idesc_f16(0, BN), IDN = idesc_f16(1, BN);
         if (err[1] != 0) {
             // test hook: a wait that nothing ends, bounded like every other wait
             const uint64_t t0 = gtimer();
@@ -261,20 +262,7 @@ __device__ __forceinline__ void cgemm_tc_body(const CUtensorMap& tmAr, const CUt
             if (!mbar_wait(full0 + 8 * s, ph, abort_flag)) break;
             fence_after();
             const uint32_t ar = lo0 + (uint32_t)s * (STAGE_BYTES >> 4);
-            const uint32_t ai = ar + (TILE_A >> 4), br = ar + (2 * TILE_A >> 4), bi = br + (TILE_B >> 4);
-            // [Dr | Di] (+)= A B^T at offsets oa and ob (16-byte units) of the 128-byte rows
-            auto product = [&](uint32_t oa, uint32_t ob, uint32_t acc) {
-                mma_f16(leader, Dr, ar + oa, br + ob, IDW, acc);
-                mma_f16(leader, Dr, ai + oa, bi + ob, IDN, 1u);
-                mma_f16(leader, Di, ai + oa, br + ob, IDP, 1u);
-            };
-#pragma unroll
-            for (uint32_t kk = 0; kk < BKE / 16; ++kk) {
-                const uint32_t hi = 2 * kk, lo = hi + 4;  // 16 halves = 32 bytes; lo 64 bytes after hi
-                product(hi, hi, kb > 0 || kk > 0 ? 1u : 0u);
-                product(hi, lo, 1u);
-                product(lo, hi, 1u);
-            }
+            tc_stage_products(leader, Dr, Di, ar, kb > 0 ? 1u : 0u);
             if (leader) mma_commit(empty0 + 8 * s);
             if (++s == STAGES) {
                 s = 0;
@@ -294,36 +282,14 @@ __device__ __forceinline__ void cgemm_tc_body(const CUtensorMap& tmAr, const CUt
         }
     }
     __syncwarp();
-    if (OUT == OUT_C32_PRE && warp >= 2) {
-        // ---------------- C tile -> TMEM while the MMAs run (warps 2-5) ----------------
-        const int qw = warp & 3;  // TMEM lane quarter this warp may access
-        const long row = (long)tm * BM + qw * 32 + lane;
-        const uint32_t lane_off = (uint32_t)(qw * 32) << 16;
-        const long col0 = (long)tn * BN;
-#pragma unroll 1
-        for (int c0 = 0; c0 < BN; c0 += 16) {
-            float cr[16], ci[16];
-#pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                const long col = col0 + c0 + q;
-                const bool in = row < m && col < n;
-                cr[q] = in ? __ldg(Cr + row + col * ldc) : 0.f;
-                ci[q] = in ? __ldg(Ci + row + col * ldc) : 0.f;
-            }
-            tmem_st16(Dr + 2 * BN + lane_off + c0, cr);
-            tmem_st16(Di + 2 * BN + lane_off + c0, ci);
-        }
-        tmem_wait_st();
-    }
-    // ---------------- epilogue: all four warps (warps 2-5 in OUT_C32_PRE) ----------------
+    // ---------------- epilogue: all four warps ----------------
     mbar_wait(done, 0, abort_flag);
     fence_before();
     __syncthreads();  // the abort decision below must be uniform: tcgen05.ld is warp-synchronous
     fence_after();
-    if (!*abort_flag && (OUT != OUT_C32_PRE || warp >= 2)) {
-        const int qw = (OUT == OUT_C32_PRE) ? (warp & 3) : warp;
-        const long row = (long)tm * BM + qw * 32 + lane;
-        const uint32_t lane_off = (uint32_t)(qw * 32) << 16;
+    if (!*abort_flag) {
+        const long row = (long)tm * BM + warp * 32 + lane;
+        const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
         const long col0 = (long)tn * BN;
         const int er = sc.e0 + (sc.eA != nullptr && row < m ? __ldg(sc.eA + row) : 0);
 #pragma unroll 1
@@ -338,21 +304,7 @@ __device__ __forceinline__ void cgemm_tc_body(const CUtensorMap& tmAr, const CUt
                 vr[q] = vr[q] * f * g;
                 vi[q] = vi[q] * f * g;
             }
-            if (OUT == OUT_C32_PRE) {
-                float cr[16], ci[16];
-                tmem_ld16x2(Dr + 2 * BN + lane_off + c0, Di + 2 * BN + lane_off + c0, cr, ci);
-                if (row < m) {
-#pragma unroll
-                    for (int q = 0; q < 16; ++q) {
-                        const long col = col0 + c0 + q;
-                        if (col < n) {
-                            const long o = row + col * ldc;
-                            Cr[o] = fmaf(beta, cr[q], alpha * vr[q]);
-                            Ci[o] = fmaf(beta, ci[q], alpha * vi[q]);
-                        }
-                    }
-                }
-            } else if (OUT == OUT_PART && row < m) {
+            if (OUT == OUT_PART && row < m) {
                 // slice z of the workspace: m x n column-major, leading dimension ldc (= m)
                 float* Pr = Cr + (long)zsplit * zstride;
                 float* Pi = Ci + (long)zsplit * zstride;
@@ -418,25 +370,219 @@ __device__ __forceinline__ void cgemm_tc_body(const CUtensorMap& tmAr, const CUt
     __syncthreads();
     if (warp == 0) {
         fence_after();
-        tmem_dealloc(tmem, tc_tmem_cols<OUT>());
+        tmem_dealloc(tmem, TMEM_COLS);
     }
     if (threadIdx.x == 0 && *abort_flag) atomicExch(err, 1);
 }
 
 template <int OUT>
-__global__ void __launch_bounds__(192, 1)
+__global__ void __launch_bounds__(128, 1)
     cgemm_tc_kernel(const __grid_constant__ CUtensorMap tmAr, const __grid_constant__ CUtensorMap tmAi,
                     const __grid_constant__ CUtensorMap tmBr, const __grid_constant__ CUtensorMap tmBi,
                     float* __restrict__ Cr, float* __restrict__ Ci, double2* __restrict__ C64, long ldc, long zstride,
-                    int m, int n, int K, int S, float alpha, float beta, int* __restrict__ err, TcScale sc,
-                    TcGate gate) {
-    if (gate.first_tile && blockIdx.x == 0 && blockIdx.y == 0) return;
+                    int m, int n, int K, int S, float alpha, float beta, int* __restrict__ err, TcScale sc) {
+    cgemm_tc_body<OUT>(tmAr, tmAi, tmBr, tmBi, Cr, Ci, C64, ldc, zstride, m, n, K, S, (int)blockIdx.z, alpha, beta,
+                       sc, err);
+}
+
+// C -= A B^T for the LU trailing updates: few K (128 of them), so loading and storing C sets the time.  One
+// persistent CTA per SM walks the 128 x 128 tiles (numbers first, first + grid, ...; row tiles fastest).  Warp 0
+// loads the operands ahead across tiles, warp 1 issues into the two accumulators in turn, and sixteen warps
+// take a tile's C into registers (64 loads in flight per thread, a quarter of the columns each) while its
+// products run, then subtract and store while the next tile's do.  Against one CTA per tile with the C tile
+// staged through tensor memory by four warps, 8064 x 8064 (63 x 63 tiles): 477 -> 270 us (3.9 TB/s of C), one tile
+// alone 18.4 -> 12.7 us; the next tile prefetched into L2 makes 10 % of it.
+constexpr int UPD_WARPS = 16, UPD_THREADS = 64 + 32 * UPD_WARPS;
+constexpr int UPD_COLS = BN / (UPD_WARPS / 4);  // columns per warp
+static_assert(UPD_COLS == 32, "a lane per column");
+__device__ __forceinline__ void tmem_ld8x2(uint32_t ta, uint32_t tb, float* va, float* vb) {
+    uint32_t a[8], b[8];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%16];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%17];\n"
+        "tcgen05.wait::ld.sync.aligned;\n"
+        : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7]), "=r"(b[0]),
+          "=r"(b[1]), "=r"(b[2]), "=r"(b[3]), "=r"(b[4]), "=r"(b[5]), "=r"(b[6]), "=r"(b[7])
+        : "r"(ta), "r"(tb)
+        : "memory");
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        va[i] = __uint_as_float(a[i]);
+        vb[i] = __uint_as_float(b[i]);
+    }
+}
+
+__global__ void __launch_bounds__(UPD_THREADS, 1)
+    cgemm_tc_upd_kernel(const __grid_constant__ CUtensorMap tmAr, const __grid_constant__ CUtensorMap tmAi,
+                        const __grid_constant__ CUtensorMap tmBr, const __grid_constant__ CUtensorMap tmBi,
+                        float* __restrict__ Cr, float* __restrict__ Ci, long ldc, int m, int n, int K,
+                        int* __restrict__ err, TcScale sc, TcGate gate) {
     if (gate.fail) {  // a factorisation that stopped before this product's block (lu_fast.cu)
         const int f = *reinterpret_cast<const volatile int*>(gate.fail);
         if (f != 0 && (f >> 1) <= gate.block) return;
     }
-    cgemm_tc_body<OUT>(tmAr, tmAi, tmBr, tmBi, Cr, Ci, C64, ldc, zstride, m, n, K, S, (int)blockIdx.z, alpha, beta,
-                       sc, err);
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    // full[S], empty[S], accfull[2], accempty[2], drain, never (the test hook's)
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 6);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    const int ntm = (m + BM - 1) / BM, ntiles = ntm * ((n + BN - 1) / BN);
+    const int nkb = (K + BKE - 1) / BKE;
+    const int first = gate.first_tile + (int)blockIdx.x, step = (int)gridDim.x;
+    const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * STAGES, accfull = empty0 + 8 * STAGES;
+    const uint32_t accempty = accfull + 16, drain = accempty + 16, never = drain + 8;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(full0 + 8 * s, 1);
+            mbar_init(empty0 + 8 * s, 1);
+        }
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(accfull + 8 * s, 1);
+            mbar_init(accempty + 8 * s, UPD_WARPS);
+        }
+        mbar_init(drain, 1);
+        mbar_init(never, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) tmem_alloc(smem_u32(tmem_slot), 2 * TMEM_COLS);
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp == 0 && lane == 0) {
+        // ---------------- TMA producer ----------------
+        int it = 0;  // stages issued
+        for (int t = first; t < ntiles && !*abort_flag; t += step) {
+            const int tm = t % ntm, tn = t / ntm;
+            for (int kb = 0; kb < nkb; ++kb, ++it) {
+                const int s = it % STAGES;
+                if (it >= STAGES && !mbar_wait(empty0 + 8 * s, (uint32_t)(it / STAGES - 1) & 1u, abort_flag)) break;
+                uint8_t* st = smem + s * STAGE_BYTES;
+                const uint32_t fb = full0 + 8 * s;
+                mbar_expect_tx(fb, STAGE_BYTES);
+                const int kx = kb * 2 * BKE;
+                tma_load_2d(smem_u32(st), &tmAr, fb, kx, tm * BM);
+                tma_load_2d(smem_u32(st + TILE_A), &tmAi, fb, kx, tm * BM);
+                tma_load_2d(smem_u32(st + 2 * TILE_A), &tmBr, fb, kx, tn * BN);
+                tma_load_2d(smem_u32(st + 2 * TILE_A + TILE_B), &tmBi, fb, kx, tn * BN);
+            }
+        }
+        if (*abort_flag) {
+            // copies already in flight land before shared memory is released
+            for (int i = (it > STAGES ? it - STAGES : 0); i < it; ++i) {
+                const uint64_t t0 = gtimer();
+                while (!mbar_try(full0 + 8 * (i % STAGES), (uint32_t)(i / STAGES) & 1u) && gtimer() - t0 < WAIT_NS) {
+                }
+            }
+        }
+    } else if (warp == 1) {
+        // ---------------- MMA issuer (the whole warp walks the loop, lane 0 issues) ----------------
+        const bool leader = lane == 0;
+        if (err[1] != 0) {  // test hook: as in cgemm_tc_body
+            const uint64_t t0 = gtimer();
+            while (!mbar_try(never, 0u) && gtimer() - t0 < TEST_WAIT_NS) {
+            }
+            *abort_flag = 1;
+        }
+        const uint32_t lo0 = desc_lo(smem_u32(smem));
+        int s = 0, j = 0;  // stage, tile of this CTA
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int t = first; t < ntiles && ok && !*abort_flag; t += step, ++j) {
+            const int buf = j & 1;
+            if (j >= 2 && !mbar_wait(accempty + 8 * buf, (uint32_t)((j >> 1) - 1) & 1u, abort_flag)) break;
+            fence_after();
+            const uint32_t Dr = tmem + (uint32_t)buf * TMEM_COLS, Di = Dr + BN;
+            for (int kb = 0; kb < nkb; ++kb) {
+                if (!mbar_wait(full0 + 8 * s, ph, abort_flag)) {
+                    ok = false;
+                    break;
+                }
+                fence_after();
+                const uint32_t ar = lo0 + (uint32_t)s * (STAGE_BYTES >> 4);
+                tc_stage_products(leader, Dr, Di, ar, kb > 0 ? 1u : 0u);
+                if (leader) mma_commit(empty0 + 8 * s);
+                if (++s == STAGES) {
+                    s = 0;
+                    ph ^= 1u;
+                }
+            }
+            if (ok && leader) mma_commit(accfull + 8 * buf);
+        }
+        __syncwarp();
+        if (leader) {
+            // the products already issued finish before TMEM and shared memory are released
+            mma_commit(drain);
+            const uint64_t t0 = gtimer();
+            while (!mbar_try(drain, 0u) && gtimer() - t0 < WAIT_NS) {
+            }
+        }
+    } else if (warp >= 2) {
+        // ---------------- C (sixteen warps) ----------------
+        const int qw = warp & 3, cg = (warp - 2) >> 2;  // TMEM lane quarter this warp may access; column group
+        const uint32_t lane_off = (uint32_t)(qw * 32) << 16;
+        int j = 0;
+        for (int t = first; t < ntiles; t += step, ++j) {
+            const int tm = t % ntm, tn = t / ntm, buf = j & 1;
+            const long row = (long)tm * BM + qw * 32 + lane;
+            const int col0 = tn * BN + cg * UPD_COLS;
+            const int nc = row < m ? min(UPD_COLS, n - col0) : 0;  // columns of this thread inside C
+            float* pr = Cr + row + (long)col0 * ldc;
+            float* pi = Ci + row + (long)col0 * ldc;
+            const int ld = (int)ldc;  // (32 columns of it fit an int)
+            if (t + step < ntiles) {  // the next tile's C into L2: a lane per column, its 32 rows of this warp a line
+                const long r2 = (long)((t + step) % ntm) * BM + qw * 32;
+                const int c2 = (t + step) / ntm * BN + cg * UPD_COLS + lane;
+                if (r2 < m && c2 < n) {
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(Cr + r2 + (long)c2 * ldc));
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(Ci + r2 + (long)c2 * ldc));
+                }
+            }
+            float cr[UPD_COLS], ci[UPD_COLS];
+#pragma unroll
+            for (int q = 0; q < UPD_COLS; ++q) {
+                cr[q] = q < nc ? __ldcg(pr + q * ld) : 0.f;
+                ci[q] = q < nc ? __ldcg(pi + q * ld) : 0.f;
+            }
+            const bool got = mbar_wait(accfull + 8 * buf, (uint32_t)(j >> 1) & 1u, abort_flag);
+            if (!__all_sync(0xffffffffu, got)) break;
+            fence_after();
+            const uint32_t D = tmem + (uint32_t)buf * TMEM_COLS + lane_off + cg * UPD_COLS;
+#pragma unroll
+            for (int c0 = 0; c0 < UPD_COLS; c0 += 8) {
+                float vr[8], vi[8];
+                tmem_ld8x2(D + c0, D + BN + c0, vr, vi);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const int e = sc.e0 + (col0 + c0 + q < n ? __ldg(sc.eB + col0 + c0 + q) : 0);
+                    const float f = -tc_pow2(e >> 1), g = tc_pow2(e - (e >> 1));
+                    cr[c0 + q] += vr[q] * f * g;
+                    ci[c0 + q] += vi[q] * f * g;
+                }
+            }
+            fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(accempty + 8 * buf);
+#pragma unroll
+            for (int q = 0; q < UPD_COLS; ++q)
+                if (q < nc) {
+                    pr[q * ld] = cr[q];
+                    pi[q * ld] = ci[q];
+                }
+        }
+    }
+    __syncwarp();  // the roles' lanes meet again: the barrier below is warp-aligned
+    fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        fence_after();
+        tmem_dealloc(tmem, 2 * TMEM_COLS);
+    }
+    if (threadIdx.x == 0 && *abort_flag) atomicExch(err, 1);
 }
 
 // One product per blockIdx.z: C_z = beta C_z + alpha A_z B_z^T for a batch of equal-shape products
@@ -501,7 +647,7 @@ namespace {
 template <int OUT>
 cudaError_t launch_tc(cudaStream_t s, dim3 grid, const void* tAr, const void* tAi, const void* tBr, const void* tBi,
                       float* Cr, float* Ci, double2* C64, long ldc, long zstride, int m, int n, int K, int S,
-                      float alpha, float beta, int* d_err, TcScale sc, TcGate gate = TcGate{}) {
+                      float alpha, float beta, int* d_err, TcScale sc) {
     static DeviceFlags attr_set;
     if (attr_set.pending()) {
         cudaError_t e =
@@ -509,10 +655,10 @@ cudaError_t launch_tc(cudaStream_t s, dim3 grid, const void* tAr, const void* tA
         if (e != cudaSuccess) return e;
         attr_set.done();
     }
-    cgemm_tc_kernel<OUT><<<grid, tc_threads<OUT>(), SMEM_BYTES, s>>>(
+    cgemm_tc_kernel<OUT><<<grid, 128, SMEM_BYTES, s>>>(
         *reinterpret_cast<const CUtensorMap*>(tAr), *reinterpret_cast<const CUtensorMap*>(tAi),
         *reinterpret_cast<const CUtensorMap*>(tBr), *reinterpret_cast<const CUtensorMap*>(tBi), Cr, Ci, C64, ldc,
-        zstride, m, n, K, S, alpha, beta, d_err, sc, gate);
+        zstride, m, n, K, S, alpha, beta, d_err, sc);
     return cudaGetLastError();
 }
 
@@ -576,17 +722,31 @@ __global__ void __launch_bounds__(TC_PACK_THREADS) pack_b_kernel(const float* __
 
 }  // namespace
 
-// C = beta C + alpha A B^T, C FP32 planar column-major (m x n, ld ldc); one K range per CTA.
+// C = alpha A B^T, C FP32 planar column-major (m x n, ld ldc); one K range per CTA.
 cudaError_t gemm_tc(cudaStream_t s, const void* tAr, const void* tAi, const void* tBr, const void* tBi, float* Cr,
-                    float* Ci, long ldc, int m, int n, int K, float alpha, float beta, TcScale sc, int* d_err,
-                    TcGate gate) {
+                    float* Ci, long ldc, int m, int n, int K, float alpha, TcScale sc, int* d_err) {
     if (m <= 0 || n <= 0 || K <= 0) return cudaSuccess;
-    dim3 grid(ceil_div(m, BM), ceil_div(n, BN), 1);
-    if (beta != 0.f)
-        return launch_tc<OUT_C32_PRE>(s, grid, tAr, tAi, tBr, tBi, Cr, Ci, nullptr, ldc, 0, m, n, K, 1, alpha,
-                                      beta, d_err, sc, gate);
-    return launch_tc<OUT_C32>(s, grid, tAr, tAi, tBr, tBi, Cr, Ci, nullptr, ldc, 0, m, n, K, 1, alpha, beta,
-                              d_err, sc, gate);
+    return launch_tc<OUT_C32>(s, dim3(ceil_div(m, BM), ceil_div(n, BN), 1), tAr, tAi, tBr, tBi, Cr, Ci, nullptr, ldc, 0,
+                              m, n, K, 1, alpha, 0.f, d_err, sc);
+}
+
+// C -= A B^T by at most `ctas` CTAs.
+cudaError_t gemm_tc_upd(cudaStream_t s, const void* tAr, const void* tAi, const void* tBr, const void* tBi, float* Cr,
+                        float* Ci, long ldc, int m, int n, int K, TcScale sc, int ctas, int* d_err, TcGate gate) {
+    if (m <= 0 || n <= 0 || K <= 0) return cudaSuccess;
+    static DeviceFlags attr_set;
+    if (attr_set.pending()) {
+        cudaError_t e = cudaFuncSetAttribute(cgemm_tc_upd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+        if (e != cudaSuccess) return e;
+        attr_set.done();
+    }
+    const int tiles = ceil_div(m, BM) * ceil_div(n, BN) - gate.first_tile;
+    if (tiles <= 0) return cudaSuccess;
+    cgemm_tc_upd_kernel<<<std::min(tiles, std::max(ctas, 1)), UPD_THREADS, SMEM_BYTES, s>>>(
+        *reinterpret_cast<const CUtensorMap*>(tAr), *reinterpret_cast<const CUtensorMap*>(tAi),
+        *reinterpret_cast<const CUtensorMap*>(tBr), *reinterpret_cast<const CUtensorMap*>(tBi), Cr, Ci, ldc, m, n, K,
+        d_err, sc, gate);
+    return cudaGetLastError();
 }
 
 // Number of K splits for a product with few output tiles: about three waves of CTAs over the

@@ -47,8 +47,10 @@ struct TcGate {
     int first_tile = 0;
 };
 cudaError_t gemm_tc(cudaStream_t s, const void* tAr, const void* tAi, const void* tBr, const void* tBi, float* Cr,
-                    float* Ci, long ldc, int m, int n, int K, float alpha, float beta, TcScale sc, int* d_err,
-                    TcGate gate = TcGate{});
+                    float* Ci, long ldc, int m, int n, int K, float alpha, TcScale sc, int* d_err);
+cudaError_t gemm_tc_upd(cudaStream_t s, const void* tAr, const void* tAi, const void* tBr, const void* tBi, float* Cr,
+                        float* Ci, long ldc, int m, int n, int K, TcScale sc, int ctas, int* d_err,
+                        TcGate gate = TcGate{});
 constexpr int TC_BM = 128;
 constexpr int TC_BN = 128;
 // destination of a split-K product: FP32 planar (re, im) or, when z is set, FP64 interleaved

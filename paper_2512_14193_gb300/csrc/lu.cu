@@ -31,6 +31,7 @@
 // (the same sums as L_bb^{-1} Y_b formed inside every step, without recomputing it in each CTA).
 #include "lu_internal.cuh"
 
+#include <climits>
 #include <map>
 #include <mutex>
 
@@ -928,10 +929,11 @@ bm_status factor_fast(bm_ctx* c, C32 F) {
         if (mm == 0) break;
         BM_PROF(c, "cgemm_tc_kernel (trailing update)");
         const C32 C = F.sub(J + FD_B, J + FD_B);
+        // (persistent CTAs on all SMs but one, which the next diagonal block takes meanwhile)
         TcGate gate{fail, J + 1, 0};
         auto update = [&](cudaStream_t st, int m) {
-            return gemm_tc(st, c->tm_lu[0], c->tm_lu[1], c->tm_lu[2], c->tm_lu[3], C.re, C.im, C.ld, m, m, FD_B, -1.0f,
-                           1.0f, TcScale{nullptr, c->d_Upe, 0}, c->d_err, gate);
+            return gemm_tc_upd(st, c->tm_lu[0], c->tm_lu[1], c->tm_lu[2], c->tm_lu[3], C.re, C.im, C.ld, m, m, FD_B,
+                               TcScale{nullptr, c->d_Upe, 0}, c->num_sms - 1, c->d_err, gate);
         };
         if (!la || mm <= FD_B) {
             LU_CUDA(update(s, mm));
@@ -1085,9 +1087,10 @@ bm_status factor_t(bm_ctx* c, V F, bool tc, int J0 = 0) {
                     }
                     C32 Cv = F.sub(J + jb, J + jb);
                     {
+                        // (a CTA per tile: the panels' clusters need SMs that come free beside the rest)
                         BM_PROF(c, "cgemm_tc_kernel (trailing update)");
-                        LU_CUDA(gemm_tc(s, c->tm_lu[0], c->tm_lu[1], c->tm_lu[2], c->tm_lu[3], Cv.re, Cv.im, Cv.ld, mm,
-                                        nnext, jb, -1.0f, 1.0f, TcScale{nullptr, c->d_Upe, 0}, c->d_err));
+                        LU_CUDA(gemm_tc_upd(s, c->tm_lu[0], c->tm_lu[1], c->tm_lu[2], c->tm_lu[3], Cv.re, Cv.im, Cv.ld, mm,
+                                        nnext, jb, TcScale{nullptr, c->d_Upe, 0}, INT_MAX, c->d_err));
                     }
                     if (la) {
                         // the rest on s2: interchanges of the columns left of this panel and right of
@@ -1099,9 +1102,9 @@ bm_status factor_t(bm_ctx* c, V F, bool tc, int J0 = 0) {
                                                     c->ldk_lu, c->d_Upe + NB));
                         if (mm > nnext) {
                             C32 Cr = F.sub(J + jb, J + jb + nnext);
-                            LU_CUDA(gemm_tc(s2, c->tm_lu[0], c->tm_lu[1], c->tm_lu[4], c->tm_lu[5], Cr.re, Cr.im, Cr.ld,
-                                            mm, mm - nnext, jb, -1.0f, 1.0f, TcScale{nullptr, c->d_Upe + NB, 0},
-                                            c->d_err));
+                            LU_CUDA(gemm_tc_upd(s2, c->tm_lu[0], c->tm_lu[1], c->tm_lu[4], c->tm_lu[5], Cr.re, Cr.im, Cr.ld,
+                                            mm, mm - nnext, jb, TcScale{nullptr, c->d_Upe + NB, 0}, INT_MAX,
+                                                c->d_err));
                         }
                         LU_CUDA(cudaEventRecord(ev_join, s2));
                     }
