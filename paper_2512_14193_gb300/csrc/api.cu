@@ -177,6 +177,7 @@ void free_solve_ws(bm_ctx* c) {
     FREE(c->d_XQ);
     FREE(c->d_Wdf);
     FREE(c->d_flow);
+    FREE(c->d_flowx);
     c->flow_len = 0;
     for (int q = 0; q < 2; ++q) {
         FREE(c->d_dx[q]);
@@ -322,6 +323,7 @@ size_t request_bytes(int N, int form, int prec, int nb, int nrhs, int resid_mode
     if (prec == BM_FP64) {
         b += (size_t)p.n * w * 16;
     } else {
+        b += (2 * (size_t)ceil_div(p.n, 64) * ceil_div((int)w, FLOW_BN) + 1) * FLOW_ITEM_BYTES;
         b += (size_t)p.nsys * w * 8 + (size_t)p.n * w * 16 + (size_t)p.nsys * w * 24 + 4 * (size_t)N * w * 16;
         if (form == BM_MIXED) b += 2 * w * (size_t)(p.ldk_schur + p.ldk_c) * 2 + 8 * w + ((size_t)64 << 20);
     }
@@ -1026,10 +1028,11 @@ bm_status ensure_ws(bm_ctx* c, int nrhs) {
             BM_TRY(alloc_t(c, &c->d_XQ, (size_t)c->nsys * w * 8));
             BM_TRY(alloc_t(c, &c->d_Wdf, (size_t)4 * c->N * w * 16));
         }
-        // two triangles x (64-row tiles) x (8-column tiles)
-        c->flow_len = 2L * ceil_div(c->n, 64) * ceil_div(w, 8);
-        BM_TRY(alloc_t(c, &c->d_flow, (size_t)(c->flow_len + 1) * sizeof(int)));  // + a flag never set (test hook)
-        BM_CUDA_TRY(cudaMemsetAsync(c->d_flow, 0, (size_t)(c->flow_len + 1) * sizeof(int), c->stream));
+        // two triangles x (64-row tiles) x (column tiles), and an item nothing writes (test hook)
+        c->flow_len = 2L * ceil_div(c->n, 64) * ceil_div(w, FLOW_BN);
+        const size_t fx = (size_t)(c->flow_len + 1) * FLOW_ITEM_BYTES;
+        BM_TRY(alloc_t(c, &c->d_flowx, fx));
+        BM_CUDA_TRY(cudaMemsetAsync(c->d_flowx, 0xff, fx, c->stream));
     }
     if (c->prec != BM_FP64) {
         // x digit planes and split-K workspace of the tensor-core residual

@@ -79,6 +79,8 @@ bm_status lu_resume_enqueue(bm_ctx* c, int stop);
 size_t lu_fast_bytes(int n);                  // work buffer of the search-free blocks (d_fd)
 size_t lu_fast_z_bytes();                     // and of the FP64 ones
 size_t swap_map_bytes();
+constexpr int FLOW_BN = 8;                  // right-hand sides per item of the FP32 triangular solve
+constexpr size_t FLOW_ITEM_BYTES = 64 * FLOW_BN * sizeof(float2);  // an item's 64 rows in its exchange buffer
 bm_status getrs_z64(bm_ctx* c, double2* Y, long ldy, int nrhs);   // in place; Y holds P B (rows gathered by perm)
 bm_status getrs_c32(bm_ctx* c, float* Yr, float* Yi, long ldy, int nrhs);
 cudaError_t launch_gather_rows_z64(cudaStream_t s, const int* perm, int n, int nrhs, const double2* B, long ldb,

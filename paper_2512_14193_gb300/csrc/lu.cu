@@ -420,132 +420,7 @@ __global__ void __launch_bounds__(256) g_form_kernel(V F, int n, const typename 
     }
 }
 
-// One step of a blocked triangular solve in G form (all right-hand sides):
-//   Y[rest0:rest0+nrest, :] -= G[rest0.., r0:r0+rb] Y[r0:r0+rb, :]
-// (each CTA one 64-row tile of the rest and BN columns; the rows it reads and writes are disjoint).
-template <class V, int BN>
-__global__ void __launch_bounds__(256) trsv_g_step_kernel(V F, V Y, int r0, int rb, int rest0, int nrest, int nrhs) {
-    using CV = typename V::cv;
-    using Rl = typename V::real;
-    constexpr int B = TS_BM;
-    extern __shared__ __align__(16) unsigned char sm[];
-    CV* Yb = reinterpret_cast<CV*>(sm);  // [BN][B]
-    CV* Ft = Yb + BN * B;                // [B][B] column-major tile of G
-    const int t = threadIdx.x;
-    const int j0 = blockIdx.y * BN;
-    const int nc = min(BN, nrhs - j0);
-    const long tr0 = (long)rest0 + (long)blockIdx.x * B;
-    const int tm = (int)min((long)B, (long)rest0 + nrest - tr0);
-    load_tile<B, B>(Ft, F, tr0, r0, tm, rb);
-    pdl_wait();
-    pdl_trigger();
-    load_tile<B, BN>(Yb, Y, r0, j0, rb, nc);
-    __syncthreads();
-    constexpr int TN = BN / 16;
-    const int tx = t % 16, ty = t / 16;
-    CV acc[4][TN];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int c = 0; c < TN; ++c) acc[a][c] = czero<Rl>();
-    // threads whose columns all lie past the last right-hand side (the ragged column tile, e.g.
-    // 65 = 4 x 16 + 1) skip the product, so their warps leave the SM early
-    const int kend = (ty < nc) ? rb : 0;
-    for (int k = 0; k < kend; ++k) {
-        CV fv[4], yv[TN];
-#pragma unroll
-        for (int a = 0; a < 4; ++a) fv[a] = Ft[k * B + tx + 16 * a];
-#pragma unroll
-        for (int c = 0; c < TN; ++c) yv[c] = Yb[(ty + 16 * c) * B + k];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int c = 0; c < TN; ++c) cfma(acc[a][c], fv[a], yv[c]);
-    }
-    // read all of this thread's outputs before writing any (the reads do not wait on the writes)
-    CV yo[4][TN];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int c = 0; c < TN; ++c) {
-            const int i = tx + 16 * a, jj = ty + 16 * c;
-            yo[a][c] = (i < tm && jj < nc) ? Y.get(tr0 + i, (long)j0 + jj) : czero<Rl>();
-        }
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int c = 0; c < TN; ++c) {
-            const int i = tx + 16 * a, jj = ty + 16 * c;
-            if (i < tm && jj < nc) {
-                CV y = yo[a][c];
-                y.x -= acc[a][c].x;
-                y.y -= acc[a][c].y;
-                Y.set(tr0 + i, (long)j0 + jj, y);
-            }
-        }
-}
-
-// Z_b = T_b Y_b for every diagonal block b at once (grid: blocks x column tiles of BN).
-template <class V, int BN>
-__global__ void __launch_bounds__(256) trsv_diag_kernel(V Y, V Z, int n, int nrhs,
-                                                        const typename V::cv* __restrict__ Tinv) {
-    using CV = typename V::cv;
-    using Rl = typename V::real;
-    constexpr int B = TS_BM;
-    extern __shared__ __align__(16) unsigned char sm[];
-    CV* Ts = reinterpret_cast<CV*>(sm);  // [B][B] column-major
-    CV* Yb = Ts + B * B;                 // [BN][B]
-    const int t = threadIdx.x;
-    const long r0 = (long)blockIdx.x * B;
-    const int rb = (int)min((long)B, n - r0);
-    const int j0 = blockIdx.y * BN;
-    const int nc = min(BN, nrhs - j0);
-    load_block<B>(Ts, Tinv + (long)blockIdx.x * B * B, rb);
-    pdl_wait();
-    pdl_trigger();
-    load_tile<B, BN>(Yb, Y, r0, j0, rb, nc);
-    __syncthreads();
-    constexpr int TN = BN / 16;
-    const int tx = t % 16, ty = t / 16;
-    CV acc[4][TN];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int c = 0; c < TN; ++c) acc[a][c] = czero<Rl>();
-    for (int k = 0; k < rb; ++k) {
-        CV tv[4], yv[TN];
-#pragma unroll
-        for (int a = 0; a < 4; ++a) tv[a] = Ts[tx + 16 * a + k * B];
-#pragma unroll
-        for (int c = 0; c < TN; ++c) yv[c] = Yb[(ty + 16 * c) * B + k];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int c = 0; c < TN; ++c) cfma(acc[a][c], tv[a], yv[c]);
-    }
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        const int i = tx + 16 * a;
-        if (i >= rb) continue;
-#pragma unroll
-        for (int c = 0; c < TN; ++c) {
-            const int jj = ty + 16 * c;
-            if (jj < nc) Z.set(r0 + i, (long)j0 + jj, acc[a][c]);
-        }
-    }
-}
-
-// Persistent blocked triangular solve in G form (C32): the block steps and the diagonal blocks of
-// one triangle (forward: lower, backward: upper) in a single cooperative launch.  Work item (i, j)
-// is tile row i (64 rows) of column tile j (16 right-hand sides).  It accumulates
-// sum_b G[i, b] Y[b, j] over the tile rows b before i (lower) or after i (upper), each as soon as
-// item (b, j) has published its final rows through the flag ready[b, j]; then it writes
-// Y[i, j] -= that sum (the rows later items read), publishes ready[i, j], and writes
-// Z[i, j] = T_i Y[i, j] with T_i the inverted diagonal block.  CTA q takes items q, q + grid, ...
-// in dependency order, so the earliest unfinished item never waits; with every CTA resident
-// (cooperative launch) no wait can deadlock.  Waits are bounded (1 s by the global timer): a
-// timeout raises *err and the item goes on with what it has.
-constexpr int FL_BN = 8;
+// Waits for a flag (bounded: 1 s by the global timer, then *err is raised).
 __device__ __forceinline__ void flow_wait(const int* flag, int* err) {
     if (*reinterpret_cast<volatile int*>(err) != 0) return;  // an earlier wait gave up: no more waiting
     uint64_t t0 = 0;
@@ -560,124 +435,171 @@ __device__ __forceinline__ void flow_wait(const int* flag, int* err) {
         }
     }
 }
-// acc[c] += sum_k M[r, k] V[k, c] for k < kn: M column-major B x B, V row-major [k][BN]
-__device__ __forceinline__ void flow_mac(float2 (&acc)[FL_BN], const float2* M, const float2* V, int r, int kn) {
-    for (int k = 0; k < kn; ++k) {
-        const float2 g = M[k * TS_BM + r];
-        const float4* v4 = reinterpret_cast<const float4*>(V + k * FL_BN);
+// Persistent blocked triangular solve in G form (C32): the block steps and the diagonal blocks of
+// one triangle (forward: lower, backward: upper) in a single cooperative launch.  Work item (i, j)
+// is tile row i (64 rows) of column tile j (8 right-hand sides).  It accumulates
+// sum_b G[i, b] Y[b, j] over the tile rows b before i (lower) or after i (upper), each as soon as item
+// (b, j) has published its final rows, publishes Y[i, j] minus that sum and writes
+// Z[i, j] = T_i Y[i, j] with T_i the inverted diagonal block.
+// The chain of tile rows bounds the launch, so a link is kept short: the published rows are their own flag
+// (xch starts as FL_UNSET words, a bit pattern that arithmetic never produces; a reader polls the 16 bytes it
+// needs, one trip to L2 instead of a flag, a fence and a read), and the tiles of G arrive by cp.async in two
+// buffers while the step before is multiplied, with one barrier per step.  65 right-hand sides, one triangle,
+// n = 4096: 305 -> 193 us; n = 8192: 990 -> 583 us; 8 right-hand sides, n = 2048: 123 -> 57 us (1.8 us a link)
+// against flags, fences and single-buffered tiles.
+// CTA q takes items q, q + grid, ... in dependency order, so the earliest unfinished item never waits; with
+// every CTA resident (cooperative launch) no wait can deadlock.  Waits are bounded (1 s by the global timer): a
+// timeout raises *err and the item goes on with what it has.
+constexpr int FL_BN = FLOW_BN, FL_T = 256, FL_TILE = 2 * TS_BM * TS_BM;  // threads; floats of a tile of G or T
+static_assert(TS_BM * FL_BN == 2 * FL_T, "a thread per pair of entries of an item");
+static_assert(FLOW_ITEM_BYTES == FL_T * sizeof(float4), "an item's rows in xch: [pair of columns][row] float4");
+constexpr uint32_t FL_UNSET = 0xffffffffu;
+__device__ __forceinline__ bool flow_load(const float4* p, float4& v) {
+    asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "l"(p)
+                 : "memory");
+    return __float_as_uint(v.x) != FL_UNSET && __float_as_uint(v.y) != FL_UNSET && __float_as_uint(v.z) != FL_UNSET &&
+           __float_as_uint(v.w) != FL_UNSET;
+}
+__device__ __forceinline__ float4 flow_take(const float4* p, int* err) {
+    float4 v;
+    if (flow_load(p, v)) return v;
+    const uint64_t t0 = gtime();
+    for (int it = 1;; ++it) {
+        if (flow_load(p, v)) return v;
+        if ((it & 31) == 0) {
+            if (*reinterpret_cast<volatile int*>(err) != 0) return v;  // an earlier wait gave up: no more waiting
+            if (gtime() - t0 > 1000000000ull) {
+                atomicExch(err, 1);
+                return v;
+            }
+        }
+    }
+}
+__device__ __forceinline__ float flow_word(float v) { return __float_as_uint(v) == FL_UNSET ? __int_as_float(0x7fffffff) : v; }
+__device__ __forceinline__ void flow_publish(float4* p, float4 v) {
+    asm volatile("st.relaxed.gpu.global.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(flow_word(v.x)),
+                 "f"(flow_word(v.y)), "f"(flow_word(v.z)), "f"(flow_word(v.w))
+                 : "memory");
+}
+// 16 bytes global -> shared, the last 16 - bytes of them zeros
+__device__ __forceinline__ void cp_async16z(void* dst, const void* src, int bytes) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(bytes) : "memory");
+}
+// acc[c] += sum_k M[r, k] V[k, c] over this thread's 16 k from k0: M column-major 64 x 64, planar (G) or
+// interleaved (T); V [pair of columns][row]
+template <bool PLANAR>
+__device__ __forceinline__ void flow_mac(float2 (&acc)[FL_BN], const float* M, const float4* V, int r, int k0) {
+#pragma unroll 4
+    for (int k = k0; k < k0 + TS_BM / 4; ++k) {
+        const float2 g = PLANAR ? make_float2(M[k * TS_BM + r], M[FL_TILE / 2 + k * TS_BM + r])
+                                : reinterpret_cast<const float2*>(M)[k * TS_BM + r];
 #pragma unroll
         for (int c2 = 0; c2 < FL_BN / 2; ++c2) {
-            const float4 y = v4[c2];
+            const float4 y = V[c2 * TS_BM + k];
             cfma(acc[2 * c2], g, make_float2(y.x, y.y));
             cfma(acc[2 * c2 + 1], g, make_float2(y.z, y.w));
         }
     }
 }
 template <bool UPPER>
-__global__ void __launch_bounds__(256, 4) trsv_flow_kernel(C32 F, C32 Y, C32 Z, int n, int nrhs,
-                                                           const float2* __restrict__ Tinv, int* ready, int* err,
-                                                           const int* never, const int* hook) {
-    constexpr int B = TS_BM, BN = FL_BN, RS = 256 / B;  // RS k-slices of the 64 rows
+__global__ void __launch_bounds__(FL_T, 3) trsv_flow_kernel(C32 F, C32 Y, C32 Z, int n, int nrhs,
+                                                            const float2* __restrict__ Tinv, float4* xch, int* err,
+                                                            const float4* never, const int* hook) {
+    constexpr int B = TS_BM, BN = FL_BN;
     extern __shared__ __align__(16) unsigned char sm[];
-    float2* Gs = reinterpret_cast<float2*>(sm);     // [B][B] column-major: G[i, b], then T_i
-    float2* Red = Gs;                               // [RS][B][BN] partial sums of the k-slices (over Gs)
-    float2* Yb = Gs + B * B;                        // [B][BN] row-major: Y[b, j], then Y[i, j]
-    float2* Yo = Yb + B * BN;                       // [B][BN] this item's own right-hand-side rows
+    float* const Gs = reinterpret_cast<float*>(sm);                 // [2] tiles of G, the last one T_i
+    float4* const Ys = reinterpret_cast<float4*>(Gs + 2 * FL_TILE);  // [2] Y[b, j], the last one Y[i, j]
     const int t = threadIdx.x;
     const int nblk = (n + B - 1) / B, ct = (nrhs + BN - 1) / BN;
     const int items = nblk * ct;
-    const int r = t % B, ks = t / B;  // this thread: row r, k in [ks B / RS, (ks + 1) B / RS)
-    const int kb0 = ks * (B / RS);
-    pdl_wait();
-    pdl_trigger();
+    // this thread: row r; columns 2 ks, 2 ks + 1 of the item's rows, k in [16 ks, 16 ks + 16) of the products
+    const int r = t % B, ks = t / B, k0 = ks * (B / 4);
     const bool hooked = never != nullptr && *hook != 0;  // test hook (set at assembly)
     for (int q = blockIdx.x; q < items; q += gridDim.x) {
         __syncthreads();  // the previous item is done with the shared buffers
         const int i = UPPER ? nblk - 1 - q / ct : q / ct, j = q % ct;
         const long r0 = (long)i * B;
         const int tm = (int)min((long)B, n - r0);
-        const int j0 = j * BN, nc = min(BN, nrhs - j0);
-        // this item's own right-hand-side rows (written only by it), fetched early
+        const int j0 = j * BN;
+        const int nsteps = UPPER ? nblk - 1 - i : i;
+        // step st's tile (the last one: T_i) into buffer st & 1, zeros outside the matrix
+        auto fetch = [&](int st) {
+            float* dst = Gs + (st & 1) * FL_TILE;
+            if (st == nsteps) {
+                const float2* T = Tinv + (long)i * B * B;
 #pragma unroll
-        for (int m = 0; m < B * BN / 256; ++m) {
-            const int e = t + 256 * m;
-            const int k = e / BN, c = e % BN;
-            Yo[e] = (k < tm && c < nc) ? Y.get(r0 + k, (long)j0 + c) : make_float2(0.f, 0.f);
-        }
+                for (int m = 0; m < FL_TILE / 4 / FL_T; ++m) {
+                    const int e = t + FL_T * m, k = e / (B / 2), x = 2 * (e % (B / 2));
+                    const int bytes = k < tm ? 8 * min(max(tm - x, 0), 2) : 0;
+                    cp_async16z(dst + 4 * e, T + k * B + x, bytes);
+                }
+            } else {
+                const long c0 = (long)(UPPER ? nblk - 1 - st : st) * B;
+                const int rb = (int)min((long)B, n - c0);
+#pragma unroll
+                for (int m = 0; m < FL_TILE / 8 / FL_T; ++m) {
+                    const int e = t + FL_T * m, k = e / (B / 4), x = 4 * (e % (B / 4));
+                    const int bytes = k < rb ? 4 * min(max(tm - x, 0), 4) : 0;
+                    const long o = bytes > 0 ? r0 + x + (c0 + k) * F.ld : 0;
+                    cp_async16z(dst + 4 * e, F.re + o, bytes);
+                    cp_async16z(dst + FL_TILE / 2 + 4 * e, F.im + o, bytes);
+                }
+            }
+            cp_async_commit();
+        };
+        fetch(0);
+        // this item's own right-hand-side rows (zeros outside)
+        float2 own[2];
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+            own[c] = r < tm && j0 + 2 * ks + c < nrhs ? Y.get(r0 + r, (long)j0 + 2 * ks + c) : make_float2(0.f, 0.f);
         float2 acc[BN];
 #pragma unroll
         for (int c = 0; c < BN; ++c) acc[c] = make_float2(0.f, 0.f);
-        const int nsteps = UPPER ? nblk - 1 - i : i;
         for (int st = 0; st < nsteps; ++st) {
             const int b = UPPER ? nblk - 1 - st : st;
-            const long c0 = (long)b * B;
-            const int rb = (int)min((long)B, n - c0);
-            __syncthreads();  // the buffers are free
-            load_tile<B, B>(Gs, F, r0, c0, tm, rb);
-            // (test hook: the last item's first wait is on a flag that nothing sets)
-            const int* wf = (hooked && q == items - 1 && st == 0) ? never : ready + b * ct + j;
-            if (t == 0) flow_wait(wf, err);
-            __syncthreads();  // item (b, j) is final
+            // (test hook: the last item's first wait is on rows that nothing publishes)
+            const float4* from = (hooked && q == items - 1 && st == 0) ? never : xch + (long)(b * ct + j) * FL_T;
+            Ys[(st & 1) * FL_T + t] = flow_take(from + t, err);
+            cp_async_wait<0>();
+            __syncthreads();  // this step's operands are there; the step before has been multiplied
+            fetch(st + 1);
+            flow_mac<true>(acc, Gs + (st & 1) * FL_TILE, Ys + (st & 1) * FL_T, r, k0);
+        }
+        // sums over the four k ranges through the buffer of G that is free, [k range][pair of columns][row]
+        float4* const Red = reinterpret_cast<float4*>(Gs + ((nsteps + 1) & 1) * FL_TILE);
+        auto reduce = [&]() {
 #pragma unroll
-            for (int m = 0; m < B * BN / 256; ++m) {
-                const int e = t + 256 * m;
-                const int k = e / BN, c = e % BN;
-                float2 v = make_float2(0.f, 0.f);
-                if (k < rb && c < nc) {
-                    const long off = (c0 + k) + (long)(j0 + c) * Y.ld;
-                    v = make_float2(__ldcg(Y.re + off), __ldcg(Y.im + off));
-                }
-                Yb[e] = v;
-            }
+            for (int c2 = 0; c2 < BN / 2; ++c2)
+                Red[(ks * (BN / 2) + c2) * B + r] =
+                    make_float4(acc[2 * c2].x, acc[2 * c2].y, acc[2 * c2 + 1].x, acc[2 * c2 + 1].y);
             __syncthreads();
-            flow_mac(acc, Gs + kb0 * B, Yb + kb0 * BN, r, min(B / RS, max(rb - kb0, 0)));
-        }
-        // combine the k-slices: the final rows of Y[i, j], published for the later items
-        __syncthreads();  // Gs is free: Red lies over it
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int c = 0; c < BN; ++c) Red[(ks * B + r) * BN + c] = acc[c];
-        __syncthreads();
-        if (ks == 0) {
-#pragma unroll
-            for (int c = 0; c < BN; ++c) {
-                float2 y = Yo[r * BN + c];
-#pragma unroll
-                for (int q2 = 0; q2 < RS; ++q2) {
-                    const float2 p2 = Red[(q2 * B + r) * BN + c];
-                    y.x -= p2.x;
-                    y.y -= p2.y;
-                }
-                if (r < tm && c < nc) Y.set(r0 + r, (long)j0 + c, y);
-                Yb[r * BN + c] = y;
+            for (int q2 = 0; q2 < 4; ++q2) {
+                const float4 p = Red[(q2 * (BN / 2) + ks) * B + r];
+                v.x += p.x, v.y += p.y, v.z += p.z, v.w += p.w;
             }
-        }
-        // the CTA barrier orders every thread's rows before thread 0's release (cumulative at gpu
-        // scope), so a reader that acquires the flag sees them
-        __syncthreads();
-        if (t == 0) asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(ready + i * ct + j), "r"(1) : "memory");
-        // Z[i, j] = T_i Y[i, j] (rows r, k-slice ks; the slices summed as above)
-        load_block<B>(Gs, Tinv + (long)i * B * B, tm);
-        __syncthreads();
-        float2 z[BN];
+            return v;
+        };
+        __syncthreads();  // the last step has been multiplied
+        float4 y = reduce();
+        y = make_float4(own[0].x - y.x, own[0].y - y.y, own[1].x - y.z, own[1].y - y.w);
+        flow_publish(xch + (long)(i * ct + j) * FL_T + t, y);
+        Ys[(nsteps & 1) * FL_T + t] = y;
+        cp_async_wait<0>();
+        __syncthreads();  // T_i and Y[i, j]
+        // Z[i, j] = T_i Y[i, j]
 #pragma unroll
-        for (int c = 0; c < BN; ++c) z[c] = make_float2(0.f, 0.f);
-        flow_mac(z, Gs + kb0 * B, Yb + kb0 * BN, r, min(B / RS, max(tm - kb0, 0)));
-        __syncthreads();  // every slice has read Gs: Red may overwrite it
-#pragma unroll
-        for (int c = 0; c < BN; ++c) Red[(ks * B + r) * BN + c] = z[c];
-        __syncthreads();
-        if (ks == 0 && r < tm) {
-#pragma unroll
-            for (int c = 0; c < BN; ++c) {
-                float2 sum = make_float2(0.f, 0.f);
-#pragma unroll
-                for (int q2 = 0; q2 < RS; ++q2) {
-                    const float2 p2 = Red[(q2 * B + r) * BN + c];
-                    sum.x += p2.x;
-                    sum.y += p2.y;
-                }
-                if (c < nc) Z.set(r0 + r, (long)j0 + c, sum);
-            }
+        for (int c = 0; c < BN; ++c) acc[c] = make_float2(0.f, 0.f);
+        flow_mac<false>(acc, Gs + (nsteps & 1) * FL_TILE, Ys + (nsteps & 1) * FL_T, r, k0);
+        const float4 z = reduce();
+        if (r < tm) {
+            if (j0 + 2 * ks < nrhs) Z.set(r0 + r, (long)j0 + 2 * ks, make_float2(z.x, z.y));
+            if (j0 + 2 * ks + 1 < nrhs) Z.set(r0 + r, (long)j0 + 2 * ks + 1, make_float2(z.z, z.w));
         }
     }
 }
@@ -1124,26 +1046,6 @@ bm_status factor_t(bm_ctx* c, V F, bool tc, int J0 = 0) {
     return BM_OK;
 }
 
-template <class V, int BN>
-cudaError_t launch_trsv_g_step(cudaStream_t s, V F, V Y, int r0, int rb, int rest0, int nrest, int nrhs) {
-    size_t smem = ((size_t)BN * TS_BM + (size_t)TS_BM * TS_BM) * sizeof(typename V::cv);
-    dim3 grid(ceil_div(nrest, TS_BM), ceil_div(nrhs, BN));
-    auto kern = trsv_g_step_kernel<V, BN>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    return launch_pdl(kern, grid, dim3(256), smem, s, F, Y, r0, rb, rest0, nrest, nrhs);
-}
-
-template <class V, int BN>
-cudaError_t launch_trsv_diag(cudaStream_t s, V Y, V Z, int n, int nrhs, const typename V::cv* Tinv) {
-    size_t smem = ((size_t)TS_BM * TS_BM + (size_t)BN * TS_BM) * sizeof(typename V::cv);
-    dim3 grid(ceil_div(n, TS_BM), ceil_div(nrhs, BN));
-    auto kern = trsv_diag_kernel<V, BN>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    return launch_pdl(kern, grid, dim3(256), smem, s, Y, Z, n, nrhs, Tinv);
-}
-
 // one cooperative launch of a persistent triangular solve: as many CTAs as the items, at most the number the
 // device keeps resident (queried once per process, device and kernel)
 template <class... KArgs, class... Args>
@@ -1186,54 +1088,25 @@ cudaError_t launch_flow(cudaStream_t s, void (*kern)(KArgs...), int threads, int
 template <class V>
 bm_status getrs_t(bm_ctx* c, V F, V Y, V Zw, int nrhs, const typename V::cv* dinvL, const typename V::cv* dinvU) {
     cudaStream_t s = c->stream;
-    const int n = c->n, bs = c->bs_solve;
-    const int nblk = ceil_div(n, bs);
-    // Column tiles of 16 right-hand sides halve each CTA's work (the steps are latency-bound) as
-    // long as the widest step still fits about one wave of resident CTAs (two per SM); beyond
-    // that, 32-wide tiles (fewer, fatter CTAs) are faster.
-    const long widest16 = (long)ceil_div(std::max(n - bs, 1), TS_BM) * ceil_div(nrhs, 16);
-    const bool narrow = nrhs <= 16 || widest16 <= (long)(1.1 * 2 * std::max(c->num_sms, 1));
+    const int n = c->n;
     if constexpr (std::is_same<V, C32>::value) {  // factors in G form
-        const int ct = ceil_div(nrhs, FL_BN), items = nblk * ct;
-        if (bs == TS_BM && c->d_flow != nullptr && 2L * items <= c->flow_len) {
-            // one persistent launch per triangle (block steps and diagonal blocks)
-            BM_PROF(c, "trsv_flow_kernel");
-            // a timed-out wait raises the handle's device-wait word, which the refinement loop reads
-            // back with every backward error (BM_ETIMEOUT)
-            // (test hook: with d_info[3] set at assembly, one wait of the forward sweep is on the
-            // never-set word after the flags)
-            LU_CUDA(cudaMemsetAsync(c->d_flow, 0, (size_t)2 * items * sizeof(int), s));
-            const int smem = (TS_BM * TS_BM + 2 * FL_BN * TS_BM) * (int)sizeof(float2);
-            LU_CUDA(launch_flow(s, trsv_flow_kernel<false>, 256, smem, items, c->num_sms, F, Y, Zw, n, nrhs, dinvL,
-                                c->d_flow, c->d_err, c->d_flow + c->flow_len, c->d_info + 3));
-            LU_CUDA(launch_flow(s, trsv_flow_kernel<true>, 256, smem, items, c->num_sms, F, Zw, Y, n, nrhs, dinvU,
-                                c->d_flow + items, c->d_err, nullptr, c->d_info + 3));
-            return BM_OK;
+        const int items = ceil_div(n, TS_BM) * ceil_div(nrhs, FL_BN);
+        if (c->d_flowx == nullptr || 2L * items > c->flow_len) {
+            bm_set_error("lu: the triangular solve's exchange buffer is missing");
+            return BM_EINVAL;
         }
-        auto gstep = [&](V Yv, int r0, int rb, int rest0, int nrest) {
-            return narrow ? launch_trsv_g_step<V, 16>(s, F, Yv, r0, rb, rest0, nrest, nrhs)
-                          : launch_trsv_g_step<V, 32>(s, F, Yv, r0, rb, rest0, nrest, nrhs);
-        };
-        auto diag = [&](V Yv, V Zv, const typename V::cv* T) {
-            return narrow ? launch_trsv_diag<V, 16>(s, Yv, Zv, n, nrhs, T)
-                          : launch_trsv_diag<V, 32>(s, Yv, Zv, n, nrhs, T);
-        };
-        for (int b = 0; b + 1 < nblk; ++b) {  // Y[below b] -= G_L Y_b
-            int r0 = b * bs, rb = std::min(bs, n - r0);
-            BM_PROF(c, "trsv_g_step_kernel");
-            LU_CUDA(gstep(Y, r0, rb, r0 + rb, n - r0 - rb));
-        }
-        {
-            BM_PROF(c, "trsv_diag_kernel");
-            LU_CUDA(diag(Y, Zw, dinvL));  // Zw = L^{-1} P B
-        }
-        for (int b = nblk - 1; b > 0; --b) {  // Zw[above b] -= G_U Zw_b
-            int r0 = b * bs, rb = std::min(bs, n - r0);
-            BM_PROF(c, "trsv_g_step_kernel");
-            LU_CUDA(gstep(Zw, r0, rb, 0, r0));
-        }
-        BM_PROF(c, "trsv_diag_kernel");
-        LU_CUDA(diag(Zw, Y, dinvU));  // Y = U^{-1} Zw
+        // one persistent launch per triangle (block steps and diagonal blocks); a timed-out wait raises the
+        // handle's device-wait word, which the refinement loop reads back with every backward error
+        // (BM_ETIMEOUT).  (Test hook: with d_info[3] set at assembly, one wait of the forward sweep is on the
+        // never-written item after the others.)
+        BM_PROF(c, "trsv_flow_kernel");
+        float4* const x = reinterpret_cast<float4*>(c->d_flowx);
+        LU_CUDA(cudaMemsetAsync(x, 0xff, 2 * items * FLOW_ITEM_BYTES, s));
+        const int smem = 2 * FL_TILE * (int)sizeof(float) + 2 * (int)FLOW_ITEM_BYTES;
+        LU_CUDA(launch_flow(s, trsv_flow_kernel<false>, FL_T, smem, items, c->num_sms, F, Y, Zw, n, nrhs, dinvL, x,
+                            c->d_err, x + c->flow_len * FL_T, c->d_info + 3));
+        LU_CUDA(launch_flow(s, trsv_flow_kernel<true>, FL_T, smem, items, c->num_sms, F, Zw, Y, n, nrhs, dinvU,
+                            x + (long)items * FL_T, c->d_err, nullptr, c->d_info + 3));
     } else {
         const int items = ceil_div(n, FZ_B) * ceil_div(nrhs, FZ_NC);
         if (c->d_flow == nullptr || 2L * items > c->flow_len) {
