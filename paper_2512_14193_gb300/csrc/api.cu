@@ -285,13 +285,12 @@ Plan make_plan(int N, int form, int prec, int nb_user, int bs, int nd, bool fast
         p.ldk_lu = tc_ldk(fast ? std::max(p.nb, 128) : p.nb);
         b += 2 * (size_t)p.n * p.ldk_lu * 4 + (size_t)p.n * 4;
         if (fast) b += lu_fast_bytes(p.n);
-        // digit planes of the operator for the tensor-core residual, their row exponents, and the
-        // row-maximum scratch of their construction
+        // digit planes of the operator for the tensor-core residual and their row exponents
         const size_t planes = (size_t)rt_digit_planes(nd) * 2;
         if (form == BM_MIXED)
-            b += planes * (2L * N * rt_ldk(N) + (size_t)N * rt_ldk(2L * N)) + 3L * N * 4 + 2L * N * 8;
+            b += planes * (2L * N * rt_ldk(N) + (size_t)N * rt_ldk(2L * N)) + 3L * N * 4;
         else
-            b += planes * 2L * N * rt_ldk(2L * N) + 2L * N * 4 + 2L * N * 8;
+            b += planes * 2L * N * rt_ldk(2L * N) + 2L * N * 4;
     }
     p.nblk = ceil_div(p.n, bs);
     b += 2 * (size_t)p.n * 4;
@@ -741,7 +740,6 @@ bm_status assemble_post(bm_ctx* c, bool run_assembly_kernel, bool wait) {
     const int N = c->N, form = c->form, prec = c->prec, nd = c->rt_nd;
     const bool c32 = prec != BM_FP64;
     const Plan& p = c->nd_plan;
-    bm_status s = BM_OK;
     c->post_pending = false;
     if (run_assembly_kernel) {
         BM_CUDA_TRY(launch_assemble(st, c));
@@ -762,25 +760,18 @@ bm_status assemble_post(bm_ctx* c, bool run_assembly_kernel, bool wait) {
             c->launches += 1;
         }
         // digit planes of the operator for the tensor-core residual
-        void* rowmax = nullptr;
-        s = ctx_alloc(c, &rowmax, 2L * N * 8);
-        if (s != BM_OK) {
-            free_problem(c);
-            return s;
-        }
         if (form == BM_MIXED) {
-            BM_CUDA_TRY(launch_digits_a(st, c->d_Mtop, c->ldtop, 2 * N, N, c->d_dge[0], c->d_dg[0], c->dg_ldk[0], rowmax,
+            BM_CUDA_TRY(launch_digits_a(st, c->d_Mtop, c->ldtop, 2 * N, N, c->d_dge[0], c->d_dg[0], c->dg_ldk[0], nullptr,
                                         nd));
-            BM_CUDA_TRY(launch_digits_a(st, c->d_Mbot, c->ldbot, N, 2 * N, c->d_dge[1], c->d_dg[1], c->dg_ldk[1], rowmax,
+            BM_CUDA_TRY(launch_digits_a(st, c->d_Mbot, c->ldbot, N, 2 * N, c->d_dge[1], c->d_dg[1], c->dg_ldk[1], nullptr,
                                         nd));
             BM_CUDA_TRY(launch_pack_solve(st, c));
-            c->launches += 7;
-        } else {
-            BM_CUDA_TRY(launch_digits_a(st, c->d_A, c->ldA, 2 * N, 2 * N, c->d_dge[0], c->d_dg[0], c->dg_ldk[0], rowmax,
-                                        nd));
             c->launches += 3;
+        } else {
+            BM_CUDA_TRY(launch_digits_a(st, c->d_A, c->ldA, 2 * N, 2 * N, c->d_dge[0], c->d_dg[0], c->dg_ldk[0], nullptr,
+                                        nd));
+            c->launches += 1;
         }
-        ctx_free(c, rowmax);  // stream-ordered: released once the digit kernels are done with it
     }
     BM_TRY(lu_setup(c, c->opt_cluster_cap, c->opt_panel_kernel));
     // test hook read by the tensor-core products (d_err[1], any nonzero value sets it); a memset keeps
@@ -860,7 +851,6 @@ bm_status factor_sequence(bm_ctx* c) {
     BM_CUDA_TRY(cudaMemsetAsync(c->d_info, 0, 2 * sizeof(int), s));
     BM_CUDA_TRY(cudaMemsetAsync(c->d_info + 4, 0, sizeof(int), s));
     if (c->prec == BM_FP64) {
-        Z64 F{c->d_F64, c->ldF};
         if (c->form == BM_MIXED) {
             BM_TRY(schur_z64(c, s));  // U33 = -[M31 M32] [M13; M23]
         } else {

@@ -278,13 +278,17 @@ __device__ __forceinline__ void atomic_max_pos(double* p, double v) {
 // its 8 warps taking every 8th column, eight loads in flight per thread.  The moduli are formed in
 // FP32 from the entries rounded to FP32 (by integer operations: the FP64 pipe is narrow) and each
 // thread sums its columns in FP32, the eight warps' sums added in FP64: a relative error of a few
-// 1e-6 at most, ample for a norm that only scales the backward error.
+// 1e-6 at most, ample for a norm that only scales the backward error.  With e, the same pass finds the row
+// exponents of the digit planes (integer maxima of the magnitudes' bits; a pass of its own took 0.19 ms at
+// N = 4096).
 __global__ void __launch_bounds__(256) rownorm_kernel(const double2* __restrict__ A, long ld, int m, int ncols,
-                                                      double add, double* out) {
+                                                      double add, double* out, int* __restrict__ e) {
     __shared__ double part[8][32];
+    __shared__ unsigned long long top[8][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i = blockIdx.x * 32 + lane;
     float sf = 0.f;
+    unsigned long long mx = 0;
     if (i < m) {
         const double2* a = A + i;
         int j = warp;
@@ -296,12 +300,14 @@ __global__ void __launch_bounds__(256) rownorm_kernel(const double2* __restrict_
             for (int u = 0; u < 8; ++u) {
                 const float x = f32_rn(v[u].x), y = f32_rn(v[u].y);
                 sf += sqrtf(fmaf(x, x, y * y));
+                mx = max(mx, max(mag_bits(v[u].x), mag_bits(v[u].y)));
             }
         }
         for (; j < ncols; j += 8) {
             const double2 v = a[(long)j * ld];
             const float x = f32_rn(v.x), y = f32_rn(v.y);
             sf += sqrtf(fmaf(x, x, y * y));
+            mx = max(mx, max(mag_bits(v.x), mag_bits(v.y)));
         }
     }
     // FP32 overflow (entries above ~1e19) falls back to the FP64 modulus for this thread's row
@@ -314,7 +320,13 @@ __global__ void __launch_bounds__(256) rownorm_kernel(const double2* __restrict_
         }
     }
     part[warp][lane] = s;
+    top[warp][lane] = mx;
     __syncthreads();
+    if (warp == 1 && e != nullptr && i < m) {
+#pragma unroll
+        for (int w = 0; w < 8; ++w) mx = max(mx, top[w][lane]);
+        e[i] = row_exponent(mx);
+    }
     if (warp == 0) {
         double t = 0.0;
         if (i < m) {
@@ -859,11 +871,15 @@ extern "C" bm_status bm_zeta_weights(int p, double* tau, double* c2) {
 cudaError_t launch_normA(cudaStream_t s, const bm_ctx* c) {
     cudaError_t e = cudaMemsetAsync(c->d_normA, 0, sizeof(double), s);
     if (e != cudaSuccess) return e;
+    // (the CF32 precisions' digit planes are scaled by row exponents, found on the way; d_dge is null in FP64)
     if (c->form == BM_MIXED) {
-        rownorm_kernel<<<ceil_div(2 * c->N, 32), 256, 0, s>>>(c->d_Mtop, c->ldtop, 2 * c->N, c->N, 1.0, c->d_normA);
-        rownorm_kernel<<<ceil_div(c->N, 32), 256, 0, s>>>(c->d_Mbot, c->ldbot, c->N, 2 * c->N, 0.0, c->d_normA);
+        rownorm_kernel<<<ceil_div(2 * c->N, 32), 256, 0, s>>>(c->d_Mtop, c->ldtop, 2 * c->N, c->N, 1.0, c->d_normA,
+                                                                  c->d_dge[0]);
+        rownorm_kernel<<<ceil_div(c->N, 32), 256, 0, s>>>(c->d_Mbot, c->ldbot, c->N, 2 * c->N, 0.0, c->d_normA,
+                                                              c->d_dge[1]);
     } else {
-        rownorm_kernel<<<ceil_div(2 * c->N, 32), 256, 0, s>>>(c->d_A, c->ldA, 2 * c->N, 2 * c->N, 0.0, c->d_normA);
+        rownorm_kernel<<<ceil_div(2 * c->N, 32), 256, 0, s>>>(c->d_A, c->ldA, 2 * c->N, 2 * c->N, 0.0, c->d_normA,
+                                                                  c->d_dge[0]);
     }
     return cudaGetLastError();
 }

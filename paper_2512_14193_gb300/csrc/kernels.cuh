@@ -142,8 +142,21 @@ void rt_plan_splits(int nprod, const long* m, const long* K, int n, int nd, int 
 bm_status rt_make_map(void* tmap, const void* base, long rows, long K, long ldk, long plane_elems, int box_rows,
                       int nd);
 bm_status rt_make_map_x(void* tmaps, const void* base, long cols, long K, long ldk, int nd);  // two blobs
+// (rowmax: scratch of `rows` words to find the row exponents e with; null: e holds them)
 cudaError_t launch_digits_a(cudaStream_t s, const double2* A, long lda, int rows, int K, int* e, void* D, long ldk,
                             void* rowmax, int nd);
+// |v| as the bits of a non-negative double, which order as the doubles do; NaN counts as zero
+__device__ __forceinline__ unsigned long long mag_bits(double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
+    return b > 0x7FF0000000000000ull ? 0ull : b;
+}
+// e with m < 2^(e - 1) of the largest magnitude m of a row, given as its bits (0 for a zero row)
+__device__ __forceinline__ int row_exponent(unsigned long long mx) {
+    const double m = __longlong_as_double((long long)mx);
+    int ex = 0;
+    if (m > 0.0) frexp(m, &ex);  // m = f 2^ex, f in [1/2, 1)
+    return m > 0.0 ? ex + 1 : 0;
+}
 cudaError_t launch_digits_x(cudaStream_t s, const double2* X, long ldx, int r0, int K, int n, int npad, int* f,
                             void* D, long ldk, long plane, int nd);
 cudaError_t gemm_rt(cudaStream_t s, const RtArgs* prods, int nprod, int n, double alpha, int* d_err, int* launched,
