@@ -218,6 +218,7 @@ void free_problem(bm_ctx* c) {
     FREE(c->d_Bp_r);
     FREE(c->d_Bp_i);
     FREE(c->d_Bpe);
+    FREE(c->d_Ape);
     FREE(c->d_Lp_r);
     FREE(c->d_Lp_i);
     FREE(c->d_Up_r);
@@ -276,7 +277,7 @@ Plan make_plan(int N, int form, int prec, int nb_user, int bs, int nd, bool fast
         b += (form == BM_MIXED) ? (size_t)p.ldtop * N * pb + (size_t)p.ldbot * 2 * N * pb : (size_t)p.ldA * 2 * N * pb;
         if (form == BM_MIXED) {
             p.ldk_schur = tc_ldk(2L * N);
-            b += 2 * (size_t)N * p.ldk_schur * 4 + (size_t)N * 4;
+            b += 2 * (size_t)N * p.ldk_schur * 4 + 2 * (size_t)N * 4;
             // [M13; M23] rows for the skinny products of the solve
             p.ldk_c = tc_ldk(N);
             b += 2 * (size_t)N * p.ldk_c * 4;
@@ -422,7 +423,7 @@ extern "C" bm_status bm_enqueue_probe(bm_ctx* c, int which, int reps) {
             } else {
                 BM_CUDA_TRY(gemm_tc(s, c->tm_schur[0], c->tm_schur[1], c->tm_schur[2], c->tm_schur[3], c->d_F32r,
                                     c->d_F32i, c->ldF, c->N, c->N, 2 * c->N, -1.0f,
-                                    TcScale{c->d_dge[1], c->d_Bpe, TC_E_DGE}, c->d_err));
+                                    schur_scale(c), c->d_err));
             }
             c->launches += 1;
         }
@@ -586,8 +587,10 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
     }
     if (c->fast_denied) p = make_plan(N, form, prec, nb, 64, nd, false, planes);
     // the captured factorisation depends on the launch settings: capture again when they change
-    if (reuse && (eager != c->eager || cl_cap != c->opt_cluster_cap || pkern != c->opt_panel_kernel))
+    const int shift = form == BM_MIXED && prec != BM_FP64 ? tc_shift_of(eps0) : 0;
+    if (reuse && (eager != c->eager || cl_cap != c->opt_cluster_cap || pkern != c->opt_panel_kernel || shift != c->tc_shift))
         drop_graphs(c);
+    c->tc_shift = shift;
     c->eager = eager;
     c->opt_cluster_cap = cl_cap;
     c->opt_panel_kernel = pkern;
@@ -656,6 +659,7 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
             if (s == BM_OK) s = alloc_t(c, &c->d_Bp_r, pb);
             if (s == BM_OK) s = alloc_t(c, &c->d_Bp_i, pb);
             if (s == BM_OK) s = alloc_t(c, &c->d_Bpe, (size_t)N * 4);
+            if (s == BM_OK) s = alloc_t(c, &c->d_Ape, (size_t)N * 4);
             size_t cb = (size_t)2 * N * p.ldk_c * 2;
             if (s == BM_OK) s = alloc_t(c, &c->d_Cp_r, cb);
             if (s == BM_OK) s = alloc_t(c, &c->d_Cp_i, cb);
@@ -766,7 +770,8 @@ bm_status assemble_post(bm_ctx* c, bool run_assembly_kernel, bool wait) {
             BM_CUDA_TRY(launch_digits_a(st, c->d_Mbot, c->ldbot, N, 2 * N, c->d_dge[1], c->d_dg[1], c->dg_ldk[1], nullptr,
                                         nd));
             BM_CUDA_TRY(launch_pack_solve(st, c));
-            c->launches += 3;
+            BM_CUDA_TRY(launch_shifted_exponents(st, c));
+            c->launches += 3 + (c->tc_shift != 0);
         } else {
             BM_CUDA_TRY(launch_digits_a(st, c->d_A, c->ldA, 2 * N, 2 * N, c->d_dge[0], c->d_dg[0], c->dg_ldk[0], nullptr,
                                         nd));
@@ -867,7 +872,7 @@ bm_status factor_sequence(bm_ctx* c) {
             BM_PROF(c, "cgemm_tc_kernel (Schur complement)");
             BM_CUDA_TRY(gemm_tc(s, c->tm_schur[0], c->tm_schur[1], c->tm_schur[2], c->tm_schur[3], c->d_F32r,
                                 c->d_F32i, c->ldF, c->N, c->N, 2 * c->N, -1.0f,
-                                TcScale{c->d_dge[1], c->d_Bpe, TC_E_DGE}, c->d_err));
+                                schur_scale(c), c->d_err));
         } else {
             BM_PROF(c, "to_c32_kernel");
             BM_CUDA_TRY(launch_to_c32(s, c->d_A, c->ldA, c->n, c->n, c->d_F32r, c->d_F32i, c->ldF));

@@ -485,12 +485,12 @@ __global__ void hankel_probe_kernel(const double2* __restrict__ z, int n, Hankel
     h1[i] = b;
 }
 
-// A operands: rows of an FP64 column-major block (rows x K) as pack rows, scaled by the digit planes' row
-// exponents e (entries below 2^(e - 1); TC_E_DGE).  One 32 x 32 tile per CTA through shared memory, so that
+// A operands: rows of an FP64 column-major block (rows x K), the columns from `half` on times w (tc_shift), as
+// pack rows scaled by row exponents e (entries below 2^(e - 1); TC_E_DGE).  One 32 x 32 tile per CTA through shared memory, so that
 // both sides are coalesced; a warp writes the 128 bytes of a row.
 __global__ void pack_rowmajor_kernel(const double2* __restrict__ M, long ldm, int rows, int K,
-                                     const int* __restrict__ e, __half* __restrict__ Pr, __half* __restrict__ Pi,
-                                     long ldk) {
+                                     int half, float w, const int* __restrict__ e, __half* __restrict__ Pr,
+                                     __half* __restrict__ Pi, long ldk) {
     __shared__ float2 t[32][33];
     const int k0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
     const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
@@ -498,7 +498,8 @@ __global__ void pack_rowmajor_kernel(const double2* __restrict__ M, long ldm, in
     for (int q = ty; q < 32; q += 8) {
         const int r = r0 + tx, k = k0 + q;
         const double2 v = (r < rows && k < K) ? M[r + (long)k * ldm] : make_double2(0, 0);
-        t[q][tx] = make_float2((float)v.x, (float)v.y);
+        const float f = k < half ? 1.f : w;
+        t[q][tx] = make_float2((float)v.x * f, (float)v.y * f);
     }
     __syncthreads();
 #pragma unroll
@@ -519,20 +520,41 @@ __global__ void pack_rowmajor_kernel(const double2* __restrict__ M, long ldm, in
     }
 }
 
-// B operand of the Schur product: column n of an FP64 block as pack row n, one CTA per column.
+// Row exponents of [M31 M32] with the columns from `half` on times 2^-shift (eps0 not near 1: tc_shift), as the
+// digit planes have them: entries below 2^(e - 1).  e starts below every exponent.
+__global__ void shifted_exponent_kernel(const double2* __restrict__ A, long lda, int rows, int K, int half, int shift,
+                                        int* __restrict__ e) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= rows) return;
+    const int j0 = blockIdx.y * 256, j1 = min(K, j0 + 256);
+    int m = -(1 << 30);
+#pragma unroll 8
+    for (int j = j0; j < j1; ++j) {
+        const double2 v = A[i + (long)j * lda];
+        const int E = (int)(max(mag_bits(v.x), mag_bits(v.y)) >> 52);  // (0: zero or subnormal)
+        if (E > 0) m = max(m, E - 1021 - (j < half ? 0 : shift));
+    }
+    atomicMax(e + i, m);
+}
+
+// B operand of the Schur product: column n of an FP64 block as pack row n, one CTA per column; the rows from
+// `half` on times w (tc_shift).
 struct ColZ64 {
     const double2* p;
+    int half;
+    float w;
     __device__ __forceinline__ float2 operator()(long k) const {
         const double2 v = p[k];
-        return make_float2((float)v.x, (float)v.y);
+        const float f = k < half ? 1.f : w;
+        return make_float2((float)v.x * f, (float)v.y * f);
     }
 };
 __global__ void __launch_bounds__(TC_PACK_THREADS) pack_colmajor_kernel(const double2* __restrict__ M, long ldm, int K,
-                                                                        __half* __restrict__ Pr,
+                                                                        int half, float w, __half* __restrict__ Pr,
                                                                         __half* __restrict__ Pi, long ldk,
                                                                         int* __restrict__ e) {
     const long n = blockIdx.x;
-    tc_pack_column(ColZ64{M + n * ldm}, K, Pr + n * ldk, Pi + n * ldk, e + n);
+    tc_pack_column(ColZ64{M + n * ldm, half, w}, K, Pr + n * ldk, Pi + n * ldk, e + n);
 }
 
 __global__ void to_c32_kernel(const double2* __restrict__ A, long lda, int m, int n, float* Fr, float* Fi, long ldf) {
@@ -942,11 +964,28 @@ cudaError_t launch_hankel_probe(cudaStream_t s, const bm_ctx* c, const double2* 
 
 // Operands of the Schur-complement product (part of the factorisation, like the FP32 copy of the
 // ordinary matrix): A = [M31 M32] row-major, B = [M13; M23] column by column.
+// The columns of M32 carry a factor eps0 and the rows of M23 one of 1 / eps1: with a single scale per row and
+// column of the packs, M31 would lose what eps0 exceeds 1 by.  A power of two near eps0 (tc_shift) is moved from
+// the one to the other, and the rows of [M31 M32] get exponents of their own then (d_Ape).
+int tc_shift_of(double eps0) {
+    return eps0 != 0.0 && std::isfinite(eps0) ? std::min(std::max(std::ilogb(eps0), -126), 126) : 0;
+}
+TcScale schur_scale(const bm_ctx* c) { return TcScale{c->tc_shift ? c->d_Ape : c->d_dge[1], c->d_Bpe, TC_E_DGE}; }
+cudaError_t launch_shifted_exponents(cudaStream_t s, const bm_ctx* c) {
+    const int N = c->N;
+    if (c->tc_shift == 0) return cudaSuccess;
+    cudaError_t e = cudaMemsetAsync(c->d_Ape, 0x80, (size_t)N * sizeof(int), s);
+    if (e != cudaSuccess) return e;
+    shifted_exponent_kernel<<<dim3(ceil_div(N, 128), ceil_div(2 * N, 256)), 128, 0, s>>>(c->d_Mbot, c->ldbot, N, 2 * N, N,
+                                                                                        c->tc_shift, c->d_Ape);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_pack_schur(cudaStream_t s, const bm_ctx* c) {
     const int N = c->N, K = 2 * N;
     pack_rowmajor_kernel<<<dim3(ceil_div(K, 32), ceil_div(N, 32)), dim3(32, 8), 0, s>>>(
-        c->d_Mbot, c->ldbot, N, K, c->d_dge[1], c->d_Ap_r, c->d_Ap_i, c->ldk_schur);
-    pack_colmajor_kernel<<<N, TC_PACK_THREADS, 0, s>>>(c->d_Mtop, c->ldtop, K, c->d_Bp_r, c->d_Bp_i, c->ldk_schur,
+        c->d_Mbot, c->ldbot, N, K, N, ldexpf(1.f, -c->tc_shift), schur_scale(c).eA, c->d_Ap_r, c->d_Ap_i, c->ldk_schur);
+    pack_colmajor_kernel<<<N, TC_PACK_THREADS, 0, s>>>(c->d_Mtop, c->ldtop, K, N, ldexpf(1.f, c->tc_shift), c->d_Bp_r, c->d_Bp_i, c->ldk_schur,
                                                        c->d_Bpe);
     return cudaGetLastError();
 }
@@ -956,7 +995,7 @@ cudaError_t launch_pack_schur(cudaStream_t s, const bm_ctx* c) {
 cudaError_t launch_pack_solve(cudaStream_t s, const bm_ctx* c) {
     const int N = c->N;
     pack_rowmajor_kernel<<<dim3(ceil_div(N, 32), ceil_div(2 * N, 32)), dim3(32, 8), 0, s>>>(
-        c->d_Mtop, c->ldtop, 2 * N, N, c->d_dge[0], c->d_Cp_r, c->d_Cp_i, c->ldk_c);
+        c->d_Mtop, c->ldtop, 2 * N, N, N, 1.f, c->d_dge[0], c->d_Cp_r, c->d_Cp_i, c->ldk_c);
     return cudaGetLastError();
 }
 

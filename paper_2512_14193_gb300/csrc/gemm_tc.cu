@@ -707,17 +707,23 @@ __global__ void splitk_reduce_z64_kernel(const float* __restrict__ Pr, const flo
 }
 
 // B operand of a skinny product: V (K x nrhs FP32 planar, column-major) -> row c of a [nrhs][ldk] pack and
-// its exponent eB[c].  One CTA per column, which it reads twice (the second time from L2).
+// its exponent eB[c], the entries from `half` on times w (tc_shift).  One CTA per column, which it reads twice
+// (the second time from L2).
 struct PlanarCol {
     const float *re, *im;
-    __device__ __forceinline__ float2 operator()(long k) const { return make_float2(__ldg(re + k), __ldg(im + k)); }
+    int half;
+    float w;
+    __device__ __forceinline__ float2 operator()(long k) const {
+        const float f = k < half ? 1.f : w;
+        return make_float2(__ldg(re + k) * f, __ldg(im + k) * f);
+    }
 };
 __global__ void __launch_bounds__(TC_PACK_THREADS) pack_b_kernel(const float* __restrict__ Vr,
-                                                                 const float* __restrict__ Vi, long ldv, int K,
-                                                                 __half* __restrict__ Br, __half* __restrict__ Bi,
+                                                                 const float* __restrict__ Vi, long ldv, int K, int half,
+                                                                 float w, __half* __restrict__ Br, __half* __restrict__ Bi,
                                                                  long ldk, int* __restrict__ eB) {
     const long c = blockIdx.x;
-    tc_pack_column(PlanarCol{Vr + c * ldv, Vi + c * ldv}, K, Br + c * ldk, Bi + c * ldk, eB + c);
+    tc_pack_column(PlanarCol{Vr + c * ldv, Vi + c * ldv, half, w}, K, Br + c * ldk, Bi + c * ldk, eB + c);
 }
 
 }  // namespace
@@ -794,10 +800,10 @@ cudaError_t gemm_tc_split(cudaStream_t s, const void* tAr, const void* tAi, cons
     return cudaGetLastError();
 }
 
-cudaError_t launch_pack_b(cudaStream_t s, const float* Vr, const float* Vi, long ldv, int K, int nrhs, __half* Br,
-                          __half* Bi, long ldk, int* eB) {
+cudaError_t launch_pack_b(cudaStream_t s, const float* Vr, const float* Vi, long ldv, int K, int half, float w, int nrhs,
+                          __half* Br, __half* Bi, long ldk, int* eB) {
     if (K <= 0 || nrhs <= 0) return cudaSuccess;
-    pack_b_kernel<<<nrhs, TC_PACK_THREADS, 0, s>>>(Vr, Vi, ldv, K, Br, Bi, ldk, eB);
+    pack_b_kernel<<<nrhs, TC_PACK_THREADS, 0, s>>>(Vr, Vi, ldv, K, half, w, Br, Bi, ldk, eB);
     return cudaGetLastError();
 }
 

@@ -37,6 +37,9 @@ struct TcScale {
     const int* eB = nullptr;
     int e0 = 0;
 };
+TcScale schur_scale(const bm_ctx* c);          // of the Schur complement's packs (and the A of the skinny product with them)
+int tc_shift_of(double eps0);                  // power of two moved from the columns of M32 to the rows of M23
+cudaError_t launch_shifted_exponents(cudaStream_t s, const bm_ctx* c);
 constexpr int TC_E_DGE = -16;  // e0 of rows scaled by the digit planes' exponents (entries below 2^(e - 1))
 constexpr int TC_SHIFT_L = 14; // L21 is packed times 2^14 (its entries are below sqrt 2 in modulus)
 // TcGate: the launch skips its first 128 x 128 tile (another launch takes it), and does nothing when the
@@ -64,7 +67,7 @@ int tc_split_k(int m, int n, int K, int num_sms);
 cudaError_t gemm_tc_split(cudaStream_t s, const void* tAr, const void* tAi, const void* tBr, const void* tBi, int m,
                           int n, int K, float alpha, float beta, TcScale sc, TcDest dst, int S, float* Pr, float* Pi,
                           int* d_err, int* launched);
-cudaError_t launch_pack_b(cudaStream_t s, const float* Vr, const float* Vi, long ldv, int K, int nrhs, __half* Br,
+cudaError_t launch_pack_b(cudaStream_t s, const float* Vr, const float* Vi, long ldv, int K, int half, float w, int nrhs, __half* Br,
                           __half* Bi, long ldk, int* eB);
 size_t tc_batch_entry_bytes();
 cudaError_t gemm_tc_batch(cudaStream_t s, int B, const void* const* maps, float* const* Cr, float* const* Ci,

@@ -234,7 +234,7 @@ bm_status factor_batch(Batch& bt, int B) {
             Cr[b] = c->d_F32r;
             Ci[b] = c->d_F32i;
             ld[b] = c->ldF;
-            sc[b] = TcScale{c->d_dge[1], c->d_Bpe, TC_E_DGE};
+            sc[b] = schur_scale(c);
         }
         SSM_CUDA(gemm_tc_batch(bt.s0, B, maps.data(), Cr.data(), Ci.data(), ld.data(), sc.data(), N, N, 2 * N, -1.0f,
                                bt.d_tc, c0->d_err));
