@@ -392,8 +392,6 @@ def roofline_from_profile(prof, N: int, nrhs: int, prec: int, iters: int, peaks:
         "swap_trsm_kernel (block row)": ("hbm", lw["swap_bytes"], hbm, "GB/s",
                                          "row interchanges of the outer panels' 2 NB rows and the U12 blocks, "
                                          "8-byte complex read + written"),
-        "trsv_g_step_kernel": ("hbm", float(iters) * N * N * 8, hbm, "GB/s",
-                               "the FP32 factors (N^2 x 8 bytes) read once per triangular-solve pair"),
         "trsv_flow_kernel": ("hbm", float(iters) * N * N * 8, hbm, "GB/s",
                              "the FP32 factors (N^2 x 8 bytes) read once per triangular-solve pair"),
         "cgemm_tc_kernel (skinny, + split-K reduction)": ("hbm", float(iters) * 4 * N * N * 8, hbm, "GB/s",
