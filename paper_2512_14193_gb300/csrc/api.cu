@@ -132,6 +132,15 @@ void drop_slot(bm_ctx::GraphSlot& g) {
     g.kernels = 0;
 }
 
+// LU without (fast) or with the pivot search.  A captured factorisation holds the one it was captured with, also
+// where buffers and block size do not tell (FP64: the default block size is the search's 64).
+void set_lu_fast(bm_ctx* c, bool fast) {
+    if (c->lu_fast == fast) return;
+    c->lu_fast = fast;
+    drop_slot(c->g_factor);
+    drop_slot(c->g_lu);
+}
+
 // Gives the optional workspace of the FP64 factorisation back (with the graphs that use it).
 void dg_release(bm_ctx* c) {
     drop_slot(c->g_factor);
@@ -595,7 +604,7 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
     c->opt_cluster_cap = cl_cap;
     c->opt_panel_kernel = pkern;
     c->fast_z = prec == BM_FP64 && nb == 0 && pkern == 0 && (cl_cap == 0 || defer_kernels);
-    c->lu_fast = prec == BM_FP64 ? c->fast_z && c->d_fd != nullptr : fast && !c->fast_denied;
+    set_lu_fast(c, prec == BM_FP64 ? c->fast_z && c->d_fd != nullptr : fast && !c->fast_denied);
     c->bs_solve = 64;
     if (!reuse && c->held + p.bytes > c->budget) {
         bm_set_error("admission: system needs " + std::to_string(p.bytes) + " bytes, budget leaves " +
@@ -822,11 +831,7 @@ void dg_reserve(bm_ctx* c) {
     if (c->fast_z && !c->d_fd && c->held + lu_fast_z_bytes() <= c->budget &&
         alloc_t(c, &c->d_fd, lu_fast_z_bytes()) != BM_OK)
         c->d_fd = nullptr;
-    if (c->lu_fast != (c->fast_z && c->d_fd)) {
-        c->lu_fast = !c->lu_fast;
-        drop_slot(c->g_factor);
-        drop_slot(c->g_lu);
-    }
+    set_lu_fast(c, c->fast_z && c->d_fd != nullptr);
     if (c->d_dgw) return;
     const size_t b = dg_request(c->N, c->form, c->lu_fast, c->num_sms);
     if (b == 0 || c->held + b > c->budget) return;
@@ -950,7 +955,7 @@ bm_status factor_result(bm_ctx* c, int* info) {
     int h[5] = {0, 0, 0, 0, 0};
     BM_CUDA_TRY(cudaMemcpyAsync(h, c->d_info, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
     BM_CUDA_TRY(cudaStreamSynchronize(c->stream));
-    if (c->lu_fast && h[1] == 0 && h[4] != 0) {
+    if (h[1] == 0 && h[4] != 0) {  // stopped: whatever enqueued it
         BM_TRY(lu_resume_enqueue(c, h[4]));
         BM_CUDA_TRY(cudaMemcpyAsync(h, c->d_info, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
         BM_CUDA_TRY(cudaStreamSynchronize(c->stream));
