@@ -532,7 +532,7 @@ __global__ void shifted_exponent_kernel(const double2* __restrict__ A, long lda,
     for (int j = j0; j < j1; ++j) {
         const double2 v = A[i + (long)j * lda];
         const int E = (int)(max(mag_bits(v.x), mag_bits(v.y)) >> 52);  // (0: zero or subnormal)
-        if (E > 0) m = max(m, E - 1021 - (j < half ? 0 : shift));
+        if (E > 0) m = max(m, E == 0x7FF ? RT_NONFINITE : E - 1021 - (j < half ? 0 : shift));
     }
     atomicMax(e + i, m);
 }

@@ -148,13 +148,15 @@ bm_status rt_make_map_x(void* tmaps, const void* base, long cols, long K, long l
 // (rowmax: scratch of `rows` words to find the row exponents e with; null: e holds them)
 cudaError_t launch_digits_a(cudaStream_t s, const double2* A, long lda, int rows, int K, int* e, void* D, long ldk,
                             void* rowmax, int nd);
-// |v| as the bits of a non-negative double, which order as the doubles do; NaN counts as zero
+// |v| as the bits of a non-negative double, which order as the doubles do; infinities and NaN are the largest
 __device__ __forceinline__ unsigned long long mag_bits(double v) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
-    return b > 0x7FF0000000000000ull ? 0ull : b;
+    return (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
 }
+// Exponent of a row or column with an infinity or a NaN: its digits are zeros and its outputs NaN
+constexpr int RT_NONFINITE = 1 << 20;
 // e with m < 2^(e - 1) of the largest magnitude m of a row, given as its bits (0 for a zero row)
 __device__ __forceinline__ int row_exponent(unsigned long long mx) {
+    if (mx >= 0x7FF0000000000000ull) return RT_NONFINITE;
     const double m = __longlong_as_double((long long)mx);
     int ex = 0;
     if (m > 0.0) frexp(m, &ex);  // m = f 2^ex, f in [1/2, 1)

@@ -451,7 +451,10 @@ __global__ void __launch_bounds__(RT_THREADS, 1) resid_tc_kernel(const __grid_co
                 for (int j = 0; j < RT_NT; ++j) {
                     if (j >= ncols) break;
                     const int col = col0 + j;
-                    const double v = ldexp((double)sh[j] + (double)sl[j], er + P.fX[col] - 14);
+                    const int fc = P.fX[col];
+                    const double v = er == RT_NONFINITE || fc == RT_NONFINITE
+                                         ? __longlong_as_double(0x7FF8000000000000ll)
+                                         : ldexp((double)sh[j] + (double)sl[j], er + fc - 14);
                     if (P.S == 1) {
                         double* o = reinterpret_cast<double*>(P.C + row + (long)col * P.ldc) + part;
                         *o += J.alpha * v;
@@ -532,8 +535,8 @@ __device__ __forceinline__ unsigned long long digit_word(double v, int ex) {
     const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
     const int E = (int)((bits >> 52) & 0x7FF);
     unsigned long long M = 0;
-    // zero and subnormals (below any row scale used here) give zero digits; so does a value that
-    // does not fit its scale (only possible for non-finite data, which the backward error reports)
+    // zero and subnormals (below any row scale used here) give zero digits; so does a value that does not fit
+    // its scale (only in a row or column with a non-finite entry, whose outputs are NaN: RT_NONFINITE)
     if (E != 0 && E != 0x7FF) {
         const unsigned long long mant = (bits & 0xFFFFFFFFFFFFFull) | (1ull << 52);
         const int sh = E - 1075 + 7 * ND - ex;  // v 2^(7 ND - ex) = mant 2^sh, mant in [2^52, 2^53)
@@ -600,20 +603,18 @@ __global__ void __launch_bounds__(256) digits_a_kernel(const double2* __restrict
 // Column exponents of x over rows [r0, r0 + K) for the n columns (one block per column).
 __global__ void col_exponent_kernel(const double2* __restrict__ X, long ldx, int r0, int K, int* __restrict__ f) {
     const int c = blockIdx.x;
-    double mx = 0.0;
+    unsigned long long mx = 0;
     for (int i = threadIdx.x; i < K; i += blockDim.x) {
         const double2 v = X[r0 + i + (long)c * ldx];
-        mx = fmax(mx, fmax(fabs(v.x), fabs(v.y)));
+        mx = max(mx, max(mag_bits(v.x), mag_bits(v.y)));
     }
-    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    __shared__ double sm[32];
+    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    __shared__ unsigned long long sm[32];
     if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = mx;
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) mx = fmax(mx, sm[w]);
-        int ex = 0;
-        if (mx > 0.0 && isfinite(mx)) frexp(mx, &ex);
-        f[c] = (mx > 0.0 && isfinite(mx)) ? ex + 1 : 0;
+        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) mx = max(mx, sm[w]);
+        f[c] = row_exponent(mx);
     }
 }
 

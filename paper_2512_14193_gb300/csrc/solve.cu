@@ -34,14 +34,15 @@ __device__ __forceinline__ void atomic_max_pos(double* p, double v) {
     atomicMax(reinterpret_cast<unsigned long long*>(p), (unsigned long long)__double_as_longlong(v));
 }
 
-// per column: eta_c = max|R| / (normA max|X| + max|B|); out[0] = max_c eta_c, out[1] = 1 if any
-// non-finite value was seen in B (the input check)
+// per column: eta_c = max|R| / (normA max|X| + max|B|), 1e300 where that or an entry of R or X is not finite
+// (the maxima alone would drop a NaN); out[0] = max_c eta_c, out[1] = 1 if any non-finite value was seen in B
+// (the input check)
 __global__ void eta_kernel(const double2* __restrict__ R, const double2* __restrict__ X,
                            const double2* __restrict__ B, long ld, int nsys, const double* __restrict__ normA,
                            double* out) {
     int c = blockIdx.x;
     double r = 0, x = 0, b = 0;
-    bool bad = false;
+    bool bad = false, lost = false;
     // magnitudes in FP32 (the ratio needs a few digits; FP64 hypot would cost the FP64 pipe)
     float rf = 0.f, xf = 0.f, bf = 0.f;
 #pragma unroll 4
@@ -50,6 +51,7 @@ __global__ void eta_kernel(const double2* __restrict__ R, const double2* __restr
         double2 bv = B[o];
         if (!isfinite(bv.x) || !isfinite(bv.y)) bad = true;
         double2 rv = R[o], xv = X[o];
+        if (!isfinite(rv.x) || !isfinite(rv.y) || !isfinite(xv.x) || !isfinite(xv.y)) lost = true;
         rf = fmaxf(rf, hypotf((float)rv.x, (float)rv.y));
         xf = fmaxf(xf, hypotf((float)xv.x, (float)xv.y));
         bf = fmaxf(bf, hypotf((float)bv.x, (float)bv.y));
@@ -58,10 +60,11 @@ __global__ void eta_kernel(const double2* __restrict__ R, const double2* __restr
     x = xf;
     b = bf;
     __shared__ double sr[32], sx[32], sb[32];
-    __shared__ int sbad;
-    if (threadIdx.x == 0) sbad = 0;
+    __shared__ int sbad, slost;
+    if (threadIdx.x == 0) sbad = slost = 0;
     __syncthreads();
     if (bad) sbad = 1;
+    if (lost) slost = 1;
     for (int o = 16; o > 0; o >>= 1) {
         r = fmax(r, __shfl_xor_sync(0xffffffffu, r, o));
         x = fmax(x, __shfl_xor_sync(0xffffffffu, x, o));
@@ -86,7 +89,7 @@ __global__ void eta_kernel(const double2* __restrict__ R, const double2* __restr
         b = fmax(b, sb[0]);
         double den = (*normA) * x + b;
         double eta = (den > 0) ? r / den : (r > 0 ? 1.0 : 0.0);
-        if (!isfinite(eta)) eta = 1e300;
+        if (slost || !isfinite(eta)) eta = 1e300;
         atomic_max_pos(out, eta);
         if (sbad) out[1] = 1.0;
     }
