@@ -228,6 +228,7 @@ void free_problem(bm_ctx* c) {
     FREE(c->d_Bp_i);
     FREE(c->d_Bpe);
     FREE(c->d_Ape);
+    FREE(c->d_bal);
     FREE(c->d_Lp_r);
     FREE(c->d_Lp_i);
     FREE(c->d_Up_r);
@@ -286,7 +287,7 @@ Plan make_plan(int N, int form, int prec, int nb_user, int bs, int nd, bool fast
         b += (form == BM_MIXED) ? (size_t)p.ldtop * N * pb + (size_t)p.ldbot * 2 * N * pb : (size_t)p.ldA * 2 * N * pb;
         if (form == BM_MIXED) {
             p.ldk_schur = tc_ldk(2L * N);
-            b += 2 * (size_t)N * p.ldk_schur * 4 + 2 * (size_t)N * 4;
+            b += 2 * (size_t)N * p.ldk_schur * 4 + (size_t)N * 4;
             // [M13; M23] rows for the skinny products of the solve
             p.ldk_c = tc_ldk(N);
             b += 2 * (size_t)N * p.ldk_c * 4;
@@ -302,6 +303,7 @@ Plan make_plan(int N, int form, int prec, int nb_user, int bs, int nd, bool fast
         else
             b += planes * 2L * N * rt_ldk(2L * N) + 2L * N * 4;
     }
+    if (form == BM_MIXED) b += (size_t)N * 4 + bal_ints(N) * 4;  // the balance of the Schur product
     p.nblk = ceil_div(p.n, bs);
     b += 2 * (size_t)p.n * 4;
     b += 2 * (size_t)p.nblk * bs * bs * (c32 ? 8 : 16);
@@ -596,10 +598,7 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
     }
     if (c->fast_denied) p = make_plan(N, form, prec, nb, 64, nd, false, planes);
     // the captured factorisation depends on the launch settings: capture again when they change
-    const int shift = form == BM_MIXED && prec != BM_FP64 ? tc_shift_of(eps0) : 0;
-    if (reuse && (eager != c->eager || cl_cap != c->opt_cluster_cap || pkern != c->opt_panel_kernel || shift != c->tc_shift))
-        drop_graphs(c);
-    c->tc_shift = shift;
+    if (reuse && (eager != c->eager || cl_cap != c->opt_cluster_cap || pkern != c->opt_panel_kernel)) drop_graphs(c);
     c->eager = eager;
     c->opt_cluster_cap = cl_cap;
     c->opt_panel_kernel = pkern;
@@ -643,6 +642,8 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
     if (s == BM_OK && form == BM_MIXED) {
         s = alloc_t(c, &c->d_Mtop, (size_t)p.ldtop * N * 16);
         if (s == BM_OK) s = alloc_t(c, &c->d_Mbot, (size_t)p.ldbot * 2 * N * 16);
+        if (s == BM_OK) s = alloc_t(c, &c->d_Ape, (size_t)N * 4);
+        if (s == BM_OK) s = alloc_t(c, &c->d_bal, bal_ints(N) * 4);
     } else if (s == BM_OK) {
         s = alloc_t(c, &c->d_A, (size_t)p.ldA * 2 * N * 16);
     }
@@ -668,7 +669,6 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
             if (s == BM_OK) s = alloc_t(c, &c->d_Bp_r, pb);
             if (s == BM_OK) s = alloc_t(c, &c->d_Bp_i, pb);
             if (s == BM_OK) s = alloc_t(c, &c->d_Bpe, (size_t)N * 4);
-            if (s == BM_OK) s = alloc_t(c, &c->d_Ape, (size_t)N * 4);
             size_t cb = (size_t)2 * N * p.ldk_c * 2;
             if (s == BM_OK) s = alloc_t(c, &c->d_Cp_r, cb);
             if (s == BM_OK) s = alloc_t(c, &c->d_Cp_i, cb);
@@ -760,7 +760,7 @@ bm_status assemble_post(bm_ctx* c, bool run_assembly_kernel, bool wait) {
     }
     BM_CUDA_TRY(launch_zeta_band(st, c));
     BM_CUDA_TRY(launch_normA(st, c));
-    c->launches += ((form == BM_MIXED) ? 2 : 1) + (c->zeta_p > 0 ? 1 : 0);
+    c->launches += ((form == BM_MIXED) ? 3 : 1) + (c->zeta_p > 0 ? 1 : 0);
     if (c32) {
         if (form == BM_MIXED) {
             if (c->planes) {
@@ -779,8 +779,7 @@ bm_status assemble_post(bm_ctx* c, bool run_assembly_kernel, bool wait) {
             BM_CUDA_TRY(launch_digits_a(st, c->d_Mbot, c->ldbot, N, 2 * N, c->d_dge[1], c->d_dg[1], c->dg_ldk[1], nullptr,
                                         nd));
             BM_CUDA_TRY(launch_pack_solve(st, c));
-            BM_CUDA_TRY(launch_shifted_exponents(st, c));
-            c->launches += 3 + (c->tc_shift != 0);
+            c->launches += 3;
         } else {
             BM_CUDA_TRY(launch_digits_a(st, c->d_A, c->ldA, 2 * N, 2 * N, c->d_dge[0], c->d_dg[0], c->dg_ldk[0], nullptr,
                                         nd));
@@ -849,7 +848,8 @@ bm_status schur_z64(bm_ctx* c, cudaStream_t s) {
     }
     BM_PROF(c, "resid_tc_kernel (Schur complement)");
     BM_CUDA_TRY(cudaMemset2DAsync(F.p, (size_t)F.ld * 16, 0, (size_t)N * 16, N, s));
-    return gemm_z64_dg(s, c->d_dgw, c->num_sms, N, N, 2 * N, -1.0, A, B, F, c->d_err);
+    return gemm_z64_dg(s, c->d_dgw, c->num_sms, N, N, 2 * N, -1.0, A, B, F, c->d_err, c->d_Ape,
+                       RtShift{c->d_bal + BAL_SHIFT, N});
 }
 
 // ------------------------------------------------------------------------------------------------

@@ -278,17 +278,30 @@ __device__ __forceinline__ void atomic_max_pos(double* p, double v) {
 // its 8 warps taking every 8th column, eight loads in flight per thread.  The moduli are formed in
 // FP32 from the entries rounded to FP32 (by integer operations: the FP64 pipe is narrow) and each
 // thread sums its columns in FP32, the eight warps' sums added in FP64: a relative error of a few
-// 1e-6 at most, ample for a norm that only scales the backward error.  With e, the same pass finds the row
-// exponents of the digit planes (integer maxima of the magnitudes' bits; a pass of its own took 0.19 ms at
-// N = 4096).
+// 1e-6 at most, ample for a norm that only scales the backward error.  The same pass finds exponents (integer
+// maxima of the magnitudes' bits; a pass of its own took 0.19 ms at N = 4096).
+struct RowExps {
+    int* e = nullptr;    // of the rows (digit planes)
+    int* he = nullptr;   // of the rows' columns before `half` and from it on, m each
+    int* g = nullptr;    // largest of he's two parts, or (he null) of the rows before `half` and from it on
+    int half = 0;
+};
 __global__ void __launch_bounds__(256) rownorm_kernel(const double2* __restrict__ A, long ld, int m, int ncols,
-                                                      double add, double* out, int* __restrict__ e) {
+                                                      double add, double* out, RowExps x) {
     __shared__ double part[8][32];
-    __shared__ unsigned long long top[8][32];
+    __shared__ unsigned long long top[2][8][32];
+    const int chalf = x.he != nullptr ? x.half : ncols;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i = blockIdx.x * 32 + lane;
     float sf = 0.f;
-    unsigned long long mx = 0;
+    unsigned long long mx[2] = {0, 0};
+    auto take = [&](double2 v, int j) {
+        const float p = f32_rn(v.x), q = f32_rn(v.y);
+        sf += sqrtf(fmaf(p, p, q * q));
+        const unsigned long long b = max(mag_bits(v.x), mag_bits(v.y));
+        if (j < chalf) mx[0] = max(mx[0], b);
+        else mx[1] = max(mx[1], b);
+    };
     if (i < m) {
         const double2* a = A + i;
         int j = warp;
@@ -297,18 +310,9 @@ __global__ void __launch_bounds__(256) rownorm_kernel(const double2* __restrict_
 #pragma unroll
             for (int u = 0; u < 8; ++u) v[u] = a[(long)(j + 8 * u) * ld];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const float x = f32_rn(v[u].x), y = f32_rn(v[u].y);
-                sf += sqrtf(fmaf(x, x, y * y));
-                mx = max(mx, max(mag_bits(v[u].x), mag_bits(v[u].y)));
-            }
+            for (int u = 0; u < 8; ++u) take(v[u], j + 8 * u);
         }
-        for (; j < ncols; j += 8) {
-            const double2 v = a[(long)j * ld];
-            const float x = f32_rn(v.x), y = f32_rn(v.y);
-            sf += sqrtf(fmaf(x, x, y * y));
-            mx = max(mx, max(mag_bits(v.x), mag_bits(v.y)));
-        }
+        for (; j < ncols; j += 8) take(a[(long)j * ld], j);
     }
     // FP32 overflow (entries above ~1e19) falls back to the FP64 modulus for this thread's row
     double s = (double)sf;
@@ -320,12 +324,32 @@ __global__ void __launch_bounds__(256) rownorm_kernel(const double2* __restrict_
         }
     }
     part[warp][lane] = s;
-    top[warp][lane] = mx;
+    top[0][warp][lane] = mx[0];
+    top[1][warp][lane] = mx[1];
     __syncthreads();
-    if (warp == 1 && e != nullptr && i < m) {
+    if (warp == 1) {
+        int h[2];
 #pragma unroll
-        for (int w = 0; w < 8; ++w) mx = max(mx, top[w][lane]);
-        e[i] = row_exponent(mx);
+        for (int q = 0; q < 2; ++q) {
+#pragma unroll
+            for (int w = 0; w < 8; ++w) mx[q] = max(mx[q], top[q][w][lane]);
+            h[q] = row_exponent(mx[q], -RT_NONFINITE);  // (no rows past m: zeros)
+        }
+        if (i < m && x.e != nullptr) x.e[i] = row_exponent(max(mx[0], mx[1]));
+        if (i < m && x.he != nullptr) {
+            x.he[i] = h[0];
+            x.he[m + i] = h[1];
+        }
+        if (x.g != nullptr && x.he == nullptr && i >= x.half) {
+            h[1] = h[0];
+            h[0] = -RT_NONFINITE;
+        }
+        if (x.g != nullptr)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int g = __reduce_max_sync(0xffffffffu, h[q]);
+                if (lane == 0) atomicMax(x.g + q, g);
+            }
     }
     if (warp == 0) {
         double t = 0.0;
@@ -485,13 +509,14 @@ __global__ void hankel_probe_kernel(const double2* __restrict__ z, int n, Hankel
     h1[i] = b;
 }
 
-// A operands: rows of an FP64 column-major block (rows x K), the columns from `half` on times w (tc_shift), as
+// A operands: rows of an FP64 column-major block (rows x K), the columns from `half` on times 2^-*shift, as
 // pack rows scaled by row exponents e (entries below 2^(e - 1); TC_E_DGE).  One 32 x 32 tile per CTA through shared memory, so that
 // both sides are coalesced; a warp writes the 128 bytes of a row.
 __global__ void pack_rowmajor_kernel(const double2* __restrict__ M, long ldm, int rows, int K,
-                                     int half, float w, const int* __restrict__ e, __half* __restrict__ Pr,
-                                     __half* __restrict__ Pi, long ldk) {
+                                     int half, const int* __restrict__ shift, const int* __restrict__ e,
+                                     __half* __restrict__ Pr, __half* __restrict__ Pi, long ldk) {
     __shared__ float2 t[32][33];
+    const float w = shift != nullptr ? tc_pow2(-*shift) : 1.f;
     const int k0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
     const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
 #pragma unroll
@@ -520,25 +545,29 @@ __global__ void pack_rowmajor_kernel(const double2* __restrict__ M, long ldm, in
     }
 }
 
-// Row exponents of [M31 M32] with the columns from `half` on times 2^-shift (eps0 not near 1: tc_shift), as the
-// digit planes have them: entries below 2^(e - 1).  e starts below every exponent.
-__global__ void shifted_exponent_kernel(const double2* __restrict__ A, long lda, int rows, int K, int half, int shift,
-                                        int* __restrict__ e) {
+// Balance of the Schur product [M31 M32] [M13; M23], for one scale per row of [M31 M32] and per column of
+// [M13; M23].  The blocks' sizes differ: M13 and M32 carry a length (of the curve) against M23 and M31, M32 a factor
+// eps0 and M23 one of 1 / eps1, and M31 has the hypersingular diagonal (about 1 / h).  With s = 0 the
+// smaller block of a row or column would lose what it is smaller by (a curve of diameter 2e-3 in FP64: solution
+// errors 1e-15 -> 1e-12; 2e-9 in CF32: no convergence).  The error of scaled entries goes with
+// max(|M31|, |M32| 2^-s) max(|M13|, |M23| 2^s), least, and no larger than the larger of |M31| |M13| and
+// |M32| |M23|, for 4^s = |M32| |M13| / (|M31| |M23|).  Also the row exponents for that s (those of
+// rownorm_kernel's pass for both blocks).
+__global__ void balance_kernel(int N, int* __restrict__ bal, int* __restrict__ e) {
+    const int g13 = bal[BAL_G], g23 = bal[BAL_G + 1], g31 = bal[BAL_G + 2], g32 = bal[BAL_G + 3];
+    const int lo = min(min(g13, g23), min(g31, g32)), hi = max(max(g13, g23), max(g31, g32));
+    int s = 0;
+    if (lo > -RT_NONFINITE && hi < RT_NONFINITE) s = min(max((g32 + g13 - g31 - g23) >> 1, -120), 120);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= rows) return;
-    const int j0 = blockIdx.y * 256, j1 = min(K, j0 + 256);
-    int m = -(1 << 30);
-#pragma unroll 8
-    for (int j = j0; j < j1; ++j) {
-        const double2 v = A[i + (long)j * lda];
-        const int E = (int)(max(mag_bits(v.x), mag_bits(v.y)) >> 52);  // (0: zero or subnormal)
-        if (E > 0) m = max(m, E == 0x7FF ? RT_NONFINITE : E - 1021 - (j < half ? 0 : shift));
-    }
-    atomicMax(e + i, m);
+    if (i == 0) bal[BAL_SHIFT] = s;
+    if (i >= N) return;
+    const int a = bal[BAL_ROWS + i], b = bal[BAL_ROWS + N + i];
+    const int m = max(a, b - s);
+    e[i] = max(a, b) == RT_NONFINITE ? RT_NONFINITE : (max(a, b) == -RT_NONFINITE ? 0 : m);
 }
 
 // B operand of the Schur product: column n of an FP64 block as pack row n, one CTA per column; the rows from
-// `half` on times w (tc_shift).
+// `half` on times 2^*shift.
 struct ColZ64 {
     const double2* p;
     int half;
@@ -550,11 +579,12 @@ struct ColZ64 {
     }
 };
 __global__ void __launch_bounds__(TC_PACK_THREADS) pack_colmajor_kernel(const double2* __restrict__ M, long ldm, int K,
-                                                                        int half, float w, __half* __restrict__ Pr,
+                                                                        int half, const int* __restrict__ shift,
+                                                                        __half* __restrict__ Pr,
                                                                         __half* __restrict__ Pi, long ldk,
                                                                         int* __restrict__ e) {
     const long n = blockIdx.x;
-    tc_pack_column(ColZ64{M + n * ldm, half, w}, K, Pr + n * ldk, Pi + n * ldk, e + n);
+    tc_pack_column(ColZ64{M + n * ldm, half, tc_pow2(*shift)}, K, Pr + n * ldk, Pi + n * ldk, e + n);
 }
 
 __global__ void to_c32_kernel(const double2* __restrict__ A, long lda, int m, int n, float* Fr, float* Fi, long ldf) {
@@ -894,14 +924,19 @@ cudaError_t launch_normA(cudaStream_t s, const bm_ctx* c) {
     cudaError_t e = cudaMemsetAsync(c->d_normA, 0, sizeof(double), s);
     if (e != cudaSuccess) return e;
     // (the CF32 precisions' digit planes are scaled by row exponents, found on the way; d_dge is null in FP64)
+    const int N = c->N;
     if (c->form == BM_MIXED) {
-        rownorm_kernel<<<ceil_div(2 * c->N, 32), 256, 0, s>>>(c->d_Mtop, c->ldtop, 2 * c->N, c->N, 1.0, c->d_normA,
-                                                                  c->d_dge[0]);
-        rownorm_kernel<<<ceil_div(c->N, 32), 256, 0, s>>>(c->d_Mbot, c->ldbot, c->N, 2 * c->N, 0.0, c->d_normA,
-                                                              c->d_dge[1]);
+        e = cudaMemsetAsync(c->d_bal, 0x80, BAL_SHIFT * sizeof(int), s);  // below every exponent
+        if (e != cudaSuccess) return e;
+        rownorm_kernel<<<ceil_div(2 * N, 32), 256, 0, s>>>(c->d_Mtop, c->ldtop, 2 * N, N, 1.0, c->d_normA,
+                                                           RowExps{c->d_dge[0], nullptr, c->d_bal + BAL_G, N});
+        rownorm_kernel<<<ceil_div(N, 32), 256, 0, s>>>(
+            c->d_Mbot, c->ldbot, N, 2 * N, 0.0, c->d_normA,
+            RowExps{c->d_dge[1], c->d_bal + BAL_ROWS, c->d_bal + BAL_G + 2, N});
+        balance_kernel<<<ceil_div(N, 256), 256, 0, s>>>(N, c->d_bal, c->d_Ape);
     } else {
-        rownorm_kernel<<<ceil_div(2 * c->N, 32), 256, 0, s>>>(c->d_A, c->ldA, 2 * c->N, 2 * c->N, 0.0, c->d_normA,
-                                                                  c->d_dge[0]);
+        rownorm_kernel<<<ceil_div(2 * N, 32), 256, 0, s>>>(c->d_A, c->ldA, 2 * N, 2 * N, 0.0, c->d_normA,
+                                                           RowExps{c->d_dge[0]});
     }
     return cudaGetLastError();
 }
@@ -964,29 +999,14 @@ cudaError_t launch_hankel_probe(cudaStream_t s, const bm_ctx* c, const double2* 
 
 // Operands of the Schur-complement product (part of the factorisation, like the FP32 copy of the
 // ordinary matrix): A = [M31 M32] row-major, B = [M13; M23] column by column.
-// The columns of M32 carry a factor eps0 and the rows of M23 one of 1 / eps1: with a single scale per row and
-// column of the packs, M31 would lose what eps0 exceeds 1 by.  A power of two near eps0 (tc_shift) is moved from
-// the one to the other, and the rows of [M31 M32] get exponents of their own then (d_Ape).
-int tc_shift_of(double eps0) {
-    return eps0 != 0.0 && std::isfinite(eps0) ? std::min(std::max(std::ilogb(eps0), -126), 126) : 0;
-}
-TcScale schur_scale(const bm_ctx* c) { return TcScale{c->tc_shift ? c->d_Ape : c->d_dge[1], c->d_Bpe, TC_E_DGE}; }
-cudaError_t launch_shifted_exponents(cudaStream_t s, const bm_ctx* c) {
-    const int N = c->N;
-    if (c->tc_shift == 0) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(c->d_Ape, 0x80, (size_t)N * sizeof(int), s);
-    if (e != cudaSuccess) return e;
-    shifted_exponent_kernel<<<dim3(ceil_div(N, 128), ceil_div(2 * N, 256)), 128, 0, s>>>(c->d_Mbot, c->ldbot, N, 2 * N, N,
-                                                                                        c->tc_shift, c->d_Ape);
-    return cudaGetLastError();
-}
+TcScale schur_scale(const bm_ctx* c) { return TcScale{c->d_Ape, c->d_Bpe, TC_E_DGE}; }
 
 cudaError_t launch_pack_schur(cudaStream_t s, const bm_ctx* c) {
     const int N = c->N, K = 2 * N;
     pack_rowmajor_kernel<<<dim3(ceil_div(K, 32), ceil_div(N, 32)), dim3(32, 8), 0, s>>>(
-        c->d_Mbot, c->ldbot, N, K, N, ldexpf(1.f, -c->tc_shift), schur_scale(c).eA, c->d_Ap_r, c->d_Ap_i, c->ldk_schur);
-    pack_colmajor_kernel<<<N, TC_PACK_THREADS, 0, s>>>(c->d_Mtop, c->ldtop, K, N, ldexpf(1.f, c->tc_shift), c->d_Bp_r, c->d_Bp_i, c->ldk_schur,
-                                                       c->d_Bpe);
+        c->d_Mbot, c->ldbot, N, K, N, c->d_bal + BAL_SHIFT, c->d_Ape, c->d_Ap_r, c->d_Ap_i, c->ldk_schur);
+    pack_colmajor_kernel<<<N, TC_PACK_THREADS, 0, s>>>(c->d_Mtop, c->ldtop, K, N, c->d_bal + BAL_SHIFT, c->d_Bp_r,
+                                                       c->d_Bp_i, c->ldk_schur, c->d_Bpe);
     return cudaGetLastError();
 }
 
@@ -995,7 +1015,7 @@ cudaError_t launch_pack_schur(cudaStream_t s, const bm_ctx* c) {
 cudaError_t launch_pack_solve(cudaStream_t s, const bm_ctx* c) {
     const int N = c->N;
     pack_rowmajor_kernel<<<dim3(ceil_div(N, 32), ceil_div(2 * N, 32)), dim3(32, 8), 0, s>>>(
-        c->d_Mtop, c->ldtop, 2 * N, N, N, 1.f, c->d_dge[0], c->d_Cp_r, c->d_Cp_i, c->ldk_c);
+        c->d_Mtop, c->ldtop, 2 * N, N, N, nullptr, c->d_dge[0], c->d_Cp_r, c->d_Cp_i, c->ldk_c);
     return cudaGetLastError();
 }
 

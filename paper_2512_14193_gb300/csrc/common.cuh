@@ -321,8 +321,8 @@ struct bm_ctx {
     __half* d_Bp_r = nullptr;  // Schur B operand [M13; M23]^T rows (N rows, K = 2N; exponents d_Bpe)
     __half* d_Bp_i = nullptr;
     int* d_Bpe = nullptr;
-    int* d_Ape = nullptr;      // exponents of A where tc_shift != 0 (a power of two moved from M32 to M23)
-    int tc_shift = 0;
+    int* d_Ape = nullptr;      // exponents of A (balance_kernel)
+    int* d_bal = nullptr;      // mixed: the balance of the Schur product (BAL_* in kernels.cuh)
     long ldk_schur = 0;
     __half* d_Lp_r = nullptr;  // LU trailing-update packs (L21 times 2^TC_SHIFT_L; exponents d_Upe of U12)
     __half* d_Lp_i = nullptr;

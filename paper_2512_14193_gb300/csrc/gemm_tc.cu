@@ -707,7 +707,7 @@ __global__ void splitk_reduce_z64_kernel(const float* __restrict__ Pr, const flo
 }
 
 // B operand of a skinny product: V (K x nrhs FP32 planar, column-major) -> row c of a [nrhs][ldk] pack and
-// its exponent eB[c], the entries from `half` on times w (tc_shift).  One CTA per column, which it reads twice
+// its exponent eB[c], the entries from `half` on times 2^*shift (balance_kernel).  One CTA per column, which it reads twice
 // (the second time from L2).
 struct PlanarCol {
     const float *re, *im;
@@ -720,9 +720,10 @@ struct PlanarCol {
 };
 __global__ void __launch_bounds__(TC_PACK_THREADS) pack_b_kernel(const float* __restrict__ Vr,
                                                                  const float* __restrict__ Vi, long ldv, int K, int half,
-                                                                 float w, __half* __restrict__ Br, __half* __restrict__ Bi,
+                                                                 const int* __restrict__ shift, __half* __restrict__ Br, __half* __restrict__ Bi,
                                                                  long ldk, int* __restrict__ eB) {
     const long c = blockIdx.x;
+    const float w = shift != nullptr ? tc_pow2(*shift) : 1.f;
     tc_pack_column(PlanarCol{Vr + c * ldv, Vi + c * ldv, half, w}, K, Br + c * ldk, Bi + c * ldk, eB + c);
 }
 
@@ -800,10 +801,10 @@ cudaError_t gemm_tc_split(cudaStream_t s, const void* tAr, const void* tAi, cons
     return cudaGetLastError();
 }
 
-cudaError_t launch_pack_b(cudaStream_t s, const float* Vr, const float* Vi, long ldv, int K, int half, float w, int nrhs,
-                          __half* Br, __half* Bi, long ldk, int* eB) {
+cudaError_t launch_pack_b(cudaStream_t s, const float* Vr, const float* Vi, long ldv, int K, int half,
+                          const int* shift, int nrhs, __half* Br, __half* Bi, long ldk, int* eB) {
     if (K <= 0 || nrhs <= 0) return cudaSuccess;
-    pack_b_kernel<<<nrhs, TC_PACK_THREADS, 0, s>>>(Vr, Vi, ldv, K, half, w, Br, Bi, ldk, eB);
+    pack_b_kernel<<<nrhs, TC_PACK_THREADS, 0, s>>>(Vr, Vi, ldv, K, half, shift, Br, Bi, ldk, eB);
     return cudaGetLastError();
 }
 

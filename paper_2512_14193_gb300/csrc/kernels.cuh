@@ -38,8 +38,12 @@ struct TcScale {
     int e0 = 0;
 };
 TcScale schur_scale(const bm_ctx* c);          // of the Schur complement's packs (and the A of the skinny product with them)
-int tc_shift_of(double eps0);                  // power of two moved from the columns of M32 to the rows of M23
-cudaError_t launch_shifted_exponents(cudaStream_t s, const bm_ctx* c);
+// Balance of the product [M31 M32] [M13; M23]: 2^s moved from the columns of M32 to the rows of M23, so that one
+// scale per row of the one and per column of the other loses neither block (balance_kernel).
+constexpr int BAL_G = 0;      // exponents of the largest entries of M13, M23, M31, M32
+constexpr int BAL_SHIFT = 4;  // s
+constexpr int BAL_ROWS = 8;   // exponents of the rows of M31, then of M32
+constexpr size_t bal_ints(long N) { return BAL_ROWS + 2 * (size_t)N; }
 constexpr int TC_E_DGE = -16;  // e0 of rows scaled by the digit planes' exponents (entries below 2^(e - 1))
 constexpr int TC_SHIFT_L = 14; // L21 is packed times 2^14 (its entries are below sqrt 2 in modulus)
 // TcGate: the launch skips its first 128 x 128 tile (another launch takes it), and does nothing when the
@@ -67,8 +71,8 @@ int tc_split_k(int m, int n, int K, int num_sms);
 cudaError_t gemm_tc_split(cudaStream_t s, const void* tAr, const void* tAi, const void* tBr, const void* tBi, int m,
                           int n, int K, float alpha, float beta, TcScale sc, TcDest dst, int S, float* Pr, float* Pi,
                           int* d_err, int* launched);
-cudaError_t launch_pack_b(cudaStream_t s, const float* Vr, const float* Vi, long ldv, int K, int half, float w, int nrhs, __half* Br,
-                          __half* Bi, long ldk, int* eB);
+cudaError_t launch_pack_b(cudaStream_t s, const float* Vr, const float* Vi, long ldv, int K, int half, const int* shift,
+                          int nrhs, __half* Br, __half* Bi, long ldk, int* eB);
 size_t tc_batch_entry_bytes();
 cudaError_t gemm_tc_batch(cudaStream_t s, int B, const void* const* maps, float* const* Cr, float* const* Ci,
                           const long* ldc, const TcScale* sc, int m, int n, int K, float alpha, void* d_entries,
@@ -145,33 +149,39 @@ void rt_plan_splits(int nprod, const long* m, const long* K, int n, int nd, int 
 bm_status rt_make_map(void* tmap, const void* base, long rows, long K, long ldk, long plane_elems, int box_rows,
                       int nd);
 bm_status rt_make_map_x(void* tmaps, const void* base, long cols, long K, long ldk, int nd);  // two blobs
+// K entries from `half` on are taken times 2^-s (A) or 2^s (x), s = *shift
+struct RtShift {
+    const int* shift = nullptr;
+    int half = 0;
+    __device__ __forceinline__ int at(int k) const { return shift != nullptr && k >= half ? __ldg(shift) : 0; }
+};
 // (rowmax: scratch of `rows` words to find the row exponents e with; null: e holds them)
 cudaError_t launch_digits_a(cudaStream_t s, const double2* A, long lda, int rows, int K, int* e, void* D, long ldk,
-                            void* rowmax, int nd);
+                            void* rowmax, int nd, RtShift sh = RtShift{});
 // |v| as the bits of a non-negative double, which order as the doubles do; infinities and NaN are the largest
 __device__ __forceinline__ unsigned long long mag_bits(double v) {
     return (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
 }
 // Exponent of a row or column with an infinity or a NaN: its digits are zeros and its outputs NaN
 constexpr int RT_NONFINITE = 1 << 20;
-// e with m < 2^(e - 1) of the largest magnitude m of a row, given as its bits (0 for a zero row)
-__device__ __forceinline__ int row_exponent(unsigned long long mx) {
+// e with m < 2^(e - 1) of the largest magnitude m of a row, given as its bits (`zero` for a zero row)
+__device__ __forceinline__ int row_exponent(unsigned long long mx, int zero = 0) {
     if (mx >= 0x7FF0000000000000ull) return RT_NONFINITE;
     const double m = __longlong_as_double((long long)mx);
     int ex = 0;
     if (m > 0.0) frexp(m, &ex);  // m = f 2^ex, f in [1/2, 1)
-    return m > 0.0 ? ex + 1 : 0;
+    return m > 0.0 ? ex + 1 : zero;
 }
 cudaError_t launch_digits_x(cudaStream_t s, const double2* X, long ldx, int r0, int K, int n, int npad, int* f,
-                            void* D, long ldk, long plane, int nd);
+                            void* D, long ldk, long plane, int nd, RtShift sh = RtShift{});
 cudaError_t gemm_rt(cudaStream_t s, const RtArgs* prods, int nprod, int n, double alpha, int* d_err, int* launched,
                     int nd);
 
 // FP64 products from nine-digit products (FP64 precision): workspace (0: the CUDA cores are the better
-// place), and C += alpha A B
+// place), and C += alpha A B (eA, sh: A's row exponents and the balance of the K entries, if they are there)
 size_t dg_bytes(int m, int n, int K, int num_sms);
 bm_status gemm_z64_dg(cudaStream_t s, void* work, int num_sms, int m, int n, int K, double alpha, Z64 A, Z64 B, Z64 C,
-                      int* d_err);
+                      int* d_err, int* eA = nullptr, RtShift sh = RtShift{});
 
 // api.cu: what an FP64 factorisation takes where the budget has room (before any capture); the Schur
 // complement of the FP64 precision into d_F64

@@ -570,7 +570,7 @@ __device__ __forceinline__ unsigned bf16_pair(float a, float b) {
 template <int ND>
 __global__ void __launch_bounds__(256) digits_a_kernel(const double2* __restrict__ A, long lda, int rows, int K,
                                                        const int* __restrict__ e, unsigned* __restrict__ D, long ldk,
-                                                       long plane) {
+                                                       long plane, RtShift sh) {
     __shared__ double2 t[32][65];
     const int k0 = blockIdx.x * 64, r0 = blockIdx.y * 32;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -582,6 +582,7 @@ __global__ void __launch_bounds__(256) digits_a_kernel(const double2* __restrict
     __syncthreads();
     const int k = k0 + 2 * tx;
     if (k >= K) return;
+    const int sa = sh.at(k), sb = sh.at(k + 1);
 #pragma unroll 1
     for (int q = ty; q < 32; q += 8) {
         const int r = r0 + q;
@@ -591,7 +592,8 @@ __global__ void __launch_bounds__(256) digits_a_kernel(const double2* __restrict
         unsigned* o = D + ((long)r * ldk + k) / 2;
 #pragma unroll
         for (int part = 0; part < 2; ++part) {
-            const unsigned long long wa = digit_word<ND>(part ? a.y : a.x, ex), wb = digit_word<ND>(part ? b.y : b.x, ex);
+            const unsigned long long wa = digit_word<ND>(part ? a.y : a.x, ex + sa),
+                                     wb = digit_word<ND>(part ? b.y : b.x, ex + sb);
 #pragma unroll
             for (int d = 0; d < ND; ++d)
                 o[(2 * d + part) * (plane / 2)] =
@@ -601,20 +603,32 @@ __global__ void __launch_bounds__(256) digits_a_kernel(const double2* __restrict
 }
 
 // Column exponents of x over rows [r0, r0 + K) for the n columns (one block per column).
-__global__ void col_exponent_kernel(const double2* __restrict__ X, long ldx, int r0, int K, int* __restrict__ f) {
-    const int c = blockIdx.x;
-    unsigned long long mx = 0;
+__global__ void col_exponent_kernel(const double2* __restrict__ X, long ldx, int r0, int K, int* __restrict__ f,
+                                    RtShift sh) {
+    const int c = blockIdx.x, half = sh.shift != nullptr ? sh.half : K;
+    unsigned long long mx[2] = {0, 0};  // of the entries before `half` and from it on
     for (int i = threadIdx.x; i < K; i += blockDim.x) {
         const double2 v = X[r0 + i + (long)c * ldx];
-        mx = max(mx, max(mag_bits(v.x), mag_bits(v.y)));
+        const unsigned long long b = max(mag_bits(v.x), mag_bits(v.y));
+        if (i < half) mx[0] = max(mx[0], b);
+        else mx[1] = max(mx[1], b);
     }
-    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    __shared__ unsigned long long sm[32];
-    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = mx;
+    __shared__ unsigned long long sm[2][32];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        for (int o = 16; o > 0; o >>= 1) mx[q] = max(mx[q], __shfl_xor_sync(0xffffffffu, mx[q], o));
+        if ((threadIdx.x & 31) == 0) sm[q][threadIdx.x >> 5] = mx[q];
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) mx = max(mx, sm[w]);
-        f[c] = row_exponent(mx);
+        for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
+            for (int q = 0; q < 2; ++q) mx[q] = max(mx[q], sm[q][w]);
+        int e = row_exponent(mx[0]);
+        if (mx[1] > 0) {
+            const int e1 = row_exponent(mx[1]), e2 = e1 == RT_NONFINITE ? e1 : e1 + sh.at(half);
+            e = mx[0] > 0 ? max(e, e2) : e2;
+        }
+        f[c] = e;
     }
 }
 
@@ -622,7 +636,8 @@ __global__ void col_exponent_kernel(const double2* __restrict__ X, long ldx, int
 // plane 2 d + part, or (nine digits: stacks) planes 3 d .. 3 d + 2 = -Im, Re, Im.  A thread takes two rows.
 template <int ND>
 __global__ void digits_x_kernel(const double2* __restrict__ X, long ldx, int r0, int K, int n, int npad,
-                                const int* __restrict__ f, unsigned* __restrict__ D, long ldk, long plane) {
+                                const int* __restrict__ f, unsigned* __restrict__ D, long ldk, long plane,
+                                RtShift sh) {
     constexpr bool STACK = ND > 7;
     const int Kp = (K + 1) / 2;
     const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -636,10 +651,10 @@ __global__ void digits_x_kernel(const double2* __restrict__ X, long ldx, int r0,
     }
     const double2* x = X + r0 + k + (long)c * ldx;
     const double2 a = x[0], b = k + 1 < K ? x[1] : make_double2(0.0, 0.0);
-    const int ex = f[c];
+    const int ea = f[c] - sh.at(k), eb = f[c] - sh.at(k + 1);
     constexpr float Z = DIGIT_ONE + 64.f;
-    const unsigned long long ra = digit_word<ND>(a.x, ex), rb = digit_word<ND>(b.x, ex);
-    const unsigned long long ia = digit_word<ND>(STACK ? -a.y : a.y, ex), ib = digit_word<ND>(STACK ? -b.y : b.y, ex);
+    const unsigned long long ra = digit_word<ND>(a.x, ea), rb = digit_word<ND>(b.x, eb);
+    const unsigned long long ia = digit_word<ND>(STACK ? -a.y : a.y, ea), ib = digit_word<ND>(STACK ? -b.y : b.y, eb);
 #pragma unroll
     for (int d = 0; d < ND; ++d) {
         const float va = digit_raw<ND>(ia, d), vb = digit_raw<ND>(ib, d);
@@ -737,7 +752,7 @@ int rt_col_tile(int nd) { return nd <= 7 ? RtCfg<7>::NT : RtCfg<9>::NT; }
 
 // Row exponents (unless rowmax is null: they are there) and digit planes of A.
 cudaError_t launch_digits_a(cudaStream_t s, const double2* A, long lda, int rows, int K, int* e, void* D, long ldk,
-                            void* rowmax, int nd) {
+                            void* rowmax, int nd, RtShift sh) {
     if (rows <= 0 || K <= 0) return cudaSuccess;
     unsigned long long* mx = reinterpret_cast<unsigned long long*>(rowmax);
     if (mx != nullptr) {
@@ -748,17 +763,17 @@ cudaError_t launch_digits_a(cudaStream_t s, const double2* A, long lda, int rows
     }
     const dim3 grid(ceil_div(K, 64), ceil_div(rows, 32));
     auto kern = nd <= 7 ? digits_a_kernel<7> : digits_a_kernel<9>;
-    kern<<<grid, 256, 0, s>>>(A, lda, rows, K, e, reinterpret_cast<unsigned*>(D), ldk, (long)rows * ldk);
+    kern<<<grid, 256, 0, s>>>(A, lda, rows, K, e, reinterpret_cast<unsigned*>(D), ldk, (long)rows * ldk, sh);
     return cudaGetLastError();
 }
 
 cudaError_t launch_digits_x(cudaStream_t s, const double2* X, long ldx, int r0, int K, int n, int npad, int* f,
-                            void* D, long ldk, long plane, int nd) {
+                            void* D, long ldk, long plane, int nd, RtShift sh) {
     if (n <= 0 || K <= 0) return cudaSuccess;
-    col_exponent_kernel<<<n, 256, 0, s>>>(X, ldx, r0, K, f);
+    col_exponent_kernel<<<n, 256, 0, s>>>(X, ldx, r0, K, f, sh);
     const long t = (long)npad * ((K + 1) / 2);
     auto kern = nd <= 7 ? digits_x_kernel<7> : digits_x_kernel<9>;
-    kern<<<ceil_div(t, 256L), 256, 0, s>>>(X, ldx, r0, K, n, npad, f, reinterpret_cast<unsigned*>(D), ldk, plane);
+    kern<<<ceil_div(t, 256L), 256, 0, s>>>(X, ldx, r0, K, n, npad, f, reinterpret_cast<unsigned*>(D), ldk, plane, sh);
     return cudaGetLastError();
 }
 
@@ -888,7 +903,7 @@ size_t dg_bytes(int m, int n, int K, int num_sms) {
 }
 
 bm_status gemm_z64_dg(cudaStream_t s, void* work, int num_sms, int m, int n, int K, double alpha, Z64 A, Z64 B, Z64 C,
-                      int* d_err) {
+                      int* d_err, int* eA, RtShift sh) {
     const DgPlan p = dg_plan(m, n, K, num_sms);
     const int nt = rt_col_tile(DG_ND);
     const long ldk = rt_ldk(K);
@@ -903,17 +918,18 @@ bm_status gemm_z64_dg(cudaStream_t s, void* work, int num_sms, int m, int n, int
     BM_TRY(rt_make_map_x(tmx, xp, p.nc, K, ldk, DG_ND));
     for (int i0 = 0; i0 < m; i0 += p.mr) {
         const int mr = std::min(p.mr, m - i0);
-        BM_CUDA_TRY(launch_digits_a(s, A.p + i0, A.ld, mr, K, ea, ap, ldk, rmax, DG_ND));
+        int* const er = eA != nullptr ? eA + i0 : ea;
+        BM_CUDA_TRY(launch_digits_a(s, A.p + i0, A.ld, mr, K, er, ap, ldk, eA != nullptr ? nullptr : rmax, DG_ND, sh));
         BM_TRY(rt_make_map(tma, ap, mr, K, ldk, (long)mr * ldk, RT_BM, DG_ND));
         for (int j0 = 0; j0 < n; j0 += p.nc) {
             const int nc = std::min(p.nc, n - j0);
             BM_CUDA_TRY(launch_digits_x(s, B.p + (long)j0 * B.ld, B.ld, 0, K, nc, ceil_div(nc, nt) * nt, fx, xp, ldk,
-                                        (long)p.nc * ldk, DG_ND));
+                                        (long)p.nc * ldk, DG_ND, sh));
             const long mq = mr, kq = K;
             int S = 1, nl = 0;
             rt_plan_splits(1, &mq, &kq, nc, DG_ND, num_sms, &S);
             while (S > 1 && (size_t)2 * S * mr * nc * 8 > p.w) --S;
-            RtArgs a{tma, tmx, ea, fx, C.p + i0 + (long)j0 * C.ld, C.ld, nullptr, nullptr, mr, K, S};
+            RtArgs a{tma, tmx, er, fx, C.p + i0 + (long)j0 * C.ld, C.ld, nullptr, nullptr, mr, K, S};
             if (S > 1) {
                 a.Wr = ws;
                 a.Wi = ws + (size_t)S * mr * nc;

@@ -368,7 +368,8 @@ bm_status correction_c32(bm_ctx* c, const double2* R, double2* X, long ld, int n
         // W3 -= [M31 M32] [W1; W2]
         {
             BM_PROF(c, "pack_b_kernel");
-            SV_CUDA(launch_pack_b(s, Wr, Wi, ldw, K, N, ldexpf(1.f, c->tc_shift), nrhs, c->d_Bx1r, c->d_Bx1i, c->ldk_schur, c->d_Bxe));
+            SV_CUDA(launch_pack_b(s, Wr, Wi, ldw, K, N, c->d_bal + BAL_SHIFT, nrhs, c->d_Bx1r, c->d_Bx1i, c->ldk_schur,
+                                  c->d_Bxe));
         }
         {
             BM_PROF(c, "cgemm_tc_kernel (skinny, + split-K reduction)");
@@ -384,7 +385,7 @@ bm_status correction_c32(bm_ctx* c, const double2* R, double2* X, long ld, int n
         // [W1; W2] -= [M13; M23] z3; the pack of z3 stays for the next residual update
         {
             BM_PROF(c, "pack_b_kernel");
-            SV_CUDA(launch_pack_b(s, Vr, Vi, ldv, N, N, 1.f, nrhs, c->d_Bx2r, c->d_Bx2i, c->ldk_c, c->d_Bxe + c->ws_nrhs));
+            SV_CUDA(launch_pack_b(s, Vr, Vi, ldv, N, N, nullptr, nrhs, c->d_Bx2r, c->d_Bx2i, c->ldk_c, c->d_Bxe + c->ws_nrhs));
         }
         {
             BM_PROF(c, "cgemm_tc_kernel (skinny, + split-K reduction)");
@@ -433,7 +434,8 @@ bm_status residual_update_c32(bm_ctx* c, double2* R, long ld, int nrhs) {
         SV_CUDA(gemm_tc_split(s, c->tm_skinny[0], c->tm_skinny[1], c->tm_skinny[4], c->tm_skinny[5], 2 * N, nrhs, N, -1.f,
                               1.f, skinny_scale(c, 0), TcDest{nullptr, nullptr, R, ld},
                               skinny_split(c, 2 * N, nrhs, N), c->d_Pkr, c->d_Pki, c->d_err, &n1));
-        SV_CUDA(launch_pack_b(s, c->d_Wr, c->d_Wi, ldw, 2 * N, N, ldexpf(1.f, c->tc_shift), nrhs, c->d_Bx1r, c->d_Bx1i, c->ldk_schur, c->d_Bxe));
+        SV_CUDA(launch_pack_b(s, c->d_Wr, c->d_Wi, ldw, 2 * N, N, c->d_bal + BAL_SHIFT, nrhs, c->d_Bx1r, c->d_Bx1i,
+                              c->ldk_schur, c->d_Bxe));
         SV_CUDA(gemm_tc_split(s, c->tm_schur[0], c->tm_schur[1], c->tm_skinny[2], c->tm_skinny[3], N, nrhs, 2 * N,
                               -1.f, 1.f, skinny_scale(c, 1), TcDest{nullptr, nullptr, R + 2 * N, ld},
                               skinny_split(c, N, nrhs, 2 * N), c->d_Pkr, c->d_Pki, c->d_err, &n2));
