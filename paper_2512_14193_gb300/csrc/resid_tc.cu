@@ -15,8 +15,11 @@
 //     2^24 (at most 7 pairs x 2 real products per complex term x 256 x 2^12), so every partial sum
 //     is an integer that FP32 represents exactly: nothing is rounded inside a chunk, whatever order
 //     the hardware adds in;
-//   * after each chunk the seven level sums are combined and added to a running double-float sum
-//     (pairs of FP32) per output; the dropped pairs (d + d' > 8) weigh below 2^-56.
+//   * after each chunk the level sums are added to two 64-bit integers per output, the upper levels and the
+//     lower ones, each weighted by its power of 128: nothing is rounded until the end, where the two are
+//     added in FP64 (pairs of FP32 per output, the first form, lose a bit or two past 2^-48 in every chunk:
+//     FP64 solutions at N = 1000 were off by 5e-14 instead of 7e-15).  The dropped pairs weigh below 2^-56
+//     (seven digits) and 2^-70.
 // The x digit tiles sit one after another in shared memory and the levels' accumulators one after
 // another in tensor memory, so one MMA multiplies A digit d by all the x digits it pairs with and
 // lands each pair in its level.  Seven digits (32 right-hand sides per CTA): four MMAs of width
@@ -68,10 +71,13 @@ struct RtCfg {
     static constexpr int A_STAGE = A_PL * RT_TILE_A;
     static constexpr int AST = STACK ? 5 : 3;           // A stages
     static constexpr int USES = 2 * D / A_PL;           // stage uses per K block
+    static constexpr int LH = D / 2;                    // last of the upper levels
     static constexpr int SMEM = AST * A_STAGE + 2 * X_BUF + 1024 + 256;
     static_assert(2 * D * NT <= 512, "the level accumulators fit tensor memory");
     static_assert(D * NT <= 256, "the widest single MMA has N <= 256");
     static_assert(D * 2 * 4096L * 64 * KB_CHUNK <= (1L << 24), "chunk sums stay exact in FP32");
+    // |upper levels' sum| < 2^14 K 128^LH, |lower levels'| < 2^(14 + 1) D K 128^(D - 2 - LH): K below 2^20
+    static_assert(14 + 7 * LH + 20 < 63 && 19 + 7 * (D - 2 - LH) + 20 < 63, "the integer sums do not overflow");
     static_assert(SMEM <= 232448, "shared memory");
 };
 
@@ -164,14 +170,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t ta, float* v) {
 __device__ constexpr uint32_t idesc_bf16(uint32_t neg_a, uint32_t n) {
     return (1u << 4) | (1u << 7) | (1u << 10) | (neg_a << 13) | ((n >> 3) << 17) | ((uint32_t)(RT_BM >> 4) << 24);
 }
-// s + t exactly as hi + lo (Knuth's TwoSum); the rn intrinsics keep the steps from being contracted
-__device__ __forceinline__ void two_sum(float& hi, float& lo, float a, float b) {
-    const float s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    lo = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-    hi = s;
-}
-
 struct RtProd {
     CUtensorMap tmA;   // the A digit planes (3-D: K, rows, 14 planes)
     CUtensorMap tmX[2];  // the x digit planes: 3-D (K, columns, 14 planes), or the two stacks (4-D)
@@ -398,54 +396,40 @@ __global__ void __launch_bounds__(RT_THREADS, 1) resid_tc_kernel(const __grid_co
         const int qw = warp & 3;  // tensor-memory lane quarter this warp may read
         const int part = warp >= 6 ? 1 : 0;
         const uint32_t lane_off = (uint32_t)(qw * 32) << 16;
-        float sh[RT_NT], sl[RT_NT];  // running double-float sums of this row's outputs
+        long long hi[RT_NT], lo[RT_NT];  // running sums of this row's outputs: levels up to LH, and past it
 #pragma unroll
-        for (int j = 0; j < RT_NT; ++j) sh[j] = sl[j] = 0.f;
+        for (int j = 0; j < RT_NT; ++j) hi[j] = lo[j] = 0;
+        // level lev of every output times w onto acc, then released to the next chunk's products
+        auto add_level = [&](long long (&acc)[RT_NT], int lev, int w) {
+#pragma unroll
+            for (int g = 0; g < RT_NT / 16; ++g) {
+                float v[16];
+                tmem_ld16(tmem + lane_off + (uint32_t)(STACK ? 2 * RT_NT * lev + RT_NT * part + g * 16
+                                                             : part * RT_D * RT_NT + lev * RT_NT + g * 16), v);
+                if (g == RT_NT / 16 - 1) {
+                    fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(levfree + 8 * lev);
+                }
+#pragma unroll
+                for (int j = 0; j < 16; ++j) acc[g * 16 + j] += (long long)__float2int_rn(v[j]) * w;
+            }
+        };
         for (int ch = 0; ch < nchunks; ++ch) {
             if (!mbar_wait(accfull, (uint32_t)ch & 1u, abort_flag)) break;
             fence_after();
-            float th[RT_NT], tl[RT_NT];
-#pragma unroll
-            for (int j = 0; j < RT_NT; ++j) th[j] = tl[j] = 0.f;
-            // level sums are exact integers; scale by 128^-l (exact) and add in double-float, the last
-            // level first, each released to the next chunk's products when it has been read
+            // (the last level first: the order in which the next chunk's products need them)
 #pragma unroll 1
-            for (int lev = RT_D - 1; lev >= 0; --lev) {
-                const float w = __int_as_float((127 - 7 * lev) << 23);  // 2^(-7 lev)
-#pragma unroll
-                for (int g = 0; g < RT_NT / 16; ++g) {
-                    float v[16];
-                    tmem_ld16(tmem + lane_off + (uint32_t)(STACK ? 2 * RT_NT * lev + RT_NT * part + g * 16
-                                                                 : part * RT_D * RT_NT + lev * RT_NT + g * 16), v);
-                    if (g == RT_NT / 16 - 1) {
-                        fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(levfree + 8 * lev);
-                    }
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        float hi, lo;
-                        two_sum(hi, lo, th[g * 16 + j], v[j] * w);
-                        th[g * 16 + j] = hi;
-                        tl[g * 16 + j] = __fadd_rn(tl[g * 16 + j], lo);
-                    }
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < RT_NT; ++j) {
-                // (sh, sl) += (th, tl)
-                float hi, lo;
-                two_sum(hi, lo, sh[j], th[j]);
-                lo = __fadd_rn(lo, __fadd_rn(sl[j], tl[j]));
-                const float s2 = __fadd_rn(hi, lo);
-                sl[j] = __fsub_rn(lo, __fsub_rn(s2, hi));
-                sh[j] = s2;
-            }
+            for (int lev = RT_D - 1; lev > Cfg::LH; --lev) add_level(lo, lev, 1 << (7 * (RT_D - 1 - lev)));
+#pragma unroll 1
+            for (int lev = Cfg::LH; lev >= 0; --lev) add_level(hi, lev, 1 << (7 * (Cfg::LH - lev)));
         }
         if (!*abort_flag) {
             const int row = row0 + qw * 32 + lane;
             if (row < P.m) {
-                // value = 128^-2 2^(e_row + f_col) sum  (digits carry 128^-d each)
+                // value = 128^-2 2^(e_row + f_col) (hi 128^-LH + lo 128^-(D - 1))  (digits carry 128^-d each)
+                constexpr int EH = -14 - 7 * Cfg::LH;
+                constexpr double LO = 1.0 / (double)(1ll << (7 * (RT_D - 1 - Cfg::LH)));
                 const int er = P.eA[row];
 #pragma unroll
                 for (int j = 0; j < RT_NT; ++j) {
@@ -454,7 +438,7 @@ __global__ void __launch_bounds__(RT_THREADS, 1) resid_tc_kernel(const __grid_co
                     const int fc = P.fX[col];
                     const double v = er == RT_NONFINITE || fc == RT_NONFINITE
                                          ? __longlong_as_double(0x7FF8000000000000ll)
-                                         : ldexp((double)sh[j] + (double)sl[j], er + fc - 14);
+                                         : ldexp(fma((double)lo[j], LO, (double)hi[j]), er + fc + EH);
                     if (P.S == 1) {
                         double* o = reinterpret_cast<double*>(P.C + row + (long)col * P.ldc) + part;
                         *o += J.alpha * v;
