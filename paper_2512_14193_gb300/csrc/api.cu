@@ -233,6 +233,7 @@ void free_problem(bm_ctx* c) {
     FREE(c->d_Lp_i);
     FREE(c->d_Up_r);
     FREE(c->d_Up_i);
+    FREE(c->d_Lpe);
     FREE(c->d_Upe);
     FREE(c->d_Cp_r);
     FREE(c->d_Cp_i);
@@ -294,7 +295,7 @@ Plan make_plan(int N, int form, int prec, int nb_user, int bs, int nd, bool fast
         }
         // packs of the trailing updates and the search-free blocks' work buffer
         p.ldk_lu = tc_ldk(fast ? std::max(p.nb, 128) : p.nb);
-        b += 2 * (size_t)p.n * p.ldk_lu * 4 + (size_t)p.n * 4;
+        b += 2 * (size_t)p.n * p.ldk_lu * 4 + 2 * (size_t)p.n * 4;
         if (fast) b += lu_fast_bytes(p.n);
         // digit planes of the operator for the tensor-core residual and their row exponents
         const size_t planes = (size_t)rt_digit_planes(nd) * 2;
@@ -304,6 +305,7 @@ Plan make_plan(int N, int form, int prec, int nb_user, int bs, int nd, bool fast
             b += planes * 2L * N * rt_ldk(2L * N) + 2L * N * 4;
     }
     if (form == BM_MIXED) b += (size_t)N * 4 + bal_ints(N) * 4;  // the balance of the Schur product
+    else if (!c32) b += 2 * (size_t)N * 4;                       // the row exponents
     p.nblk = ceil_div(p.n, bs);
     b += 2 * (size_t)p.n * 4;
     b += 2 * (size_t)p.nblk * bs * bs * (c32 ? 8 : 16);
@@ -648,6 +650,7 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
         s = alloc_t(c, &c->d_A, (size_t)p.ldA * 2 * N * 16);
     }
     if (s == BM_OK && !c32) s = alloc_t(c, &c->d_F64, (size_t)p.ldF * p.n * 16);
+    if (s == BM_OK && !c32 && form == BM_ORDINARY) s = alloc_t(c, &c->d_dge[0], 2 * (size_t)N * 4);  // inner scale
     if (s == BM_OK && planes >= 1) {
         if (form == BM_MIXED) {
             s = alloc_t(c, &c->d_Ptop, (size_t)p.ldtop * N * 16);
@@ -678,6 +681,7 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
         if (s == BM_OK) s = alloc_t(c, &c->d_Lp_i, lb);
         if (s == BM_OK) s = alloc_t(c, &c->d_Up_r, lb);
         if (s == BM_OK) s = alloc_t(c, &c->d_Up_i, lb);
+        if (s == BM_OK) s = alloc_t(c, &c->d_Lpe, (size_t)p.n * 4);
         if (s == BM_OK) s = alloc_t(c, &c->d_Upe, (size_t)p.n * 4);
         if (s == BM_OK && c32 && c->lu_fast) s = alloc_t(c, &c->d_fd, lu_fast_bytes(p.n));
     }

@@ -923,7 +923,8 @@ extern "C" bm_status bm_zeta_weights(int p, double* tau, double* c2) {
 cudaError_t launch_normA(cudaStream_t s, const bm_ctx* c) {
     cudaError_t e = cudaMemsetAsync(c->d_normA, 0, sizeof(double), s);
     if (e != cudaSuccess) return e;
-    // (the CF32 precisions' digit planes are scaled by row exponents, found on the way; d_dge is null in FP64)
+    // (the exponents found on the way scale the CF32 precisions' digit planes and the LU's updates; the mixed system
+    // has none of its rows in FP64)
     const int N = c->N;
     if (c->form == BM_MIXED) {
         e = cudaMemsetAsync(c->d_bal, 0x80, BAL_SHIFT * sizeof(int), s);  // below every exponent

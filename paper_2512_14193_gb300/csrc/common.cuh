@@ -324,10 +324,11 @@ struct bm_ctx {
     int* d_Ape = nullptr;      // exponents of A (balance_kernel)
     int* d_bal = nullptr;      // mixed: the balance of the Schur product (BAL_* in kernels.cuh)
     long ldk_schur = 0;
-    __half* d_Lp_r = nullptr;  // LU trailing-update packs (L21 times 2^TC_SHIFT_L; exponents d_Upe of U12)
+    __half* d_Lp_r = nullptr;  // LU trailing-update packs (exponents d_Lpe of L21's rows, d_Upe of U12's columns)
     __half* d_Lp_i = nullptr;
     __half* d_Up_r = nullptr;
     __half* d_Up_i = nullptr;
+    int* d_Lpe = nullptr;
     int* d_Upe = nullptr;
     long ldk_lu = 0;
     __half* d_Cp_r = nullptr;  // [M13; M23] rows, K = N (2N rows; exponents d_dge[0]): A operand of the skinny

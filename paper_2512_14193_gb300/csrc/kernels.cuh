@@ -45,7 +45,6 @@ constexpr int BAL_SHIFT = 4;  // s
 constexpr int BAL_ROWS = 8;   // exponents of the rows of M31, then of M32
 constexpr size_t bal_ints(long N) { return BAL_ROWS + 2 * (size_t)N; }
 constexpr int TC_E_DGE = -16;  // e0 of rows scaled by the digit planes' exponents (entries below 2^(e - 1))
-constexpr int TC_SHIFT_L = 14; // L21 is packed times 2^14 (its entries are below sqrt 2 in modulus)
 // TcGate: the launch skips its first 128 x 128 tile (another launch takes it), and does nothing when the
 // word *fail, if any, names a block of the factorisation up to `block` (lu_fast.cu)
 struct TcGate {
@@ -149,11 +148,21 @@ void rt_plan_splits(int nprod, const long* m, const long* K, int n, int nd, int 
 bm_status rt_make_map(void* tmap, const void* base, long rows, long K, long ldk, long plane_elems, int box_rows,
                       int nd);
 bm_status rt_make_map_x(void* tmaps, const void* base, long cols, long K, long ldk, int nd);  // two blobs
-// K entries from `half` on are taken times 2^-s (A) or 2^s (x), s = *shift
+// Inner scale of a block's product L21 U12 of an LU: column k of L21 times 2^d, row k of U12 times 2^-d, d the
+// difference of the exponents `re` of the matrix's rows that became the block's rows k and 0.  U12's rows have
+// the size of those rows (the ordinary system's two block rows differ by beta), L21's columns its inverse, and a block
+// where the two meet would otherwise lose the smaller under one scale per row and column.
+__device__ __forceinline__ int inner_exponent(int ek, int e0) { return min(max(ek - e0, -100), 100); }
+// K entries k are taken times 2^-at(k) (A) or 2^at(k) (x): from `half` on at = *shift, or the inner scale
+// of a block whose rows have the exponents re[0], re[1], ..
 struct RtShift {
     const int* shift = nullptr;
     int half = 0;
-    __device__ __forceinline__ int at(int k) const { return shift != nullptr && k >= half ? __ldg(shift) : 0; }
+    const int* re = nullptr;
+    __device__ __forceinline__ int at(int k) const {
+        if (shift != nullptr) return k >= half ? __ldg(shift) : 0;
+        return re != nullptr ? -inner_exponent(re[k], re[0]) : 0;
+    }
 };
 // (rowmax: scratch of `rows` words to find the row exponents e with; null: e holds them)
 cudaError_t launch_digits_a(cudaStream_t s, const double2* A, long lda, int rows, int K, int* e, void* D, long ldk,
@@ -161,6 +170,13 @@ cudaError_t launch_digits_a(cudaStream_t s, const double2* A, long lda, int rows
 // |v| as the bits of a non-negative double, which order as the doubles do; infinities and NaN are the largest
 __device__ __forceinline__ unsigned long long mag_bits(double v) {
     return (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
+}
+// the bits of v 2^d from those of |v| (0 below the normal range)
+__device__ __forceinline__ unsigned long long scaled_mag(unsigned long long b, int d) {
+    if (d == 0 || b >= 0x7FF0000000000000ull) return b;
+    const int e = (int)(b >> 52), n = e + d;
+    if (e == 0 || n < 1) return 0;
+    return (b & 0xFFFFFFFFFFFFFull) | (unsigned long long)min(n, 2046) << 52;
 }
 // Exponent of a row or column with an infinity or a NaN: its digits are zeros and its outputs NaN
 constexpr int RT_NONFINITE = 1 << 20;

@@ -74,7 +74,8 @@ constexpr int ST_KC = 32;  // L11 columns per shared-memory chunk when L11 does 
 template <class V>
 __global__ void __launch_bounds__(ST_WARPS * 32) swap_trsm_kernel(V A, const SwapMap* __restrict__ map, int a0, int a1,
                                                                    int b0, int b1, int t0, int tb, __half* Upr,
-                                                                   __half* Upi, long ldk, int* Upe, int l_in_smem) {
+                                                                   __half* Upi, long ldk, int* Upe, const int* re,
+                                                                   const int* perm, int l_in_smem) {
     using CV = typename V::cv;
     using Rl = typename V::real;
     constexpr int QMAX = 8;  // rows per lane: tb <= 256
@@ -229,47 +230,66 @@ __global__ void __launch_bounds__(ST_WARPS * 32) swap_trsm_kernel(V A, const Swa
             if (i < tb) A.set((long)t0 + i, col, x[q]);
         }
         if (Upr != nullptr) {
-            // pack row col - b0 (tb is a multiple of 32: the last panel has no pack) and its exponent, which
-            // also takes L21's shift back
+            // pack row col - b0 (tb is a multiple of 32: the last panel has no pack) and its exponent
             const long rowp = col - b0;
-            float mx = 0.f;
+            float mx = 0.f, w[QMAX];
 #pragma unroll
             for (int q = 0; q < QMAX; ++q)
-                if (lane + 32 * q < tb) mx = fmaxf(mx, fmaxf(fabsf((float)x[q].x), fabsf((float)x[q].y)));
+                if (lane + 32 * q < tb) {
+                    w[q] = re != nullptr ? tc_pow2(-inner_exponent(re[perm[t0 + lane + 32 * q]], re[perm[t0]])) : 1.f;
+                    mx = fmaxf(mx, w[q] * fmaxf(fabsf((float)x[q].x), fabsf((float)x[q].y)));
+                }
             for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
             const TcRowScale sc(mx);
-            if (lane == 0) Upe[rowp] = sc.ex - 15 - TC_SHIFT_L;
+            if (lane == 0) Upe[rowp] = sc.ex - 15;
             __half* pr = Upr + rowp * ldk + lane;
             __half* pi = Upi + rowp * ldk + lane;
 #pragma unroll
             for (int q = 0; q < QMAX; ++q)
                 if (lane + 32 * q < tb) {
-                    tc_split(sc((float)x[q].x), pr[64 * q], pr[64 * q + 32]);
-                    tc_split(sc((float)x[q].y), pi[64 * q], pi[64 * q + 32]);
+                    tc_split(sc(w[q] * (float)x[q].x), pr[64 * q], pr[64 * q + 32]);
+                    tc_split(sc(w[q] * (float)x[q].y), pi[64 * q], pi[64 * q + 32]);
                 }
         }
     }
 }
 
-// L21 pack: rows [r0, r0+m) x columns [c0, c0+kb) of A (kb a multiple of 32) -> pack rows, times 2^TC_SHIFT_L.
-__global__ void pack_L_kernel(C32 A, long r0, long c0, int m, __half* Pr, __half* Pi, long ldk) {
+// L21 pack: rows [r0, r0+m) x columns [c0, c0+kb) of A (kb a multiple of 32) -> pack rows and their exponents: the
+// maxima of 32 rows, then the pack through 32 x 32 tiles (the second reads come from L2).
+__global__ void pack_L_kernel(C32 A, long r0, long c0, int m, int kb, __half* Pr, __half* Pi, long ldk, int* Le,
+                              const int* re, const int* perm) {
     __shared__ float2 t[32][33];
-    const int k0 = blockIdx.x * 32, i0 = blockIdx.y * 32;
+    auto w = [&](int k) { return re != nullptr ? tc_pow2(inner_exponent(re[perm[c0 + k]], re[perm[c0]])) : 1.f; };
+    __shared__ float top[8][32];
+    const int i0 = blockIdx.x * 32;
     const int tx = threadIdx.x, ty = threadIdx.y;
-    for (int q = ty; q < 32; q += 8) {
-        const int i = i0 + tx;
-        t[q][tx] = i < m ? A.get(r0 + i, c0 + k0 + q) : make_float2(0.f, 0.f);
+    const bool in = i0 + tx < m;
+    float mx = 0.f;
+#pragma unroll 8
+    for (int k = ty; k < kb; k += 8) {
+        const float2 v = in ? A.get(r0 + i0 + tx, c0 + k) : make_float2(0.f, 0.f);
+        mx = fmaxf(mx, w(k) * fmaxf(fabsf(v.x), fabsf(v.y)));
     }
-    __syncthreads();
-    const TcRowScale sc(TC_SHIFT_L);
-    for (int q = ty; q < 32; q += 8) {
-        const int i = i0 + q;
-        if (i >= m) continue;
-        const float2 v = t[tx][q];
-        __half* pr = Pr + (long)i * ldk + 2 * k0 + tx;
-        __half* pi = Pi + (long)i * ldk + 2 * k0 + tx;
-        tc_split(sc(v.x), pr[0], pr[32]);
-        tc_split(sc(v.y), pi[0], pi[32]);
+    top[ty][tx] = mx;
+    for (int k0 = 0; k0 < kb; k0 += 32) {
+        __syncthreads();  // the maxima are there; the tile before has been packed
+        for (int q = ty; q < 32; q += 8) t[q][tx] = in ? A.get(r0 + i0 + tx, c0 + k0 + q) : make_float2(0.f, 0.f);
+        __syncthreads();
+        const float wk = w(k0 + tx);
+        for (int q = ty; q < 32; q += 8) {
+            const int i = i0 + q;
+            if (i >= m) continue;
+            float mi = 0.f;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) mi = fmaxf(mi, top[w][q]);
+            const TcRowScale sc(mi);
+            if (k0 == 0 && tx == 0) Le[i] = sc.ex - 15;
+            const float2 v = t[tx][q];
+            __half* pr = Pr + (long)i * ldk + 2 * k0 + tx;
+            __half* pi = Pi + (long)i * ldk + 2 * k0 + tx;
+            tc_split(sc(wk * v.x), pr[0], pr[32]);
+            tc_split(sc(wk * v.y), pi[0], pi[32]);
+        }
     }
 }
 
@@ -748,7 +768,8 @@ __global__ void gather_rows_c32_kernel(const int* __restrict__ perm, int n, int 
 
 template <class V>
 cudaError_t launch_swap_trsm(cudaStream_t s, V A, const SwapMap* map, int a0, int a1, int b0, int b1, int t0, int tb,
-                             __half* Upr, __half* Upi, long ldk, int* Upe) {
+                             __half* Upr, __half* Upi, long ldk, int* Upe, const int* re = nullptr,
+                             const int* perm = nullptr) {
     using CV = typename V::cv;
     long ncols = (long)(a1 - a0) + (b1 - b0);
     if (ncols <= 0) return cudaSuccess;
@@ -763,7 +784,7 @@ cudaError_t launch_swap_trsm(cudaStream_t s, V A, const SwapMap* map, int a0, in
     }
     int grid = ceil_div(ncols, ST_WARPS * ST_COLS);
     return launch_pdl(kern, dim3(grid), dim3(ST_WARPS * 32), smem, s, A, map, a0, a1, b0, b1, t0, tb, Upr, Upi, ldk,
-                      Upe, l_in_smem);
+                      Upe, re, perm, l_in_smem);
 }
 
 cudaError_t gemm_any(cudaStream_t s, int m, int n, int k, Z64 A, Z64 B, Z64 C) {
@@ -772,6 +793,10 @@ cudaError_t gemm_any(cudaStream_t s, int m, int n, int k, Z64 A, Z64 B, Z64 C) {
 cudaError_t gemm_any(cudaStream_t s, int m, int n, int k, C32 A, C32 B, C32 C) {
     return gemm_c32(s, m, n, k, -1.0f, A, false, B, 1.0f, C);
 }
+
+// Exponents of the rows of the factored matrix for the inner scale of its updates: the ordinary system's, whose
+// block rows differ (the Schur complement's rows do not).
+const int* row_exponents(const bm_ctx* c) { return c->form == BM_ORDINARY ? c->d_dge[0] : nullptr; }
 
 // What the solves need besides the factors: the inverted diagonal blocks and (FP32) the G form.
 template <class V>
@@ -833,7 +858,7 @@ bm_status factor_fast(bm_ctx* c, C32 F) {
         iota_kernel<<<ceil_div(n, 256), 256, 0, s>>>(c->d_perm, c->d_ipiv, n);
         LU_CUDA(cudaGetLastError());
     }
-    const TcPacks packs{c->d_Lp_r, c->d_Lp_i, c->d_Up_r, c->d_Up_i, c->d_Upe, c->ldk_lu};
+    const TcPacks packs{c->d_Lp_r, c->d_Lp_i, c->d_Up_r, c->d_Up_i, c->d_Lpe, c->d_Upe, row_exponents(c), c->ldk_lu};
     bool rest = false;  // a trailing update is under way on s2
     for (int J = 0; J < n; J += FD_B) {
         const int db = std::min(FD_B, n - J), mm = n - J - db;
@@ -855,7 +880,7 @@ bm_status factor_fast(bm_ctx* c, C32 F) {
         TcGate gate{fail, J + 1, 0};
         auto update = [&](cudaStream_t st, int m) {
             return gemm_tc_upd(st, c->tm_lu[0], c->tm_lu[1], c->tm_lu[2], c->tm_lu[3], C.re, C.im, C.ld, m, m, FD_B,
-                               TcScale{nullptr, c->d_Upe, 0}, c->num_sms - 1, c->d_err, gate);
+                               TcScale{c->d_Lpe, c->d_Upe, 0}, c->num_sms - 1, c->d_err, gate);
         };
         if (!la || mm <= FD_B) {
             LU_CUDA(update(s, mm));
@@ -875,6 +900,13 @@ bm_status factor_fast(bm_ctx* c, C32 F) {
         LU_CUDA(cudaStreamWaitEvent(c->stream, ev_done, 0));
     }
     return BM_OK;
+}
+
+// the inner scale of the product of the columns and rows from J on (rows in place: no interchange so far)
+RtShift inner_z(const bm_ctx* c, int J) {
+    RtShift sh;
+    if (const int* re = row_exponents(c)) sh.re = re + J;
+    return sh;
 }
 
 // The FP64 LU in blocks of FZ_BLOCK columns without a pivot search (lu_fast_z.cu), outer blocks of FZ_OUTER:
@@ -914,7 +946,8 @@ bm_status factor_fast_z(bm_ctx* c, Z64 F) {
         BM_PROF(c, "cgemm_simt_kernel (trailing update)");
         const size_t need = dg_bytes(m, m, k, c->num_sms);
         if (need > 0 && need <= c->dgw_bytes)
-            BM_TRY(gemm_z64_dg(s, c->d_dgw, c->num_sms, m, m, k, -1.0, F.sub(je, J), F.sub(J, je), F.sub(je, je), c->d_err));
+            BM_TRY(gemm_z64_dg(s, c->d_dgw, c->num_sms, m, m, k, -1.0, F.sub(je, J), F.sub(J, je), F.sub(je, je), c->d_err,
+                               nullptr, inner_z(c, J)));
         else
             LU_CUDA(gemm_z64(s, m, m, k, -1.0, F.sub(je, J), false, F.sub(J, je), 1.0, F.sub(je, je)));
     }
@@ -996,15 +1029,16 @@ bm_status factor_t(bm_ctx* c, V F, bool tc, int J0 = 0) {
             // on s: the next big panel's columns (all trailing columns without look-ahead), and the
             // columns left of this panel unless the rest stream takes them
             LU_CUDA(launch_swap_trsm<V>(s, F, d_map, 0, la ? 0 : J, J + jb, J + jb + nnext, J, jb,
-                                        pack ? c->d_Up_r : nullptr, pack ? c->d_Up_i : nullptr, c->ldk_lu, c->d_Upe));
+                                        pack ? c->d_Up_r : nullptr, pack ? c->d_Up_i : nullptr, c->ldk_lu, c->d_Upe,
+                                        row_exponents(c), c->d_perm));
         }
         if (mm > 0) {
             if (tc) {
                 if constexpr (std::is_same<V, C32>::value) {
-                    dim3 blk2(32, 8), grid(ceil_div(jb, 32), ceil_div(mm, 32));
                     {
                         BM_PROF(c, "pack_L_kernel");
-                        pack_L_kernel<<<grid, blk2, 0, s>>>(F, J + jb, J, mm, c->d_Lp_r, c->d_Lp_i, c->ldk_lu);
+                        pack_L_kernel<<<ceil_div(mm, 32), dim3(32, 8), 0, s>>>(F, J + jb, J, mm, jb, c->d_Lp_r, c->d_Lp_i,
+                                                                               c->ldk_lu, c->d_Lpe, row_exponents(c), c->d_perm);
                         LU_CUDA(cudaGetLastError());
                     }
                     C32 Cv = F.sub(J + jb, J + jb);
@@ -1012,7 +1046,7 @@ bm_status factor_t(bm_ctx* c, V F, bool tc, int J0 = 0) {
                         // (a CTA per tile: the panels' clusters need SMs that come free beside the rest)
                         BM_PROF(c, "cgemm_tc_kernel (trailing update)");
                         LU_CUDA(gemm_tc_upd(s, c->tm_lu[0], c->tm_lu[1], c->tm_lu[2], c->tm_lu[3], Cv.re, Cv.im, Cv.ld, mm,
-                                        nnext, jb, TcScale{nullptr, c->d_Upe, 0}, INT_MAX, c->d_err));
+                                        nnext, jb, TcScale{c->d_Lpe, c->d_Upe, 0}, INT_MAX, c->d_err));
                     }
                     if (la) {
                         // the rest on s2: interchanges of the columns left of this panel and right of
@@ -1021,11 +1055,11 @@ bm_status factor_t(bm_ctx* c, V F, bool tc, int J0 = 0) {
                         LU_CUDA(cudaStreamWaitEvent(s2, ev_fork, 0));
                         LU_CUDA(launch_swap_trsm<V>(s2, F, d_map, 0, J, J + jb + nnext, n, J, jb,
                                                     c->d_Up_r + (long)NB * c->ldk_lu, c->d_Up_i + (long)NB * c->ldk_lu,
-                                                    c->ldk_lu, c->d_Upe + NB));
+                                                    c->ldk_lu, c->d_Upe + NB, row_exponents(c), c->d_perm));
                         if (mm > nnext) {
                             C32 Cr = F.sub(J + jb, J + jb + nnext);
                             LU_CUDA(gemm_tc_upd(s2, c->tm_lu[0], c->tm_lu[1], c->tm_lu[4], c->tm_lu[5], Cr.re, Cr.im, Cr.ld,
-                                            mm, mm - nnext, jb, TcScale{nullptr, c->d_Upe + NB, 0}, INT_MAX,
+                                            mm, mm - nnext, jb, TcScale{c->d_Lpe, c->d_Upe + NB, 0}, INT_MAX,
                                                 c->d_err));
                         }
                         LU_CUDA(cudaEventRecord(ev_join, s2));

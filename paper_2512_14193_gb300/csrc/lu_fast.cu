@@ -362,6 +362,7 @@ __global__ void __launch_bounds__(RT, 2) lu_trsm_kernel(C32 F, int J, int db, in
     float* Xr = Ti + FD_PACK;  // [k][row]
     float* Xi = Xr + B * XP;
     __shared__ float2 piv_s[B];
+    __shared__ float w_s[B];  // inner scale of the packs
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     {
         const int f = *reinterpret_cast<volatile int*>(fail);
@@ -412,6 +413,10 @@ __global__ void __launch_bounds__(RT, 2) lu_trsm_kernel(C32 F, int J, int db, in
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     }
     piv_s[tid] = t.piv[tid];
+    {
+        const int d = packs.re != nullptr ? inner_exponent(packs.re[J + tid], packs.re[J]) : 0;
+        w_s[tid] = tc_pow2(rows ? d : -d);
+    }
     static_assert(RT == B, "a thread per pivot, row and K index");
     if (rows) {
         const int r = lane;
@@ -520,28 +525,30 @@ __global__ void __launch_bounds__(RT, 2) lu_trsm_kernel(C32 F, int J, int db, in
                 F.im[o] = Xi[tid * XP + c];
             }
     }
-    // packs of L21 rows (times 2^TC_SHIFT_L) and U12 columns (by their exponents, which take that shift back)
+    // packs of the L21 rows and U12 columns and their exponents (the rows' own: with beta far from i / k or a low
+    // frequency the ordinary system's lower rows of L21 are small, and a fixed scale would lose them)
     __shared__ float mx_s[RT / 32][R];
-    if (!rows) {
-        float mx = 0.f;  // of a quarter of column `lane`
+    {
+        float mx = 0.f;  // of a quarter of row or column `lane`
 #pragma unroll 8
         for (int k = warp; k < B; k += RT / 32)
-            mx = fmaxf(mx, fmaxf(fabsf(Xr[k * XP + lane]), fabsf(Xi[k * XP + lane])));
+            mx = fmaxf(mx, w_s[k] * fmaxf(fabsf(Xr[k * XP + lane]), fabsf(Xi[k * XP + lane])));
         mx_s[warp][lane] = mx;
         __syncthreads();
     }
+    const float w = w_s[tid];
+    int* const pe = rows ? packs.Le : packs.Ue;
     __half* Pr = (rows ? packs.Lr : packs.Ur) + tc_pos(tid);
     __half* Pi = (rows ? packs.Li : packs.Ui) + tc_pos(tid);
 #pragma unroll 4
     for (int r = 0; r < R; ++r)
         if (x0 + r < mm) {
-            const TcRowScale sc = rows ? TcRowScale(TC_SHIFT_L)
-                                       : TcRowScale(fmaxf(fmaxf(mx_s[0][r], mx_s[1][r]), fmaxf(mx_s[2][r], mx_s[3][r])));
-            if (!rows && tid == 0) packs.Ue[x0 + r] = sc.ex - 15 - TC_SHIFT_L;
+            const TcRowScale sc(fmaxf(fmaxf(mx_s[0][r], mx_s[1][r]), fmaxf(mx_s[2][r], mx_s[3][r])));
+            if (tid == 0) pe[x0 + r] = sc.ex - 15;
             __half* pr = Pr + (long)(x0 + r) * packs.ldk;
             __half* pi = Pi + (long)(x0 + r) * packs.ldk;
-            tc_split(sc(Xr[tid * XP + r]), pr[0], pr[32]);
-            tc_split(sc(Xi[tid * XP + r]), pi[0], pi[32]);
+            tc_split(sc(w * Xr[tid * XP + r]), pr[0], pr[32]);
+            tc_split(sc(w * Xi[tid * XP + r]), pi[0], pi[32]);
         }
 }
 

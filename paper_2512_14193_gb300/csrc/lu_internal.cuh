@@ -548,9 +548,10 @@ struct FdBackup {
 };
 inline size_t fd_work_floats(long n) { return (size_t)FD_T + 2 * FD_B * FD_B + 4 * (size_t)n * FD_B; }
 cudaError_t launch_lu_diag(cudaStream_t s, C32 F, int J, int db, float* work, int* fail);
-struct TcPacks {  // the trailing update's packs and U12's exponents
+struct TcPacks {  // the trailing update's packs and the exponents of L21's rows and U12's columns
     __half *Lr, *Li, *Ur, *Ui;
-    int* Ue;
+    int *Le, *Ue;
+    const int* re;  // exponents of the matrix's rows, or null: no inner scale (inner_exponent)
     long ldk;
 };
 cudaError_t launch_lu_trsm(cudaStream_t s, C32 F, int J, int db, int mm, float* work, long n, TcPacks packs, int* fail);

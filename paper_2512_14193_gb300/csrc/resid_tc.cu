@@ -480,12 +480,13 @@ __global__ void rt_reduce_kernel(const double* __restrict__ Wr, const double* __
 // 256 columns, combined by an atomic maximum on the bit patterns (non-negative doubles order as
 // their bits).  mx must start at zero.
 __global__ void row_max_kernel(const double2* __restrict__ A, long lda, int rows, int K,
-                               unsigned long long* __restrict__ mx) {
+                               unsigned long long* __restrict__ mx, RtShift sh) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= rows) return;
     const int j0 = blockIdx.y * 256, j1 = min(K, j0 + 256);
     // (integer maxima: FP64 compares run on the narrow FP64 pipe)
     unsigned long long m = 0;
+    auto take = [&](double2 v, int j) { m = max(m, scaled_mag(max(mag_bits(v.x), mag_bits(v.y)), -sh.at(j))); };
     const double2* a = A + i;
     int j = j0;
     for (; j + 8 <= j1; j += 8) {
@@ -493,12 +494,9 @@ __global__ void row_max_kernel(const double2* __restrict__ A, long lda, int rows
 #pragma unroll
         for (int u = 0; u < 8; ++u) v[u] = a[(long)(j + u) * lda];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) m = max(m, max(mag_bits(v[u].x), mag_bits(v[u].y)));
+        for (int u = 0; u < 8; ++u) take(v[u], j + u);
     }
-    for (; j < j1; ++j) {
-        const double2 v = a[(long)j * lda];
-        m = max(m, max(mag_bits(v.x), mag_bits(v.y)));
-    }
+    for (; j < j1; ++j) take(a[(long)j * lda], j);
     atomicMax(mx + i, m);
 }
 // e_i with max_j max(|Re|, |Im|) < 2^(e_i - 1) (0 for a zero row)
@@ -589,30 +587,19 @@ __global__ void __launch_bounds__(256) digits_a_kernel(const double2* __restrict
 // Column exponents of x over rows [r0, r0 + K) for the n columns (one block per column).
 __global__ void col_exponent_kernel(const double2* __restrict__ X, long ldx, int r0, int K, int* __restrict__ f,
                                     RtShift sh) {
-    const int c = blockIdx.x, half = sh.shift != nullptr ? sh.half : K;
-    unsigned long long mx[2] = {0, 0};  // of the entries before `half` and from it on
+    const int c = blockIdx.x;
+    unsigned long long mx = 0;
     for (int i = threadIdx.x; i < K; i += blockDim.x) {
         const double2 v = X[r0 + i + (long)c * ldx];
-        const unsigned long long b = max(mag_bits(v.x), mag_bits(v.y));
-        if (i < half) mx[0] = max(mx[0], b);
-        else mx[1] = max(mx[1], b);
+        mx = max(mx, scaled_mag(max(mag_bits(v.x), mag_bits(v.y)), sh.at(i)));
     }
-    __shared__ unsigned long long sm[2][32];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        for (int o = 16; o > 0; o >>= 1) mx[q] = max(mx[q], __shfl_xor_sync(0xffffffffu, mx[q], o));
-        if ((threadIdx.x & 31) == 0) sm[q][threadIdx.x >> 5] = mx[q];
-    }
+    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    __shared__ unsigned long long sm[32];
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = mx;
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
-            for (int q = 0; q < 2; ++q) mx[q] = max(mx[q], sm[q][w]);
-        int e = row_exponent(mx[0]);
-        if (mx[1] > 0) {
-            const int e1 = row_exponent(mx[1]), e2 = e1 == RT_NONFINITE ? e1 : e1 + sh.at(half);
-            e = mx[0] > 0 ? max(e, e2) : e2;
-        }
-        f[c] = e;
+        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) mx = max(mx, sm[w]);
+        f[c] = row_exponent(mx);
     }
 }
 
@@ -742,7 +729,7 @@ cudaError_t launch_digits_a(cudaStream_t s, const double2* A, long lda, int rows
     if (mx != nullptr) {
         cudaError_t err = cudaMemsetAsync(mx, 0, (size_t)rows * 8, s);
         if (err != cudaSuccess) return err;
-        row_max_kernel<<<dim3(ceil_div(rows, 128), ceil_div(K, 256)), 128, 0, s>>>(A, lda, rows, K, mx);
+        row_max_kernel<<<dim3(ceil_div(rows, 128), ceil_div(K, 256)), 128, 0, s>>>(A, lda, rows, K, mx, sh);
         row_exponent_kernel<<<ceil_div(rows, 128), 128, 0, s>>>(mx, rows, e);
     }
     const dim3 grid(ceil_div(K, 64), ceil_div(rows, 32));
