@@ -330,7 +330,7 @@ static size_t dg_request(int N, int form, bool fast, int num_sms) {
 size_t request_bytes(int N, int form, int prec, int nb, int nrhs, int resid_mode, bool optional, int num_sms) {
     Plan p = make_plan(N, form, prec, nb, 64, 9, optional && prec != BM_FP64 && nb == 0,
                        planes_needed(form, prec, resid_mode));
-    if (optional && prec == BM_FP64) p.bytes += dg_request(N, form, true, num_sms) + lu_fast_z_bytes();
+    if (optional && prec == BM_FP64) p.bytes += dg_request(N, form, true, num_sms) + lu_fast_z_bytes(p.n);
     const size_t w = (size_t)std::max(nrhs, 8);
     size_t b = p.bytes + 7 * (size_t)N * 8 + (size_t)p.nsys * w * 16 * 3 + (size_t)p.n * w * 16 * 2;
     if (prec == BM_FP64) {
@@ -831,8 +831,8 @@ bm_status assemble_post(bm_ctx* c, bool run_assembly_kernel, bool wait) {
 // (without it the panels search) and the digit workspace (without it the products run on the CUDA cores).
 void dg_reserve(bm_ctx* c) {
     if (c->prec != BM_FP64) return;
-    if (c->fast_z && !c->d_fd && c->held + lu_fast_z_bytes() <= c->budget &&
-        alloc_t(c, &c->d_fd, lu_fast_z_bytes()) != BM_OK)
+    if (c->fast_z && !c->d_fd && c->held + lu_fast_z_bytes(c->n) <= c->budget &&
+        alloc_t(c, &c->d_fd, lu_fast_z_bytes(c->n)) != BM_OK)
         c->d_fd = nullptr;
     set_lu_fast(c, c->fast_z && c->d_fd != nullptr);
     if (c->d_dgw) return;

@@ -42,11 +42,13 @@ template <class VC> BM_HD typename VC::cv from_acc(float2 v) {
 
 // VA, VB, VC: storage views of A, B, C; R: arithmetic precision
 template <class VA, class VB, class VC, class R, bool AT, int BM, int BN>
-__global__ void __launch_bounds__(256) cgemm_simt_kernel(int m, int n, int k, VA A, VB B, VC C, R alpha, R beta) {
+__global__ void __launch_bounds__(256) cgemm_simt_kernel(int m, int n, int k, VA A, VB B, VC C, R alpha, R beta,
+                                                         const int* stop) {
     using CV = cplx_t<R>;
     constexpr int TM = BM / 16, TN = BN / 16;
     pdl_wait();
     pdl_trigger();
+    if (stop != nullptr && *stop != 0) return;  // a factorisation that stopped (lu_fast_z.cu)
     __shared__ CV As[BK][BM + 1];
     __shared__ CV Bs[BK][BN + 1];
     const int t = threadIdx.x;
@@ -134,11 +136,12 @@ __global__ void __launch_bounds__(256) cgemm_simt_kernel(int m, int n, int k, VA
 }
 
 template <class VA, class VB, class VC, class R, bool AT>
-cudaError_t launch_impl(cudaStream_t s, int m, int n, int k, VA A, VB B, VC C, R alpha, R beta) {
+cudaError_t launch_impl(cudaStream_t s, int m, int n, int k, VA A, VB B, VC C, R alpha, R beta,
+                        const int* stop = nullptr) {
     if (m <= 0 || n <= 0) return cudaSuccess;
     // every launch may overlap the previous kernel's tail: the kernel waits (pdl_wait) before it
     // reads anything
-    auto go = [&](auto kern, dim3 grid) { return launch_pdl(kern, grid, dim3(256), 0, s, m, n, k, A, B, C, alpha, beta); };
+    auto go = [&](auto kern, dim3 grid) { return launch_pdl(kern, grid, dim3(256), 0, s, m, n, k, A, B, C, alpha, beta, stop); };
     // Few right-hand sides (n <= 80, e.g. 65): one column tile covers them all, so A is streamed
     // once; 32-row tiles when 64-row ones would leave SMs idle.
     if (n > 32 && n <= 80) {
@@ -305,10 +308,10 @@ cudaError_t gemm_z64_skinny(cudaStream_t s, int num_sms, int m, int n, int k, do
 }
 
 cudaError_t gemm_z64(cudaStream_t s, int m, int n, int k, double alpha, Z64 A, bool a_trans, Z64 B, double beta,
-                     Z64 C) {
+                     Z64 C, const int* stop) {
     if (k <= 0 && beta == 1.0) return cudaSuccess;
-    return a_trans ? launch_impl<Z64, Z64, Z64, double, true>(s, m, n, k, A, B, C, alpha, beta)
-                   : launch_impl<Z64, Z64, Z64, double, false>(s, m, n, k, A, B, C, alpha, beta);
+    return a_trans ? launch_impl<Z64, Z64, Z64, double, true>(s, m, n, k, A, B, C, alpha, beta, stop)
+                   : launch_impl<Z64, Z64, Z64, double, false>(s, m, n, k, A, B, C, alpha, beta, stop);
 }
 
 cudaError_t gemm_c32(cudaStream_t s, int m, int n, int k, float alpha, C32 A, bool a_trans, C32 B, float beta,

@@ -21,7 +21,9 @@ cudaError_t launch_pack_solve(cudaStream_t s, const bm_ctx* c);  // [M13; M23] r
 cudaError_t launch_to_c32(cudaStream_t s, const double2* A, long lda, int m, int n, float* Fr, float* Fi, long ldf);
 
 // gemm_simt.cu
-cudaError_t gemm_z64(cudaStream_t s, int m, int n, int k, double alpha, Z64 A, bool a_trans, Z64 B, double beta, Z64 C);
+// (stop: the launch does nothing when this word is not zero)
+cudaError_t gemm_z64(cudaStream_t s, int m, int n, int k, double alpha, Z64 A, bool a_trans, Z64 B, double beta, Z64 C,
+                     const int* stop = nullptr);
 cudaError_t gemm_z64_skinny(cudaStream_t s, int num_sms, int m, int n, int k, double alpha, Z64 A, Z64 B, double beta,
                             Z64 C);
 cudaError_t gemm_c32(cudaStream_t s, int m, int n, int k, float alpha, C32 A, bool a_trans, C32 B, float beta, C32 C);
@@ -83,7 +85,7 @@ bm_status lu_factor_enqueue(bm_ctx* c);       // factor d_F64 / d_F32 in place (
 // continue a factorisation that stopped at a block (the value of its stop word) with the pivot search
 bm_status lu_resume_enqueue(bm_ctx* c, int stop);
 size_t lu_fast_bytes(int n);                  // work buffer of the search-free blocks (d_fd)
-size_t lu_fast_z_bytes();                     // and of the FP64 ones
+size_t lu_fast_z_bytes(int n);                // and of the FP64 ones
 size_t swap_map_bytes();
 constexpr int FLOW_BN = 8;                  // right-hand sides per item of the FP32 triangular solve
 constexpr size_t FLOW_ITEM_BYTES = 64 * FLOW_BN * sizeof(float2);  // an item's 64 rows in its exchange buffer
@@ -166,7 +168,7 @@ struct RtShift {
 };
 // (rowmax: scratch of `rows` words to find the row exponents e with; null: e holds them)
 cudaError_t launch_digits_a(cudaStream_t s, const double2* A, long lda, int rows, int K, int* e, void* D, long ldk,
-                            void* rowmax, int nd, RtShift sh = RtShift{});
+                            void* rowmax, int nd, RtShift sh = RtShift{}, const int* stop = nullptr);
 // |v| as the bits of a non-negative double, which order as the doubles do; infinities and NaN are the largest
 __device__ __forceinline__ unsigned long long mag_bits(double v) {
     return (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
@@ -189,15 +191,16 @@ __device__ __forceinline__ int row_exponent(unsigned long long mx, int zero = 0)
     return m > 0.0 ? ex + 1 : zero;
 }
 cudaError_t launch_digits_x(cudaStream_t s, const double2* X, long ldx, int r0, int K, int n, int npad, int* f,
-                            void* D, long ldk, long plane, int nd, RtShift sh = RtShift{});
+                            void* D, long ldk, long plane, int nd, RtShift sh = RtShift{}, const int* stop = nullptr);
 cudaError_t gemm_rt(cudaStream_t s, const RtArgs* prods, int nprod, int n, double alpha, int* d_err, int* launched,
-                    int nd);
+                    int nd, const int* stop = nullptr);
 
 // FP64 products from nine-digit products (FP64 precision): workspace (0: the CUDA cores are the better
-// place), and C += alpha A B (eA, sh: A's row exponents and the balance of the K entries, if they are there)
+// place), and C += alpha A B (eA, sh: A's row exponents and the balance of the K entries, if they are there; stop:
+// nothing is done when this word is not zero)
 size_t dg_bytes(int m, int n, int K, int num_sms);
 bm_status gemm_z64_dg(cudaStream_t s, void* work, int num_sms, int m, int n, int K, double alpha, Z64 A, Z64 B, Z64 C,
-                      int* d_err, int* eA = nullptr, RtShift sh = RtShift{});
+                      int* d_err, int* eA = nullptr, RtShift sh = RtShift{}, const int* stop = nullptr);
 
 // api.cu: what an FP64 factorisation takes where the budget has room (before any capture); the Schur
 // complement of the FP64 precision into d_F64

@@ -909,10 +909,21 @@ RtShift inner_z(const bm_ctx* c, int J) {
     return sh;
 }
 
+// A[e:, e:] -= A[e:, J:e] A[J:e, e:], by digits on the tensor cores where that is the faster (dg_bytes) and the
+// workspace is there, else on the FP64 pipe.
+bm_status update_z(bm_ctx* c, Z64 F, int J, int c1, int e, const int* stop) {
+    const int m = c->n - e, k = c1 - J;
+    const size_t need = dg_bytes(m, m, k, c->num_sms);
+    if (need > 0 && need <= c->dgw_bytes)
+        return gemm_z64_dg(c->stream, c->d_dgw, c->num_sms, m, m, k, -1.0, F.sub(e, J), F.sub(J, e), F.sub(e, e), c->d_err,
+                           nullptr, inner_z(c, J), stop);
+    LU_CUDA(gemm_z64(c->stream, m, m, k, -1.0, F.sub(e, J), false, F.sub(J, e), 1.0, F.sub(e, e), stop));
+    return BM_OK;
+}
+
 // The FP64 LU in blocks of FZ_BLOCK columns without a pivot search (lu_fast_z.cu), outer blocks of FZ_OUTER:
 // inside one, each block updates the rest of the outer block's columns and rows on the FP64 pipe; then the
-// trailing matrix takes the outer block's product, by digits on the tensor cores where that is the faster
-// (dg_bytes), else on the FP64 pipe.
+// trailing matrix takes the outer block's product.
 bm_status factor_fast_z(bm_ctx* c, Z64 F) {
     const int n = c->n;
     cudaStream_t s = c->stream;
@@ -933,23 +944,17 @@ bm_status factor_fast_z(bm_ctx* c, Z64 F) {
             }
             {
                 BM_PROF(c, "lu_trsm_z_kernel");
-                LU_CUDA(launch_lu_trsm_z(s, F, j, db, mm, work, fail));
+                LU_CUDA(launch_lu_trsm_z(s, F, j, db, mm, work, n, fail));
             }
             if (mm == 0 || e >= je) continue;
             BM_PROF(c, "cgemm_simt_kernel (panel update)");
-            LU_CUDA(gemm_z64(s, mm, je - e, db, -1.0, F.sub(e, j), false, F.sub(j, e), 1.0, F.sub(e, e)));
+            LU_CUDA(gemm_z64(s, mm, je - e, db, -1.0, F.sub(e, j), false, F.sub(j, e), 1.0, F.sub(e, e), fail));
             if (je < n)
-                LU_CUDA(gemm_z64(s, je - e, n - je, db, -1.0, F.sub(e, j), false, F.sub(j, je), 1.0, F.sub(e, je)));
+                LU_CUDA(gemm_z64(s, je - e, n - je, db, -1.0, F.sub(e, j), false, F.sub(j, je), 1.0, F.sub(e, je), fail));
         }
-        const int m = n - je, k = je - J;
-        if (m == 0) break;
+        if (je == n) break;
         BM_PROF(c, "cgemm_simt_kernel (trailing update)");
-        const size_t need = dg_bytes(m, m, k, c->num_sms);
-        if (need > 0 && need <= c->dgw_bytes)
-            BM_TRY(gemm_z64_dg(s, c->d_dgw, c->num_sms, m, m, k, -1.0, F.sub(je, J), F.sub(J, je), F.sub(je, je), c->d_err,
-                               nullptr, inner_z(c, J)));
-        else
-            LU_CUDA(gemm_z64(s, m, m, k, -1.0, F.sub(je, J), false, F.sub(J, je), 1.0, F.sub(je, je)));
+        BM_TRY(update_z(c, F, J, je, je, fail));
     }
     return finish_t<Z64>(c, F, s);
 }
@@ -1208,23 +1213,25 @@ bm_status lu_factor_enqueue(bm_ctx* c) {
 }
 
 bm_status lu_resume_enqueue(bm_ctx* c, int stop) {
-    if (c->prec == BM_FP64) {  // from the start, with the matrix formed again
-        LU_CUDA(cudaMemsetAsync(c->d_info + 4, 0, sizeof(int), c->stream));
-        if (c->form == BM_MIXED)
-            BM_TRY(schur_z64(c, c->stream));
-        else
-            LU_CUDA(launch_copy_z64(c->stream, c->d_A, c->ldA, c->n, c->n, c->d_F64, c->ldF));
-        return factor_t<Z64>(c, Z64{c->d_F64, c->ldF}, false);
+    const int J = (stop >> 1) - 1;
+    LU_CUDA(cudaMemsetAsync(c->d_info + 4, 0, sizeof(int), c->stream));
+    if (c->prec == BM_FP64) {
+        const Z64 F{c->d_F64, c->ldF};
+        const int db = std::min(FZ_BLOCK, c->n - J), o = J / FZ_OUTER * FZ_OUTER, oe = std::min(o + FZ_OUTER, c->n);
+        if (stop & 1)
+            LU_CUDA(launch_lu_restore_z(c->stream, F, J, db, c->n - J - db, reinterpret_cast<double2*>(c->d_fd), c->n));
+        // what lies past the outer block still lacks the products of its blocks before this one
+        if (J > o && oe < c->n) BM_TRY(update_z(c, F, o, J, oe, nullptr));
+        return factor_t<Z64>(c, F, false, J);
     }
     C32 F{c->d_F32r, c->d_F32i, c->ldF};
-    const int J = (stop >> 1) - 1, db = std::min(FD_B, c->n - J);
-    LU_CUDA(cudaMemsetAsync(c->d_info + 4, 0, sizeof(int), c->stream));
+    const int db = std::min(FD_B, c->n - J);
     if (stop & 1) LU_CUDA(launch_lu_restore(c->stream, F, J, db, c->n - J - db, c->d_fd, c->n));
     return factor_t<C32>(c, F, true, J);
 }
 
 size_t lu_fast_bytes(int n) { return fd_work_floats(n) * sizeof(float); }
-size_t lu_fast_z_bytes() { return FZ_T * sizeof(double2); }
+size_t lu_fast_z_bytes(int n) { return fz_work(n) * sizeof(double2); }
 
 // Y holds P B already (rows gathered with d_perm); solves L U X = Y in place.
 bm_status getrs_z64(bm_ctx* c, double2* Y, long ldy, int nrhs) {

@@ -1,7 +1,7 @@
 // FP64 LU with the pivots kept on the diagonal while partial pivoting would keep them there (the FP64
 // counterpart of lu_fast.cu): blocks of 32 columns without a pivot search, every candidate compared with
-// its pivot.  When one is larger (or a pivot is zero or a NaN) *fail is set, the remaining kernels of the
-// sequence return or compute values nobody reads, and the host factors the matrix again with the search.
+// its pivot.  When one is larger (or a pivot is zero or a NaN) *fail names the block, the remaining kernels of the
+// sequence return, and the host restores the block and goes on from it with the search (lu_resume_enqueue).
 //
 // An SM does two FP64 multiply-adds a cycle, so a warp instruction costs 16 cycles of its pipe whatever the
 // number of active lanes: the diagonal block stays small (32 columns, ~20 us on one SM), the solves and the
@@ -168,10 +168,11 @@ __global__ void __launch_bounds__(256, 1) lu_diag_z_kernel(Z64 F, int J, int db,
 
 // L21 = A21 U11^{-1} by rows and U12 = L11^{-1} A12 by columns, x T = a in chunks of 8 entries as in
 // lu_trsm_kernel: a CTA takes 16 rows or columns, eight threads each (one entry of a chunk per thread).
-// FP64-bound: 320 warp instructions per four rows.  The last CTA writes the diagonal block's factors.
+// FP64-bound: 320 warp instructions per four rows.  The last CTA writes the diagonal block's factors.  Every
+// CTA saves what it overwrites.
 constexpr int R = 16;
 __global__ void __launch_bounds__(128) lu_trsm_z_kernel(Z64 F, int J, int db, int mm, const double2* __restrict__ T,
-                                                        int* fail) {
+                                                        double2* __restrict__ bk, long n, int* fail) {
     __shared__ double2 Ts[B * B];
     __shared__ double2 Xs[R][P];
     __shared__ double2 piv_s[B];
@@ -181,12 +182,16 @@ __global__ void __launch_bounds__(128) lu_trsm_z_kernel(Z64 F, int J, int db, in
         if (f != 0 && f != 2 * (J + 1) + 1) return;
     }
     const FzT t(const_cast<double2*>(T));
+    const FzBackup b(bk, n);
     const int nr = (mm + R - 1) / R;
     if ((int)blockIdx.x == 2 * nr) {
 #pragma unroll
         for (int q = 0; q < B / 4; ++q) {
             const int j = warp + 4 * q;
-            if (lane < db && j < db) F.set(J + lane, J + j, t.F[lane * B + j]);
+            if (lane < db && j < db) {
+                b.D[lane + j * B] = F.get(J + lane, J + j);
+                F.set(J + lane, J + j, t.F[lane * B + j]);
+            }
         }
         return;
     }
@@ -201,13 +206,23 @@ __global__ void __launch_bounds__(128) lu_trsm_z_kernel(Z64 F, int J, int db, in
 #pragma unroll
         for (int q = 0; q < B / 8; ++q) {
             const int k = k0 + 8 * q;
-            Xs[r][k] = x0 + r < mm ? F.get(J + B + x0 + r, J + k) : make_double2(0.0, 0.0);
+            double2 v = make_double2(0.0, 0.0);
+            if (x0 + r < mm) {
+                v = F.get(J + B + x0 + r, J + k);
+                b.L[x0 + r + k * n] = v;
+            }
+            Xs[r][k] = v;
         }
     } else {
 #pragma unroll
         for (int q = 0; q < R / 4; ++q) {
             const int c = warp + 4 * q;
-            Xs[c][lane] = x0 + c < mm ? F.get(J + lane, J + B + x0 + c) : make_double2(0.0, 0.0);
+            double2 v = make_double2(0.0, 0.0);
+            if (x0 + c < mm) {
+                v = F.get(J + lane, J + B + x0 + c);
+                b.U[lane + (long)(x0 + c) * B] = v;
+            }
+            Xs[c][lane] = v;
         }
     }
     __syncthreads();
@@ -250,6 +265,23 @@ __global__ void __launch_bounds__(128) lu_trsm_z_kernel(Z64 F, int J, int db, in
     }
 }
 
+// the entries lu_trsm_z_kernel overwrote, back into the matrix
+__global__ void lu_restore_z_kernel(Z64 F, int J, int db, int mm, double2* __restrict__ bk, long n) {
+    const FzBackup b(bk, n);
+    const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long nl = (long)mm * B;
+    if (e < nl) {
+        const long r = e % mm, k = e / mm;
+        F.set(J + B + r, J + k, b.L[r + k * n]);
+    } else if (e < 2 * nl) {
+        const long k = (e - nl) % B, c = (e - nl) / B;
+        F.set(J + k, J + B + c, b.U[k + c * B]);
+    } else if (e - 2 * nl < B * B) {
+        const int i = (int)((e - 2 * nl) % B), j = (int)((e - 2 * nl) / B);
+        if (i < db && j < db) F.set(J + i, J + j, b.D[i + j * B]);
+    }
+}
+
 }  // namespace
 
 cudaError_t launch_lu_diag_z(cudaStream_t s, Z64 F, int J, int db, double2* work, int* fail) {
@@ -257,9 +289,15 @@ cudaError_t launch_lu_diag_z(cudaStream_t s, Z64 F, int J, int db, double2* work
     return cudaGetLastError();
 }
 
-cudaError_t launch_lu_trsm_z(cudaStream_t s, Z64 F, int J, int db, int mm, const double2* work, int* fail) {
+cudaError_t launch_lu_trsm_z(cudaStream_t s, Z64 F, int J, int db, int mm, double2* work, long n, int* fail) {
     if (mm > 0 && db != B) return cudaErrorInvalidValue;
-    lu_trsm_z_kernel<<<2 * ceil_div(mm, R) + 1, 128, 0, s>>>(F, J, db, mm, work, fail);
+    lu_trsm_z_kernel<<<2 * ceil_div(mm, R) + 1, 128, 0, s>>>(F, J, db, mm, work, work + FZ_T, n, fail);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_lu_restore_z(cudaStream_t s, Z64 F, int J, int db, int mm, double2* work, long n) {
+    const long t = 2L * mm * B + B * B;
+    lu_restore_z_kernel<<<ceil_div(t, 256), 256, 0, s>>>(F, J, db, mm, work + FZ_T, n);
     return cudaGetLastError();
 }
 

@@ -518,8 +518,14 @@ struct FzT {
     BM_HD explicit FzT(double2* w)
         : U(w), L(w + FZ_BLOCK * FZ_BLOCK), F(w + 2 * FZ_BLOCK * FZ_BLOCK), piv(w + 3 * FZ_BLOCK * FZ_BLOCK) {}
 };
+struct FzBackup {
+    double2 *D, *L, *U;  // diagonal block; A21 (column-major, ld n); A12 (ld FZ_BLOCK)
+    BM_HD FzBackup(double2* w, long n) : D(w), L(w + FZ_BLOCK * FZ_BLOCK), U(L + n * FZ_BLOCK) {}
+};
+constexpr size_t fz_work(long n) { return FZ_T + FZ_BLOCK * FZ_BLOCK + 2 * (size_t)n * FZ_BLOCK; }  // complex numbers
 cudaError_t launch_lu_diag_z(cudaStream_t s, Z64 F, int J, int db, double2* work, int* fail);
-cudaError_t launch_lu_trsm_z(cudaStream_t s, Z64 F, int J, int db, int mm, const double2* work, int* fail);
+cudaError_t launch_lu_trsm_z(cudaStream_t s, Z64 F, int J, int db, int mm, double2* work, long n, int* fail);
+cudaError_t launch_lu_restore_z(cudaStream_t s, Z64 F, int J, int db, int mm, double2* work, long n);
 int query_cluster_max_c32();
 
 // lu_fast.cu: blocks of FD_B columns whose pivots stay on the diagonal.  The work buffer holds the

@@ -186,7 +186,9 @@ struct RtJob {
     int nprod, n, ntile_n;  // right-hand sides, column tiles
     double alpha;
     int first_unit[3];
+    const int* stop;  // the launch does nothing when this word is not zero
 };
+__device__ __forceinline__ bool stopped(const int* stop) { return stop != nullptr && *stop != 0; }
 
 template <int D>
 __global__ void __launch_bounds__(RT_THREADS, 1) resid_tc_kernel(const __grid_constant__ RtJob J, int* __restrict__ err) {
@@ -194,6 +196,7 @@ __global__ void __launch_bounds__(RT_THREADS, 1) resid_tc_kernel(const __grid_co
     constexpr int RT_D = D, RT_KB_CHUNK = Cfg::KB_CHUNK, RT_X_BUF = Cfg::X_BUF, RT_AST = Cfg::AST;
     constexpr int RT_NT = Cfg::NT, RT_TILE_X = Cfg::TILE_X, RT_A_STAGE = Cfg::A_STAGE, USES = Cfg::USES;
     constexpr bool STACK = Cfg::STACK;
+    if (stopped(J.stop)) return;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* sA = smem;                               // RT_AST stages of digit tiles of A
@@ -461,7 +464,8 @@ __global__ void __launch_bounds__(RT_THREADS, 1) resid_tc_kernel(const __grid_co
 
 // C += alpha sum_z W[z]  (z in order; W: S planes of n columns of m rows, Re and Im)
 __global__ void rt_reduce_kernel(const double* __restrict__ Wr, const double* __restrict__ Wi, int S, int m, int n,
-                                 double alpha, double2* __restrict__ C, long ldc) {
+                                 double alpha, double2* __restrict__ C, long ldc, const int* stop) {
+    if (stopped(stop)) return;
     const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
     const long zs = (long)m * n;
     if (idx >= zs) return;
@@ -480,9 +484,9 @@ __global__ void rt_reduce_kernel(const double* __restrict__ Wr, const double* __
 // 256 columns, combined by an atomic maximum on the bit patterns (non-negative doubles order as
 // their bits).  mx must start at zero.
 __global__ void row_max_kernel(const double2* __restrict__ A, long lda, int rows, int K,
-                               unsigned long long* __restrict__ mx, RtShift sh) {
+                               unsigned long long* __restrict__ mx, RtShift sh, const int* stop) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= rows) return;
+    if (i >= rows || stopped(stop)) return;
     const int j0 = blockIdx.y * 256, j1 = min(K, j0 + 256);
     // (integer maxima: FP64 compares run on the narrow FP64 pipe)
     unsigned long long m = 0;
@@ -552,7 +556,8 @@ __device__ __forceinline__ unsigned bf16_pair(float a, float b) {
 template <int ND>
 __global__ void __launch_bounds__(256) digits_a_kernel(const double2* __restrict__ A, long lda, int rows, int K,
                                                        const int* __restrict__ e, unsigned* __restrict__ D, long ldk,
-                                                       long plane, RtShift sh) {
+                                                       long plane, RtShift sh, const int* stop) {
+    if (stopped(stop)) return;
     __shared__ double2 t[32][65];
     const int k0 = blockIdx.x * 64, r0 = blockIdx.y * 32;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -586,7 +591,8 @@ __global__ void __launch_bounds__(256) digits_a_kernel(const double2* __restrict
 
 // Column exponents of x over rows [r0, r0 + K) for the n columns (one block per column).
 __global__ void col_exponent_kernel(const double2* __restrict__ X, long ldx, int r0, int K, int* __restrict__ f,
-                                    RtShift sh) {
+                                    RtShift sh, const int* stop) {
+    if (stopped(stop)) return;
     const int c = blockIdx.x;
     unsigned long long mx = 0;
     for (int i = threadIdx.x; i < K; i += blockDim.x) {
@@ -608,7 +614,8 @@ __global__ void col_exponent_kernel(const double2* __restrict__ X, long ldx, int
 template <int ND>
 __global__ void digits_x_kernel(const double2* __restrict__ X, long ldx, int r0, int K, int n, int npad,
                                 const int* __restrict__ f, unsigned* __restrict__ D, long ldk, long plane,
-                                RtShift sh) {
+                                RtShift sh, const int* stop) {
+    if (stopped(stop)) return;
     constexpr bool STACK = ND > 7;
     const int Kp = (K + 1) / 2;
     const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -723,28 +730,29 @@ int rt_col_tile(int nd) { return nd <= 7 ? RtCfg<7>::NT : RtCfg<9>::NT; }
 
 // Row exponents (unless rowmax is null: they are there) and digit planes of A.
 cudaError_t launch_digits_a(cudaStream_t s, const double2* A, long lda, int rows, int K, int* e, void* D, long ldk,
-                            void* rowmax, int nd, RtShift sh) {
+                            void* rowmax, int nd, RtShift sh, const int* stop) {
     if (rows <= 0 || K <= 0) return cudaSuccess;
     unsigned long long* mx = reinterpret_cast<unsigned long long*>(rowmax);
     if (mx != nullptr) {
         cudaError_t err = cudaMemsetAsync(mx, 0, (size_t)rows * 8, s);
         if (err != cudaSuccess) return err;
-        row_max_kernel<<<dim3(ceil_div(rows, 128), ceil_div(K, 256)), 128, 0, s>>>(A, lda, rows, K, mx, sh);
+        row_max_kernel<<<dim3(ceil_div(rows, 128), ceil_div(K, 256)), 128, 0, s>>>(A, lda, rows, K, mx, sh, stop);
         row_exponent_kernel<<<ceil_div(rows, 128), 128, 0, s>>>(mx, rows, e);
     }
     const dim3 grid(ceil_div(K, 64), ceil_div(rows, 32));
     auto kern = nd <= 7 ? digits_a_kernel<7> : digits_a_kernel<9>;
-    kern<<<grid, 256, 0, s>>>(A, lda, rows, K, e, reinterpret_cast<unsigned*>(D), ldk, (long)rows * ldk, sh);
+    kern<<<grid, 256, 0, s>>>(A, lda, rows, K, e, reinterpret_cast<unsigned*>(D), ldk, (long)rows * ldk, sh, stop);
     return cudaGetLastError();
 }
 
 cudaError_t launch_digits_x(cudaStream_t s, const double2* X, long ldx, int r0, int K, int n, int npad, int* f,
-                            void* D, long ldk, long plane, int nd, RtShift sh) {
+                            void* D, long ldk, long plane, int nd, RtShift sh, const int* stop) {
     if (n <= 0 || K <= 0) return cudaSuccess;
-    col_exponent_kernel<<<n, 256, 0, s>>>(X, ldx, r0, K, f, sh);
+    col_exponent_kernel<<<n, 256, 0, s>>>(X, ldx, r0, K, f, sh, stop);
     const long t = (long)npad * ((K + 1) / 2);
     auto kern = nd <= 7 ? digits_x_kernel<7> : digits_x_kernel<9>;
-    kern<<<ceil_div(t, 256L), 256, 0, s>>>(X, ldx, r0, K, n, npad, f, reinterpret_cast<unsigned*>(D), ldk, plane, sh);
+    kern<<<ceil_div(t, 256L), 256, 0, s>>>(X, ldx, r0, K, n, npad, f, reinterpret_cast<unsigned*>(D), ldk, plane, sh,
+                                           stop);
     return cudaGetLastError();
 }
 
@@ -770,7 +778,7 @@ void rt_plan_splits(int nprod, const long* m, const long* K, int n, int nd, int 
 // The products of one residual (at most two, sharing n and alpha): C += alpha A x each.  A product
 // with S > 1 K splits writes S m n doubles (Re and Im) to its workspace, reduced in order afterwards.
 cudaError_t gemm_rt(cudaStream_t s, const RtArgs* prods, int nprod, int n, double alpha, int* d_err, int* launched,
-                    int nd) {
+                    int nd, const int* stop) {
     if (nprod < 1 || nprod > 2 || n <= 0 || (nd != 7 && nd != 9)) return cudaSuccess;
     static DeviceFlags attr7, attr9;
     if (nd == 7 && attr7.pending()) {
@@ -790,6 +798,7 @@ cudaError_t gemm_rt(cudaStream_t s, const RtArgs* prods, int nprod, int n, doubl
     J.n = n;
     J.ntile_n = ceil_div(n, rt_col_tile(nd));
     J.alpha = alpha;
+    J.stop = stop;
     int u = 0;
     for (int q = 0; q < 2; ++q) {
         J.first_unit[q] = u;
@@ -822,7 +831,7 @@ cudaError_t gemm_rt(cudaStream_t s, const RtArgs* prods, int nprod, int n, doubl
         const RtArgs& a = prods[q];
         if (a.S > 1 && a.m > 0 && a.K > 0) {
             const long t = (long)a.m * n;
-            rt_reduce_kernel<<<ceil_div(t, 256L), 256, 0, s>>>(a.Wr, a.Wi, a.S, a.m, n, alpha, a.C, a.ldc);
+            rt_reduce_kernel<<<ceil_div(t, 256L), 256, 0, s>>>(a.Wr, a.Wi, a.S, a.m, n, alpha, a.C, a.ldc, stop);
             *launched += 1;
         }
     }
@@ -874,7 +883,7 @@ size_t dg_bytes(int m, int n, int K, int num_sms) {
 }
 
 bm_status gemm_z64_dg(cudaStream_t s, void* work, int num_sms, int m, int n, int K, double alpha, Z64 A, Z64 B, Z64 C,
-                      int* d_err, int* eA, RtShift sh) {
+                      int* d_err, int* eA, RtShift sh, const int* stop) {
     const DgPlan p = dg_plan(m, n, K, num_sms);
     const int nt = rt_col_tile(DG_ND);
     const long ldk = rt_ldk(K);
@@ -890,12 +899,12 @@ bm_status gemm_z64_dg(cudaStream_t s, void* work, int num_sms, int m, int n, int
     for (int i0 = 0; i0 < m; i0 += p.mr) {
         const int mr = std::min(p.mr, m - i0);
         int* const er = eA != nullptr ? eA + i0 : ea;
-        BM_CUDA_TRY(launch_digits_a(s, A.p + i0, A.ld, mr, K, er, ap, ldk, eA != nullptr ? nullptr : rmax, DG_ND, sh));
+        BM_CUDA_TRY(launch_digits_a(s, A.p + i0, A.ld, mr, K, er, ap, ldk, eA != nullptr ? nullptr : rmax, DG_ND, sh, stop));
         BM_TRY(rt_make_map(tma, ap, mr, K, ldk, (long)mr * ldk, RT_BM, DG_ND));
         for (int j0 = 0; j0 < n; j0 += p.nc) {
             const int nc = std::min(p.nc, n - j0);
             BM_CUDA_TRY(launch_digits_x(s, B.p + (long)j0 * B.ld, B.ld, 0, K, nc, ceil_div(nc, nt) * nt, fx, xp, ldk,
-                                        (long)p.nc * ldk, DG_ND, sh));
+                                        (long)p.nc * ldk, DG_ND, sh, stop));
             const long mq = mr, kq = K;
             int S = 1, nl = 0;
             rt_plan_splits(1, &mq, &kq, nc, DG_ND, num_sms, &S);
@@ -905,7 +914,7 @@ bm_status gemm_z64_dg(cudaStream_t s, void* work, int num_sms, int m, int n, int
                 a.Wr = ws;
                 a.Wi = ws + (size_t)S * mr * nc;
             }
-            BM_CUDA_TRY(gemm_rt(s, &a, 1, nc, alpha, d_err, &nl, DG_ND));
+            BM_CUDA_TRY(gemm_rt(s, &a, 1, nc, alpha, d_err, &nl, DG_ND, stop));
         }
     }
     return BM_OK;
