@@ -65,13 +65,10 @@ cudaMemPool_t device_pool(int dev) {
 }
 }  // namespace
 
-namespace {
-void dg_release(bm_ctx* c);
-}
 bm_status ctx_alloc(bm_ctx* c, void** p, size_t bytes) {
     *p = nullptr;
     if (bytes == 0) return BM_OK;
-    if (c->held + bytes > c->budget && c->d_dgw) dg_release(c);
+    if (c->held + bytes > c->budget) opt_release(c, c->held + bytes - c->budget);
     if (c->held + bytes > c->budget) {
         bm_set_error("allocation of " + std::to_string(bytes) + " bytes exceeds the HBM budget");
         return BM_ENOMEM;
@@ -84,9 +81,9 @@ bm_status ctx_alloc(bm_ctx* c, void** p, size_t bytes) {
         return pool ? cudaMallocFromPoolAsync(p, bytes, pool, c->stream) : cudaMallocAsync(p, bytes, c->stream);
     };
     cudaError_t e = get();
-    if (e != cudaSuccess && c->d_dgw) {
+    if (e != cudaSuccess && (c->d_dgw || c->d_fd)) {
         cudaGetLastError();
-        dg_release(c);
+        opt_release(c, ~(size_t)0);
         e = get();
     }
     if (e != cudaSuccess) {
@@ -141,14 +138,6 @@ void set_lu_fast(bm_ctx* c, bool fast) {
     drop_slot(c->g_lu);
 }
 
-// Gives the optional workspace of the FP64 factorisation back (with the graphs that use it).
-void dg_release(bm_ctx* c) {
-    drop_slot(c->g_factor);
-    drop_slot(c->g_lu);
-    FREE(c->d_dgw);
-    c->dgw_bytes = 0;
-}
-
 void drop_solve_graphs(bm_ctx* c) {
     for (auto& kv : c->g_solve) drop_slot(kv.second);
     c->g_solve.clear();
@@ -197,6 +186,7 @@ void free_solve_ws(bm_ctx* c) {
     c->pk_elems = 0;
     c->ws_nrhs = 0;
     c->last_nrhs = 0;
+    c->ws_held = 0;
     drop_solve_graphs(c);
 }
 
@@ -238,12 +228,12 @@ void free_problem(bm_ctx* c) {
     FREE(c->d_Cp_r);
     FREE(c->d_Cp_i);
     FREE(c->d_fd);
+    c->fd_bytes = 0;
     for (int q = 0; q < 2; ++q) {
         FREE(c->d_dg[q]);
         FREE(c->d_dge[q]);
     }
     c->assembled = c->factored = c->singular = false;
-    c->fast_denied = false;
     c->tm_ok = false;
     c->tc_skinny = false;
 }
@@ -262,8 +252,14 @@ int planes_needed(int form, int prec, int resid_mode) {
     return form == BM_ORDINARY ? 1 : 0;
 }
 
-// fast: the FP32 LU in search-free blocks (lu_fast.cu), with its work buffer
-Plan make_plan(int N, int form, int prec, int nb_user, int bs, int nd, bool fast, int planes) {
+// Digits of the tensor-core residual (0: the mode forms its residuals elsewhere).
+int digits_of(int resid_mode) {
+    return resid_mode == BM_RESID_TC_ALL ? 9 : (resid_mode == BM_RESID_TC_UPDATE ? 7 : 0);
+}
+// Rows of an inverted diagonal block of the triangular solves.
+int solve_block(int prec) { return prec == BM_FP64 ? 16 : 64; }
+
+Plan make_plan(int N, int form, int prec, int nb_user, int bs, int nd, int planes) {
     Plan p;
     const bool c32 = prec != BM_FP64;
     p.n = (form == BM_MIXED) ? N : 2 * N;
@@ -293,19 +289,20 @@ Plan make_plan(int N, int form, int prec, int nb_user, int bs, int nd, bool fast
             p.ldk_c = tc_ldk(N);
             b += 2 * (size_t)N * p.ldk_c * 4;
         }
-        // packs of the trailing updates and the search-free blocks' work buffer
-        p.ldk_lu = tc_ldk(fast ? std::max(p.nb, 128) : p.nb);
+        // packs of the trailing updates (of the search-free LU's blocks too: its block size is the default)
+        p.ldk_lu = tc_ldk(p.nb);
         b += 2 * (size_t)p.n * p.ldk_lu * 4 + 2 * (size_t)p.n * 4;
-        if (fast) b += lu_fast_bytes(p.n);
-        // digit planes of the operator for the tensor-core residual and their row exponents
-        const size_t planes = (size_t)rt_digit_planes(nd) * 2;
+        // the operator's row exponents, and its digit planes where the tensor cores form residuals
+        b += (form == BM_MIXED ? 3L : 2L) * N * 4;
+        const size_t planes = nd > 0 ? (size_t)rt_digit_planes(nd) * 2 : 0;
         if (form == BM_MIXED)
-            b += planes * (2L * N * rt_ldk(N) + (size_t)N * rt_ldk(2L * N)) + 3L * N * 4;
+            b += planes * (2L * N * rt_ldk(N) + (size_t)N * rt_ldk(2L * N));
         else
-            b += planes * 2L * N * rt_ldk(2L * N) + 2L * N * 4;
+            b += planes * 2L * N * rt_ldk(2L * N);
     }
     if (form == BM_MIXED) b += (size_t)N * 4 + bal_ints(N) * 4;  // the balance of the Schur product
     else if (!c32) b += 2 * (size_t)N * 4;                       // the row exponents
+    // pivots and rows; inverted diagonal blocks of bs x bs
     p.nblk = ceil_div(p.n, bs);
     b += 2 * (size_t)p.n * 4;
     b += 2 * (size_t)p.nblk * bs * bs * (c32 ? 8 : 16);
@@ -315,11 +312,17 @@ Plan make_plan(int N, int form, int prec, int nb_user, int bs, int nd, bool fast
 
 }  // namespace
 
-// Digit workspace of an FP64 factorisation: the Schur complement's, and the first trailing update's
-static size_t dg_request(int N, int form, bool fast, int num_sms) {
+// Optional workspaces: the search-free LU's, and the FP64 digit products' (the Schur complement's, and the first
+// trailing update's)
+static size_t fd_request(int N, int form, int prec) {
+    const int n = form == BM_MIXED ? N : 2 * N;
+    return prec == BM_FP64 ? lu_fast_z_bytes(n) : lu_fast_bytes(n);
+}
+static size_t dg_request(int N, int form, int prec, int num_sms) {
+    if (prec != BM_FP64) return 0;
     size_t b = form == BM_MIXED ? dg_bytes(N, N, 2 * N, num_sms) : 0;
     const int m = (form == BM_MIXED ? N : 2 * N) - 128;
-    if (fast && m > 0) b = std::max(b, dg_bytes(m, m, 128, num_sms));
+    if (m > 0) b = std::max(b, dg_bytes(m, m, 128, num_sms));
     return b;
 }
 
@@ -328,9 +331,8 @@ static size_t dg_request(int N, int form, bool fast, int num_sms) {
 // margin for the split-K partial sums).  optional: with what a handle also takes when its budget has room
 // (the search-free LU's buffers, the FP64 digit workspace).
 size_t request_bytes(int N, int form, int prec, int nb, int nrhs, int resid_mode, bool optional, int num_sms) {
-    Plan p = make_plan(N, form, prec, nb, 64, 9, optional && prec != BM_FP64 && nb == 0,
-                       planes_needed(form, prec, resid_mode));
-    if (optional && prec == BM_FP64) p.bytes += dg_request(N, form, true, num_sms) + lu_fast_z_bytes(p.n);
+    Plan p = make_plan(N, form, prec, nb, solve_block(prec), digits_of(resid_mode), planes_needed(form, prec, resid_mode));
+    if (optional) p.bytes += (nb == 0 ? fd_request(N, form, prec) : 0) + dg_request(N, form, prec, num_sms);
     const size_t w = (size_t)std::max(nrhs, 8);
     size_t b = p.bytes + 7 * (size_t)N * 8 + (size_t)p.nsys * w * 16 * 3 + (size_t)p.n * w * 16 * 2;
     if (prec == BM_FP64) {
@@ -581,32 +583,26 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
     BM_CUDA_TRY(cudaSetDevice(c->device));
     cudaStreamSynchronize(c->stream);
     const int rmode = opts ? opts->refine_residual : BM_RESID_TC_UPDATE;
-    const int nd = rmode == BM_RESID_TC_ALL ? 9 : 7;
+    const int nd = digits_of(rmode);
     // LU in search-free blocks, unless a block size or a panel setting asks for the panels (the contour
     // solver's deferred assembly sets a cluster size for what its factorisations continue with)
-    const bool fast = prec != BM_FP64 && nb == 0 && pkern == 0 && (cl_cap == 0 || defer_kernels);
+    const bool fast = nb == 0 && pkern == 0 && (cl_cap == 0 || defer_kernels);
     const int planes = planes_needed(form, prec, rmode);
-    Plan p = make_plan(N, form, prec, nb, 64, nd, fast, planes);
+    Plan p = make_plan(N, form, prec, nb, solve_block(prec), nd, planes);
     // Same shape as the assembled system: assemble again into the same buffers (no device
     // allocation or release - cudaFree would wait for every stream of the device - and the cached
     // graphs and tensor maps stay valid, as they depend only on these pointers and sizes).
     const bool reuse = c->assembled && c->N == N && c->form == form && c->prec == prec && c->nb == p.nb &&
-                       (prec == BM_FP64 || (c->d_fd != nullptr || c->fast_denied) == fast) && c->rt_nd == nd && c->planes == planes &&
-                       curve->kind != BM_CURVE_USER;
-    if (!reuse) {
-        free_problem(c);
-        // a budget without room for the search-free LU's buffers keeps the panels
-        c->fast_denied = fast && c->held + p.bytes > c->budget;
-    }
-    if (c->fast_denied) p = make_plan(N, form, prec, nb, 64, nd, false, planes);
+                       c->rt_nd == nd && c->planes == planes && curve->kind != BM_CURVE_USER;
+    if (!reuse) free_problem(c);
     // the captured factorisation depends on the launch settings: capture again when they change
     if (reuse && (eager != c->eager || cl_cap != c->opt_cluster_cap || pkern != c->opt_panel_kernel)) drop_graphs(c);
     c->eager = eager;
     c->opt_cluster_cap = cl_cap;
     c->opt_panel_kernel = pkern;
-    c->fast_z = prec == BM_FP64 && nb == 0 && pkern == 0 && (cl_cap == 0 || defer_kernels);
-    set_lu_fast(c, prec == BM_FP64 ? c->fast_z && c->d_fd != nullptr : fast && !c->fast_denied);
-    c->bs_solve = 64;
+    c->want_fast = fast;
+    set_lu_fast(c, fast && c->d_fd != nullptr && !c->no_optional);
+    c->bs_solve = solve_block(prec);
     if (!reuse && c->held + p.bytes > c->budget) {
         bm_set_error("admission: system needs " + std::to_string(p.bytes) + " bytes, budget leaves " +
                      std::to_string(c->budget - c->held));
@@ -683,19 +679,14 @@ bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, b
         if (s == BM_OK) s = alloc_t(c, &c->d_Up_i, lb);
         if (s == BM_OK) s = alloc_t(c, &c->d_Lpe, (size_t)p.n * 4);
         if (s == BM_OK) s = alloc_t(c, &c->d_Upe, (size_t)p.n * 4);
-        if (s == BM_OK && c32 && c->lu_fast) s = alloc_t(c, &c->d_fd, lu_fast_bytes(p.n));
     }
     if (s == BM_OK && c32) {
         // [0] Mtop (2N x N) or A (2N x 2N), [1] Mbot (N x 2N)
-        const int np = rt_digit_planes(nd);
-        const long rows0 = 2L * N, k0 = (form == BM_MIXED) ? N : 2L * N;
-        c->dg_ldk[0] = rt_ldk(k0);
-        s = alloc_t(c, &c->d_dg[0], (size_t)np * rows0 * c->dg_ldk[0] * 2);
-        if (s == BM_OK) s = alloc_t(c, &c->d_dge[0], (size_t)rows0 * 4);
-        if (s == BM_OK && form == BM_MIXED) {
-            c->dg_ldk[1] = rt_ldk(2L * N);
-            s = alloc_t(c, &c->d_dg[1], (size_t)np * N * c->dg_ldk[1] * 2);
-            if (s == BM_OK) s = alloc_t(c, &c->d_dge[1], (size_t)N * 4);
+        for (int q = 0; q < (form == BM_MIXED ? 2 : 1) && s == BM_OK; ++q) {
+            const long rows = q == 0 ? 2L * N : N, K = form == BM_MIXED && q == 0 ? N : 2L * N;
+            s = alloc_t(c, &c->d_dge[q], (size_t)rows * 4);
+            c->dg_ldk[q] = rt_ldk(K);
+            if (s == BM_OK && nd > 0) s = alloc_t(c, &c->d_dg[q], (size_t)rt_digit_planes(nd) * rows * c->dg_ldk[q] * 2);
         }
     }
     if (s == BM_OK) s = alloc_t(c, &c->d_ipiv, (size_t)p.n * 4);
@@ -777,16 +768,19 @@ bm_status assemble_post(bm_ctx* c, bool run_assembly_kernel, bool wait) {
             c->launches += 1;
         }
         // digit planes of the operator for the tensor-core residual
-        if (form == BM_MIXED) {
+        if (nd > 0 && form == BM_MIXED) {
             BM_CUDA_TRY(launch_digits_a(st, c->d_Mtop, c->ldtop, 2 * N, N, c->d_dge[0], c->d_dg[0], c->dg_ldk[0], nullptr,
                                         nd));
             BM_CUDA_TRY(launch_digits_a(st, c->d_Mbot, c->ldbot, N, 2 * N, c->d_dge[1], c->d_dg[1], c->dg_ldk[1], nullptr,
                                         nd));
-            BM_CUDA_TRY(launch_pack_solve(st, c));
-            c->launches += 3;
-        } else {
+            c->launches += 2;
+        } else if (nd > 0) {
             BM_CUDA_TRY(launch_digits_a(st, c->d_A, c->ldA, 2 * N, 2 * N, c->d_dge[0], c->d_dg[0], c->dg_ldk[0], nullptr,
                                         nd));
+            c->launches += 1;
+        }
+        if (form == BM_MIXED) {
+            BM_CUDA_TRY(launch_pack_solve(st, c));
             c->launches += 1;
         }
     }
@@ -806,7 +800,7 @@ bm_status assemble_post(bm_ctx* c, bool run_assembly_kernel, bool wait) {
             BM_TRY(tc_make_map(c->tm_skinny[1], c->d_Cp_i, 2L * N, N, p.ldk_c, TC_BM));
             c->tc_skinny = true;
         }
-        {
+        if (nd > 0) {
             const long rows0 = 2L * N, k0 = (form == BM_MIXED) ? N : 2L * N;
             BM_TRY(rt_make_map(c->tm_dg[0], c->d_dg[0], rows0, k0, c->dg_ldk[0], rows0 * c->dg_ldk[0], 128, nd));
             if (form == BM_MIXED)
@@ -827,18 +821,40 @@ bm_status assemble_post(bm_ctx* c, bool run_assembly_kernel, bool wait) {
     return BM_OK;
 }
 
-// Reserves, where the budget and the device have room, the small buffer of the search-free FP64 blocks
-// (without it the panels search) and the digit workspace (without it the products run on the CUDA cores).
-void dg_reserve(bm_ctx* c) {
-    if (c->prec != BM_FP64) return;
-    if (c->fast_z && !c->d_fd && c->held + lu_fast_z_bytes(c->n) <= c->budget &&
-        alloc_t(c, &c->d_fd, lu_fast_z_bytes(c->n)) != BM_OK)
-        c->d_fd = nullptr;
-    set_lu_fast(c, c->fast_z && c->d_fd != nullptr);
-    if (c->d_dgw) return;
-    const size_t b = dg_request(c->N, c->form, c->lu_fast, c->num_sms);
-    if (b == 0 || c->held + b > c->budget) return;
-    if (alloc_t(c, &c->d_dgw, b) == BM_OK) c->dgw_bytes = b;
+// Gives optional workspaces back, with the graphs that use them, until `bytes` are free: the digit workspace (its
+// products run on the CUDA cores without it), then the search-free LU's buffer (the panels search without it).
+void opt_release(bm_ctx* c, size_t bytes) {
+    const size_t held = c->held;
+    if (c->d_dgw && bytes > 0) {
+        drop_slot(c->g_factor);
+        drop_slot(c->g_lu);
+        FREE(c->d_dgw);
+        c->dgw_bytes = 0;
+    }
+    if (c->d_fd && held - c->held < bytes) {
+        set_lu_fast(c, false);
+        FREE(c->d_fd);
+        c->fd_bytes = 0;
+    }
+}
+
+// Takes the optional workspaces that the budget has room for beside the system alone: a solve workspace in the way
+// goes (the next solve makes it again), so that a factorisation does not depend on what the handle solved before.
+void opt_reserve(bm_ctx* c) {
+    const size_t base = c->held - c->ws_held - c->fd_bytes - c->dgw_bytes;
+    size_t fd = c->want_fast && !c->no_optional ? fd_request(c->N, c->form, c->prec) : 0;
+    if (base + fd > c->budget) fd = 0;
+    size_t dg = c->no_optional ? 0 : dg_request(c->N, c->form, c->prec, c->num_sms);
+    if (base + fd + dg > c->budget) dg = 0;
+    const size_t more = (c->d_fd ? 0 : fd) + (c->d_dgw ? 0 : dg);
+    if (c->held + more > c->budget) free_solve_ws(c);
+    if (fd > 0 && !c->d_fd && alloc_t(c, &c->d_fd, fd) == BM_OK) c->fd_bytes = fd;
+    if (dg > 0 && !c->d_dgw && alloc_t(c, &c->d_dgw, dg) == BM_OK) {
+        c->dgw_bytes = dg;
+        drop_slot(c->g_factor);
+        drop_slot(c->g_lu);
+    }
+    set_lu_fast(c, fd > 0 && c->d_fd != nullptr);
 }
 
 bm_status schur_z64(bm_ctx* c, cudaStream_t s) {
@@ -995,7 +1011,7 @@ extern "C" bm_status bm_factor(bm_ctx* c, int* info) {
         return BM_ESTATE;
     }
     BM_CUDA_TRY(cudaSetDevice(c->device));
-    dg_reserve(c);
+    opt_reserve(c);
     BM_TRY(run_captured(c, &c->g_factor, [&]() { return factor_sequence(c); }));
     return factor_result(c, info);
 }
@@ -1003,18 +1019,27 @@ extern "C" bm_status bm_factor(bm_ctx* c, int* info) {
 // ------------------------------------------------------------------------------------------------
 namespace {
 
+bm_status make_ws(bm_ctx* c, int nrhs);
 bm_status ensure_ws(bm_ctx* c, int nrhs) {
     if (nrhs <= c->ws_nrhs) return BM_OK;
     free_solve_ws(c);
+    auto others = [&]() { return c->held - c->fd_bytes - c->dgw_bytes; };  // (optional workspaces may go meanwhile)
+    const size_t before = others();
+    const bm_status s = make_ws(c, nrhs);
+    c->ws_held = others() - before;
+    return s;
+}
+
+bm_status make_ws(bm_ctx* c, int nrhs) {
     int w = std::max(nrhs, 8);
     size_t zb = (size_t)c->nsys * w * 16;
     BM_TRY(alloc_t(c, &c->d_X, zb));
     BM_TRY(alloc_t(c, &c->d_R, zb));
     BM_TRY(alloc_t(c, &c->d_Bw, zb));
-    size_t yb = (size_t)c->n * w * 16;
-    BM_TRY(alloc_t(c, &c->d_Y64, yb));
-    BM_TRY(alloc_t(c, &c->d_Y64b, yb));
     if (c->prec == BM_FP64) {
+        const size_t yb = (size_t)c->n * w * 16;
+        BM_TRY(alloc_t(c, &c->d_Y64, yb));
+        BM_TRY(alloc_t(c, &c->d_Y64b, yb));
         BM_TRY(alloc_t(c, &c->d_Zw64, yb));
         c->flow_len = 2L * ceil_div(c->n, 16) * ceil_div(w, 4);  // two triangles x (16-row tiles) x (4-column tiles)
         BM_TRY(alloc_t(c, &c->d_flow, (size_t)c->flow_len * sizeof(int)));
@@ -1038,7 +1063,7 @@ bm_status ensure_ws(bm_ctx* c, int nrhs) {
         BM_TRY(alloc_t(c, &c->d_flowx, fx));
         BM_CUDA_TRY(cudaMemsetAsync(c->d_flowx, 0xff, fx, c->stream));
     }
-    if (c->prec != BM_FP64) {
+    if (c->prec != BM_FP64 && c->rt_nd > 0) {
         // x digit planes and split-K workspace of the tensor-core residual
         const int N = c->N, np = rt_x_planes(c->rt_nd);
         const int npad = (int)round_up(w, rt_col_tile(c->rt_nd));

@@ -290,8 +290,14 @@ struct bm_ctx {
 
     // factorisation storage
     double2* d_F64 = nullptr;  // FP64 LU (n x n, ld ldF)
-    void* d_dgw = nullptr;     // FP64: workspace of the digit products of the factorisation.  Optional: it
-    size_t dgw_bytes = 0;      //   is given back when another allocation needs the room (ctx_alloc)
+    // Optional workspaces: taken at bm_factor where the budget has room beside the system (opt_reserve) and given
+    // back when another allocation needs it (opt_release).
+    void* d_dgw = nullptr;     // FP64: digit products of the factorisation
+    size_t dgw_bytes = 0;
+    float* d_fd = nullptr;     // work buffer of the LU without a pivot search (lu_fast.cu, lu_fast_z.cu)
+    size_t fd_bytes = 0;
+    bool no_optional = false;  // none are taken (a server request admitted without them)
+    size_t ws_held = 0;        // bytes of the solve workspace
     float* d_F32r = nullptr;   // FP32 planar LU
     float* d_F32i = nullptr;
     long ldF = 0;
@@ -299,10 +305,8 @@ struct bm_ctx {
     int* d_perm = nullptr;
     int* d_info = nullptr;
     int* d_err = nullptr;      // d_info + 1; d_info[2..3] test hooks, d_info[4] stop word of lu_fast.cu
-    bool lu_fast = false;      // FP32 LU in blocks without a pivot search (lu_fast.cu) and their
-    float* d_fd = nullptr;     //   work buffer: the default, unless bm_opts.nb or a panel setting is set
-    bool fast_z = false;       // FP64: the same (lu_fast_z.cu), where dg_reserve finds room
-    bool fast_denied = false;  //   or the budget has no room for the buffer
+    bool want_fast = false;    // LU without a pivot search: the default, unless bm_opts.nb or a panel setting is set
+    bool lu_fast = false;      // and its work buffer is there
     void* d_maps = nullptr;    // row-interchange maps used by the factorisation: big panel (even),
                                // sub-panel, big panel (odd)
     // look-ahead of the FP32 factorisation: the panel chain on la_hi (high priority), the rest of

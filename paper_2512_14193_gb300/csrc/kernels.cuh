@@ -202,9 +202,10 @@ size_t dg_bytes(int m, int n, int K, int num_sms);
 bm_status gemm_z64_dg(cudaStream_t s, void* work, int num_sms, int m, int n, int K, double alpha, Z64 A, Z64 B, Z64 C,
                       int* d_err, int* eA = nullptr, RtShift sh = RtShift{}, const int* stop = nullptr);
 
-// api.cu: what an FP64 factorisation takes where the budget has room (before any capture); the Schur
+// api.cu: what a factorisation takes where the budget has room (before any capture), and gives back; the Schur
 // complement of the FP64 precision into d_F64
-void dg_reserve(bm_ctx* c);
+void opt_reserve(bm_ctx* c);
+void opt_release(bm_ctx* c, size_t bytes);
 bm_status schur_z64(bm_ctx* c, cudaStream_t s);
 // api.cu: assembly in two halves (the batched contour solver assembles many handles at once)
 bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, bm_c64 k_in, bm_formulation form,

@@ -26,6 +26,7 @@ struct Job {
     unsigned long long id;
     bm_request req;
     size_t bytes;
+    bool optional;  // admitted with the optional workspaces
     clk::time_point t_submit;
 };
 
@@ -59,6 +60,7 @@ bm_result run_request(bm_server* s, int slot, const Job& j) {
     bm_result res{};
     res.slot = slot;
     res.bytes = j.bytes;
+    h->no_optional = !j.optional;
     bm_status st = bm_assemble(h, &r.curve, r.N, r.k_out, r.k_in, (bm_formulation)r.formulation, &s->opts);
     int info = 0;
     if (st == BM_OK) st = bm_factor(h, &info);
@@ -145,7 +147,8 @@ extern "C" bm_status bm_server_submit(bm_server* s, const bm_request* r, unsigne
     if (r->ldb < nsys || r->ldx < nsys) return BM_EINVAL;
     const int sms = s->handles[0]->num_sms;
     size_t bytes = request_bytes(r->N, r->formulation, s->opts.prec, s->opts.nb, r->nrhs, s->opts.refine_residual, true, sms);
-    if (bytes > s->budget)
+    const bool optional = bytes <= s->budget;
+    if (!optional)
         bytes = request_bytes(r->N, r->formulation, s->opts.prec, s->opts.nb, r->nrhs, s->opts.refine_residual, false, sms);
     if (bytes > s->budget) {
         bm_set_error("bm_server_submit: the request needs " + std::to_string(bytes) + " bytes, more than the budget " +
@@ -155,7 +158,7 @@ extern "C" bm_status bm_server_submit(bm_server* s, const bm_request* r, unsigne
     {
         std::lock_guard<std::mutex> lk(s->mu);
         if (s->stopping) return BM_ESTATE;
-        Job j{s->next_id++, *r, bytes, clk::now()};
+        Job j{s->next_id++, *r, bytes, optional, clk::now()};
         *ticket = j.id;
         s->queue.push_back(j);
         s->submitted += 1;

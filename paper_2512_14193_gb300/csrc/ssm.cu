@@ -198,6 +198,9 @@ Batch* take_cached(const std::vector<long>& key) {
 }
 
 void give_cached(Batch* b) {
+    // an idle batch keeps no FP64 digit workspaces (up to a GB per point)
+    for (bm_ctx* c : b->h)
+        if (c && c->d_dgw) opt_release(c, 1);
     std::lock_guard<std::mutex> lock(g_cache_mu);
     for (size_t i = 0; i < g_cache.size(); ++i)
         if (g_cache[i]->key == b->key) {  // keep the newer batch of a shape
@@ -215,6 +218,7 @@ void give_cached(Batch* b) {
 bm_status factor_batch(Batch& bt, int B) {
     bm_ctx* c0 = bt.h[0];
     const int N = c0->N;
+    for (int b = 0; b < B; ++b) opt_reserve(bt.h[b]);
     // the pivot / timeout words of every point, cleared ahead of everything that may set them
     for (int b = 0; b < B; ++b) {
         SSM_CUDA(cudaMemsetAsync(bt.h[b]->d_info, 0, 2 * sizeof(int), bt.s0));
@@ -244,7 +248,6 @@ bm_status factor_batch(Batch& bt, int B) {
     } else {
         for (int b = 0; b < B; ++b) {
             bm_ctx* c = bt.h[b];
-            dg_reserve(c);
             if (c->form == BM_MIXED) {
                 BM_TRY(schur_z64(c, c->stream));
             } else if (c->prec == BM_FP64) {
