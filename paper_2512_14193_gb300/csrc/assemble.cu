@@ -532,7 +532,7 @@ __global__ void pack_rowmajor_kernel(const double2* __restrict__ M, long ldm, in
         const int r = r0 + q;
         if (r >= rows) continue;
         // lanes 0-15: the hi parts of entries 2 l and 2 l + 1, lanes 16-31: the lo parts
-        const TcRowScale sc(-TC_E_DGE - e[r]);
+        const TcExpScale sc(-TC_E_DGE - e[r]);
         const int l = 2 * (tx & 15);
         __half2 hr, lr, hi, li;
         tc_split(sc(t[l][q].x), hr.x, lr.x);

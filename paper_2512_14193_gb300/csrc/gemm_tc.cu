@@ -531,7 +531,9 @@ __global__ void __launch_bounds__(UPD_THREADS, 1)
             const long row = (long)tm * BM + qw * 32 + lane;
             const int col0 = tn * BN + cg * UPD_COLS;
             const int nc = row < m ? min(UPD_COLS, n - col0) : 0;  // columns of this thread inside C
-            const int er = sc.e0 + (row < m ? __ldg(sc.eA + row) : 0);
+            // minus the row's factor; it and the columns' are normal numbers (TcRowScale), and a product times the
+            // first is about L21's entry times 2^15
+            const float rf = -tc_pow2(row < m ? __ldg(sc.eA + row) : 0);
             float* pr = Cr + row + (long)col0 * ldc;
             float* pi = Ci + row + (long)col0 * ldc;
             const int ld = (int)ldc;  // (32 columns of it fit an int)
@@ -559,10 +561,9 @@ __global__ void __launch_bounds__(UPD_THREADS, 1)
                 tmem_ld8x2(D + c0, D + BN + c0, vr, vi);
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
-                    const int e = er + (col0 + c0 + q < n ? __ldg(sc.eB + col0 + c0 + q) : 0);
-                    const float f = -tc_pow2(e >> 1), g = tc_pow2(e - (e >> 1));
-                    cr[c0 + q] += vr[q] * f * g;
-                    ci[c0 + q] += vi[q] * f * g;
+                    const float cf = tc_pow2(col0 + c0 + q < n ? __ldg(sc.eB + col0 + c0 + q) : 0);
+                    cr[c0 + q] = fmaf(vr[q] * rf, cf, cr[c0 + q]);
+                    ci[c0 + q] = fmaf(vi[q] * rf, cf, ci[c0 + q]);
                 }
             }
             fence_before();

@@ -413,10 +413,6 @@ __global__ void __launch_bounds__(RT, 2) lu_trsm_kernel(C32 F, int J, int db, in
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     }
     piv_s[tid] = t.piv[tid];
-    {
-        const int d = packs.re != nullptr ? inner_exponent(packs.re[J + tid], packs.re[J]) : 0;
-        w_s[tid] = tc_pow2(rows ? d : -d);
-    }
     static_assert(RT == B, "a thread per pivot, row and K index");
     if (rows) {
         const int r = lane;
@@ -448,6 +444,10 @@ __global__ void __launch_bounds__(RT, 2) lu_trsm_kernel(C32 F, int J, int db, in
             Xr[tid * XP + c] = vr;
             Xi[tid * XP + c] = vi;
         }
+    }
+    {
+        const int d = packs.re != nullptr ? inner_exponent(packs.re[J + tid], packs.re[J]) : 0;
+        w_s[tid] = tc_pow2(rows ? d : -d);
     }
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     __syncthreads();

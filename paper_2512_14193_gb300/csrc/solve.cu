@@ -34,8 +34,8 @@ __device__ __forceinline__ void atomic_max_pos(double* p, double v) {
     atomicMax(reinterpret_cast<unsigned long long*>(p), (unsigned long long)__double_as_longlong(v));
 }
 
-// per column: eta_c = max|R| / (normA max|X| + max|B|), 1e300 where that or an entry of R or X is not finite
-// (the maxima alone would drop a NaN); out[0] = max_c eta_c, out[1] = 1 if any non-finite value was seen in B
+// per column: eta_c = max|R| / (normA max|X| + max|B|), 1e300 where that is not finite or an entry of R or X is
+// a NaN (the maxima alone would drop it); out[0] = max_c eta_c, out[1] = 1 if any non-finite value was seen in B
 // (the input check)
 __global__ void eta_kernel(const double2* __restrict__ R, const double2* __restrict__ X,
                            const double2* __restrict__ B, long ld, int nsys, const double* __restrict__ normA,
@@ -51,9 +51,10 @@ __global__ void eta_kernel(const double2* __restrict__ R, const double2* __restr
         double2 bv = B[o];
         if (!isfinite(bv.x) || !isfinite(bv.y)) bad = true;
         double2 rv = R[o], xv = X[o];
-        if (!isfinite(rv.x) || !isfinite(rv.y) || !isfinite(xv.x) || !isfinite(xv.y)) lost = true;
-        rf = fmaxf(rf, hypotf((float)rv.x, (float)rv.y));
-        xf = fmaxf(xf, hypotf((float)xv.x, (float)xv.y));
+        const float rm = hypotf((float)rv.x, (float)rv.y), xm = hypotf((float)xv.x, (float)xv.y);
+        lost = lost || rm != rm || xm != xm;
+        rf = fmaxf(rf, rm);
+        xf = fmaxf(xf, xm);
         bf = fmaxf(bf, hypotf((float)bv.x, (float)bv.y));
     }
     r = rf;

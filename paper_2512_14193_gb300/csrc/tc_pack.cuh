@@ -8,21 +8,23 @@
 // 2^e, e clamped to the normal range
 __device__ __forceinline__ float tc_pow2(int e) { return __int_as_float((min(max(e, -126), 127) + 127) << 23); }
 
-// The scale 2^(15 - ex) of a row whose largest |Re| or |Im| is mx < 2^ex: exact factors f g (one may not reach).
-// Zero and non-finite rows take ex = 0 (infinities and NaN stay what they are).
+// The scale 2^(15 - ex) of a row whose largest |Re| or |Im| is mx < 2^ex.  Zero and non-finite rows take ex = 0
+// (infinities and NaN stay what they are); ex stops at -111, so that the scale and its inverse are normal numbers
+// (a row below 2^-112 still keeps its 22 bits down to FP32's own limit).
 struct TcRowScale {
-    float f, g;
+    float f;
     int ex;
     __device__ __forceinline__ explicit TcRowScale(float mx) {
         ex = 0;
-        if (mx > 0.f && mx < __int_as_float(0x7f800000)) ex = max((__float_as_int(mx) >> 23) - 126, -125);
-        set(15 - ex);
+        if (mx > 0.f && mx < __int_as_float(0x7f800000)) ex = max((__float_as_int(mx) >> 23) - 126, -111);
+        f = tc_pow2(15 - ex);
     }
-    __device__ __forceinline__ explicit TcRowScale(int shift) : ex(0) { set(shift); }
-    __device__ __forceinline__ void set(int e) {
-        f = tc_pow2(e >> 1);
-        g = tc_pow2(e - (e >> 1));
-    }
+    __device__ __forceinline__ float operator()(float v) const { return v * f; }
+};
+// 2^e for any e, as exact factors f g (one may not reach)
+struct TcExpScale {
+    float f, g;
+    __device__ __forceinline__ explicit TcExpScale(int e) : f(tc_pow2(e >> 1)), g(tc_pow2(e - (e >> 1))) {}
     __device__ __forceinline__ float operator()(float v) const { return v * f * g; }
 };
 
