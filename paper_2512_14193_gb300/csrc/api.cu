@@ -81,9 +81,10 @@ bm_status ctx_alloc(bm_ctx* c, void** p, size_t bytes) {
         return pool ? cudaMallocFromPoolAsync(p, bytes, pool, c->stream) : cudaMallocAsync(p, bytes, c->stream);
     };
     cudaError_t e = get();
-    if (e != cudaSuccess && (c->d_dgw || c->d_fd)) {
+    if (e != cudaSuccess) {  // no memory: optional workspaces go, this handle's and the idle contour batches'
         cudaGetLastError();
         opt_release(c, ~(size_t)0);
+        ssm_yield_optional(c->device);
         e = get();
     }
     if (e != cudaSuccess) {

@@ -206,6 +206,7 @@ bm_status gemm_z64_dg(cudaStream_t s, void* work, int num_sms, int m, int n, int
 // complement of the FP64 precision into d_F64
 void opt_reserve(bm_ctx* c);
 void opt_release(bm_ctx* c, size_t bytes);
+void ssm_yield_optional(int device);  // ssm.cu
 bm_status schur_z64(bm_ctx* c, cudaStream_t s);
 // api.cu: assembly in two halves (the batched contour solver assembles many handles at once)
 bm_status assemble_impl(bm_ctx* c, const bm_curve* curve, int N, bm_c64 k_out, bm_c64 k_in, bm_formulation form,

@@ -198,9 +198,6 @@ Batch* take_cached(const std::vector<long>& key) {
 }
 
 void give_cached(Batch* b) {
-    // an idle batch keeps no FP64 digit workspaces (up to a GB per point)
-    for (bm_ctx* c : b->h)
-        if (c && c->d_dgw) opt_release(c, 1);
     std::lock_guard<std::mutex> lock(g_cache_mu);
     for (size_t i = 0; i < g_cache.size(); ++i)
         if (g_cache[i]->key == b->key) {  // keep the newer batch of a shape
@@ -576,6 +573,19 @@ extern "C" bm_status bm_ssm(int device, const bm_curve* curve, int N, bm_formula
         for (int q = 0; q < 3; ++q) info->tune_ms[q] = tune[q] != 0.0 ? tune[q] : bt.tune[q];
     }
     return BM_OK;
+}
+
+// Idle batches of a device give their optional workspaces back (another handle's allocation found no memory).
+void ssm_yield_optional(int device) {
+    std::lock_guard<std::mutex> lock(g_cache_mu);
+    for (Batch* b : g_cache) {
+        if (b->key[0] != device) continue;
+        for (bm_ctx* c : b->h)
+            if (c) {
+                opt_release(c, ~(size_t)0);
+                cudaStreamSynchronize(c->stream);  // (the releases are ordered on it)
+            }
+    }
 }
 
 extern "C" bm_status bm_ssm_release(int device) {
