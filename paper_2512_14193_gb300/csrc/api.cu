@@ -236,7 +236,6 @@ void free_problem(bm_ctx* c) {
     }
     c->assembled = c->factored = c->singular = false;
     c->tm_ok = false;
-    c->tc_skinny = false;
 }
 
 bool finite_c(bm_c64 z) { return std::isfinite(z.re) && std::isfinite(z.im); }
@@ -434,7 +433,7 @@ extern "C" bm_status bm_enqueue_probe(bm_ctx* c, int which, int reps) {
         drop_slot(c->g_factor);
         for (int r = 0; r < reps; ++r) {
             if (c->prec == BM_FP64) {
-                BM_CUDA_TRY(gemm_z64(s, c->N, c->N, 2 * c->N, -1.0, Z64{c->d_Mbot, c->ldbot}, false,
+                BM_CUDA_TRY(gemm_z64(s, c->N, c->N, 2 * c->N, -1.0, Z64{c->d_Mbot, c->ldbot},
                                      Z64{c->d_Mtop, c->ldtop}, 0.0, Z64{c->d_F64, c->ldF}));
             } else {
                 BM_CUDA_TRY(gemm_tc(s, c->tm_schur[0], c->tm_schur[1], c->tm_schur[2], c->tm_schur[3], c->d_F32r,
@@ -799,7 +798,6 @@ bm_status assemble_post(bm_ctx* c, bool run_assembly_kernel, bool wait) {
             BM_TRY(tc_make_map(c->tm_schur[3], c->d_Bp_i, N, 2L * N, p.ldk_schur, TC_BN));
             BM_TRY(tc_make_map(c->tm_skinny[0], c->d_Cp_r, 2L * N, N, p.ldk_c, TC_BM));
             BM_TRY(tc_make_map(c->tm_skinny[1], c->d_Cp_i, 2L * N, N, p.ldk_c, TC_BM));
-            c->tc_skinny = true;
         }
         if (nd > 0) {
             const long rows0 = 2L * N, k0 = (form == BM_MIXED) ? N : 2L * N;
@@ -864,7 +862,7 @@ bm_status schur_z64(bm_ctx* c, cudaStream_t s) {
     const size_t b = dg_bytes(N, N, 2 * N, c->num_sms);
     if (b == 0 || b > c->dgw_bytes) {
         BM_PROF(c, "cgemm_simt_kernel<Z64> (Schur complement)");
-        BM_CUDA_TRY(gemm_z64(s, N, N, 2 * N, -1.0, A, false, B, 0.0, F));
+        BM_CUDA_TRY(gemm_z64(s, N, N, 2 * N, -1.0, A, B, 0.0, F));
         return BM_OK;
     }
     BM_PROF(c, "resid_tc_kernel (Schur complement)");
@@ -1095,7 +1093,7 @@ bm_status make_ws(bm_ctx* c, int nrhs) {
         if (wsz) BM_TRY(alloc_t(c, &c->d_rtw, wsz * 8));
         c->rtw_elems = wsz;
     }
-    if (c->tc_skinny) {
+    if (c->prec != BM_FP64 && c->form == BM_MIXED) {
         const int N = c->N;
         BM_TRY(alloc_t(c, &c->d_Bx1r, (size_t)w * c->ldk_schur * 2));
         BM_TRY(alloc_t(c, &c->d_Bx1i, (size_t)w * c->ldk_schur * 2));

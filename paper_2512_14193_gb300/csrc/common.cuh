@@ -338,7 +338,6 @@ struct bm_ctx {
     __half* d_Cp_r = nullptr;  // [M13; M23] rows, K = N (2N rows; exponents d_dge[0]): A operand of the skinny
     __half* d_Cp_i = nullptr;  //   products [M13; M23] z of the mixed correction and residual update
     long ldk_c = 0;
-    float* d_O32r = nullptr;  // ordinary: FP32 copy of A is the LU buffer (d_F32*)
 
     // solve workspace (sized for the largest nrhs seen)
     int ws_nrhs = 0;
@@ -390,7 +389,6 @@ struct bm_ctx {
     // skinny products: [0,1] [M13; M23] pack, [2,3] B pack of [W1; W2], [4,5] B pack of z3
     alignas(64) unsigned char tm_skinny[6][128];
     bool tm_ok = false;
-    bool tc_skinny = false;  // mixed CF32: skinny products of the solve on the tensor cores
     int num_sms = 0;
 
     // panel launch configuration

@@ -1,16 +1,13 @@
-// Complex GEMM on the CUDA cores: C = beta C + alpha op(A) B for column-major views.
+// Complex GEMM on the CUDA cores: C = beta C + alpha A B for column-major views.
 //
-// FP64 (Z64, interleaved double2): the engine of the FP64 path (Schur complement
-// U33 = -[M31 M32][M13; M23] of Theorem thm:LU, LU trailing updates, the FP64 residual of
-// refinement).  GB300 executes FP64 on the CUDA cores only, so this kernel is bound by the FP64
+// FP64 (Z64, interleaved double2): the products of the FP64 path that are too small for digits (resid_tc.cu
+// gemm_z64_dg), or have no room for them: Schur complement, LU updates; with few columns (right-hand sides)
+// skinny_z64_kernel.  GB300 executes FP64 on the CUDA cores only, so this kernel is bound by the FP64
 // pipe; it keeps a 64 x BN tile per CTA (BN = 16, 32 or 64, whichever pads the column count
 // least) with 4 x BN/16 complex accumulators per thread staged through shared memory.
-// FP32 (C32, planar): skinny updates inside the LU panel and the FP32 correction solves.
-// Mixed (A and C FP64 storage, B FP32, FP32 arithmetic): the refinement residual update
-// r -= A d for a small correction d.
-//
-// op(A) = A (m x k view) or, with a_trans, A is given as its transpose stored column-major
-// (k x m view), i.e. row-major A - the layout of the tensor-core operand packs.
+// FP32 (C32, planar): updates inside the LU panels of the pivot search.
+// Mixed (A hi parts of split planes, C FP64, B FP32, FP32 arithmetic): the ordinary system's refinement
+// residual update r -= A d for a small correction d.
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -24,7 +21,6 @@ constexpr int BK = 16;
 template <class R> BM_HD cplx_t<R> conv(double2 v);
 template <class R> BM_HD cplx_t<R> conv(float2 v);
 template <> BM_HD double2 conv<double>(double2 v) { return v; }
-template <> BM_HD float2 conv<float>(double2 v) { return make_float2((float)v.x, (float)v.y); }
 template <> BM_HD float2 conv<float>(float2 v) { return v; }
 
 template <class VC> BM_HD typename VC::cv from_acc(double2 v) {
@@ -41,7 +37,7 @@ template <class VC> BM_HD typename VC::cv from_acc(float2 v) {
 }
 
 // VA, VB, VC: storage views of A, B, C; R: arithmetic precision
-template <class VA, class VB, class VC, class R, bool AT, int BM, int BN>
+template <class VA, class VB, class VC, class R, int BM, int BN>
 __global__ void __launch_bounds__(256) cgemm_simt_kernel(int m, int n, int k, VA A, VB B, VC C, R alpha, R beta,
                                                          const int* stop) {
     using CV = cplx_t<R>;
@@ -63,18 +59,11 @@ __global__ void __launch_bounds__(256) cgemm_simt_kernel(int m, int n, int k, VA
     for (int k0 = 0; k0 < k; k0 += BK) {
 #pragma unroll
         for (int e = t; e < BM * BK; e += 256) {
-            int ii, kk;
-            if (AT) {
-                kk = e % BK;
-                ii = e / BK;
-            } else {
-                ii = e % BM;
-                kk = e / BM;
-            }
+            const int ii = e % BM, kk = e / BM;
             long gi = i0 + ii;
             int gk = k0 + kk;
             CV v = czero<R>();
-            if (gi < m && gk < k) v = conv<R>(AT ? A.get(gk, gi) : A.get(gi, gk));
+            if (gi < m && gk < k) v = conv<R>(A.get(gi, gk));
             As[kk][ii] = v;
         }
 #pragma unroll
@@ -135,7 +124,7 @@ __global__ void __launch_bounds__(256) cgemm_simt_kernel(int m, int n, int k, VA
     }
 }
 
-template <class VA, class VB, class VC, class R, bool AT>
+template <class VA, class VB, class VC, class R>
 cudaError_t launch_impl(cudaStream_t s, int m, int n, int k, VA A, VB B, VC C, R alpha, R beta,
                         const int* stop = nullptr) {
     if (m <= 0 || n <= 0) return cudaSuccess;
@@ -146,8 +135,8 @@ cudaError_t launch_impl(cudaStream_t s, int m, int n, int k, VA A, VB B, VC C, R
     // once; 32-row tiles when 64-row ones would leave SMs idle.
     if (n > 32 && n <= 80) {
         if ((long)ceil_div(m, 64) >= 2 * 152)
-            return go(cgemm_simt_kernel<VA, VB, VC, R, AT, 64, 80>, dim3(ceil_div(m, 64), 1));
-        return go(cgemm_simt_kernel<VA, VB, VC, R, AT, 32, 80>, dim3(ceil_div(m, 32), 1));
+            return go(cgemm_simt_kernel<VA, VB, VC, R, 64, 80>, dim3(ceil_div(m, 64), 1));
+        return go(cgemm_simt_kernel<VA, VB, VC, R, 32, 80>, dim3(ceil_div(m, 32), 1));
     }
     // FP64 products too small to fill the GPU with 64-row tiles (the FP64 pipe gives each SM only
     // ~8 GFLOP/s, so idle SMs cost directly): 32 x 16 tiles
@@ -162,7 +151,7 @@ cudaError_t launch_impl(cudaStream_t s, int m, int n, int k, VA A, VB B, VC C, R
                 sms = 1;
         }
         if ((long)ceil_div(m, 64) * ceil_div(n, 64) < sms)
-            return go(cgemm_simt_kernel<VA, VB, VC, R, AT, 32, 16>, dim3(ceil_div(m, 32), ceil_div(n, 16)));
+            return go(cgemm_simt_kernel<VA, VB, VC, R, 32, 16>, dim3(ceil_div(m, 32), ceil_div(n, 16)));
     }
     // otherwise the column tile with the least padding (ties go to the wider tile)
     int bn = 64;
@@ -174,9 +163,9 @@ cudaError_t launch_impl(cudaStream_t s, int m, int n, int k, VA A, VB B, VC C, R
             bn = cand;
         }
     }
-    if (bn == 16) return go(cgemm_simt_kernel<VA, VB, VC, R, AT, 64, 16>, dim3(ceil_div(m, 64), ceil_div(n, 16)));
-    if (bn == 32) return go(cgemm_simt_kernel<VA, VB, VC, R, AT, 64, 32>, dim3(ceil_div(m, 64), ceil_div(n, 32)));
-    return go(cgemm_simt_kernel<VA, VB, VC, R, AT, 64, 64>, dim3(ceil_div(m, 64), ceil_div(n, 64)));
+    if (bn == 16) return go(cgemm_simt_kernel<VA, VB, VC, R, 64, 16>, dim3(ceil_div(m, 64), ceil_div(n, 16)));
+    if (bn == 32) return go(cgemm_simt_kernel<VA, VB, VC, R, 64, 32>, dim3(ceil_div(m, 64), ceil_div(n, 32)));
+    return go(cgemm_simt_kernel<VA, VB, VC, R, 64, 64>, dim3(ceil_div(m, 64), ceil_div(n, 64)));
 }
 
 // FP64 products with few columns (right-hand sides): C = beta C + alpha A B.  The tiles of the kernel above
@@ -287,7 +276,7 @@ cudaError_t launch_skinny_z64(cudaStream_t s, dim3 grid, int m, int n, int k, do
 cudaError_t gemm_z64_skinny(cudaStream_t s, int num_sms, int m, int n, int k, double alpha, Z64 A, Z64 B, double beta,
                             Z64 C) {
     if (m <= 0 || n <= 0) return cudaSuccess;
-    if (k <= 0) return gemm_z64(s, m, n, k, alpha, A, false, B, beta, C);
+    if (k <= 0) return gemm_z64(s, m, n, k, alpha, A, B, beta, C);
     const int t = ceil_div(n, 9), nc = ceil_div(n, t), rt = ceil_div(m, 32);
     const int S = (int)std::max(1L, std::min(std::min(8L, (long)ceil_div(k, SK_K)), (long)ceil_div(2L * num_sms, (long)rt * t)));
     auto go = [&](auto w) {
@@ -307,28 +296,19 @@ cudaError_t gemm_z64_skinny(cudaStream_t s, int num_sms, int m, int n, int k, do
     }
 }
 
-cudaError_t gemm_z64(cudaStream_t s, int m, int n, int k, double alpha, Z64 A, bool a_trans, Z64 B, double beta,
-                     Z64 C, const int* stop) {
+cudaError_t gemm_z64(cudaStream_t s, int m, int n, int k, double alpha, Z64 A, Z64 B, double beta, Z64 C,
+                     const int* stop) {
     if (k <= 0 && beta == 1.0) return cudaSuccess;
-    return a_trans ? launch_impl<Z64, Z64, Z64, double, true>(s, m, n, k, A, B, C, alpha, beta, stop)
-                   : launch_impl<Z64, Z64, Z64, double, false>(s, m, n, k, A, B, C, alpha, beta, stop);
+    return launch_impl<Z64, Z64, Z64, double>(s, m, n, k, A, B, C, alpha, beta, stop);
 }
 
-cudaError_t gemm_c32(cudaStream_t s, int m, int n, int k, float alpha, C32 A, bool a_trans, C32 B, float beta,
-                     C32 C) {
+cudaError_t gemm_c32(cudaStream_t s, int m, int n, int k, float alpha, C32 A, C32 B, float beta, C32 C) {
     if (k <= 0 && beta == 1.0f) return cudaSuccess;
-    return a_trans ? launch_impl<C32, C32, C32, float, true>(s, m, n, k, A, B, C, alpha, beta)
-                   : launch_impl<C32, C32, C32, float, false>(s, m, n, k, A, B, C, alpha, beta);
-}
-
-// C (FP64) += alpha A (FP64 storage) B (FP32 planar), products and sums in FP32
-cudaError_t gemm_update_z64_c32(cudaStream_t s, int m, int n, int k, float alpha, Z64 A, C32 B, Z64 C) {
-    if (k <= 0) return cudaSuccess;
-    return launch_impl<Z64, C32, Z64, float, false>(s, m, n, k, A, B, C, alpha, 1.0f);
+    return launch_impl<C32, C32, C32, float>(s, m, n, k, A, B, C, alpha, beta);
 }
 
 // C (FP64) += alpha A_hi (FP32 hi parts of split planes) B (FP32 planar), FP32 arithmetic
 cudaError_t gemm_update_f4hi_c32(cudaStream_t s, int m, int n, int k, float alpha, F4Hi A, C32 B, Z64 C) {
     if (k <= 0) return cudaSuccess;
-    return launch_impl<F4Hi, C32, Z64, float, false>(s, m, n, k, A, B, C, alpha, 1.0f);
+    return launch_impl<F4Hi, C32, Z64, float>(s, m, n, k, A, B, C, alpha, 1.0f);
 }

@@ -22,12 +22,11 @@ cudaError_t launch_to_c32(cudaStream_t s, const double2* A, long lda, int m, int
 
 // gemm_simt.cu
 // (stop: the launch does nothing when this word is not zero)
-cudaError_t gemm_z64(cudaStream_t s, int m, int n, int k, double alpha, Z64 A, bool a_trans, Z64 B, double beta, Z64 C,
+cudaError_t gemm_z64(cudaStream_t s, int m, int n, int k, double alpha, Z64 A, Z64 B, double beta, Z64 C,
                      const int* stop = nullptr);
 cudaError_t gemm_z64_skinny(cudaStream_t s, int num_sms, int m, int n, int k, double alpha, Z64 A, Z64 B, double beta,
                             Z64 C);
-cudaError_t gemm_c32(cudaStream_t s, int m, int n, int k, float alpha, C32 A, bool a_trans, C32 B, float beta, C32 C);
-cudaError_t gemm_update_z64_c32(cudaStream_t s, int m, int n, int k, float alpha, Z64 A, C32 B, Z64 C);
+cudaError_t gemm_c32(cudaStream_t s, int m, int n, int k, float alpha, C32 A, C32 B, float beta, C32 C);
 
 // gemm_tc.cu (tensor maps are CUtensorMap, passed as opaque 128-byte blobs)
 bm_status tc_make_map(void* tmap, const __half* base, long rows, long K, long ldk, int box_rows);

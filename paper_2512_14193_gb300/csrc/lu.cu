@@ -341,10 +341,10 @@ __device__ __forceinline__ void load_block(CV* dst, const CV* __restrict__ src, 
 // (the reciprocals 1 / U_kk are formed before the sweep).
 // Entries outside the rb x rb leading block are zero.
 constexpr int TI_B = 64;
-template <class V, bool UPPER>
-__global__ void __launch_bounds__(256) tri_inv_kernel(V F, int n, typename V::cv* __restrict__ out, const int* fail) {
-    using CV = typename V::cv;
-    using Rl = typename V::real;
+template <bool UPPER>
+__global__ void __launch_bounds__(256) tri_inv_kernel(C32 F, int n, float2* __restrict__ out, const int* fail) {
+    using CV = float2;
+    using Rl = float;
     if (*fail != 0) return;  // the factorisation stopped (lu_fast.cu) and is continued first
     constexpr int B = TI_B, M = B * B / 256;
     extern __shared__ __align__(16) unsigned char sm[];
@@ -393,11 +393,10 @@ constexpr int TS_BM = 64;
 // G form of the factors (C32): every off-diagonal bs x bs tile F[it, b] (it != b) becomes
 // F[it, b] T_b with T_b = L_bb^{-1} below the diagonal and U_bb^{-1} above it.  One CTA per tile,
 // in place (each CTA reads its whole tile before writing it).  bs == TS_BM == 64.
-template <class V>
-__global__ void __launch_bounds__(256) g_form_kernel(V F, int n, const typename V::cv* __restrict__ dinvL,
-                                                     const typename V::cv* __restrict__ dinvU, const int* fail) {
-    using CV = typename V::cv;
-    using Rl = typename V::real;
+__global__ void __launch_bounds__(256) g_form_kernel(C32 F, int n, const float2* __restrict__ dinvL,
+                                                     const float2* __restrict__ dinvU, const int* fail) {
+    using CV = float2;
+    using Rl = float;
     constexpr int B = TS_BM;
     const int it = blockIdx.x, b = blockIdx.y;
     if (it == b || *fail != 0) return;
@@ -788,10 +787,10 @@ cudaError_t launch_swap_trsm(cudaStream_t s, V A, const SwapMap* map, int a0, in
 }
 
 cudaError_t gemm_any(cudaStream_t s, int m, int n, int k, Z64 A, Z64 B, Z64 C) {
-    return gemm_z64(s, m, n, k, -1.0, A, false, B, 1.0, C);
+    return gemm_z64(s, m, n, k, -1.0, A, B, 1.0, C);
 }
 cudaError_t gemm_any(cudaStream_t s, int m, int n, int k, C32 A, C32 B, C32 C) {
-    return gemm_c32(s, m, n, k, -1.0f, A, false, B, 1.0f, C);
+    return gemm_c32(s, m, n, k, -1.0f, A, B, 1.0f, C);
 }
 
 // Exponents of the rows of the factored matrix for the inner scale of its updates: the ordinary system's, whose
@@ -799,42 +798,33 @@ cudaError_t gemm_any(cudaStream_t s, int m, int n, int k, C32 A, C32 B, C32 C) {
 const int* row_exponents(const bm_ctx* c) { return c->form == BM_ORDINARY ? c->d_dge[0] : nullptr; }
 
 // What the solves need besides the factors: the inverted diagonal blocks and (FP32) the G form.
-template <class V>
-bm_status finish_t(bm_ctx* c, V F, cudaStream_t s) {
-    const int n = c->n;
+bm_status finish_t(bm_ctx* c, Z64 F, cudaStream_t s) {
+    BM_PROF(c, "tri_inv16_kernel");
+    tri_inv16_kernel<<<dim3(ceil_div(ceil_div(c->n, FZ_B), 2), 2), 32, 0, s>>>(
+        F, c->n, reinterpret_cast<double2*>(c->d_dinvL), reinterpret_cast<double2*>(c->d_dinvU), c->d_info + 4);
+    LU_CUDA(cudaGetLastError());
+    return BM_OK;
+}
+bm_status finish_t(bm_ctx* c, C32 F, cudaStream_t s) {
+    const int n = c->n, nblk = ceil_div(n, TI_B);
     const int* const fail = c->d_info + 4;
-    using CV = typename V::cv;
-    if constexpr (std::is_same<V, Z64>::value) {
+    float2* const dinvL = reinterpret_cast<float2*>(c->d_dinvL);
+    float2* const dinvU = reinterpret_cast<float2*>(c->d_dinvU);
+    static_assert(TI_B == TS_BM, "one block size for the inverses and the G form");
+    constexpr int smem = (TI_B * TI_B + 3 * TI_B) * (int)sizeof(float2), gsm = 2 * TS_BM * TS_BM * (int)sizeof(float2);
+    LU_CUDA(cudaFuncSetAttribute(tri_inv_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    LU_CUDA(cudaFuncSetAttribute(tri_inv_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    {
         BM_PROF(c, "tri_inv_kernel");
-        tri_inv16_kernel<<<dim3(ceil_div(ceil_div(n, FZ_B), 2), 2), 32, 0, s>>>(
-            F, n, reinterpret_cast<double2*>(c->d_dinvL), reinterpret_cast<double2*>(c->d_dinvU), fail);
-        LU_CUDA(cudaGetLastError());
-        return BM_OK;
-    }
-    const int bs = c->bs_solve;
-    if (bs != TI_B || bs != TS_BM) {
-        bm_set_error("lu: the solve block size must be 64");
-        return BM_EINVAL;
-    }
-    const int nblk = ceil_div(n, bs);
-    size_t smem = ((size_t)bs * bs + 3 * (size_t)bs) * sizeof(typename V::cv);
-    if constexpr (std::is_same<V, C32>::value) {
-        LU_CUDA(cudaFuncSetAttribute(tri_inv_kernel<V, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        LU_CUDA(cudaFuncSetAttribute(tri_inv_kernel<V, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        BM_PROF(c, "tri_inv_kernel");
-        tri_inv_kernel<V, false><<<nblk, 256, smem, s>>>(F, n, reinterpret_cast<CV*>(c->d_dinvL), fail);
-        tri_inv_kernel<V, true><<<nblk, 256, smem, s>>>(F, n, reinterpret_cast<CV*>(c->d_dinvU), fail);
+        tri_inv_kernel<false><<<nblk, 256, smem, s>>>(F, n, dinvL, fail);
+        tri_inv_kernel<true><<<nblk, 256, smem, s>>>(F, n, dinvU, fail);
         LU_CUDA(cudaGetLastError());
     }
-    if constexpr (std::is_same<V, C32>::value) {
-        if (nblk > 1) {
-            BM_PROF(c, "g_form_kernel");
-            const size_t gsm = 2 * (size_t)TS_BM * TS_BM * sizeof(CV);
-            LU_CUDA(cudaFuncSetAttribute(g_form_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm));
-            g_form_kernel<V><<<dim3(nblk, nblk), 256, gsm, s>>>(F, n, reinterpret_cast<const CV*>(c->d_dinvL),
-                                                                reinterpret_cast<const CV*>(c->d_dinvU), fail);
-            LU_CUDA(cudaGetLastError());
-        }
+    if (nblk > 1) {
+        BM_PROF(c, "g_form_kernel");
+        LU_CUDA(cudaFuncSetAttribute(g_form_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, gsm));
+        g_form_kernel<<<dim3(nblk, nblk), 256, gsm, s>>>(F, n, dinvL, dinvU, fail);
+        LU_CUDA(cudaGetLastError());
     }
     return BM_OK;
 }
@@ -894,7 +884,7 @@ bm_status factor_fast(bm_ctx* c, C32 F) {
         LU_CUDA(cudaEventRecord(ev_join, s2));
         rest = true;
     }
-    BM_TRY(finish_t<C32>(c, F, s));
+    BM_TRY(finish_t(c, F, s));
     if (la) {  // join the handle's stream
         LU_CUDA(cudaEventRecord(ev_done, s));
         LU_CUDA(cudaStreamWaitEvent(c->stream, ev_done, 0));
@@ -914,10 +904,12 @@ RtShift inner_z(const bm_ctx* c, int J) {
 bm_status update_z(bm_ctx* c, Z64 F, int J, int c1, int e, const int* stop) {
     const int m = c->n - e, k = c1 - J;
     const size_t need = dg_bytes(m, m, k, c->num_sms);
-    if (need > 0 && need <= c->dgw_bytes)
+    const bool digits = need > 0 && need <= c->dgw_bytes;
+    BM_PROF(c, digits ? "resid_tc_kernel (trailing update)" : "cgemm_simt_kernel (trailing update)");
+    if (digits)
         return gemm_z64_dg(c->stream, c->d_dgw, c->num_sms, m, m, k, -1.0, F.sub(e, J), F.sub(J, e), F.sub(e, e), c->d_err,
                            nullptr, inner_z(c, J), stop);
-    LU_CUDA(gemm_z64(c->stream, m, m, k, -1.0, F.sub(e, J), false, F.sub(J, e), 1.0, F.sub(e, e), stop));
+    LU_CUDA(gemm_z64(c->stream, m, m, k, -1.0, F.sub(e, J), F.sub(J, e), 1.0, F.sub(e, e), stop));
     return BM_OK;
 }
 
@@ -939,7 +931,7 @@ bm_status factor_fast_z(bm_ctx* c, Z64 F) {
         for (int j = J; j < je; j += FZ_BLOCK) {
             const int db = std::min(FZ_BLOCK, n - j), e = j + db, mm = n - e;
             {
-                BM_PROF(c, "panel_kernel");  // (the profile keeps one name for the panels' elimination)
+                BM_PROF(c, "lu_diag_z_kernel");
                 LU_CUDA(launch_lu_diag_z(s, F, j, db, work, fail));
             }
             {
@@ -948,15 +940,14 @@ bm_status factor_fast_z(bm_ctx* c, Z64 F) {
             }
             if (mm == 0 || e >= je) continue;
             BM_PROF(c, "cgemm_simt_kernel (panel update)");
-            LU_CUDA(gemm_z64(s, mm, je - e, db, -1.0, F.sub(e, j), false, F.sub(j, e), 1.0, F.sub(e, e), fail));
+            LU_CUDA(gemm_z64(s, mm, je - e, db, -1.0, F.sub(e, j), F.sub(j, e), 1.0, F.sub(e, e), fail));
             if (je < n)
-                LU_CUDA(gemm_z64(s, je - e, n - je, db, -1.0, F.sub(e, j), false, F.sub(j, je), 1.0, F.sub(e, je), fail));
+                LU_CUDA(gemm_z64(s, je - e, n - je, db, -1.0, F.sub(e, j), F.sub(j, je), 1.0, F.sub(e, je), fail));
         }
         if (je == n) break;
-        BM_PROF(c, "cgemm_simt_kernel (trailing update)");
         BM_TRY(update_z(c, F, J, je, je, fail));
     }
-    return finish_t<Z64>(c, F, s);
+    return finish_t(c, F, s);
 }
 
 // The LU with the pivot search, from column J0 on (the columns before it are factored, their
@@ -1077,7 +1068,7 @@ bm_status factor_t(bm_ctx* c, V F, bool tc, int J0 = 0) {
         }
     }
     if (la) LU_CUDA(cudaStreamWaitEvent(s, ev_join, 0));
-    BM_TRY(finish_t<V>(c, F, s));
+    BM_TRY(finish_t(c, F, s));
     if (la) {  // join the handle's stream
         LU_CUDA(cudaEventRecord(ev_done, s));
         LU_CUDA(cudaStreamWaitEvent(c->stream, ev_done, 0));

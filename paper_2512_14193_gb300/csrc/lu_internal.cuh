@@ -171,16 +171,6 @@ __device__ __forceinline__ void warp_best(uint32_t& vbits, uint32_t& idx) {
     idx = __reduce_min_sync(0xffffffffu, vbits == vm ? idx : 0xffffffffu);
     vbits = vm;
 }
-// 1 / a by Smith's scaling, with IEEE reciprocals instead of divisions
-__device__ __forceinline__ float2 cinv_rcp(float2 a) {
-    if (fabsf(a.x) >= fabsf(a.y)) {
-        const float r = a.y * __frcp_rn(a.x), id = __frcp_rn(fmaf(a.y, r, a.x));
-        return make_float2(id, -r * id);
-    }
-    const float r = a.x * __frcp_rn(a.y), id = __frcp_rn(fmaf(a.x, r, a.y));
-    return make_float2(r * id, -id);
-}
-
 // 1 / a for a != 0: a is scaled by a power of two (exact) to |a|_inf in [1, 2), and
 // conj(a) / |a|^2 uses one hardware reciprocal refined by a Newton step (a few ulps, no overflow or
 // underflow for any finite a).
