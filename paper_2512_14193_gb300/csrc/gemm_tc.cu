@@ -293,7 +293,7 @@ __device__ __forceinline__ void cgemm_tc_body(const CUtensorMap& tmAr, const CUt
         const long col0 = (long)tn * BN;
         const int er = sc.e0 + (sc.eA != nullptr && row < m ? __ldg(sc.eA + row) : 0);
 #pragma unroll 1
-        for (int c0 = 0; c0 < BN; c0 += 16) {
+        for (int c0 = 0; c0 < BN && col0 + c0 < n; c0 += 16) {  // (few right-hand sides: few chunks)
             float vr[16], vi[16];
             tmem_ld16x2(Dr + lane_off + c0, Di + lane_off + c0, vr, vi);
 #pragma unroll

@@ -109,6 +109,8 @@ __global__ void __launch_bounds__(DT, 1) lu_diag_kernel(C32 F, int J, int db, fl
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (*reinterpret_cast<volatile int*>(fail) != 0) return;
     if (tid == 0) bad = 0;
+    const int be = (db + W - 1) & ~(W - 1);  // past it the block is the identity's, which needs no elimination
+    if (tid >= be && tid < B) inv_s[tid] = piv_s[tid] = make_float2(1.f, 0.f);
     {
         // lane = 8 rows x 4 columns: 32-byte sectors of the matrix, all 32 shared banks
         const int r = warp * 8 + (lane & 7), cs = lane >> 3;
@@ -126,8 +128,8 @@ __global__ void __launch_bounds__(DT, 1) lu_diag_kernel(C32 F, int J, int db, fl
     if (warp == 0) ok = diag16(Sr, Si, 0, inv_s, piv_s);
     __syncthreads();
 #pragma unroll 1
-    for (int c0 = 0; c0 + W < B; c0 += W) {
-        const int rest = B - c0 - W;
+    for (int c0 = 0; c0 + W < be; c0 += W) {
+        const int rest = be - c0 - W;
         if (tid < rest) {  // a row of L21
             float* pr = Sr + (c0 + W + tid) * PITCH + c0;
             float* pi = Si + (c0 + W + tid) * PITCH + c0;

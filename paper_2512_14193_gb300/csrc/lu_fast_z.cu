@@ -81,6 +81,8 @@ __global__ void __launch_bounds__(256, 1) lu_diag_z_kernel(Z64 F, int J, int db,
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (*reinterpret_cast<volatile int*>(fail) != 0) return;
     if (tid == 0) bad = 0;
+    const int be = (db + W - 1) & ~(W - 1);  // past it the block is the identity's, which needs no elimination
+    if (tid >= be && tid < B) inv_s[tid] = piv_s[tid] = make_double2(1.0, 0.0);
 #pragma unroll
     for (int q = 0; q < B / 8; ++q) {
         const int c = warp + 8 * q;
@@ -90,10 +92,10 @@ __global__ void __launch_bounds__(256, 1) lu_diag_z_kernel(Z64 F, int J, int db,
     __syncthreads();
     bool ok = true;
 #pragma unroll 1
-    for (int c0 = 0; c0 < B; c0 += W) {
+    for (int c0 = 0; c0 < be; c0 += W) {
         if (warp == 0) ok = diag8(S, c0, inv_s, piv_s) && ok;
         __syncthreads();
-        const int t0 = c0 + W, rest = B - t0;
+        const int t0 = c0 + W, rest = be - t0;
         if (warp == 0 && lane < rest) {  // a row below
             double2* row = S + (t0 + lane) * P + c0;
             double2 a[W];
