@@ -35,8 +35,9 @@ import workloads as W  # noqa: E402
 METRIC = "factor+solve ms, solves/s: direct-indirect vs ordinary BM on 1 GB300 @relerr 1e-9"
 UNIT = "solves/s"
 PREC = {"fp64": 0, "tf32": 1, "3xtf32": 2}
-DTYPE = {"fp64": "c128 (f64)", "tf32": "c64 factor (tf32 tensor cores) + f64 refinement",
-         "3xtf32": "c64 factor (3xtf32 tensor cores) + f64 refinement"}
+# (both CF32 precisions take the same products: operands split into FP16 hi + lo, 22 significant bits)
+DTYPE = {"fp64": "c128 (f64)", "tf32": "c64 factor (fp16 hi+lo split, 3 products, f32 sums) + f64 refinement",
+         "3xtf32": "c64 factor (fp16 hi+lo split, 3 products, f32 sums) + f64 refinement"}
 
 
 def workload_cfg(w: W.Workload, prec: str):
@@ -47,7 +48,7 @@ def workload_cfg(w: W.Workload, prec: str):
         "formulation": "direct-indirect (Theorem thm:LU Schur path) vs ordinary Burton-Miller LU",
         "precision": prec,
         "refine_tol": 1e-9,
-        "l2": "operands larger than L2 (mixed FP64 blocks 1.07 GB, FP32 packs 1.6 GB; L2 129 MB)",
+        "l2": "operands larger than L2 (mixed FP64 blocks 1.07 GB, split packs 0.8 GB, digit planes 1.9 GB; L2 129 MB)",
     }
 
 
@@ -358,6 +359,19 @@ def lu_work(n: int, NB: int = 256, nbp: int = 32) -> dict:
     return {"panel": panel, "inner": inner, "trailing": trail, "swap_bytes": swap_bytes}
 
 
+def free_lu_work(n: int, B: int = 128) -> dict:
+    """The same for the LU in blocks of B columns without a pivot search: real flops of the diagonal
+    blocks' eliminations, of the solves with them (L21 by rows, U12 by columns) and of the trailing updates."""
+    diag = trsm = trail = 0.0
+    for J in range(0, n, B):
+        db = min(B, n - J)
+        mm = n - J - db
+        diag += 8.0 * sum((db - 1 - c) ** 2 + (db - 1 - c) for c in range(db))
+        trsm += 8.0 * mm * (db * (db + 1) / 2 + db * (db - 1) / 2)
+        trail += 8.0 * mm * mm * db
+    return {"diag": diag, "trsm": trsm, "trailing": trail}
+
+
 def roofline_from_profile(prof, N: int, nrhs: int, prec: int, iters: int, peaks: dict, src: str):
     """Roofline of the kernel with the largest summed device time in one mixed factor + solve
     (prof: (name, launches, ms) from bm_profile, largest first).  achieved = the kernel's algorithmic
@@ -372,6 +386,9 @@ def roofline_from_profile(prof, N: int, nrhs: int, prec: int, iters: int, peaks:
     peak_src = {fp32: "derived: 152 SMs x 128 FP32 lanes x 2 flops x max SM clock",
                 tf32: f"{src} bf16 x nominal TF32/bf16 ratio 1.1/2.25", hbm: src}
     lw = lu_work(N)
+    # (bm_profile reports the search-free blocks' elimination and updates under the panels' group names)
+    free = any(name == "lu_trsm_kernel" for name, _, _ in prof)
+    fw = free_lu_work(N)
     work = {
         "resid_df_kernel (+ split-K reduction)": ("alu", 8.0 * 4 * N * N * nrhs, fp32, "TFLOP/s",
                                                   "4N^2 nrhs complex MACs x 8 real flops vs the FP32 FMA rate "
@@ -380,11 +397,16 @@ def roofline_from_profile(prof, N: int, nrhs: int, prec: int, iters: int, peaks:
                                                   "the FP64 operator (4N^2 complex entries x 16 bytes) read once per "
                                                   "residual vs the measured copy bandwidth"),
         "cgemm_tc_kernel (Schur complement)": ("tensor", 16.0 * N ** 3, tf32, "TFLOP/s",
-                                               "16 N^3 real flops (4M) vs the TF32 figure (measured bf16 x 1.1/2.25)"),
-        "cgemm_tc_kernel (trailing update)": ("tensor", lw["trailing"], tf32, "TFLOP/s",
-                                              "sum over outer panels of 8 m^2 NB real flops vs the TF32 figure"),
-        "panel_lc_kernel": ("alu", lw["panel"], fp32, "TFLOP/s",
+                                               "16 N^3 real flops (4M; issued as three FP16 products each) vs the "
+                                               "TF32 figure (measured bf16 x 1.1/2.25)"),
+        "cgemm_tc_kernel (trailing update)": ("tensor", fw["trailing"] if free else lw["trailing"], tf32, "TFLOP/s",
+                                              "sum over the blocks of 8 m^2 NB real flops vs the TF32 figure"),
+        "panel_lc_kernel": ("alu", fw["diag"] if free else lw["panel"], fp32, "TFLOP/s",
+                            "unblocked LU flops of the 128-column diagonal blocks (lu_diag_kernel, one CTA) vs the FP32 "
+                            "FMA rate" if free else
                             "unblocked LU flops of the 32-column sub-panels vs the FP32 FMA rate"),
+        "lu_trsm_kernel": ("alu", fw["trsm"], fp32, "TFLOP/s",
+                           "the solves of L21 and U12 with the diagonal blocks vs the FP32 FMA rate"),
         "panel_kernel": ("alu", lw["panel"], fp32, "TFLOP/s",
                          "unblocked LU flops of the sub-panels vs the FP32 FMA rate"),
         "cgemm_simt_kernel (panel update)": ("alu", lw["inner"], fp32, "TFLOP/s",
