@@ -52,7 +52,10 @@ typedef enum {
 typedef enum { BM_MIXED = 0, BM_ORDINARY = 1 } bm_formulation;
 
 /* Arithmetic of the factorisation.
- *  BM_FP64          : FP64 throughout (assembly, Schur GEMM, LU, solve).
+ *  BM_FP64          : FP64 accuracy throughout (assembly, Schur GEMM, LU, solve).  Large products (the Schur
+ *                     complement, trailing updates) are formed exactly from nine base-128 digits per operand on the
+ *                     tensor cores and rounded once, where the budget has room for the digits (bm_factor takes
+ *                     it, any other allocation may take it back); else by FP64 multiply-adds.
  *  BM_CF32_3XTF32_IR: FP64 assembly; Schur GEMM and LU trailing updates on the tensor cores (FP32
  *                     accumulation) from operands split hi/lo (11 + 11 significant bits, three products,
  *                     about FP32 accuracy), diagonal blocks or panels and triangular solves in FP32;
@@ -92,12 +95,13 @@ typedef struct {
  *  nb            : outer LU block size, a multiple of 32 in [32, 256] (0 = library default).  The CF32
  *     precisions' default factors blocks of 128 columns without a pivot search, checks every candidate
  *     against its pivot and continues with the search from the first block that needs an interchange
- *     (the same pivots); a block size or a panel setting below asks for the search from the start.
+ *     (the same pivots up to the rounding of the magnitudes compared), FP64's the same with 32; a block
+ *     size or a panel setting below asks for the search from the start.
  *  refine_residual: how refinement forms r = b - A x (bm_refine_residual):
  *     BM_RESID_TC_UPDATE (0, default): the first residual from exact integer products on the
  *        tensor cores - A (once, after assembly) and x split into seven base-128 digits per row /
  *        column scale, digit pairs multiplied in bf16 with exact FP32 sums over chunks of 256 and
- *        double-float sums across chunks (FP64-level accuracy, ~1e-15 of |A||x|); later ones
+ *        integer sums across chunks (FP64-level accuracy, ~1e-15 of |A||x|); later ones
  *        updated as r -= A d with the product in FP32 (d, the last correction, is small by then,
  *        so the update error stays far below refine_tol);
  *     BM_RESID_FP64_UPDATE (1): the first residual in FP64, later ones updated as above;
@@ -106,7 +110,7 @@ typedef struct {
  *        FP64 operand split into two FP32 parts, exact products, compensated sums: ~1e-12 of
  *        |A||x|), later ones updated as in mode 0;
  *     BM_RESID_TC_ALL (4): every residual from exact tensor-core digit products as in mode 0, with
- *        nine digits per operand (~2^-64 of the row and column scales).
+ *        nine digits per operand (~2^-61 of the row and column scales).
  *  The updated residuals of modes 0, 1 and 3 carry the FP32 product error of each update, so the
  *  backward error they track is reliable down to about 1e-12; refine_tol below 1e-12 needs
  *  BM_RESID_FP64_ALL or BM_RESID_TC_ALL (bm_assemble returns BM_EINVAL otherwise).
@@ -436,9 +440,9 @@ bm_status bm_enqueue_probe(bm_ctx* ctx, int which, int reps);
  * launched directly (no graph replay) and each launch bracketed by two events on the handle's
  * stream, and reports the launches grouped by kernel name: count and summed device time.  The
  * factors and X are those of a normal call; the times add up to the serial device time of the two
- * calls (kernels that a normal call overlaps are timed one after another here).  The FP32
- * factorisation's panel eliminations are one group, panel_lc_kernel, whether they ran with or
- * without the pivot search.
+ * calls (kernels that a normal call overlaps are timed one after another here).  Two groups of the
+ * FP32 factorisation hold what does one job with or without the pivot search: panel_lc_kernel
+ * (without: lu_diag_kernel) and cgemm_tc_kernel (trailing update) (cgemm_tc_upd_kernel).
  *  out: cap entries (may be NULL to query the count); *count receives the number of groups.
  * Errors: those of bm_factor and bm_solve. */
 typedef struct {

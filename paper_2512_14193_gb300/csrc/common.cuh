@@ -276,7 +276,7 @@ struct bm_ctx {
     void* d_dg[2] = {nullptr, nullptr};
     int* d_dge[2] = {nullptr, nullptr};
     long dg_ldk[2] = {0, 0};
-    int rt_nd = 7;            // digits per operand (8 for BM_RESID_TC_ALL)
+    int rt_nd = 7;            // digits per operand (9 for BM_RESID_TC_ALL, 0: no tensor-core residual)
     alignas(64) unsigned char tm_dg[2][128];
     // x digit planes for the two products (K ranges [2N, 3N) and [0, 2N) mixed; [0, 2N) ordinary),
     // their column exponents, and the split-K workspace of the tensor-core residual
@@ -316,11 +316,11 @@ struct bm_ctx {
     // inverted diagonal blocks of L and U (getrs), bs x bs each, n/bs blocks
     void* d_dinvL = nullptr;
     void* d_dinvU = nullptr;
-    int bs_solve = 64;
+    int bs_solve = 64;  // rows of an inverted diagonal block (FP64: 16)
 
     // tensor-core operand packs (tc_pack.cuh; planar, ldk halves a row) and the exponents of their rows that
     // are not the digit planes' d_dge
-    __half* d_Ap_r = nullptr;  // Schur A operand [M31 M32] (N rows, K = 2N; exponents d_dge[1])
+    __half* d_Ap_r = nullptr;  // Schur A operand [M31 M32] (N rows, K = 2N; exponents d_Ape)
     __half* d_Ap_i = nullptr;
     __half* d_Bp_r = nullptr;  // Schur B operand [M13; M23]^T rows (N rows, K = 2N; exponents d_Bpe)
     __half* d_Bp_i = nullptr;

@@ -390,8 +390,10 @@ __global__ void __launch_bounds__(128, 1)
 // loads the operands ahead across tiles, warp 1 issues into the two accumulators in turn, and sixteen warps
 // take a tile's C into registers (64 loads in flight per thread, a quarter of the columns each) while its
 // products run, then subtract and store while the next tile's do.  Against one CTA per tile with the C tile
-// staged through tensor memory by four warps, 8064 x 8064 (63 x 63 tiles): 477 -> 270 us (3.9 TB/s of C), one tile
-// alone 18.4 -> 12.7 us; the next tile prefetched into L2 makes 10 % of it.
+// staged through tensor memory by four warps, 8064 x 8064 (63 x 63 tiles): 477 -> 206 us (5.0 TB/s of C), one tile
+// alone 18.4 -> 11.6 us; the next tile prefetched into L2 makes 10 % of it.  An entry takes one product with its
+// row's factor and one multiply-add with its column's, which is uniform in the warp (a factor per entry from both
+// exponents: 10 % slower).
 constexpr int UPD_WARPS = 16, UPD_THREADS = 64 + 32 * UPD_WARPS;
 constexpr int UPD_COLS = BN / (UPD_WARPS / 4);  // columns per warp
 static_assert(UPD_COLS == 32, "a lane per column");

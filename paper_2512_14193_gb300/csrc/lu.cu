@@ -1,7 +1,10 @@
 // Dense complex LU with partial pivoting on the GPU (the N x N Schur complement U33 of
 // Theorem thm:LU, or the 2N x 2N ordinary matrix of Eq. dis_BM), and the triangular solves.
 //
-// Right-looking blocked LU with two block sizes:
+// By default blocks of columns are factored without a pivot search while partial pivoting keeps its pivots on the
+// diagonal (lu_fast.cu, lu_fast_z.cu: every candidate is checked); from the first block that needs an interchange
+// on, and where a block size or a panel setting asks for it, the search below factors.  Right-looking, with two
+// block sizes:
 //   for each big panel of NB columns (C32: 256, Z64: 64):
 //     for each sub-panel of nbp columns:
 //        panel kernel      : unblocked LU with partial pivoting of rows [j, n) x nbp columns on a
@@ -22,13 +25,13 @@
 // records the 1-based column in *info and skips the scaling, as LAPACK getrf does.
 //
 // Solves (getrs): Y = P B, then block forward substitution with the unit L and block back
-// substitution with U; the bs x bs diagonal blocks are inverted once after the factorisation so
-// that every step is a small matrix product.  For C32 the off-diagonal bs x bs tiles of each
+// substitution with U, each triangle one persistent launch whose items wait for the block rows they need
+// (trsv_flow_kernel, trsv_flow_z64_kernel).  The diagonal blocks (64 x 64, FP64: 16 x 16) are inverted once after
+// the factorisation so that every step is a small matrix product.  For C32 the off-diagonal tiles of each
 // block column are then multiplied by that column's inverted diagonal block (the "G form"), so
 // that a step is one product with no dependence on the inverse:
-//   forward:  Y[below b] -= (L[below b, b] L_bb^{-1}) Y_b,  then Z_b = L_bb^{-1} Y_b for all b at once
-//   backward: Z[above b] -= (U[above b, b] U_bb^{-1}) Z_b,  then X_b = U_bb^{-1} Z_b for all b at once
-// (the same sums as L_bb^{-1} Y_b formed inside every step, without recomputing it in each CTA).
+//   forward:  Y[below b] -= (L[below b, b] L_bb^{-1}) Y_b,  Z_b = L_bb^{-1} Y_b
+//   backward: Z[above b] -= (U[above b, b] U_bb^{-1}) Z_b,  X_b = U_bb^{-1} Z_b
 #include "lu_internal.cuh"
 
 #include <climits>

@@ -7,7 +7,8 @@
 // elimination forms is compared with its pivot, and the first block where one is larger (or a pivot
 // is zero or a NaN) stops the sequence: *fail = 2 (J + 1) + stage names the block, later kernels return
 // at once, and the host restores that block's columns and rows and continues from it with the pivot
-// search (factor_t in lu.cu).  So the pivots are always those of partial pivoting.
+// search (factor_t in lu.cu).  So the pivots are those of partial pivoting up to the rounding of the magnitudes
+// compared: below the diagonal block a candidate is formed again from its multiplier and pivot.
 //
 // Per block of FD_B = 128 columns at J:
 //   lu_diag_kernel  one CTA: LU of the diagonal block (stage 0 of the check)

@@ -4,7 +4,8 @@
 // sequence return, and the host restores the block and goes on from it with the search (lu_resume_enqueue).
 //
 // An SM does two FP64 multiply-adds a cycle, so a warp instruction costs 16 cycles of its pipe whatever the
-// number of active lanes: the diagonal block stays small (32 columns, ~20 us on one SM), the solves and the
+// number of active lanes: the diagonal block stays small (32 columns, 67 us on one SM, of which its FP64
+// instructions take a third: the elimination's chain is the rest), the solves and the
 // rest of the trailing matrix are spread over all SMs, and outer blocks of 128 columns are applied by the
 // tensor cores (gemm_z64_dg).
 #include "lu_internal.cuh"

@@ -17,9 +17,9 @@
 //     the hardware adds in;
 //   * after each chunk the level sums are added to two 64-bit integers per output, the upper levels and the
 //     lower ones, each weighted by its power of 128: nothing is rounded until the end, where the two are
-//     added in FP64 (pairs of FP32 per output, the first form, lose a bit or two past 2^-48 in every chunk:
-//     FP64 solutions at N = 1000 were off by 5e-14 instead of 7e-15).  The dropped pairs weigh below 2^-56
-//     (seven digits) and 2^-70.
+//     added in FP64 (pairs of FP32 per output, the form before, round near 2^-48 in every chunk: errors of FP64
+//     solutions were three times as large).  The dropped pairs of one term add up to below 2^-48 (seven
+//     digits) or 2^-62 (nine) of the row's and column's scales.
 // The x digit tiles sit one after another in shared memory and the levels' accumulators one after
 // another in tensor memory, so one MMA multiplies A digit d by all the x digits it pairs with and
 // lands each pair in its level.  Seven digits (32 right-hand sides per CTA): four MMAs of width
@@ -552,7 +552,7 @@ __device__ __forceinline__ unsigned bf16_pair(float a, float b) {
 // Digit planes of A: plane 2d + part holds digit d of the real (part 0) or imaginary (1) parts, K-major
 // ([row][ldk]); through a 32-row x 64-column shared tile so that both sides are coalesced, a lane taking two
 // columns and writing 4 bytes per plane.  Integer work bounded it when each digit was peeled off with its
-// carry and built bit by bit: N = 4096, both operators, 1.39 -> 0.65 ms (3.7 TB/s read and written).
+// carry and built bit by bit: N = 4096, both operators, 1.39 -> 0.65 ms (3.5 GB read and written: 5.3 TB/s).
 template <int ND>
 __global__ void __launch_bounds__(256) digits_a_kernel(const double2* __restrict__ A, long lda, int rows, int K,
                                                        const int* __restrict__ e, unsigned* __restrict__ D, long ldk,
@@ -840,10 +840,12 @@ cudaError_t gemm_rt(cudaStream_t s, const RtArgs* prods, int nprod, int n, doubl
 
 // ------------------------------------------------------------------------------------------------
 // FP64 products C += alpha A B (column-major, C initialised) from nine-digit products: the Schur
-// complement and the trailing updates of the FP64 precision.  Each row of A and column of B is good to
-// 2^-64 of its largest entry, ten bits past FP64's own rounding of that entry, and sums are kept in
-// double-float: the error against 64 bits is that of an FP64 product or below (N = 1000 Schur
-// complement 14.0 -> 0.9 ms; the FP64 pipe runs 304 multiply-adds a cycle on the whole chip).
+// complement and the trailing updates of the FP64 precision.  A product of two entries is good to about 2^-61 of
+// the scales of its row of A and column of B (the last digits, and the dropped pairs), its sum over K is exact and
+// rounded once.  The scales have to fit the entries that matter: the Schur complement's blocks are balanced
+// (balance_kernel), the LU's columns and rows scaled against each other (inner_exponent).  Solution errors against extended
+// precision over N = 256 .. 1024, four curves: 0.29 times those with FP64 multiply-adds (geometric mean; 0.64 at
+// most).  N = 1000 Schur complement 14.0 -> 0.9 ms; the FP64 pipe runs 304 multiply-adds a cycle on the whole chip.
 // The operands' digit planes are made per call in the workspace, in chunks of rows and columns when it
 // does not hold them all.
 // ------------------------------------------------------------------------------------------------
