@@ -53,9 +53,10 @@ typedef enum { BM_MIXED = 0, BM_ORDINARY = 1 } bm_formulation;
 
 /* Arithmetic of the factorisation.
  *  BM_FP64          : FP64 accuracy throughout (assembly, Schur GEMM, LU, solve).  Large products (the Schur
- *                     complement, trailing updates) are formed exactly from nine base-128 digits per operand on the
- *                     tensor cores and rounded once, where the budget has room for the digits (bm_factor takes
- *                     it, any other allocation may take it back); else by FP64 multiply-adds.
+ *                     complement, trailing updates) come from nine base-128 digits per operand on the tensor
+ *                     cores (to about 2^-61 of the row's and column's scales, summed exactly, rounded once)
+ *                     where the budget has room for the digits (bm_factor takes it, any other allocation may
+ *                     take it back), else from FP64 multiply-adds.
  *  BM_CF32_3XTF32_IR: FP64 assembly; Schur GEMM and LU trailing updates on the tensor cores (FP32
  *                     accumulation) from operands split hi/lo (11 + 11 significant bits, three products,
  *                     about FP32 accuracy), diagonal blocks or panels and triangular solves in FP32;
